@@ -301,3 +301,86 @@ def tolerance(case):
     else:
         K = case["C"] * case["k"] ** 2
     return {"rel": max(1.6e-5 if case["beta_a"] == 1 else 2e-6, 5e-9 * K)}
+
+
+# --------------------------------------------------------------------------------------------------------------
+# The same results in 64 bits
+# --------------------------------------------------------------------------------------------------------------
+def _group_means(x, beta):
+    """Mean magnitude of each run of ``beta`` elements of a row (a shorter last run has its own length)."""
+    G = -(-x.shape[1] // beta)
+    n = torch.full((G,), float(beta), dtype=torch.float64, device=x.device)
+    n[-1] = x.shape[1] - (G - 1) * beta
+    mag = torch.nn.functional.pad(x.abs(), (0, G * beta - x.shape[1]))
+    return mag.view(-1, G, beta).sum(2) / n
+
+
+def _spread(d, beta, K):
+    return d.repeat_interleave(beta, 1)[:, :K]
+
+
+def _binarized(x, beta, scales):
+    """delta (.) Sign(x), Sign(0) = +1; scales stored as bf16 are rounded as stored."""
+    x = x.double()
+    d = _group_means(x, beta)
+    if scales == "bf16":
+        d = d.bfloat16().double()
+    return torch.where(x < 0, -1.0, 1.0) * _spread(d, beta, x.shape[1])
+
+
+def _exact_linear(case, gen):
+    dims, out = [int(d) for d in case["dims"].split("-")], []
+    for K, N in zip(dims, dims[1:]):
+        x = _normal((case["M"], K), gen, DTYPES[case["x"]][0])
+        w = _normal((N, K), gen, scale=math.sqrt(2.0 / K))
+        out.append(_binarized(x, case["beta_a"], case["scales"]) @ _binarized(w, case["beta_w"], case["scales"]).t())
+    return out
+
+
+def _conv64(x, w, case, N):
+    """x NCHW in 64 bits, w the binarized filters [N, C kh kw]: the product [B Ho Wo, N], image by image."""
+    k, st = case["k"], case["stride"]
+    out = []
+    for img in x:
+        cols = torch.nn.functional.unfold(img[None], k, padding=k // 2, stride=st)[0].t()
+        out.append((cols if case["beta_a"] == 1 else _binarized(cols, case["beta_a"], case["scales"])) @ w.t())
+    return torch.cat(out)
+
+
+def _exact_conv(case, gen):
+    geom, M, K = _geometry(case)
+    B, C, H, W_, N = case["B"], case["C"], case["H"], case["W"], case["N"]
+    w = _binarized(_normal((N, K), gen, scale=math.sqrt(2.0 / K)), case["beta_w"], case["scales"])
+    if not case["chain"]:
+        return _conv64(_normal((B, C, H, W_), gen, DTYPES[case["x"]][0]).double(), w, case, N)
+    x = _normal((B, H, W_, C), gen, torch.bfloat16).double()
+    w2 = _binarized(_normal((N, N * 9), gen, scale=math.sqrt(2.0 / (N * 9))), case["beta_w"], case["scales"])
+    bn = [(torch.rand(N, generator=gen, device="cuda") + 0.5, _normal((N,), gen, scale=0.1)) for _ in range(2)]
+    ys = []
+    for wd, (scale, shift) in zip((w, w2), bn):                                # each layer's result is stored as bf16
+        y = _conv64(x.permute(0, 3, 1, 2), wd, case, N).relu() * scale.double() + shift.double()
+        x = y.bfloat16().double().view(B, H, W_, N)
+        ys.append(x)
+    return [ys[0], ys[1].view(M, N)]
+
+
+def _exact_train(case, gen):
+    M, K, N, beta = case["M"], case["K"], case["N"], case["beta"]
+    x, w = _normal((M, K), gen), _normal((N, K), gen, scale=math.sqrt(2.0 / K))
+    gw = _normal((N, K), gen, scale=1e-2).double()
+    C = _binarized(x, beta, case["scales"]) @ _binarized(w, beta, case["scales"]).t()
+    # the gradient of delta (.) Sign(w) with respect to w: through the group's mean, and straight through the sign
+    # where |w| <= 1
+    w = w.double()
+    sign, G = torch.where(w < 0, -1.0, 1.0), -(-K // beta)
+    n = torch.full((G,), float(beta), dtype=torch.float64, device=w.device)
+    n[-1] = K - (G - 1) * beta
+    dot = torch.nn.functional.pad(gw * sign, (0, G * beta - K)).view(N, G, beta).sum(2) / n
+    gx = sign * _spread(dot, beta, K) + torch.where(w.abs() <= 1, _spread(_group_means(w, beta), beta, K) * gw, 0.0)
+    return [C, _binarized(w, beta, "fp32").bfloat16().double(), gx]
+
+
+def exact(case, seed):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    return {"linear": _exact_linear, "conv": _exact_conv, "train": _exact_train}[case["kind"]](case, gen)
