@@ -100,7 +100,7 @@ inline bool workspace_ok(const void* ws, size_t have, size_t need) {
 // The integer-pipe contraction that fits the operands: matrix-vector shaped, sub-word segments, or tiled.
 cudaError_t popc_any(const PackedView& a, const PackedView& w, float* C, int64_t ldc, cudaStream_t stream) {
   if (gemv_popc_supported(a, w)) return launch_gemv_popc(a, w, C, ldc, stream);
-  return gemm_subword(a, w) ? launch_gemm_popc_sub(a, w, C, ldc, stream) : launch_gemm_popc(a, w, C, ldc, stream);
+  return gemm_popc_tile_supported(a, w) ? launch_gemm_popc_tile(a, w, C, ldc, stream) : launch_gemm_popc(a, w, C, ldc, stream);
 }
 
 hbmm_status gemm_checked(const hbmm_operand* A, const hbmm_operand* W, float* C, int64_t ldc,

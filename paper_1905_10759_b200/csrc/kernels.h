@@ -69,9 +69,12 @@ cudaError_t launch_partials_popc(const PackedView& A, const PackedView& W, int32
 bool gemv_popc_supported(const PackedView& A, const PackedView& W);
 cudaError_t launch_gemv_popc(const PackedView& A, const PackedView& W, float* C, int64_t ldc, cudaStream_t stream);
 
-// The same for sub-word segments (the finer grouping is 2, 4, 8 or 16 elements): masked popcounts inside a word.
+// The same in 32 x 32 warp tiles with the K range split between warps: segments of 2, 4, 8, 16 bits or 1, 2, 4, 8 words.
+bool gemm_popc_tile_supported(const PackedView& A, const PackedView& W);
+cudaError_t launch_gemm_popc_tile(const PackedView& A, const PackedView& W, float* C, int64_t ldc, cudaStream_t stream);
+
+// Integer partial sums of sub-word segments (the finer grouping is 2, 4, 8 or 16 elements).
 bool gemm_subword(const PackedView& A, const PackedView& W);
-cudaError_t launch_gemm_popc_sub(const PackedView& A, const PackedView& W, float* C, int64_t ldc, cudaStream_t stream);
 cudaError_t launch_partials_popc_sub(const PackedView& A, const PackedView& W, int32_t* D, cudaStream_t stream);
 
 // Packed x packed contraction on the legacy b1 tensor instruction (segment multiple of 128 bits).
