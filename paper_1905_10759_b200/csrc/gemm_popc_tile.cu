@@ -17,11 +17,13 @@
 // beta 16 28.5 -> 9.7 us, 82 x 536 x 3768 at beta 64 90 -> 9.2 us, 4050 x 280 x 4368 at beta 16 203 -> 104 us; on the
 // conv3_x matrix (50176 x 128 x 1152) beta 2 / 4 / 8 / 16 / 32 / 128: 1337 / 660 / 332 / 172 / 90 / 81 ->
 // 926 / 640 / 326 / 153 / 83 / 71 us.  Scalar fp32 instead of the paired instructions: 5 % slower.
-#include <cuda_bf16.h>
 #include "kernels.h"
+#include "popc_common.cuh"
 
 namespace hbmm {
 namespace {
+
+using namespace popc;
 
 constexpr int kWarps = 8;
 constexpr int kThreads = kWarps * 32;
@@ -49,11 +51,6 @@ struct Cfg {
   static constexpr int SMEM_WORDS = WARP_WORDS > TS * TS ? WARP_WORDS : TS * TS;   // ... which its partial sums reuse
 };
 
-__device__ __forceinline__ float load_scale(const void* s, int bf16, int64_t idx) {
-  if (bf16) return __uint_as_float(static_cast<uint32_t>(__ldg(reinterpret_cast<const unsigned short*>(s) + idx)) << 16);
-  return __ldg(reinterpret_cast<const float*>(s) + idx);
-}
-
 // The CW packed words of one row from word w0 on (rows are padded to a multiple of four words).
 template <int CW>
 __device__ __forceinline__ void load_words(const uint32_t* row, int64_t w0, int64_t ld, bool in, uint32_t (&v)[CW]) {
@@ -76,34 +73,6 @@ __device__ __forceinline__ void load_words(const uint32_t* row, int64_t w0, int6
   }
 }
 
-// The scales of SPC consecutive segments of one row from segment s0 on; 0 past the last group.  One group per segment
-// and fp32: 16-byte loads (s0 is a multiple of SPC, rows are 16-byte vectors); otherwise one load per segment.
-template <int SPC>
-__device__ __forceinline__ void load_scales(const void* s, int bf16, int64_t row_off, int64_t s0, int64_t r, int64_t G, bool in, float (&v)[SPC]) {
-#pragma unroll
-  for (int i = 0; i < SPC; i++) v[i] = 0.0f;
-  if (!in) return;
-  if (SPC >= 4 && r == 1 && !bf16) {
-#pragma unroll
-    for (int q = 0; q < SPC / 4; q++)
-      if (s0 + 4 * q < G) {
-        const float4 x = __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(s) + row_off + s0 + 4 * q));
-        v[(4 * q) % SPC] = x.x;
-        if (s0 + 4 * q + 1 < G) v[(4 * q + 1) % SPC] = x.y;
-        if (s0 + 4 * q + 2 < G) v[(4 * q + 2) % SPC] = x.z;
-        if (s0 + 4 * q + 3 < G) v[(4 * q + 3) % SPC] = x.w;
-      }
-    return;
-  }
-  int64_t g = s0, rem = 0;
-  if (r != 1) { g = s0 / r; rem = s0 - g * r; }
-#pragma unroll
-  for (int i = 0; i < SPC; i++) {
-    if (g < G) v[i] = load_scale(s, bf16, row_off + g);
-    if (++rem >= r) { rem = 0; g++; }
-  }
-}
-
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
   uint64_t v;
   asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
@@ -116,17 +85,6 @@ __device__ __forceinline__ void add_term(uint64_t& acc, uint32_t c0, uint32_t c1
   asm("add.rn.f32x2 %0, %0, %1;" : "+l"(f) : "l"(neg_bias));
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(s) : "l"(sa), "l"(sw));
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(s), "l"(f));
-}
-
-// Doubled counts of a word's segments p, p + PARTS, p + 2 PARTS, .. (PARTS = 8 / SEG) as the four bytes of a word: the
-// fields of the part are brought one bit above the bottom of their bytes by a rotation.
-template <int SEG>
-__device__ __forceinline__ uint32_t doubled_counts(uint32_t x, int p) {
-  const uint32_t c2 = x - ((x >> 1) & 0x55555555u);
-  if constexpr (SEG == 2) return __funnelshift_r(c2, c2, 2 * p + 31) & 0x06060606u;
-  const uint32_t c4 = (c2 & 0x33333333u) + ((c2 >> 2) & 0x33333333u);
-  if constexpr (SEG == 4) return __funnelshift_r(c4, c4, 4 * p + 31) & 0x0E0E0E0Eu;
-  return ((c4 << 1) & 0x0E0E0E0Eu) + ((c4 >> 3) & 0x0E0E0E0Eu);
 }
 
 template <int SEG>

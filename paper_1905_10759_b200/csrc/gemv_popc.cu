@@ -2,17 +2,20 @@
 // shaped product that is bound by reading the packed weights once (Section 4.2: K / 8 bytes of sign bits plus
 // 4 K / beta bytes of scales per weight row) and by launch latency, not by arithmetic.
 //
-// One warp per weight row.  The activation rows (bits and the per-segment scales) sit in shared memory; a lane
+// One warp per weight row.  For groups of whole words the activation rows (bits and the per-segment scales) sit in shared
+// memory (groups shorter than a word: the second kernel below); a lane
 // walks the weight row in 16-byte pieces (four K-words, a whole number of segments), forms per segment the
 // signed +-1 dot D = n_valid - 2 popc(a ^ w) in integers (Eq. 7) and adds (deltaA deltaW) D in fp32; the lanes'
 // partial sums meet in a shuffle tree.  Segments of one, two or four K-words (beta 32, 64, 128 and their
 // mixes); K any length (rows are padded with zero words to a multiple of four, pad bits are zero in both
 // operands and the tail segment counts only its valid bits).
-#include <cuda_bf16.h>
 #include "kernels.h"
+#include "popc_common.cuh"
 
 namespace hbmm {
 namespace {
+
+using namespace popc;
 
 constexpr int kWarps = 8;
 constexpr int kMaxRows = 8;
@@ -24,14 +27,10 @@ struct GemvArgs {
   int64_t N, K, lda_w, ldw_w, lda_s, ldw_s, ldc;
   int32_t M, a_bf16, w_bf16;
   int32_t ra, rw;        // segments per A group / per W group
+  int64_t Ga, Gw;        // groups per row
   int32_t n_quads;       // 16-byte pieces per row: ceil(K / 128)
   int32_t T;             // segments per row
 };
-
-__device__ __forceinline__ float load_scale(const void* s, int bf16, int64_t idx) {
-  if (bf16) return __uint_as_float(static_cast<uint32_t>(__ldg(reinterpret_cast<const unsigned short*>(s) + idx)) << 16);
-  return __ldg(reinterpret_cast<const float*>(s) + idx);
-}
 
 // SW: K-words per segment; MR: activation rows held in registers.
 template <int SW, int MR>
@@ -95,13 +94,73 @@ gemv_popc_kernel(const GemvArgs g) {
   }
 }
 
+// Segments of SEG = 2, 4, 8 or 16 bits: a lane takes one word of the weight row at a time, so the 32 / SEG scales it needs
+// are one vector and a warp's loads are contiguous; the activation rows are read the same way (they are a few KB, in L1
+// after the first warp), so nothing is staged and no barrier stands between the launch and the first weight load.
+// Bound by the scales: at beta 16 they are four times the bits.  3 x 3200 x 6592 at beta 16: 24 us in 32-row tiles (three
+// rows of each used), 17 us here; with one row 7.4 us.  Against the folded tensor-core kernel with its weight expansion,
+// which the automatic choice took before when K is whole words: 8 rows of 4096 x 9216 at beta 2 / 16 1580 / 315 us -> 119 / 34.
+template <int SEG, int MR>
+__global__ void __launch_bounds__(kWarps * 32)
+gemv_popc_sub_kernel(const GemvArgs g) {
+  constexpr int SPW = 32 / SEG, PARTS = SEG <= 8 ? 8 / SEG : 1;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n_words = static_cast<int>((g.K + 31) / 32);
+  for (int64_t n = static_cast<int64_t>(blockIdx.x) * kWarps + warp; n < g.N; n += static_cast<int64_t>(gridDim.x) * kWarps) {
+    const uint32_t* wrow = g.w_bits + n * g.ldw_w;
+    float acc[MR];
+#pragma unroll
+    for (int m = 0; m < MR; m++) acc[m] = 0.0f;
+#pragma unroll 2
+    for (int q = lane; q < n_words; q += 32) {
+      const uint32_t w = __ldg(wrow + q);
+      float sw[SPW];
+      load_scales<SPW>(g.w_scales, g.w_bf16, n * g.ldw_s, static_cast<int64_t>(q) * SPW, g.rw, g.Gw, true, sw);
+      const int64_t left = g.K - static_cast<int64_t>(q) * 32;          // valid bits from the word's start
+#pragma unroll
+      for (int m = 0; m < MR; m++) {
+        const bool in = m < g.M;
+        const uint32_t x = w ^ (in ? __ldg(g.a_bits + m * g.lda_w + q) : 0u);
+        float sa[SPW];
+        load_scales<SPW>(g.a_scales, g.a_bf16, m * g.lda_s, static_cast<int64_t>(q) * SPW, g.ra, g.Ga, in, sa);
+        uint32_t cnt[PARTS];
+        if constexpr (SEG <= 8) {
+#pragma unroll
+          for (int p = 0; p < PARTS; p++) cnt[p] = doubled_counts<SEG>(x, p);
+        }
+#pragma unroll
+        for (int t = 0; t < SPW; t++) {
+          const int64_t lt = left - t * SEG;
+          const int nv = lt >= SEG ? SEG : (lt > 0 ? static_cast<int>(lt) : 0);
+          int twice;
+          if constexpr (SEG <= 8) twice = static_cast<int>((cnt[t % PARTS] >> (8 * (t / PARTS))) & 0xFFu);
+          else twice = 2 * __popc(t == 0 ? (x & 0xFFFFu) : (x >> 16));
+          acc[m] = fmaf(sa[t] * sw[t], static_cast<float>(nv - twice), acc[m]);
+        }
+      }
+    }
+#pragma unroll
+    for (int m = 0; m < MR; m++) {
+      float v = acc[m];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+      if (lane == 0 && m < g.M) g.C[m * g.ldc + n] = v;
+    }
+  }
+}
+
+// Elements per segment: the finer grouping, or that of the operand with more than one group per row.
+int64_t segment_of(const PackedView& A, const PackedView& W) {
+  return A.beta >= A.K ? W.beta : (W.beta >= W.K ? A.beta : (A.beta < W.beta ? A.beta : W.beta));
+}
+
 bool make_args(const PackedView& A, const PackedView& W, GemvArgs& g) {
   if (A.rows > kMaxRows || A.rows < 1 || A.K != W.K) return false;
   const bool a_one = A.beta >= A.K, w_one = W.beta >= W.K;
-  if ((!a_one && A.beta % 32 != 0) || (!w_one && W.beta % 32 != 0)) return false;
   if (a_one && w_one) return false;
-  const int64_t seg = a_one ? W.beta : (w_one ? A.beta : (A.beta < W.beta ? A.beta : W.beta));
-  if (seg != 32 && seg != 64 && seg != 128) return false;
+  const int64_t seg = segment_of(A, W);
+  if (seg != 2 && seg != 4 && seg != 8 && seg != 16 && seg != 32 && seg != 64 && seg != 128) return false;
+  if ((!a_one && A.beta % seg != 0) || (!w_one && W.beta % seg != 0)) return false;
   const int64_t T = (A.K + seg - 1) / seg, quads = (A.K + 127) / 128;
   if (T > (int64_t{1} << 24)) return false;
   g.a_bits = A.bits; g.a_scales = A.scales; g.w_bits = W.bits; g.w_scales = W.scales; g.C = nullptr;
@@ -109,6 +168,8 @@ bool make_args(const PackedView& A, const PackedView& W, GemvArgs& g) {
   g.M = static_cast<int32_t>(A.rows); g.a_bf16 = A.scale_bf16; g.w_bf16 = W.scale_bf16;
   g.ra = static_cast<int32_t>(a_one ? T : A.beta / seg);
   g.rw = static_cast<int32_t>(w_one ? T : W.beta / seg);
+  g.Ga = num_groups(A.K, A.beta);
+  g.Gw = num_groups(W.K, W.beta);
   g.n_quads = static_cast<int32_t>(quads);
   g.T = static_cast<int32_t>(T);
   return true;
@@ -134,13 +195,26 @@ cudaError_t launch_sw(const GemvArgs& g, int sms, cudaStream_t stream) {
   return cudaGetLastError();
 }
 
+template <int SEG>
+cudaError_t launch_sub(const GemvArgs& g, int sms, cudaStream_t stream) {
+  int64_t blocks = (g.N + kWarps - 1) / kWarps;
+  if (blocks > static_cast<int64_t>(sms) * 8) blocks = static_cast<int64_t>(sms) * 8;
+  const unsigned grid = static_cast<unsigned>(blocks);
+  if (g.M <= 1) gemv_popc_sub_kernel<SEG, 1><<<grid, kWarps * 32, 0, stream>>>(g);
+  else if (g.M <= 2) gemv_popc_sub_kernel<SEG, 2><<<grid, kWarps * 32, 0, stream>>>(g);
+  else if (g.M <= 4) gemv_popc_sub_kernel<SEG, 4><<<grid, kWarps * 32, 0, stream>>>(g);
+  else gemv_popc_sub_kernel<SEG, 8><<<grid, kWarps * 32, 0, stream>>>(g);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
-// At most eight activation rows, groups of whole words with a finer grouping of 32, 64 or 128 elements, and
-// the activation rows fit the default 48 KB of shared memory.
+// At most eight activation rows with a finer grouping of 2 .. 16, 32, 64 or 128 elements; for the latter three (groups of
+// whole words) the activation rows have to fit the default 48 KB of shared memory.
 bool gemv_popc_supported(const PackedView& A, const PackedView& W) {
   GemvArgs g;
   if (!make_args(A, W, g)) return false;
+  if (segment_of(A, W) < 32) return true;
   return smem_bytes(g, 8, 1) <= 48 * 1024;
 }
 
@@ -150,10 +224,13 @@ cudaError_t launch_gemv_popc(const PackedView& A, const PackedView& W, float* C,
   g.C = C; g.ldc = ldc;
   int dev = 0, sms = 0;
   if (current_device(&dev, &sms) != cudaSuccess) return cudaErrorInvalidDevice;
-  const int sw = static_cast<int>(((A.beta >= A.K) ? W.beta : ((W.beta >= W.K) ? A.beta : (A.beta < W.beta ? A.beta : W.beta))) / 32);
-  switch (sw) {
-    case 1: return launch_sw<1>(g, sms, stream);
-    case 2: return launch_sw<2>(g, sms, stream);
+  switch (segment_of(A, W)) {
+    case 2: return launch_sub<2>(g, sms, stream);
+    case 4: return launch_sub<4>(g, sms, stream);
+    case 8: return launch_sub<8>(g, sms, stream);
+    case 16: return launch_sub<16>(g, sms, stream);
+    case 32: return launch_sw<1>(g, sms, stream);
+    case 64: return launch_sw<2>(g, sms, stream);
     default: return launch_sw<4>(g, sms, stream);
   }
 }

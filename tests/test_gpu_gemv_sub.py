@@ -1,0 +1,30 @@
+"""The matrix-vector kernel on groups shorter than a word (gemv_popc.cu): one to eight rows, K ending inside a word and
+inside a group, a row shorter than a warp's stride, mixed groups, one group per row, bf16 scales -- against the oracle."""
+import pytest
+import torch
+
+import oracle
+from paper_1905_10759_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+CASES = [(M, N, K, b, b, 0) for b in (2, 4, 8, 16) for M, N, K in ((1, 9, 31), (3, 33, 1056), (8, 17, 2055))]
+CASES += [(5, 40, 777, 2, 64, 0), (2, 41, 777, 32, 8, 1), (4, 7, 333, 333, 16, 0), (6, 8, 100, 4, 4, 1), (7, 1500, 96, 16, 2, 0)]
+
+
+@pytest.mark.parametrize("M,N,K,ba,bw,sdt", CASES)
+def test_gemv_of_sub_word_groups_matches_oracle(M, N, K, ba, bw, sdt):
+    import gpu_util as gu
+    from paper_1905_10759_b200 import hbmm
+    a, w = inputs.normal((M, K), 4200 + M + K + ba), inputs.he_normal(N, K, 5200 + N + K + bw)
+    A, da, sa = gu.oracle_operand(a, ba, sdt)
+    W, dw, sw = gu.oracle_operand(w, bw, sdt)
+    ea, ew = gu.eff_beta(ba, K), gu.eff_beta(bw, K)
+    c_ref, absref = oracle.hbmm_from_quantized(da, sa, ea, dw, sw, ew)
+    T = -(-K // min(ea, ew))
+    for path in (hbmm.PATH_POPC, hbmm.PATH_AUTO):
+        C = torch.full((M, (N + 3) // 4 * 4 + 4), float("nan"), device="cuda")
+        hbmm.gemm_ex(A, W, C, path)
+        assert torch.isnan(C[:, N:]).all()
+        # two roundings per segment, one per segment of a lane's sum and five in the tree that joins the lanes
+        gu.assert_close_rel_absref(C[:, :N].cpu().numpy(), c_ref, absref, (T + 5 + 2) * gu.U, "gemv")
