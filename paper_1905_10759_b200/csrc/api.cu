@@ -162,7 +162,10 @@ hbmm_status gemm_checked(const hbmm_operand* A, const hbmm_operand* W, float* C,
     case HBMM_PATH_FOLDED:
       if (!gemm_fold_supported(a, w)) return HBMM_ERR_UNSUPPORTED;
       if (!workspace_ok(workspace, workspace_bytes, fold_workspace(a, w))) return HBMM_ERR_WORKSPACE;
-      e = launch_gemm_fold(a, w, C, ldc, workspace, stream, w_prepared);
+      // the earlier call may have been an automatic one, which leaves no expanded weights behind for a handful of rows
+      // with sub-word groups: those take the kernel that needs none
+      if (w_prepared && gemm_subword(a, w) && gemv_popc_supported(a, w)) e = launch_gemv_popc(a, w, C, ldc, stream);
+      else e = launch_gemm_fold(a, w, C, ldc, workspace, stream, w_prepared);
       break;
     default:
       // a handful of activation rows: reading the packed weights once beats any tile kernel (and the expanded

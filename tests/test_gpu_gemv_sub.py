@@ -28,3 +28,20 @@ def test_gemv_of_sub_word_groups_matches_oracle(M, N, K, ba, bw, sdt):
         assert torch.isnan(C[:, N:]).all()
         # two roundings per segment, one per segment of a lane's sum and five in the tree that joins the lanes
         gu.assert_close_rel_absref(C[:, :N].cpu().numpy(), c_ref, absref, (T + 5 + 2) * gu.U, "gemv")
+
+
+def test_prepared_call_after_an_automatic_one_on_a_few_rows():
+    """An automatic call leaves no expanded weights for these operands; a prepared call that follows has to be right."""
+    import gpu_util as gu
+    from paper_1905_10759_b200 import hbmm
+    M, N, K, b = 4, 40, 320, 8
+    a, w = inputs.normal((M, K), 4300), inputs.he_normal(N, K, 5300)
+    A, da, sa = gu.oracle_operand(a, b, 0)
+    W, dw, sw = gu.oracle_operand(w, b, 0)
+    c_ref, absref = oracle.hbmm_from_quantized(da, sa, b, dw, sw, b)
+    ws = torch.zeros(hbmm.gemm_workspace_bytes(A, W), dtype=torch.uint8, device="cuda")
+    C = torch.full((M, N), float("nan"), device="cuda")
+    hbmm.gemm(A, W, C, ws)
+    C.fill_(float("nan"))
+    hbmm.gemm_ex(A, W, C, hbmm.PATH_FOLDED_PREPARED, ws)
+    gu.assert_close_rel_absref(C.cpu().numpy(), c_ref, absref, 1e-5, "prepared")
