@@ -8,8 +8,10 @@
 // product is exact in the fp32 accumulator, and the cross products
 //     A1 W1^T + A1 W2^T + A2 W1^T
 // are one accumulation in tensor memory over the whole of K: per 16 K-elements three MMAs of 128 x TN x 16
-// (A1 against W1, A2 against W1, A1 against W2) add into the same TN accumulator columns (the 64-column tile
-// forms A1 W1 and A1 W2 with one MMA of 128 columns instead and adds the blocks in the epilogue).  The fourth product A2 W2^T is left out: both second pieces are
+// (A1 against W1, A2 against W1, A1 against W2) add into the same TN accumulator columns.  Where tensor memory has room the
+// two cross products, 2^-11 of the first, add into columns of their own and the epilogue adds the blocks, so that the large
+// sum takes a third of the fp32 roundings: the 64-column tile (which forms A1 W1 and A1 W2 with one MMA of 128
+// columns) and a tile split between CTAs (whose second accumulator is free).  The fourth product A2 W2^T is left out: both second pieces are
 // constant inside a scale group and at most 2^-11 of the first, so it equals sum_g (a2_g w2_g) D_g, at
 // most 2^-22 of sum_g |deltaA deltaW D_g| -- forty times below the 1e-5 the result is held to.
 // There is no per-group step; the epilogue runs once per tile and divides the rows' and columns' powers of
@@ -35,6 +37,7 @@
 // CTA-wide abort flag that all other waits observe, and the kernel drains and frees its TMEM before returning.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+#include <atomic>
 #include "kernels.h"
 #include "tensor_map.h"
 #include "umma_common.cuh"
@@ -124,6 +127,21 @@ row_max_kernel(const float* __restrict__ scales, int64_t ld, int64_t M, float* _
   if (lane == 0) out[m] = __uint_as_float(x);
 }
 
+// Producer and scout warps: the first tile's row factors are in shared memory.
+__device__ __forceinline__ void first_rows_barrier() {
+  asm volatile("bar.sync 1, %0;" ::"n"((kProducerWarps + kScoutWarps) * 32) : "memory");
+}
+
+// Split mode: byte offset of the 16-byte piece u of row `row` of a partial tile.
+constexpr int kMaxSplit = 8;            // CTAs that may share a tile (the portable cluster size)
+template <int TN>
+__device__ __forceinline__ int split_piece(int row, int u) { return row * (TN * 4) + ((u ^ (row & 7)) << 4); }
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+
 // Walks the stages a producer thread owns (every second stage of the CTA's stream of tiles) and keeps
 // the row pointers of the tile it is in.
 struct StageCursor {
@@ -137,9 +155,11 @@ struct StageCursor {
 // ASUB: scale groups per packed word of A (1: groups of whole words; 2 .. 16: beta_a = 16 .. 2).
 // FUSE: the epilogue runs the activation / affine map / dense or binarized output chain of epilogue.cuh instead of
 // storing the product as fp32.
-// BAL: the balanced schedule (runs of (tile, stage) pairs, partial tiles reduced by the last CTA to arrive); the plain
-// instantiation carries none of its code.
-template <int TN, int ASUB, bool FUSE, bool BAL>
+// MODE: how the tiles are shared out.  kPlain: whole tiles, round robin.  kBalanced: runs of (tile, stage) pairs, partial
+// tiles reduced by the last CTA to arrive.  kSplit: a cluster of g.split CTAs per tile, each with an equal part of the K
+// range; the partial accumulators meet through distributed shared memory.  Each instantiation carries its own code only.
+enum Mode : int { kPlain = 0, kBalanced = 1, kSplit = 2 };
+template <int TN, int ASUB, bool FUSE, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
 hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
   using S = Smem<TN>;
@@ -169,24 +189,27 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
   // The CTA's work is a list of segments (tile, first stage, one past the last stage).  Plain schedule: whole tiles
   // blockIdx.x, blockIdx.x + gridDim.x, ...  Balanced schedule: the run [u0, u1) of the tile-major (tile, stage)
   // sequence -- consecutive tiles, the first possibly entered mid-way, the last possibly left early.
+  constexpr bool BAL = MODE == kBalanced, SPLIT = MODE == kSplit;
   constexpr bool balanced = BAL;
+  const int64_t sp_rank = SPLIT ? blockIdx.x % g.split : 0, sp_tile = SPLIT ? blockIdx.x / g.split : 0;
+  const int64_t sp_begin = SPLIT ? sp_rank * n_stages / g.split : 0, sp_end = SPLIT ? (sp_rank + 1) * n_stages / g.split : n_stages;
   const int64_t u0 = balanced ? static_cast<int64_t>(blockIdx.x) * g.sk_units : 0;
   const int64_t u_end = balanced ? ((u0 + g.sk_units < n_tiles * n_stages) ? u0 + g.sk_units : n_tiles * n_stages) : 0;
   const int64_t sk_t0 = balanced ? u0 / n_stages : 0;                                  // first tile of the run
   const int64_t sk_first = balanced ? u0 - sk_t0 * n_stages : 0;                       // first stage inside it
   const int64_t sk_t1 = (balanced && u_end > u0) ? (u_end - 1) / n_stages : 0;         // last tile of the run
   const int64_t sk_last_end = (balanced && u_end > u0) ? u_end - sk_t1 * n_stages : 0; // one past its last stage
-  const int64_t my_tiles = balanced ? (u_end > u0 ? sk_t1 - sk_t0 + 1 : 0)
+  const int64_t my_tiles = SPLIT ? 1 : balanced ? (u_end > u0 ? sk_t1 - sk_t0 + 1 : 0)
                                     : (blockIdx.x < n_tiles ? (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0);
-  const int64_t my_stages = balanced ? (u_end > u0 ? u_end - u0 : 0) : my_tiles * n_stages;
+  const int64_t my_stages = SPLIT ? sp_end - sp_begin : balanced ? (u_end > u0 ? u_end - u0 : 0) : my_tiles * n_stages;
   // Order of work in a balanced run: the two tiles shared with the neighbouring runs first (the tail of the run's first
   // tile, then the head of its last), the whole tiles after them -- so partial accumulators are handed in early and
   // the CTA that completes a shared tile does so in the shadow of the MMAs of its whole tiles, not at the kernel's end.
   const bool reorder = balanced && my_tiles >= 3;
   auto seg_nat = [&](int64_t ti) -> int64_t { return !reorder ? ti : (ti == 0 ? 0 : (ti == 1 ? my_tiles - 1 : ti - 1)); };
-  auto seg_tile = [&](int64_t ti) -> int64_t { return balanced ? sk_t0 + seg_nat(ti) : blockIdx.x + ti * gridDim.x; };
-  auto seg_begin = [&](int64_t ti) -> int64_t { return (balanced && ti < my_tiles && seg_nat(ti) == 0) ? sk_first : 0; };
-  auto seg_end = [&](int64_t ti) -> int64_t { return (balanced && ti < my_tiles && seg_nat(ti) == my_tiles - 1) ? sk_last_end : n_stages; };
+  auto seg_tile = [&](int64_t ti) -> int64_t { return SPLIT ? sp_tile : balanced ? sk_t0 + seg_nat(ti) : blockIdx.x + ti * gridDim.x; };
+  auto seg_begin = [&](int64_t ti) -> int64_t { return SPLIT ? sp_begin : (balanced && ti < my_tiles && seg_nat(ti) == 0) ? sk_first : 0; };
+  auto seg_end = [&](int64_t ti) -> int64_t { return SPLIT ? sp_end : (balanced && ti < my_tiles && seg_nat(ti) == my_tiles - 1) ? sk_last_end : n_stages; };
 
   pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
   if (tid == 0) {
@@ -212,6 +235,12 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
   tc_fence_after();
   const uint32_t tmem_base = *tmem_base_ptr;
 
+  // The first tile's row factors are found by the producer warps, two threads per row, while their first words and scales
+  // are on the way: nothing can be expanded before they are known, and the scouts (two rows per thread) take several
+  // memory round trips for a long row.  (Where a row has few scales and a CTA many tiles this costs 1 %: the scouts' later
+  // tiles start later.  It runs for split tiles and for sub-word groups.)
+  const bool scan_first = (SPLIT || ASUB > 1) && my_tiles > 0 && !(ASUB > 1 && g.a_rowmax);
+
   // The CTA is persistent: it walks tiles blockIdx.x, blockIdx.x + gridDim.x, ... and the stage ring
   // simply continues across tiles (gst counts stages since launch).
   if (warp >= kFirstProducerWarp && warp < kMmaWarp) {
@@ -235,7 +264,7 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
     };
     auto carry_over = [&](StageCursor& c) {        // moves a stage index past its segment's end into the segments after it
       if (c.st >= c.end) {
-        if (!balanced) {
+        if (!balanced && !SPLIT) {
           do { c.st -= n_stages; c.ti++; } while (c.st >= n_stages);
         } else {
           do { const int64_t over = c.st - c.end; c.ti++; c.st = seg_begin(c.ti) + over; c.end = seg_end(c.ti); } while (c.st >= c.end);
@@ -288,6 +317,16 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
     float sc[kDepth][2 * ASUB];
 #pragma unroll
     for (int u = 0; u < kDepth; u++) { fetch(pf, w[u], sc[u]); advance(pf); }
+    if (scan_first) {
+      const int r = pt >> 1;
+      const int64_t m = (seg_tile(0) / tiles_n) * TM + r;
+      uint32_t mx = m < g.M ? row_max_part<2>(g.a_scales, g.a_bf16, m * g.lda_s, g.lda_s, pt & 1) : 0u;
+      mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, 1));
+      float up0 = 0.0f, down0 = 1.0f;
+      if (m < g.M) norm_factors(__uint_as_float(mx), up0, down0);
+      if ((pt & 1) == 0) { rowup[r] = up0; rowdown[r] = down0; }
+      first_rows_barrier();
+    }
     int64_t up_tile = -1;
     float up = 0.0f;
     bool ok = true;
@@ -358,7 +397,9 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
       const int slot = static_cast<int>(ti & (kRowSlots - 1));
       if (ti >= kRowSlots && !mbar_wait(&rowempty[slot], static_cast<uint32_t>(((ti / kRowSlots) & 1) ^ 1), abort_flag, 8)) break;
       const int64_t tile = seg_tile(ti);
-      if (ASUB > 1 && g.a_rowmax) {
+      if (ti == 0 && scan_first) {
+        first_rows_barrier();          // the producers have stored them
+      } else if (ASUB > 1 && g.a_rowmax) {
         // long rows of scales: a kernel of its own has reduced every row to its largest scale
         const int64_t ma = (tile / tiles_n) * TM + p0, mb = ma + kScoutWarps * 32;
         float up = 0.0f, down = 1.0f;
@@ -468,7 +509,12 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
             for (int ks = 0; ks < KB / 16; ks++) {        // 16 K-elements = 8 TMEM columns of A, 32 bytes along the swizzled rows of W
               if constexpr (S::STACKED) {
                 umma_f16_ts(d_tmem, a1 + ks * 8, db_hi | (b1_lo + ks * 2), idesc2, (st | ks) != 0 ? 1u : 0u);   // A1 [W1; W2]
-                umma_f16_ts(d_tmem, a2 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, 1u);                           // A2 W1
+                umma_f16_ts(d_tmem + TN, a2 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, 1u);                      // A2 W1, to A1 W2
+              } else if constexpr (SPLIT) {
+                // one tile only: the second accumulator takes the two cross products
+                umma_f16_ts(d_tmem, a1 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, (st | ks) != 0 ? 1u : 0u);
+                umma_f16_ts(d_tmem + S::ACC_COLS, a2 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, (st | ks) != 0 ? 1u : 0u);
+                umma_f16_ts(d_tmem + S::ACC_COLS, a1 + ks * 8, db_hi | (b2_lo + ks * 2), idesc, 1u);
               } else {
                 umma_f16_ts(d_tmem, a1 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, (st | ks) != 0 ? 1u : 0u);
                 umma_f16_ts(d_tmem, a2 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, 1u);
@@ -531,11 +577,12 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
       if (lane == 0) mbar_arrive(&rowempty[slot]);
       float* dst = g.C + m * g.ldc + nb;
       float carry = 0.0f;                                   // |z| sum of a group wider than a 32-column chunk
-      // raw accumulator of chunk c (32 columns of this thread's row): the two stacked blocks added for the narrow tile
+      // raw accumulator of chunk c (32 columns of this thread's row): the block of A1 W1 and the block of the cross
+      // products added, where they are apart
       auto load_chunk = [&](int c, uint32_t (&v1)[32]) {
         const uint32_t t_addr = tmem_base + t_lane + buf * S::ACC_COLS + c * 32;
         tmem_ld32(t_addr, v1);
-        if constexpr (S::STACKED) {      // the A1 W2 block sits TN columns further on
+        if constexpr (S::STACKED || SPLIT) {      // the cross products sit TN columns further on
           uint32_t v2[32];
           tmem_ld32(t_addr + TN, v2);
           tmem_ld_wait();
@@ -582,6 +629,19 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
           }
         }
       };
+      if constexpr (SPLIT) {
+        // The partial accumulator goes to the weight ring (every copy into it has been consumed, every MMA that read it
+        // has retired), row-major with the row's 16-byte pieces permuted so that eight rows hit eight bank groups.
+#pragma unroll
+        for (int c = 0; c < TN / 32; c++) {
+          uint32_t v1[32];
+          load_chunk(c, v1);
+#pragma unroll
+          for (int j = 0; j < 8; j++)
+            *reinterpret_cast<uint4*>(smem + S::OFF_B + split_piece<TN>(row, c * 8 + j)) = make_uint4(v1[4 * j], v1[4 * j + 1], v1[4 * j + 2], v1[4 * j + 3]);
+        }
+        break;
+      }
       const bool whole = !BAL || (seg_begin(ti) == 0 && seg_end(ti) == n_stages);
       if (whole) {
 #pragma unroll
@@ -639,6 +699,39 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
     }
   }
 
+  if constexpr (SPLIT) {
+    // Every CTA of the cluster finishes its share of the tile's rows: the partial sums of all of them in rank order (the
+    // same sum in every run), the powers of two divided out, whole 16-byte pieces of consecutive columns per lane.
+    __syncwarp();
+    cluster_sync_all();
+    const int r0 = static_cast<int>(sp_rank) * TM / g.split, r1 = (static_cast<int>(sp_rank) + 1) * TM / g.split;
+    const int64_t mb = (sp_tile / tiles_n) * TM, nb = (sp_tile % tiles_n) * TN;
+    for (int i = tid; i < (r1 - r0) * (TN / 4); i += kThreads) {
+      const int row = r0 + i / (TN / 4), u = i % (TN / 4);
+      const int64_t m = mb + row, n = nb + 4 * u;
+      if (m >= g.M || n >= g.N) continue;
+      const float4 fw = __ldg(reinterpret_cast<const float4*>(g.w_down + n));
+      const uint32_t at = smem_u32(smem + S::OFF_B + split_piece<TN>(row, u));
+      float4 v[kMaxSplit];
+#pragma unroll
+      for (int q = 0; q < kMaxSplit; q++)
+        if (q < g.split) v[q] = ld_cluster_f4(mapa_rank(at, q));
+      float4 sum = v[0];
+#pragma unroll
+      for (int q = 1; q < kMaxSplit; q++)
+        if (q < g.split) { sum.x += v[q].x; sum.y += v[q].y; sum.z += v[q].z; sum.w += v[q].w; }
+      const float fa = rowdown[row];
+      float o[4] = {sum.x * fa, sum.y * fa, sum.z * fa, sum.w * fa};
+      o[0] *= fw.x; o[1] *= fw.y; o[2] *= fw.z; o[3] *= fw.w;
+      float* dst = g.C + m * g.ldc + n;
+      if (n + 3 < g.N) *reinterpret_cast<float4*>(dst) = make_float4(o[0], o[1], o[2], o[3]);
+      else
+        for (int e = 0; e < 4; e++)
+          if (n + e < g.N) dst[e] = o[e];
+    }
+    __syncwarp();
+    cluster_sync_all();          // nobody's shared memory goes away while another CTA reads it
+  }
   // ---- teardown: everyone meets here (aborted threads too), then the allocating warp frees TMEM
   tc_fence_before();
   __syncthreads();
@@ -683,6 +776,7 @@ Args make_args(const PackedView& A, const PackedView& W, float* C, int64_t ldc) 
   g.ep = plain_epilogue();
   g.sk_units = 0; g.sk_counters = nullptr; g.sk_counter_count = 0; g.sk_partials = nullptr;
   g.a_staged = 0; g.a_rowmax = nullptr;
+  g.split = 1;
   return g;
 }
 
@@ -697,6 +791,10 @@ constexpr int64_t kMaxBalancedCtas = 256;
 constexpr int64_t kBalancedWaves = 4;
 constexpr int64_t kBalancedMinStages = 4;
 constexpr int64_t kBalancedMaxShare = 4;
+// Split mode: 256 x 256 x 256 (four stages) takes 7.4 us whole and 7.8 us in two parts; from six stages on parts of two
+// stages win (64 x 1024 x 1024, 16 stages: 17.4 -> 8.0 us in eight parts).
+constexpr int64_t kSplitMinStages = 2;
+constexpr int64_t kSplitFromStages = 6;
 template <int TN>
 int64_t tile_count(const Args& g) { return ((g.M + TM - 1) / TM) * ((g.N + TN - 1) / TN); }
 template <int TN>
@@ -737,6 +835,41 @@ void set_balanced_area(Args& g, void* workspace) {
   g.sk_partials = reinterpret_cast<float*>(area + counters_bytes<TN>(g));
 }
 
+// Split mode: the largest number of CTAs per tile (2 .. 8, at least two stages each) for which every tile's cluster is
+// resident at once; 1: not worth it.  Taken where the tiles cover at most half of the machine.  Against the balanced
+// schedule, whose last CTA adds the partial tiles through global memory (12 .. 20 rounds of loads by four warps):
+// 256 x 1000 x 4096 28.4 -> 16.2 us, 256 x 4096 x 4096 39 -> 30, 256 x 4096 x 9216 61.5 -> 56, 49 x 512 x 4608 26.6 -> 12.2,
+// 1024^3 24.2 -> 13.2 us; and the second accumulator brings the error of a result from 4e-7 .. 4e-6 to 1e-7 .. 1.8e-6.  (All instantiations take a whole SM per CTA, so they share what was asked once.)
+template <typename Kernel>
+int choose_split(Kernel kernel, int smem_bytes, int dev, int sms, int64_t tiles, int64_t n_stages) {
+  static std::atomic<int> resident[64][kMaxSplit + 1];           // clusters of each size the device holds, plus one; 0: not asked yet
+  if (2 * tiles > sms || n_stages < kSplitFromStages || dev < 0 || dev >= 64) return 1;
+  int64_t most = n_stages / kSplitMinStages;
+  if (most > kMaxSplit) most = kMaxSplit;
+  for (int s = static_cast<int>(most); s >= 2; s--) {
+    if (tiles * s > sms) continue;
+    int n = resident[dev][s].load(std::memory_order_relaxed);
+    if (n == 0) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(static_cast<unsigned>(s));
+      cfg.blockDim = dim3(kThreads);
+      cfg.dynamicSmemBytes = static_cast<size_t>(smem_bytes);
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = static_cast<unsigned>(s);
+      attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      int got = 0;
+      if (cudaOccupancyMaxActiveClusters(&got, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); got = 0; }
+      n = got + 1;
+      resident[dev][s].store(n, std::memory_order_relaxed);
+    }
+    if (tiles <= n - 1) return s;
+  }
+  return 1;
+}
+
 template <int TN, int ASUB, bool FUSE = false>
 cudaError_t launch_fold(Args g, void* workspace, cudaStream_t stream, bool w_prepared) {
   using S = Smem<TN>;
@@ -747,10 +880,14 @@ cudaError_t launch_fold(Args g, void* workspace, cudaStream_t stream, bool w_pre
   int dev = 0, sms = 0;
   if (current_device(&dev, &sms) != cudaSuccess) return cudaErrorInvalidDevice;
   if (configured.pending(dev)) {
-    cudaError_t e = cudaFuncSetAttribute(hbmm_fold_kernel<TN, ASUB, FUSE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+    cudaError_t e = cudaFuncSetAttribute(hbmm_fold_kernel<TN, ASUB, FUSE, kPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
     if (e != cudaSuccess) return e;
     if (kHasBalanced) {
-      e = cudaFuncSetAttribute(hbmm_fold_kernel<TN, ASUB, FUSE, kHasBalanced>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+      e = cudaFuncSetAttribute(hbmm_fold_kernel<TN, ASUB, FUSE, kHasBalanced ? kBalanced : kPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+      if (e != cudaSuccess) return e;
+    }
+    if (!FUSE) {
+      e = cudaFuncSetAttribute(hbmm_fold_kernel<TN, ASUB, FUSE, FUSE ? kPlain : kSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
       if (e != cudaSuccess) return e;
     }
     configured.mark(dev);
@@ -792,6 +929,14 @@ cudaError_t launch_fold(Args g, void* workspace, cudaStream_t stream, bool w_pre
     if (e != cudaSuccess) return e;
   }
   const int64_t tiles = ((g.M + TM - 1) / TM) * tiles_n;
+  if constexpr (!FUSE) {
+    const int split = choose_split(hbmm_fold_kernel<TN, ASUB, FUSE, kSplit>, kBytes, dev, sms, tiles, n_stages);
+    if (split > 1) {
+      g.split = split;
+      return launch_pdl_cluster(hbmm_fold_kernel<TN, ASUB, FUSE, kSplit>, dim3(static_cast<unsigned>(tiles * split)), dim3(kThreads),
+                                static_cast<unsigned>(split), kBytes, stream, g, s_map);
+    }
+  }
   // equal runs of (tile, stage) pairs, one per CTA, when that shortens the longest CTA's walk by a tenth or more
   const int64_t units = tiles * n_stages;
   int64_t ctas = units / kBalancedMinStages < sms ? units / kBalancedMinStages : sms;
@@ -805,10 +950,10 @@ cudaError_t launch_fold(Args g, void* workspace, cudaStream_t stream, bool w_pre
   if (kHasBalanced && balanced_possible<TN>(g, sms) && run * 10 <= plain_walk * 9) {
     ctas = (units + run - 1) / run;                     // no CTA without work
     g.sk_units = run;
-    return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kHasBalanced>, dim3(static_cast<unsigned>(ctas)), dim3(kThreads), kBytes, stream, g, s_map);
+    return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kHasBalanced ? kBalanced : kPlain>, dim3(static_cast<unsigned>(ctas)), dim3(kThreads), kBytes, stream, g, s_map);
   }
   const unsigned grid = static_cast<unsigned>(tiles < sms ? tiles : sms);   // one persistent CTA per SM
-  return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, false>, dim3(grid), dim3(kThreads), kBytes, stream, g, s_map);
+  return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kPlain>, dim3(grid), dim3(kThreads), kBytes, stream, g, s_map);
 }
 
 template <int TN>

@@ -128,6 +128,29 @@ __device__ __forceinline__ void row_max_scale2(const void* s, int bf16, int64_t 
   max_b = __uint_as_float(mb);
 }
 
+// The same for one row shared by PARTS consecutive lanes: consecutive lanes take consecutive vectors, eight of each lane's in
+// flight.  Returns the bit pattern of this lane's largest.
+template <int PARTS>
+__device__ __forceinline__ uint32_t row_max_part(const void* s, int bf16, int64_t row_off, int64_t ld, int part) {
+  uint32_t mx = 0;
+  const int64_t n_vec = bf16 ? ld / 8 : ld / 4;
+  const uint4* p = bf16 ? reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned short*>(s) + row_off)
+                        : reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(s) + row_off);
+#pragma unroll 1
+  for (int64_t i = part; i < n_vec; i += 8 * PARTS) {
+    uint4 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; u++) v[u] = i + PARTS * u < n_vec ? __ldg(p + i + PARTS * u) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int u = 0; u < 8; u++) {
+      const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+      for (int e = 0; e < 4; e++) mx = max(mx, bf16 ? max(w[e] << 16, w[e] & 0xFFFF0000u) : w[e]);
+    }
+  }
+  return mx;
+}
+
 // Powers of two for a row whose largest scale is mx: mx * up lies in [2^14, 2^15), down = 1 / up.
 // Rows whose scales are all below 2^-100 (an all-zero row included) are treated as if their largest
 // were 2^-100, which keeps both factors normal numbers.

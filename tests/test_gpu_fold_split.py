@@ -1,0 +1,47 @@
+"""The folded contraction with a tile's K range split between the CTAs of a cluster (gemm_fold.cu): one to eight parts, parts
+of unequal length, a last stage of one word, ragged rows and columns, both tile widths, sub-word activation groups, scales
+stored as bf16 -- against the oracle, and the same bits from run to run."""
+import pytest
+import torch
+
+import oracle
+from paper_1905_10759_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # M, N, K, beta_a, beta_w, scale dtype
+    (49, 100, 352, 32, 32, 0),        # six stages, the last of one word: three parts
+    (9, 64, 320, 32, 32, 0),          # five stages: not split
+    (128, 128, 1024, 64, 64, 0),      # eight parts of two stages
+    (129, 130, 1088, 32, 32, 0),      # four tiles, 17 stages in eight unequal parts
+    (10, 33, 4608, 32, 32, 1),        # narrow tile, bf16 scales
+    (300, 700, 960, 32, 64, 0),       # 18 tiles: as many CTAs per tile as fit
+    (1100, 1000, 512, 32, 32, 0),     # 72 tiles: pairs of CTAs
+    (200, 72, 1152, 16, 16, 0),
+    (130, 200, 2304, 4, 4, 0),        # scales through the shared-memory ring
+    (70, 60, 1088, 2, 16, 0),         # 544 scales per row: row maxima from their own kernel
+    (70, 150, 768, 8, 8, 1),
+    (40, 50, 640, 640, 32, 0),        # one activation group per row
+]
+
+
+@pytest.mark.parametrize("M,N,K,ba,bw,sdt", CASES)
+def test_split_tiles_match_oracle(M, N, K, ba, bw, sdt):
+    import gpu_util as gu
+    from paper_1905_10759_b200 import hbmm
+    a, w = inputs.normal((M, K), 4400 + M + K + ba), inputs.he_normal(N, K, 5400 + N + K + bw)
+    A, da, sa = gu.oracle_operand(a, ba, sdt)
+    W, dw, sw = gu.oracle_operand(w, bw, sdt)
+    ea, ew = gu.eff_beta(ba, K), gu.eff_beta(bw, K)
+    c_ref, absref = oracle.hbmm_from_quantized(da, sa, ea, dw, sw, ew)
+    fine = gu.elementwise_magnitude(da, ea, dw, ew, K)
+    ws = torch.empty(hbmm.gemm_workspace_bytes(A, W), dtype=torch.uint8, device="cuda")
+    ldc = (N + 3) // 4 * 4 + 4
+    outs = [torch.full((M, ldc), float("nan"), device="cuda") for _ in range(3)]
+    for C, path in zip(outs, (hbmm.PATH_FOLDED, hbmm.PATH_FOLDED_PREPARED, hbmm.PATH_FOLDED_PREPARED)):
+        hbmm.gemm_ex(A, W, C, path, ws)
+        assert torch.isnan(C[:, N:]).all()
+        assert torch.equal(C[:, :N], outs[0][:, :N])
+    gu.assert_close_rel_absref(outs[0][:, :N].cpu().numpy(), c_ref, absref, 1e-5, "split", fine)
+    assert hbmm.last_device_error() == 0
