@@ -10,8 +10,8 @@
 // are one accumulation in tensor memory over the whole of K: per 16 K-elements three MMAs of 128 x TN x 16
 // (A1 against W1, A2 against W1, A1 against W2) add into the same TN accumulator columns.  Where tensor memory has room the
 // two cross products, 2^-11 of the first, add into columns of their own and the epilogue adds the blocks, so that the large
-// sum takes a third of the fp32 roundings: the 64-column tile (which forms A1 W1 and A1 W2 with one MMA of 128
-// columns) and a tile split between CTAs (whose second accumulator is free).  The fourth product A2 W2^T is left out: both second pieces are
+// sum takes a third of the fp32 roundings: the 64-column tile, long 128-column tiles and tiles split between CTAs, which form
+// A1 W1 and A1 W2 side by side with one MMA of twice the columns.  The fourth product A2 W2^T is left out: both second pieces are
 // constant inside a scale group and at most 2^-11 of the first, so it equals sum_g (a2_g w2_g) D_g, at
 // most 2^-22 of sum_g |deltaA deltaW D_g| -- forty times below the 1e-5 the result is held to.
 // There is no per-group step; the epilogue runs once per tile and divides the rows' and columns' powers of
@@ -159,7 +159,8 @@ struct StageCursor {
 // tiles reduced by the last CTA to arrive.  kSplit: a cluster of g.split CTAs per tile, each with an equal part of the K
 // range; the partial accumulators meet through distributed shared memory.  Each instantiation carries its own code only.
 enum Mode : int { kPlain = 0, kBalanced = 1, kSplit = 2 };
-template <int TN, int ASUB, bool FUSE, int MODE>
+// WIDE (128-column tiles): one accumulator of 256 columns instead of two of 128 (see the MMA issuer).
+template <int TN, int ASUB, bool FUSE, int MODE, bool WIDE>
 __global__ void __launch_bounds__(kThreads, 1)
 hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
   using S = Smem<TN>;
@@ -191,6 +192,8 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
   // sequence -- consecutive tiles, the first possibly entered mid-way, the last possibly left early.
   constexpr bool BAL = MODE == kBalanced, SPLIT = MODE == kSplit;
   constexpr bool balanced = BAL;
+  constexpr bool STACK = S::STACKED || WIDE;                     // A1 W1 and A1 W2 from one instruction, side by side
+  constexpr int NBUF = WIDE ? 1 : 2;                             // accumulators
   const int64_t sp_rank = SPLIT ? blockIdx.x % g.split : 0, sp_tile = SPLIT ? blockIdx.x / g.split : 0;
   const int64_t sp_begin = SPLIT ? sp_rank * n_stages / g.split : 0, sp_end = SPLIT ? (sp_rank + 1) * n_stages / g.split : n_stages;
   const int64_t u0 = balanced ? static_cast<int64_t>(blockIdx.x) * g.sk_units : 0;
@@ -479,6 +482,11 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
     __syncwarp();
   } else if (warp == kMmaWarp) {
     // =========================== MMA issuer ===========================
+    // The tensor core's queue holds a few MMAs, whatever their size: with 128-column instructions (64 clk each) the barrier,
+    // the fence and the commit around a stage's twelve, and the producers' stores to tensor memory in between, drain it --
+    // 1100 clk per stage instead of the 768 the MMAs take.  WIDE forms A1 [W1; W2] as one instruction of 256 columns
+    // (128 clk), which rides over these, and as a side effect keeps the large products' sum apart from the small ones'.  Its
+    // accumulator takes the room of both: the epilogue is then exposed at every tile's end, so a tile has to be long.
     // The whole warp walks the loop so that ring indices and descriptors stay warp-uniform values; one
     // lane issues the MMAs and commits.
     {
@@ -492,9 +500,9 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
       uint32_t s = 0, full_par = 0;
       bool ok = true;
       for (int64_t ti = 0; ti < my_tiles && ok; ti++) {
-        const uint32_t buf = static_cast<uint32_t>(ti & 1);
-        if (ti >= 2) {      // the epilogue must have drained this accumulator (used by tile ti - 2)
-          if (!mbar_wait_a(tempty_a + buf * 8, static_cast<uint32_t>(((ti >> 1) & 1) ^ 1), abort_flag, 3)) { ok = false; break; }
+        const uint32_t buf = static_cast<uint32_t>(ti % NBUF);
+        if (ti >= NBUF) {      // the epilogue must have drained this accumulator (used by tile ti - NBUF)
+          if (!mbar_wait_a(tempty_a + buf * 8, static_cast<uint32_t>(((ti / NBUF) & 1) ^ 1), abort_flag, 3)) { ok = false; break; }
           tc_fence_after();
         }
         const uint32_t d_tmem = tmem_base + buf * S::ACC_COLS;
@@ -507,14 +515,9 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
           if (leader) {
 #pragma unroll
             for (int ks = 0; ks < KB / 16; ks++) {        // 16 K-elements = 8 TMEM columns of A, 32 bytes along the swizzled rows of W
-              if constexpr (S::STACKED) {
+              if constexpr (STACK) {
                 umma_f16_ts(d_tmem, a1 + ks * 8, db_hi | (b1_lo + ks * 2), idesc2, (st | ks) != 0 ? 1u : 0u);   // A1 [W1; W2]
                 umma_f16_ts(d_tmem + TN, a2 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, 1u);                      // A2 W1, to A1 W2
-              } else if constexpr (SPLIT) {
-                // one tile only: the second accumulator takes the two cross products
-                umma_f16_ts(d_tmem, a1 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, (st | ks) != 0 ? 1u : 0u);
-                umma_f16_ts(d_tmem + S::ACC_COLS, a2 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, (st | ks) != 0 ? 1u : 0u);
-                umma_f16_ts(d_tmem + S::ACC_COLS, a1 + ks * 8, db_hi | (b2_lo + ks * 2), idesc, 1u);
               } else {
                 umma_f16_ts(d_tmem, a1 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, (st | ks) != 0 ? 1u : 0u);
                 umma_f16_ts(d_tmem, a2 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, 1u);
@@ -546,7 +549,7 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
     const int row = warp * 32 + lane;               // TMEM lane = tile row
     const uint32_t t_lane = static_cast<uint32_t>(warp * 32) << 16;
     for (int64_t ti = 0; ti < my_tiles; ti++) {
-      const uint32_t buf = static_cast<uint32_t>(ti & 1);
+      const uint32_t buf = static_cast<uint32_t>(ti % NBUF);
       const int slot = static_cast<int>(ti & (kRowSlots - 1));
       const int64_t tile = seg_tile(ti);
       const int64_t m = (tile / tiles_n) * TM + row, nb = (tile % tiles_n) * TN;
@@ -560,7 +563,7 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
         fsc[i] = (FUSE && g.ep.bn_scale && n < g.N) ? __ldg(g.ep.bn_scale + n) : 1.0f;
         fsh[i] = (FUSE && g.ep.bn_shift && n < g.N) ? __ldg(g.ep.bn_shift + n) : 0.0f;
       }
-      if (!mbar_wait(&tfull[buf], static_cast<uint32_t>((ti >> 1) & 1), abort_flag, 5)) break;
+      if (!mbar_wait(&tfull[buf], static_cast<uint32_t>((ti / NBUF) & 1), abort_flag, 5)) break;
       if (!mbar_wait(&rowfull[slot], static_cast<uint32_t>((ti / kRowSlots) & 1), abort_flag, 5)) break;   // long complete
       tc_fence_after();
       const float fa = rowdown[slot * TM + row];
@@ -582,7 +585,7 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
       auto load_chunk = [&](int c, uint32_t (&v1)[32]) {
         const uint32_t t_addr = tmem_base + t_lane + buf * S::ACC_COLS + c * 32;
         tmem_ld32(t_addr, v1);
-        if constexpr (S::STACKED || SPLIT) {      // the cross products sit TN columns further on
+        if constexpr (STACK) {      // the cross products sit TN columns further on
           uint32_t v2[32];
           tmem_ld32(t_addr + TN, v2);
           tmem_ld_wait();
@@ -648,11 +651,14 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
         for (int c = 0; c < TN / 32; c++) {
           uint32_t v1[32];
           load_chunk(c, v1);
+          if (c == TN / 32 - 1) {      // the accumulator is in registers: the next tile may start
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&tempty[buf]);
+          }
           finish(c, v1);
         }
-        tc_fence_before();
-        __syncwarp();          // also: every lane is done with the warp's column factors
-        if (lane == 0) mbar_arrive(&tempty[buf]);
+        __syncwarp();          // every lane is done with the warp's column factors
       } else if constexpr (BAL) {
         // Part of the tile's K range: the raw partial accumulator goes to this CTA's slot (first slot for the tile
         // its run starts in, second for the tile it ends in), the accumulator is handed back, and the warp
@@ -794,6 +800,10 @@ constexpr int64_t kBalancedMaxShare = 4;
 // Split mode: 256 x 256 x 256 (four stages) takes 7.4 us whole and 7.8 us in two parts; from six stages on parts of two
 // stages win (64 x 1024 x 1024, 16 stages: 17.4 -> 8.0 us in eight parts).
 constexpr int64_t kSplitMinStages = 2;
+// 128-column tiles: the wide accumulator from this many stages per tile on.  50176 x 128 x 1152 (18 stages) 40.4 -> 43.5 us,
+// 4096 x 4096 x 512 (8) 47 -> 52, 4096 x 4096 x 1024 (16) 84 -> 85; 3000 x 3000 x 1472 (23) 75 -> 68, 4096 x 4096 x 2048 (32)
+// 159 -> 152, 3136 x 512 x 4608 (72) 50 -> 45 us.
+constexpr int64_t kWideFromStages = 20;
 constexpr int64_t kSplitFromStages = 6;
 template <int TN>
 int64_t tile_count(const Args& g) { return ((g.M + TM - 1) / TM) * ((g.N + TN - 1) / TN); }
@@ -870,24 +880,25 @@ int choose_split(Kernel kernel, int smem_bytes, int dev, int sms, int64_t tiles,
   return 1;
 }
 
-template <int TN, int ASUB, bool FUSE = false>
-cudaError_t launch_fold(Args g, void* workspace, cudaStream_t stream, bool w_prepared) {
+template <int TN, int ASUB, bool FUSE, bool WIDE>
+cudaError_t launch_fold_wide(Args g, void* workspace, cudaStream_t stream, bool w_prepared) {
   using S = Smem<TN>;
   constexpr bool kHasBalanced = ASUB == 1;           // the balanced schedule is built for activation groups of whole words
   constexpr int kBytes = ScaleRing<TN, ASUB>::BYTES;
+  constexpr bool kSplitWide = TN == 128 && !FUSE;
   static_assert(kBytes <= 227 * 1024, "weight stages and the scale ring fit one CTA's shared memory");
   static DeviceOnce configured;
   int dev = 0, sms = 0;
   if (current_device(&dev, &sms) != cudaSuccess) return cudaErrorInvalidDevice;
   if (configured.pending(dev)) {
-    cudaError_t e = cudaFuncSetAttribute(hbmm_fold_kernel<TN, ASUB, FUSE, kPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+    cudaError_t e = cudaFuncSetAttribute(hbmm_fold_kernel<TN, ASUB, FUSE, kPlain, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
     if (e != cudaSuccess) return e;
     if (kHasBalanced) {
-      e = cudaFuncSetAttribute(hbmm_fold_kernel<TN, ASUB, FUSE, kHasBalanced ? kBalanced : kPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+      e = cudaFuncSetAttribute(hbmm_fold_kernel<TN, ASUB, FUSE, kHasBalanced ? kBalanced : kPlain, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
       if (e != cudaSuccess) return e;
     }
     if (!FUSE) {
-      e = cudaFuncSetAttribute(hbmm_fold_kernel<TN, ASUB, FUSE, FUSE ? kPlain : kSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+      e = cudaFuncSetAttribute(hbmm_fold_kernel<TN, ASUB, FUSE, FUSE ? kPlain : kSplit, kSplitWide>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
       if (e != cudaSuccess) return e;
     }
     configured.mark(dev);
@@ -930,10 +941,10 @@ cudaError_t launch_fold(Args g, void* workspace, cudaStream_t stream, bool w_pre
   }
   const int64_t tiles = ((g.M + TM - 1) / TM) * tiles_n;
   if constexpr (!FUSE) {
-    const int split = choose_split(hbmm_fold_kernel<TN, ASUB, FUSE, kSplit>, kBytes, dev, sms, tiles, n_stages);
+    const int split = choose_split(hbmm_fold_kernel<TN, ASUB, FUSE, kSplit, kSplitWide>, kBytes, dev, sms, tiles, n_stages);
     if (split > 1) {
       g.split = split;
-      return launch_pdl_cluster(hbmm_fold_kernel<TN, ASUB, FUSE, kSplit>, dim3(static_cast<unsigned>(tiles * split)), dim3(kThreads),
+      return launch_pdl_cluster(hbmm_fold_kernel<TN, ASUB, FUSE, kSplit, kSplitWide>, dim3(static_cast<unsigned>(tiles * split)), dim3(kThreads),
                                 static_cast<unsigned>(split), kBytes, stream, g, s_map);
     }
   }
@@ -950,10 +961,17 @@ cudaError_t launch_fold(Args g, void* workspace, cudaStream_t stream, bool w_pre
   if (kHasBalanced && balanced_possible<TN>(g, sms) && run * 10 <= plain_walk * 9) {
     ctas = (units + run - 1) / run;                     // no CTA without work
     g.sk_units = run;
-    return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kHasBalanced ? kBalanced : kPlain>, dim3(static_cast<unsigned>(ctas)), dim3(kThreads), kBytes, stream, g, s_map);
+    return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kHasBalanced ? kBalanced : kPlain, WIDE>, dim3(static_cast<unsigned>(ctas)), dim3(kThreads), kBytes, stream, g, s_map);
   }
   const unsigned grid = static_cast<unsigned>(tiles < sms ? tiles : sms);   // one persistent CTA per SM
-  return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kPlain>, dim3(grid), dim3(kThreads), kBytes, stream, g, s_map);
+  return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kPlain, WIDE>, dim3(grid), dim3(kThreads), kBytes, stream, g, s_map);
+}
+
+template <int TN, int ASUB, bool FUSE = false>
+cudaError_t launch_fold(const Args& g, void* workspace, cudaStream_t stream, bool w_prepared) {
+  const int64_t n_stages = (g.n_words + WPS - 1) / WPS;
+  if (TN == 128 && n_stages >= kWideFromStages) return launch_fold_wide<TN, ASUB, FUSE, TN == 128>(g, workspace, stream, w_prepared);
+  return launch_fold_wide<TN, ASUB, FUSE, false>(g, workspace, stream, w_prepared);
 }
 
 template <int TN>

@@ -45,3 +45,30 @@ def test_split_tiles_match_oracle(M, N, K, ba, bw, sdt):
         assert torch.equal(C[:, :N], outs[0][:, :N])
     gu.assert_close_rel_absref(outs[0][:, :N].cpu().numpy(), c_ref, absref, 1e-5, "split", fine)
     assert hbmm.last_device_error() == 0
+
+
+@pytest.mark.parametrize("M,N,K,ba,bw", [
+    (1300, 1030, 1248, 32, 32),       # 20 stages, 99 tiles: wide accumulator under the balanced schedule
+    (1300, 1030, 1216, 32, 32),       # 19: two narrow ones
+    (2500, 1000, 1312, 16, 16),       # 160 tiles, whole ones, the last stage of one word
+    (2400, 1001, 1280, 8, 8),
+])
+def test_long_tiles_match_oracle(M, N, K, ba, bw):
+    import gpu_util as gu
+    from paper_1905_10759_b200 import hbmm
+    a, w = inputs.normal((M, K), 4500 + M + K + ba), inputs.he_normal(N, K, 5500 + N + K + bw)
+    A, da, sa = gu.oracle_operand(a, ba, 0)
+    W, dw, sw = gu.oracle_operand(w, bw, 0)
+    ws = torch.empty(hbmm.gemm_workspace_bytes(A, W), dtype=torch.uint8, device="cuda")
+    C = torch.full((M, (N + 3) // 4 * 4 + 4), float("nan"), device="cuda")
+    hbmm.gemm_ex(A, W, C, hbmm.PATH_FOLDED, ws)
+    assert torch.isnan(C[:, N:]).all()
+    rows = list(range(0, M, 97)) + [M - 1]
+    c_ref, absref = oracle.hbmm_from_quantized(da[rows], sa[rows], ba, dw, sw, bw)
+    fine = gu.elementwise_magnitude(da[rows], ba, dw, bw, K)
+    gu.assert_close_rel_absref(C[rows, :N].cpu().numpy(), c_ref, absref, 1e-5, "long tiles", fine)
+    # all the other rows: the same product on the integer pipe, which the oracle holds to 1e-5 as well
+    P = torch.empty_like(C)
+    hbmm.gemm_ex(A, W, P, hbmm.PATH_POPC)
+    diff = (C[:, :N] - P[:, :N]).double()
+    assert float(diff.norm() / P[:, :N].double().norm()) < 1e-5
