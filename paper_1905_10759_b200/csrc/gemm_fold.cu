@@ -210,7 +210,15 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
   // the CTA that completes a shared tile does so in the shadow of the MMAs of its whole tiles, not at the kernel's end.
   const bool reorder = balanced && my_tiles >= 3;
   auto seg_nat = [&](int64_t ti) -> int64_t { return !reorder ? ti : (ti == 0 ? 0 : (ti == 1 ? my_tiles - 1 : ti - 1)); };
-  auto seg_tile = [&](int64_t ti) -> int64_t { return SPLIT ? sp_tile : balanced ? sk_t0 + seg_nat(ti) : blockIdx.x + ti * gridDim.x; };
+  // Plain schedule: where the expanded weights are larger than what the L2 keeps, the tiles are walked in blocks of
+  // g.group_n column tiles, row by row inside a block, so that all row tiles of a block read the same few columns' weights.
+  auto in_blocks = [&](int64_t t) -> int64_t {
+    if (g.group_n == 0 || t >= n_tiles) return t;
+    const int64_t blk = t / (g.group_n * tiles_m), r = t - blk * (g.group_n * tiles_m);
+    const int64_t n0 = blk * g.group_n, w = tiles_n - n0 < g.group_n ? tiles_n - n0 : g.group_n;
+    return (r / w) * tiles_n + n0 + r % w;
+  };
+  auto seg_tile = [&](int64_t ti) -> int64_t { return SPLIT ? sp_tile : balanced ? sk_t0 + seg_nat(ti) : in_blocks(blockIdx.x + ti * gridDim.x); };
   auto seg_begin = [&](int64_t ti) -> int64_t { return SPLIT ? sp_begin : (balanced && ti < my_tiles && seg_nat(ti) == 0) ? sk_first : 0; };
   auto seg_end = [&](int64_t ti) -> int64_t { return SPLIT ? sp_end : (balanced && ti < my_tiles && seg_nat(ti) == my_tiles - 1) ? sk_last_end : n_stages; };
 
@@ -783,6 +791,7 @@ Args make_args(const PackedView& A, const PackedView& W, float* C, int64_t ldc) 
   g.sk_units = 0; g.sk_counters = nullptr; g.sk_counter_count = 0; g.sk_partials = nullptr;
   g.a_staged = 0; g.a_rowmax = nullptr;
   g.split = 1;
+  g.group_n = 0;
   return g;
 }
 
@@ -800,11 +809,17 @@ constexpr int64_t kBalancedMaxShare = 4;
 // Split mode: 256 x 256 x 256 (four stages) takes 7.4 us whole and 7.8 us in two parts; from six stages on parts of two
 // stages win (64 x 1024 x 1024, 16 stages: 17.4 -> 8.0 us in eight parts).
 constexpr int64_t kSplitMinStages = 2;
+constexpr int64_t kSplitFromStages = 6;
 // 128-column tiles: the wide accumulator from this many stages per tile on.  50176 x 128 x 1152 (18 stages) 40.4 -> 43.5 us,
 // 4096 x 4096 x 512 (8) 47 -> 52, 4096 x 4096 x 1024 (16) 84 -> 85; 3000 x 3000 x 1472 (23) 75 -> 68, 4096 x 4096 x 2048 (32)
 // 159 -> 152, 3136 x 512 x 4608 (72) 50 -> 45 us.
 constexpr int64_t kWideFromStages = 20;
-constexpr int64_t kSplitFromStages = 6;
+// Plain schedule: above this many bytes of expanded weights the tiles are walked in blocks of as many columns as hold
+// kBlockBytes of them.  Row by row over all columns every wave of CTAs read all of the weights again, from memory once they
+// exceed the L2 (8192^3: 268 MB a wave, 7.5 GB in all, under the power cap): 3.29 -> 2.49 ms with blocks of 8, 18 or 36 MB
+// (2.49 / 2.51 / 2.53), 4096^3 (67 MB) 304 -> 289 us.  Below, the L2 holds them whatever the order.
+constexpr size_t kWeightsInL2 = size_t{48} << 20;
+constexpr size_t kBlockBytes = size_t{18} << 20;
 template <int TN>
 int64_t tile_count(const Args& g) { return ((g.M + TM - 1) / TM) * ((g.N + TN - 1) / TN); }
 template <int TN>
@@ -964,6 +979,10 @@ cudaError_t launch_fold_wide(Args g, void* workspace, cudaStream_t stream, bool 
     return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kHasBalanced ? kBalanced : kPlain, WIDE>, dim3(static_cast<unsigned>(ctas)), dim3(kThreads), kBytes, stream, g, s_map);
   }
   const unsigned grid = static_cast<unsigned>(tiles < sms ? tiles : sms);   // one persistent CTA per SM
+  if (stage_bytes<TN>(g) > kWeightsInL2) {
+    g.group_n = static_cast<int64_t>(kBlockBytes / (static_cast<size_t>(n_stages) * S::B_STAGE));
+    if (g.group_n < 1) g.group_n = 1;
+  }
   return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kPlain, WIDE>, dim3(grid), dim3(kThreads), kBytes, stream, g, s_map);
 }
 

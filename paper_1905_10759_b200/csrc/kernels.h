@@ -135,6 +135,7 @@ struct FoldArgs {
   int64_t sk_counter_count;
   float* sk_partials;            // [2 * CTAs][128][TN]
   float* a_rowmax;               // sub-word groups: largest scale of every activation row (nullptr: the scouts scan the rows)
+  int64_t group_n;               // column tiles per block of the plain schedule's walk; 0: row by row over all columns
   int32_t split;                 // CTAs (one cluster) that share a tile's K range in split mode
   int32_t a_staged;              // sub-word groups: the activation scales of a stage reach the producers through shared memory
 };

@@ -72,3 +72,23 @@ def test_long_tiles_match_oracle(M, N, K, ba, bw):
     hbmm.gemm_ex(A, W, P, hbmm.PATH_POPC)
     diff = (C[:, :N] - P[:, :N]).double()
     assert float(diff.norm() / P[:, :N].double().norm()) < 1e-5
+
+
+def test_tiles_walked_in_blocks_of_columns():
+    """More expanded weights than the L2 keeps: every tile is still formed once (blocks of 11 columns, a last one of 10; row
+    and column remainders).  Against the integer pipe, which the oracle holds to 1e-5 elsewhere."""
+    from paper_1905_10759_b200 import hbmm
+    M, N, K, b = 2500, 4090, 3200, 32
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(7)
+    x, w = (torch.randn((r, K), generator=gen, device="cuda") for r in (M, N))
+    A, W = hbmm.quantize(x, hbmm.alloc_operand(M, K, b)), hbmm.quantize(w, hbmm.alloc_operand(N, K, b))
+    ws = torch.empty(hbmm.gemm_workspace_bytes(A, W), dtype=torch.uint8, device="cuda")
+    C = torch.full((M, 4096), float("nan"), device="cuda")
+    P = torch.empty_like(C)
+    hbmm.gemm_ex(A, W, C, hbmm.PATH_FOLDED, ws)
+    hbmm.gemm_ex(A, W, P, hbmm.PATH_POPC)
+    assert torch.isnan(C[:, N:]).all()
+    diff, ref = (C[:, :N] - P[:, :N]).double(), P[:, :N].double()
+    assert float(diff.norm() / ref.norm()) < 1e-5
+    assert float(diff.abs().max()) < 1e-3 * float(ref.abs().max())
