@@ -158,8 +158,7 @@ bool launch_rows(int64_t beta, unsigned blocks, cudaStream_t stream, const float
 cudaError_t launch_binarize_backward(const float* x, int64_t ldx, const float* gy, int64_t ldg, int64_t rows, int64_t K, int32_t beta,
                                      float* gx, int64_t ldo, cudaStream_t stream) {
   int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  current_device(&dev, &sms);
   const int64_t beff = beta >= K ? K : beta;
   const bool aligned = reinterpret_cast<uintptr_t>(x) % 16 == 0 && reinterpret_cast<uintptr_t>(gy) % 16 == 0 &&
                        reinterpret_cast<uintptr_t>(gx) % 16 == 0;

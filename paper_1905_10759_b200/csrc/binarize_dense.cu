@@ -192,8 +192,7 @@ cudaError_t launch_typed(const float* x, int64_t ldx, int64_t rows, int64_t K, i
 cudaError_t launch_binarize_dense(const float* x, int64_t ldx, int64_t rows, int64_t K, int32_t beta, void* out, bool out_bf16,
                                   int64_t ldo, cudaStream_t stream) {
   int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  current_device(&dev, &sms);
   const int64_t beff = beta >= K ? K : beta;
   if (out_bf16) return launch_typed(x, ldx, rows, K, beff, static_cast<__nv_bfloat16*>(out), ldo, sms, stream);
   return launch_typed(x, ldx, rows, K, beff, static_cast<float*>(out), ldo, sms, stream);

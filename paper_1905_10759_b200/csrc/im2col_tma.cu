@@ -477,8 +477,7 @@ bool im2col_quantize_tma_supported(const void* x, int x_bf16, const ConvGeom& g,
 cudaError_t launch_im2col_quantize_tma(const void* x, const ConvGeom& g, int32_t beta, uint32_t* bits, int64_t ld_words, void* scales,
                                        int64_t ld_scales, int scale_bf16, cudaStream_t stream, const UmmaPrepJob* prep) {
   int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  current_device(&dev, &sms);
   const int mode = tma_mode(x, 0, g, beta);
   Plan p;
   size_t smem;

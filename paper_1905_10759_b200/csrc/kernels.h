@@ -15,11 +15,16 @@ struct DeviceOnce {
   bool pending(int dev) const { return dev < 0 || dev >= 64 || !((mask.load(std::memory_order_acquire) >> dev) & 1u); }
   void mark(int dev) { if (dev >= 0 && dev < 64) mask.fetch_or(uint64_t{1} << dev, std::memory_order_release); }
 };
-// Current device and its multiprocessor count.
+// Current device and its multiprocessor count (asked for once per device).
 inline cudaError_t current_device(int* dev, int* sms) {
+  static std::atomic<int> known[64];
   cudaError_t e = cudaGetDevice(dev);
   if (e != cudaSuccess) return e;
-  return cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, *dev);
+  const bool cached = *dev >= 0 && *dev < 64;
+  if (cached && (*sms = known[*dev].load(std::memory_order_relaxed)) > 0) return cudaSuccess;
+  e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, *dev);
+  if (e == cudaSuccess && cached) known[*dev].store(*sms, std::memory_order_relaxed);
+  return e;
 }
 
 // Device-side view of one packed Hadamard-binary operand (validated by the caller).

@@ -413,8 +413,7 @@ cudaError_t launch_quantize(const void* x, int x_bf16, int64_t rows, int64_t K, 
   const int wpw = x_bf16 ? 8 : 4;
   const bool pow2 = (beta_words & (beta_words - 1)) == 0;
   int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  current_device(&dev, &sms);
   if (!one_group && vec_ok && ldx == K && K % 32 == 0 && K % beta == 0 && K / 32 < (int64_t{1} << 31) && rows < (int64_t{1} << 31)) {
     const int64_t total_words = rows * (K / 32);
     int64_t blocks = ((total_words + 15) / 16 + (kThreads / 32) - 1) / (kThreads / 32);
