@@ -90,10 +90,106 @@ struct ScaleRing {
   }
 };
 
-template <int TN>
-__global__ void __launch_bounds__(TN)
-prepare_w_fold_kernel(const Args g, unsigned char* __restrict__ out, float* __restrict__ w_down) {
-  prepare_w_task<TN>(g, out, w_down, blockIdx.x, blockIdx.y, threadIdx.x);
+// The whole weight expansion as a launch of its own: a CTA takes one column tile and `spc` stages.  Bound by its writes (4 K
+// bytes per weight row), so eight consecutive lanes fill the 128 bytes of one tile row (a warp's store is four whole lines;
+// one thread per row leaves every 16-byte store in a line of its own) and a row's scales are scanned once per CTA by 256 / TN
+// threads -- or, with 512 scales and more per row, once per call by a kernel of their own (known_down).  4096 x 4096 at
+// beta 64: 36 us in the one-thread-per-row tasks of two stages that the convolution front end runs, 15.3 us here; 4096 x 9216
+// at beta 2 (each of 72 tasks scanned 4608 scales per row): 1.46 ms against 0.06.
+constexpr int kPrepThreads = 256;
+template <int TN, int SUB>
+__global__ void __launch_bounds__(kPrepThreads)
+prepare_w_fold_kernel(const Args g, unsigned char* __restrict__ out, float* __restrict__ w_down, int spc, int known_down) {
+  using S = Smem<TN>;
+  __shared__ float s_up[TN];
+  constexpr int PARTS = kPrepThreads / TN;
+  const int tid = threadIdx.x;
+  const int64_t n_stages = (g.n_words + WPS - 1) / WPS, tile_n = blockIdx.y;
+  if (g.sk_counters != nullptr) {
+    // the per-tile arrival counters of the balanced schedule start at zero; every launch leaves them there
+    const int64_t ctas = static_cast<int64_t>(gridDim.x) * gridDim.y, cta = blockIdx.y * static_cast<int64_t>(gridDim.x) + blockIdx.x;
+    for (int64_t i = cta * kPrepThreads + tid; i < g.sk_counter_count; i += ctas * kPrepThreads) g.sk_counters[i] = 0;
+  }
+  {
+    const int row = tid / PARTS;
+    const int64_t n = tile_n * TN + row;
+    float up = 0.0f, down = 1.0f;
+    if (known_down) {
+      if (n < g.N) up = __uint_as_float((254u << 23) - __float_as_uint(__ldg(w_down + n)));      // 1 / a power of two
+    } else {
+      uint32_t mx = n < g.N ? row_max_part<PARTS>(g.w_scales, g.w_bf16, n * g.ldw_s, g.ldw_s, tid % PARTS) : 0u;
+#pragma unroll
+      for (int o = 1; o < PARTS; o <<= 1) mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+      if (n < g.N) norm_factors(__uint_as_float(mx), up, down);
+      if (blockIdx.x == 0 && tid % PARTS == 0) w_down[n] = down;
+    }
+    if (tid % PARTS == 0) s_up[row] = up;
+  }
+  __syncthreads();
+  const int64_t st0 = static_cast<int64_t>(blockIdx.x) * spc, st1 = st0 + spc < n_stages ? st0 + spc : n_stages;
+  for (int64_t st = st0; st < st1; st++) {
+    unsigned char* base = out + (tile_n * n_stages + st) * S::B_STAGE;
+#pragma unroll
+    for (int i = tid; i < TN * 8; i += kPrepThreads) {
+      // physical piece j of the row holds logical piece j ^ (row % 8): word slot q, element pairs 4 c .. 4 c + 3 of the word
+      const int row = i >> 3, j = i & 7, lp = j ^ (row & 7), q = lp >> 2, c = lp & 3;
+      const int64_t n = tile_n * TN + row, wi = st * WPS + q;
+      uint32_t o1[4] = {0u, 0u, 0u, 0u}, o2[4] = {0u, 0u, 0u, 0u};
+      if (n < g.N && wi < g.n_words) {
+        const uint32_t nw = ~__ldg(g.w_bits + n * g.ldw_w + wi);
+        const float up = s_up[row];
+        uint32_t h1[4], h2[4];
+        if constexpr (SUB == 1) {
+          const float sc = load_scale(g.w_scales, g.w_bf16, n * g.ldw_s + wi / g.w_gw) * up;
+          const __half d1 = __float2half_rn(sc), d2 = __float2half_rn(sc - __half2float(d1));
+#pragma unroll
+          for (int e = 0; e < 4; e++) {
+            h1[e] = static_cast<uint32_t>(__half_as_ushort(d1)) * 0x10001u;
+            h2[e] = static_cast<uint32_t>(__half_as_ushort(d2)) * 0x10001u;
+          }
+        } else {
+          constexpr int BETA = 32 / SUB, HALF = SUB / 2;
+#pragma unroll
+          for (int e = 0; e < 4; e++) {
+            if (e > 0 && BETA > 1 && (BETA >= 4 || e % BETA != 0)) { h1[e] = h1[e - 1]; h2[e] = h2[e - 1]; continue; }
+            const int t = (4 * c + e) / BETA;          // low half: group t of the word, high half: group t + SUB / 2
+            const int64_t idx = n * g.ldw_s + wi * SUB + t;
+            const float lo = load_scale(g.w_scales, g.w_bf16, idx) * up, hi = load_scale(g.w_scales, g.w_bf16, idx + HALF) * up;
+            const __half2 d1 = __floats2half2_rn(lo, hi);
+            const float2 back = __half22float2(d1);
+            const __half2 d2 = __floats2half2_rn(lo - back.x, hi - back.y);
+            h1[e] = *reinterpret_cast<const uint32_t*>(&d1);
+            h2[e] = *reinterpret_cast<const uint32_t*>(&d2);
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+          const uint32_t m = (nw << (15 - (4 * c + e))) & 0x80008000u;
+          o1[e] = m ^ h1[e];
+          o2[e] = m ^ h2[e];
+        }
+      }
+      *reinterpret_cast<uint4*>(base + row * 128 + j * 16) = make_uint4(o1[0], o1[1], o1[2], o1[3]);
+      *reinterpret_cast<uint4*>(base + S::B_PIECE + row * 128 + j * 16) = make_uint4(o2[0], o2[1], o2[2], o2[3]);
+    }
+  }
+}
+
+// The power of two that undoes the normalisation of every weight row, for rows of many scales: one warp per row; rows past
+// the operand (to the end of the last tile) get 1.
+__global__ void __launch_bounds__(256)
+w_down_kernel(const Args g, int64_t rows_padded, float* __restrict__ w_down) {
+  const int lane = threadIdx.x & 31;
+  const int64_t n = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
+  if (n >= rows_padded) return;
+  float up = 0.0f, down = 1.0f;
+  if (n < g.N) {
+    uint32_t mx = row_max_part<32>(g.w_scales, g.w_bf16, n * g.ldw_s, g.ldw_s, lane);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+    norm_factors(__uint_as_float(mx), up, down);
+  }
+  if (lane == 0) w_down[n] = down;
 }
 
 // Largest scale of every row of an operand with many scales per row (sub-word groups): one warp per row, consecutive
@@ -895,6 +991,24 @@ int choose_split(Kernel kernel, int smem_bytes, int dev, int sms, int64_t tiles,
   return 1;
 }
 
+template <int TN>
+void launch_prepare(const Args& g, unsigned char* stages, float* down, int sms, cudaStream_t stream) {
+  const int64_t tiles_n = (g.N + TN - 1) / TN, n_stages = (g.n_words + WPS - 1) / WPS;
+  // two to sixteen stages per CTA: few enough that every SM has several CTAs, many enough to pay for the scan of the rows
+  int64_t spc = n_stages * tiles_n / (static_cast<int64_t>(sms) * 4);
+  spc = spc < 2 ? 2 : (spc > 16 ? 16 : spc);
+  const bool long_rows = g.ldw_s >= kRowMaxFrom;
+  if (long_rows) w_down_kernel<<<static_cast<unsigned>((tiles_n * TN + 7) / 8), 256, 0, stream>>>(g, tiles_n * TN, down);
+  const dim3 grid(static_cast<unsigned>((n_stages + spc - 1) / spc), static_cast<unsigned>(tiles_n));
+  switch (g.w_sub) {
+    case 2: prepare_w_fold_kernel<TN, 2><<<grid, kPrepThreads, 0, stream>>>(g, stages, down, static_cast<int>(spc), long_rows); break;
+    case 4: prepare_w_fold_kernel<TN, 4><<<grid, kPrepThreads, 0, stream>>>(g, stages, down, static_cast<int>(spc), long_rows); break;
+    case 8: prepare_w_fold_kernel<TN, 8><<<grid, kPrepThreads, 0, stream>>>(g, stages, down, static_cast<int>(spc), long_rows); break;
+    case 16: prepare_w_fold_kernel<TN, 16><<<grid, kPrepThreads, 0, stream>>>(g, stages, down, static_cast<int>(spc), long_rows); break;
+    default: prepare_w_fold_kernel<TN, 1><<<grid, kPrepThreads, 0, stream>>>(g, stages, down, static_cast<int>(spc), long_rows); break;
+  }
+}
+
 template <int TN, int ASUB, bool FUSE, bool WIDE>
 cudaError_t launch_fold_wide(Args g, void* workspace, cudaStream_t stream, bool w_prepared) {
   using S = Smem<TN>;
@@ -922,10 +1036,7 @@ cudaError_t launch_fold_wide(Args g, void* workspace, cudaStream_t stream, bool 
   unsigned char* stages = static_cast<unsigned char*>(workspace);
   float* down = reinterpret_cast<float*>(stages + stage_bytes<TN>(g));
   set_balanced_area<TN>(g, workspace);
-  if (!w_prepared) {
-    dim3 pgrid(static_cast<unsigned>((n_stages + kPrepStages - 1) / kPrepStages), static_cast<unsigned>(tiles_n));
-    prepare_w_fold_kernel<TN><<<pgrid, TN, 0, stream>>>(g, stages, down);
-  }
+  if (!w_prepared) launch_prepare<TN>(g, stages, down, sms, stream);
   g.w_prep = stages;
   g.w_down = down;
   // sub-word groups: the activation scales as a 2-D tensor [M][lda_s] of fp32 for the per-stage block copies
