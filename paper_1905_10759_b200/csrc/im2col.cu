@@ -123,6 +123,53 @@ im2col_quantize_groups_kernel(const void* __restrict__ x, int x_bf16, const Conv
   }
 }
 
+// Groups shorter than a word: one thread per (row m, K-word), 32 consecutive rows per warp as above; a thread emits the word
+// and the means of its 32 / BETA groups.  One thread per row leaves most of the machine idle and walks all of K serially:
+// 3136 rows of 4608 at beta 4 from bf16 1019 us against 43 here, 3025 rows of 12800 at beta 8 2.1 ms against 86 us.
+template <int BETA>
+__global__ void __launch_bounds__(256)
+im2col_quantize_words_kernel(const void* __restrict__ x, int x_bf16, const ConvGeom g, int64_t M, int64_t K, int64_t G, int64_t n_words,
+                             uint32_t* __restrict__ bits, int64_t ld_words, void* __restrict__ scales, int64_t ld_scales, int scale_bf16) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t m = static_cast<int64_t>(blockIdx.x) * 32 + lane;
+  const int64_t wi = static_cast<int64_t>(blockIdx.y) * 8 + warp;
+  if (m >= M || wi >= n_words) return;
+  const int xo = static_cast<int>(m % g.Wo);
+  const int yo = static_cast<int>((m / g.Wo) % g.Ho);
+  const int64_t b = m / (static_cast<int64_t>(g.Wo) * g.Ho);
+  const int taps = g.kh * g.kw;
+  const int64_t HW = static_cast<int64_t>(g.H) * g.W, base = b * g.C * HW;
+  const int y0 = yo * g.sh - g.ph, x0 = xo * g.sw - g.pw;
+  const int64_t k0 = wi * 32;
+  int c = static_cast<int>(k0 / taps);
+  const int r = static_cast<int>(k0 - static_cast<int64_t>(c) * taps);
+  int i = r / g.kw, j = r - i * g.kw;
+  uint32_t word = 0;
+#pragma unroll
+  for (int t = 0; t < 32 / BETA; t++) {
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int e = 0; e < BETA; e++) {
+      if (k0 + t * BETA + e < K) {
+        const int y = y0 + i, xx = x0 + j;
+        float v = 0.0f;
+        if (y >= 0 && y < g.H && xx >= 0 && xx < g.W) v = load_x(x, x_bf16, base + c * HW + static_cast<int64_t>(y) * g.W + xx);
+        word |= (v >= 0.0f ? 1u : 0u) << (t * BETA + e);
+        s[e & 3] += fabsf(v);
+        if (++j == g.kw) { j = 0; if (++i == g.kh) { i = 0; c++; } }
+      }
+    }
+    const int64_t left = K - (k0 + t * BETA);
+    if (left > 0)
+      store_scale(scales, scale_bf16, m * ld_scales + wi * (32 / BETA) + t, ((s[0] + s[1]) + (s[2] + s[3])) / static_cast<float>(left < BETA ? left : BETA));
+  }
+  bits[m * ld_words + wi] = word;
+  if (wi == n_words - 1) {
+    for (int64_t w = n_words; w < ld_words; w++) bits[m * ld_words + w] = 0u;
+    for (int64_t z = G; z < ld_scales; z++) store_scale(scales, scale_bf16, m * ld_scales + z, 0.0f);
+  }
+}
+
 __global__ void __launch_bounds__(256)
 im2col_bf16_kernel(const void* __restrict__ x, int x_bf16, const ConvGeom g, int64_t M, int64_t K,
                    __nv_bfloat16* __restrict__ out, int64_t ld) {
@@ -406,6 +453,14 @@ cudaError_t launch_im2col_quantize(const void* x, int x_bf16, const ConvGeom& g,
     dim3 grid(static_cast<unsigned>((M + 31) / 32), static_cast<unsigned>((G + 7) / 8));
     im2col_quantize_groups_kernel<<<grid, 256, 0, stream>>>(x, x_bf16, g, M, K, beta / 32, G, (K + 31) / 32, bits,
                                                              ld_words, scales, ld_scales, scale_bf16);
+    return cudaGetLastError();
+  }
+  const int64_t n_words = (K + 31) / 32, word_blocks = (n_words + 7) / 8;
+  if (beta < K && (beta == 2 || beta == 4 || beta == 8 || beta == 16) && word_blocks <= 65535) {
+    const dim3 grid(static_cast<unsigned>((M + 31) / 32), static_cast<unsigned>(word_blocks));
+#define HBMM_IW(B) case B: im2col_quantize_words_kernel<B><<<grid, 256, 0, stream>>>(x, x_bf16, g, M, K, G, n_words, bits, ld_words, scales, ld_scales, scale_bf16); break;
+    switch (beta) { HBMM_IW(2) HBMM_IW(4) HBMM_IW(8) HBMM_IW(16) }
+#undef HBMM_IW
     return cudaGetLastError();
   }
   const int64_t blocks = (M + kThreads - 1) / kThreads;

@@ -1,0 +1,52 @@
+"""Packed convolution front end on strided filters (tensor-copy tiles of fewer rows, whole channel planes) and on the gather
+for groups shorter than a word (bf16 images, odd widths, large filters, K ending inside a word): the packed operand left in
+the workspace against the oracle's binarization of the im2col rows."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1905_10759_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # B, C, H, W, k, stride, beta, bf16
+    (2, 64, 56, 56, 3, 2, 32, False),     # two tiles fit only with fewer output rows
+    (3, 40, 28, 28, 3, 2, 64, False),     # short last channel chunk, groups of two words
+    (2, 64, 14, 14, 3, 2, 32, False),     # whole planes
+    (2, 32, 13, 16, 3, 2, 8, False),
+    (2, 64, 8, 8, 1, 2, 4, False),
+    (1, 32, 60, 60, 5, 3, 32, False),
+    (2, 100, 9, 9, 3, 1, 16, False),      # odd width, K = 900
+    (2, 33, 7, 7, 5, 1, 2, False),        # K = 825
+    (2, 48, 12, 12, 3, 2, 4, True),       # bf16 image
+    (1, 5, 11, 10, 3, 1, 8, True),        # K = 45: two words, a short group
+]
+
+
+@pytest.mark.parametrize("B,C,H,W,k,st,beta,bf16", CASES)
+def test_packed_rows_match_oracle(B, C, H, W, k, st, beta, bf16):
+    import gpu_util as gu
+    from paper_1905_10759_b200 import hbmm
+    K, pad = C * k * k, k // 2
+    x = inputs.normal((B * C * H, W), 650 + C + H).reshape(B, C, H, W)
+    if bf16:
+        x = torch.from_numpy(x).bfloat16().float().numpy()
+    Wop = hbmm.quantize(torch.from_numpy(inputs.he_normal(40, K, 651)).cuda(), hbmm.alloc_operand(40, K, max(beta, 32)))
+    geom = hbmm.make_geom(B, C, H, W, k, k, (st, st), (pad, pad))
+    M = B * ((H + 2 * pad - k) // st + 1) * ((W + 2 * pad - k) // st + 1)
+    ws = torch.empty(hbmm.conv_workspace_bytes(geom, beta, hbmm.F32, Wop), dtype=torch.uint8, device="cuda").fill_(0xAB)
+    xd = torch.from_numpy(x).cuda()
+    hbmm.conv_im2col(xd.bfloat16() if bf16 else xd, geom, beta, hbmm.F32, Wop, None, ws, flags=hbmm.CONV_PACK_ONLY)
+    bb, sb, lw, ls = hbmm.operand_bytes(M, K, beta, hbmm.F32)
+    bits = ws[:bb].view(torch.int32).reshape(M, lw)
+    off = (bb + 255) // 256 * 256
+    sc = ws[off: off + sb].view(torch.float32).reshape(M, ls).cpu().numpy().astype(np.float64)
+    da, sa = oracle.quantize(oracle.im2col(x, k, k, (st, st), (pad, pad)), beta)
+    assert np.array_equal(gu.host_bits(bits), oracle.pack(sa, lw))
+    G = da.shape[1]
+    assert np.all(sc[:, G:] == 0.0)
+    # four partial sums of a word's or group's elements in turn, joined pairwise, one division
+    np.testing.assert_allclose(sc[:, :G], da, rtol=(min(beta, 32) // 4 + int(np.ceil(np.log2(beta))) + 3) * gu.U, atol=0)
+    assert hbmm.last_device_error() == 0
