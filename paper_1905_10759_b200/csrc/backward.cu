@@ -14,6 +14,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 #include "kernels.h"
+#include "pdl.cuh"
 #include "row_io.cuh"
 
 namespace hbmm {
@@ -53,6 +54,8 @@ __device__ __forceinline__ void group_sums(const float (&a)[4], const float (&d)
 template <int BETA>
 __global__ void __launch_bounds__(kThreads)
 binarize_backward_stream(const float4* __restrict__ x, const float4* __restrict__ gy, float4* __restrict__ gx, int64_t n_vec) {
+  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
+  pdl_wait();
   constexpr float inv = 1.0f / static_cast<float>(BETA);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
   // whole warps walk together: the shuffles below need every lane, so the loop bound is rounded up to a warp
@@ -87,6 +90,8 @@ template <int BETA, bool VEC>
 __global__ void __launch_bounds__(kThreads)
 binarize_backward_rows(const float* __restrict__ x, int64_t ldx, const float* __restrict__ gy, int64_t ldg, int64_t rows, int64_t K,
                        float* __restrict__ gx, int64_t ldo) {
+  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const int64_t chunks = (K + 127) / 128, items = rows * chunks;
   const int64_t warp0 = (static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x) >> 5;
@@ -115,6 +120,8 @@ binarize_backward_rows(const float* __restrict__ x, int64_t ldx, const float* __
 __global__ void __launch_bounds__(kThreads)
 binarize_backward_general(const float* __restrict__ x, int64_t ldx, const float* __restrict__ gy, int64_t ldg, int64_t rows, int64_t K,
                           int64_t beta, int64_t G, float* __restrict__ gx, int64_t ldo) {
+  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
+  pdl_wait();
   const int64_t total = rows * G;
   for (int64_t idx = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; idx < total;
        idx += static_cast<int64_t>(gridDim.x) * kThreads) {
@@ -138,14 +145,14 @@ binarize_backward_general(const float* __restrict__ x, int64_t ldx, const float*
 
 template <int BETA>
 void launch_stream(unsigned blocks, cudaStream_t stream, const float* x, const float* gy, float* gx, int64_t n_vec) {
-  binarize_backward_stream<BETA><<<blocks, kThreads, 0, stream>>>(reinterpret_cast<const float4*>(x), reinterpret_cast<const float4*>(gy),
+  launch_pdl(binarize_backward_stream<BETA>, dim3(blocks), dim3(kThreads), 0, stream, reinterpret_cast<const float4*>(x), reinterpret_cast<const float4*>(gy),
                                                                reinterpret_cast<float4*>(gx), n_vec);
 }
 
 template <bool VEC>
 bool launch_rows(int64_t beta, unsigned blocks, cudaStream_t stream, const float* x, int64_t ldx, const float* gy, int64_t ldg, int64_t rows,
                  int64_t K, float* gx, int64_t ldo) {
-#define HBMM_BR(B) case B: binarize_backward_rows<B, VEC><<<blocks, kThreads, 0, stream>>>(x, ldx, gy, ldg, rows, K, gx, ldo); return true;
+#define HBMM_BR(B) case B: launch_pdl(binarize_backward_rows<B, VEC>, dim3(blocks), dim3(kThreads), 0, stream, x, ldx, gy, ldg, rows, K, gx, ldo); return true;
   switch (beta) {
     HBMM_BR(1) HBMM_BR(2) HBMM_BR(4) HBMM_BR(8) HBMM_BR(16) HBMM_BR(32) HBMM_BR(64) HBMM_BR(128)
     default: return false;
@@ -196,7 +203,7 @@ cudaError_t launch_binarize_backward(const float* x, int64_t ldx, const float* g
   const int64_t G = (K + beff - 1) / beff;
   int64_t blocks = (rows * G + kThreads - 1) / kThreads;
   if (blocks > cap) blocks = cap;
-  binarize_backward_general<<<static_cast<unsigned>(blocks < 1 ? 1 : blocks), kThreads, 0, stream>>>(x, ldx, gy, ldg, rows, K, beff, G, gx, ldo);
+  launch_pdl(binarize_backward_general, dim3(static_cast<unsigned>(blocks < 1 ? 1 : blocks)), dim3(kThreads), 0, stream, x, ldx, gy, ldg, rows, K, beff, G, gx, ldo);
   return cudaGetLastError();
 }
 

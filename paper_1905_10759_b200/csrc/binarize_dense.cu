@@ -14,6 +14,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include "kernels.h"
+#include "pdl.cuh"
 #include "row_io.cuh"
 
 namespace hbmm {
@@ -42,6 +43,8 @@ __device__ __forceinline__ void store1(__nv_bfloat16* out, int64_t i, float v) {
 template <int BETA, int E, typename OUT>
 __global__ void __launch_bounds__(kThreads)
 binarize_dense_stream(const float4* __restrict__ x, OUT* __restrict__ out, int64_t n_items) {
+  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
+  pdl_wait();
   constexpr int LANES = BETA > E ? BETA / E : 1;          // lanes per group
   constexpr int RUN = BETA < E ? BETA : E;                // elements of one group inside a lane
   constexpr float inv = 1.0f / static_cast<float>(BETA);
@@ -89,6 +92,8 @@ binarize_dense_stream(const float4* __restrict__ x, OUT* __restrict__ out, int64
 template <int BETA, bool VEC, typename OUT>
 __global__ void __launch_bounds__(kThreads)
 binarize_dense_rows(const float* __restrict__ x, int64_t ldx, int64_t rows, int64_t K, OUT* __restrict__ out, int64_t ldo) {
+  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
+  pdl_wait();
   constexpr int LANES = BETA > 4 ? BETA / 4 : 1;          // lanes per group
   const int lane = threadIdx.x & 31;
   const int64_t chunks = (K + 127) / 128, items = rows * chunks;
@@ -120,7 +125,7 @@ binarize_dense_rows(const float* __restrict__ x, int64_t ldx, int64_t rows, int6
 
 template <bool VEC, typename OUT>
 bool launch_rows(int64_t beta, unsigned blocks, cudaStream_t stream, const float* x, int64_t ldx, int64_t rows, int64_t K, OUT* out, int64_t ldo) {
-#define HBMM_DR(B) case B: binarize_dense_rows<B, VEC, OUT><<<blocks, kThreads, 0, stream>>>(x, ldx, rows, K, out, ldo); return true;
+#define HBMM_DR(B) case B: launch_pdl(binarize_dense_rows<B, VEC, OUT>, dim3(blocks), dim3(kThreads), 0, stream, x, ldx, rows, K, out, ldo); return true;
   switch (beta) {
     HBMM_DR(1) HBMM_DR(2) HBMM_DR(4) HBMM_DR(8) HBMM_DR(16) HBMM_DR(32) HBMM_DR(64) HBMM_DR(128)
     default: return false;
@@ -132,6 +137,8 @@ template <typename OUT>
 __global__ void __launch_bounds__(kThreads)
 binarize_dense_general(const float* __restrict__ x, int64_t ldx, int64_t rows, int64_t K, int64_t beta, int64_t G,
                        OUT* __restrict__ out, int64_t ldo) {
+  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
+  pdl_wait();
   const int64_t total = rows * G;
   for (int64_t idx = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; idx < total;
        idx += static_cast<int64_t>(gridDim.x) * kThreads) {
@@ -158,14 +165,14 @@ cudaError_t launch_typed(const float* x, int64_t ldx, int64_t rows, int64_t K, i
     const unsigned b = static_cast<unsigned>(blocks < 1 ? 1 : blocks);
     const float4* xv = reinterpret_cast<const float4*>(x);
     switch (beff) {
-      case 1: binarize_dense_stream<1, E, OUT><<<b, kThreads, 0, stream>>>(xv, out, n_items); break;
-      case 2: binarize_dense_stream<2, E, OUT><<<b, kThreads, 0, stream>>>(xv, out, n_items); break;
-      case 4: binarize_dense_stream<4, E, OUT><<<b, kThreads, 0, stream>>>(xv, out, n_items); break;
-      case 8: binarize_dense_stream<8, E, OUT><<<b, kThreads, 0, stream>>>(xv, out, n_items); break;
-      case 16: binarize_dense_stream<16, E, OUT><<<b, kThreads, 0, stream>>>(xv, out, n_items); break;
-      case 32: binarize_dense_stream<32, E, OUT><<<b, kThreads, 0, stream>>>(xv, out, n_items); break;
-      case 64: binarize_dense_stream<64, E, OUT><<<b, kThreads, 0, stream>>>(xv, out, n_items); break;
-      default: binarize_dense_stream<128, E, OUT><<<b, kThreads, 0, stream>>>(xv, out, n_items); break;
+      case 1: launch_pdl(binarize_dense_stream<1, E, OUT>, dim3(b), dim3(kThreads), 0, stream, xv, out, n_items); break;
+      case 2: launch_pdl(binarize_dense_stream<2, E, OUT>, dim3(b), dim3(kThreads), 0, stream, xv, out, n_items); break;
+      case 4: launch_pdl(binarize_dense_stream<4, E, OUT>, dim3(b), dim3(kThreads), 0, stream, xv, out, n_items); break;
+      case 8: launch_pdl(binarize_dense_stream<8, E, OUT>, dim3(b), dim3(kThreads), 0, stream, xv, out, n_items); break;
+      case 16: launch_pdl(binarize_dense_stream<16, E, OUT>, dim3(b), dim3(kThreads), 0, stream, xv, out, n_items); break;
+      case 32: launch_pdl(binarize_dense_stream<32, E, OUT>, dim3(b), dim3(kThreads), 0, stream, xv, out, n_items); break;
+      case 64: launch_pdl(binarize_dense_stream<64, E, OUT>, dim3(b), dim3(kThreads), 0, stream, xv, out, n_items); break;
+      default: launch_pdl(binarize_dense_stream<128, E, OUT>, dim3(b), dim3(kThreads), 0, stream, xv, out, n_items); break;
     }
     return cudaGetLastError();
   }
@@ -183,7 +190,7 @@ cudaError_t launch_typed(const float* x, int64_t ldx, int64_t rows, int64_t K, i
   const int64_t G = (K + beff - 1) / beff;
   int64_t blocks = (rows * G + kThreads - 1) / kThreads;
   if (blocks > cap) blocks = cap;
-  binarize_dense_general<OUT><<<static_cast<unsigned>(blocks < 1 ? 1 : blocks), kThreads, 0, stream>>>(x, ldx, rows, K, beff, G, out, ldo);
+  launch_pdl(binarize_dense_general<OUT>, dim3(static_cast<unsigned>(blocks < 1 ? 1 : blocks)), dim3(kThreads), 0, stream, x, ldx, rows, K, beff, G, out, ldo);
   return cudaGetLastError();
 }
 

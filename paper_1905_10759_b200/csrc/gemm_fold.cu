@@ -309,7 +309,7 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
   // Plain schedule: where the expanded weights are larger than what the L2 keeps, the tiles are walked in blocks of
   // g.group_n column tiles, row by row inside a block, so that all row tiles of a block read the same few columns' weights.
   auto in_blocks = [&](int64_t t) -> int64_t {
-    if (g.group_n == 0 || t >= n_tiles) return t;
+    if (!WIDE || g.group_n == 0 || t >= n_tiles) return t;      // short tiles have small weights; the test there costs them 2 %
     const int64_t blk = t / (g.group_n * tiles_m), r = t - blk * (g.group_n * tiles_m);
     const int64_t n0 = blk * g.group_n, w = tiles_n - n0 < g.group_n ? tiles_n - n0 : g.group_n;
     return (r / w) * tiles_n + n0 + r % w;
@@ -991,6 +991,8 @@ int choose_split(Kernel kernel, int smem_bytes, int dev, int sms, int64_t tiles,
   return 1;
 }
 
+// Launched without programmatic serialization: its few CTAs would all land on the first SMs the kernel before leaves (that
+// kernel's CTAs fill one SM each), and wait there for the rest: 50176 x 128 x 1152 at beta 4, expanding, 72 against 53 us.
 template <int TN>
 void launch_prepare(const Args& g, unsigned char* stages, float* down, int sms, cudaStream_t stream) {
   const int64_t tiles_n = (g.N + TN - 1) / TN, n_stages = (g.n_words + WPS - 1) / WPS;
@@ -1090,7 +1092,7 @@ cudaError_t launch_fold_wide(Args g, void* workspace, cudaStream_t stream, bool 
     return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kHasBalanced ? kBalanced : kPlain, WIDE>, dim3(static_cast<unsigned>(ctas)), dim3(kThreads), kBytes, stream, g, s_map);
   }
   const unsigned grid = static_cast<unsigned>(tiles < sms ? tiles : sms);   // one persistent CTA per SM
-  if (stage_bytes<TN>(g) > kWeightsInL2) {
+  if (WIDE && stage_bytes<TN>(g) > kWeightsInL2) {
     g.group_n = static_cast<int64_t>(kBlockBytes / (static_cast<size_t>(n_stages) * S::B_STAGE));
     if (g.group_n < 1) g.group_n = 1;
   }

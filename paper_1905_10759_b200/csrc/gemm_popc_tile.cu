@@ -18,6 +18,7 @@
 // conv3_x matrix (50176 x 128 x 1152) beta 2 / 4 / 8 / 16 / 32 / 128: 1337 / 660 / 332 / 172 / 90 / 81 ->
 // 926 / 640 / 326 / 153 / 83 / 71 us.  Scalar fp32 instead of the paired instructions: 5 % slower.
 #include "kernels.h"
+#include "pdl.cuh"
 #include "popc_common.cuh"
 
 namespace hbmm {
@@ -90,6 +91,8 @@ __device__ __forceinline__ void add_term(uint64_t& acc, uint32_t c0, uint32_t c1
 template <int SEG>
 __global__ void __launch_bounds__(kThreads, 2)
 gemm_popc_tile_kernel(const TileArgs g) {
+  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
+  pdl_wait();
   using P = Cfg<SEG>;
   // The next chunk waits in registers, except for the finest segments: their counts and scales need those registers
   // (spills otherwise), and a chunk is 1000 instructions and more, which the other warps fill a load's latency with.
@@ -278,7 +281,7 @@ cudaError_t launch_seg(TileArgs g, int sms, cudaStream_t stream) {
   while (g.ks_log2 < 3 && (tiles_m * tiles_n << g.ks_log2) < want && (2ll << g.ks_log2) <= g.n_chunks) g.ks_log2++;
   const int64_t per_cta = kWarps >> g.ks_log2;
   const dim3 grid(static_cast<unsigned>(tiles_n), static_cast<unsigned>((tiles_m + per_cta - 1) / per_cta));
-  gemm_popc_tile_kernel<SEG><<<grid, kThreads, 0, stream>>>(g);
+  launch_pdl(gemm_popc_tile_kernel<SEG>, dim3(grid), dim3(kThreads), 0, stream, g);
   return cudaGetLastError();
 }
 

@@ -10,6 +10,7 @@
 // mixes); K any length (rows are padded with zero words to a multiple of four, pad bits are zero in both
 // operands and the tail segment counts only its valid bits).
 #include "kernels.h"
+#include "pdl.cuh"
 #include "popc_common.cuh"
 
 namespace hbmm {
@@ -36,6 +37,8 @@ struct GemvArgs {
 template <int SW, int MR>
 __global__ void __launch_bounds__(kWarps * 32)
 gemv_popc_kernel(const GemvArgs g) {
+  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
+  pdl_wait();
   constexpr int SEGS = 4 / SW;                          // segments per 16-byte piece
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint4* a_bits = reinterpret_cast<uint4*>(smem_raw);                                    // [MR][n_quads]
@@ -103,6 +106,8 @@ gemv_popc_kernel(const GemvArgs g) {
 template <int SEG, int MR>
 __global__ void __launch_bounds__(kWarps * 32)
 gemv_popc_sub_kernel(const GemvArgs g) {
+  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
+  pdl_wait();
   constexpr int SPW = 32 / SEG, PARTS = SEG <= 8 ? 8 / SEG : 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_words = static_cast<int>((g.K + 31) / 32);
@@ -187,10 +192,10 @@ cudaError_t launch_sw(const GemvArgs& g, int sms, cudaStream_t stream) {
   if (blocks > static_cast<int64_t>(sms) * 8) blocks = static_cast<int64_t>(sms) * 8;
   const unsigned grid = static_cast<unsigned>(blocks);
   switch (mr) {
-    case 1: gemv_popc_kernel<SW, 1><<<grid, kWarps * 32, smem, stream>>>(g); break;
-    case 2: gemv_popc_kernel<SW, 2><<<grid, kWarps * 32, smem, stream>>>(g); break;
-    case 4: gemv_popc_kernel<SW, 4><<<grid, kWarps * 32, smem, stream>>>(g); break;
-    default: gemv_popc_kernel<SW, 8><<<grid, kWarps * 32, smem, stream>>>(g); break;
+    case 1: launch_pdl(gemv_popc_kernel<SW, 1>, dim3(grid), dim3(kWarps * 32), smem, stream, g); break;
+    case 2: launch_pdl(gemv_popc_kernel<SW, 2>, dim3(grid), dim3(kWarps * 32), smem, stream, g); break;
+    case 4: launch_pdl(gemv_popc_kernel<SW, 4>, dim3(grid), dim3(kWarps * 32), smem, stream, g); break;
+    default: launch_pdl(gemv_popc_kernel<SW, 8>, dim3(grid), dim3(kWarps * 32), smem, stream, g); break;
   }
   return cudaGetLastError();
 }
@@ -200,10 +205,10 @@ cudaError_t launch_sub(const GemvArgs& g, int sms, cudaStream_t stream) {
   int64_t blocks = (g.N + kWarps - 1) / kWarps;
   if (blocks > static_cast<int64_t>(sms) * 8) blocks = static_cast<int64_t>(sms) * 8;
   const unsigned grid = static_cast<unsigned>(blocks);
-  if (g.M <= 1) gemv_popc_sub_kernel<SEG, 1><<<grid, kWarps * 32, 0, stream>>>(g);
-  else if (g.M <= 2) gemv_popc_sub_kernel<SEG, 2><<<grid, kWarps * 32, 0, stream>>>(g);
-  else if (g.M <= 4) gemv_popc_sub_kernel<SEG, 4><<<grid, kWarps * 32, 0, stream>>>(g);
-  else gemv_popc_sub_kernel<SEG, 8><<<grid, kWarps * 32, 0, stream>>>(g);
+  if (g.M <= 1) launch_pdl(gemv_popc_sub_kernel<SEG, 1>, dim3(grid), dim3(kWarps * 32), 0, stream, g);
+  else if (g.M <= 2) launch_pdl(gemv_popc_sub_kernel<SEG, 2>, dim3(grid), dim3(kWarps * 32), 0, stream, g);
+  else if (g.M <= 4) launch_pdl(gemv_popc_sub_kernel<SEG, 4>, dim3(grid), dim3(kWarps * 32), 0, stream, g);
+  else launch_pdl(gemv_popc_sub_kernel<SEG, 8>, dim3(grid), dim3(kWarps * 32), 0, stream, g);
   return cudaGetLastError();
 }
 

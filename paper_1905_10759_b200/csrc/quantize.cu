@@ -8,6 +8,7 @@
 // (log2(beta) + 2) * 2^-24 relative.
 #include <cuda_bf16.h>
 #include "kernels.h"
+#include "pdl.cuh"
 
 namespace hbmm {
 namespace {
@@ -121,6 +122,8 @@ __global__ void __launch_bounds__(kThreads)
 quantize_small_beta(const void* __restrict__ x, int64_t rows, int64_t K, int64_t ldx, bool vec_ok,
                     uint32_t* __restrict__ bits, int64_t ld_words, void* __restrict__ scales, int64_t ld_scales,
                     int scale_bf16, int beta_words, int64_t G) {
+  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
+  pdl_wait();
   constexpr int EPT = In<BF16>::EPT;
   constexpr int LPW = 32 / EPT;  // lanes per word
   constexpr int WPW = EPT;       // words per warp item (32 lanes * EPT elements / 32)
@@ -187,6 +190,8 @@ template <bool BF16, int BETA>
 __global__ void __launch_bounds__(kThreads)
 quantize_stream(const void* __restrict__ x, int64_t total_words, uint32_t n_words, uint32_t* __restrict__ bits, int64_t ld_words,
                 void* __restrict__ scales, int64_t ld_scales, int scale_bf16, uint32_t G) {
+  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const int64_t warp0 = (static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x) >> 5;
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * kThreads) >> 5;
@@ -254,7 +259,7 @@ quantize_stream(const void* __restrict__ x, int64_t total_words, uint32_t n_word
 template <bool BF16>
 bool launch_stream(int beta, unsigned blocks, cudaStream_t stream, const void* x, int64_t total_words, uint32_t n_words, uint32_t* bits,
                    int64_t ld_words, void* scales, int64_t ld_scales, int scale_bf16, uint32_t G) {
-#define HBMM_QS(B) case B: quantize_stream<BF16, B><<<blocks, kThreads, 0, stream>>>(x, total_words, n_words, bits, ld_words, scales, ld_scales, scale_bf16, G); return true;
+#define HBMM_QS(B) case B: launch_pdl(quantize_stream<BF16, B>, dim3(blocks), dim3(kThreads), 0, stream, x, total_words, n_words, bits, ld_words, scales, ld_scales, scale_bf16, G); return true;
   switch (beta) {
     HBMM_QS(2) HBMM_QS(4) HBMM_QS(8) HBMM_QS(16) HBMM_QS(32) HBMM_QS(64) HBMM_QS(128) HBMM_QS(256) HBMM_QS(512)
     default: return false;
@@ -272,6 +277,8 @@ __global__ void __launch_bounds__(kThreads)
 quantize_subword(const void* __restrict__ x, int64_t rows, int64_t K, int64_t ldx, bool vec_ok,
                  uint32_t* __restrict__ bits, int64_t ld_words, void* __restrict__ scales, int64_t ld_scales,
                  int scale_bf16, int64_t G) {
+  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
+  pdl_wait();
   using L = In<BF16>;
   constexpr int EPT = L::EPT;
   constexpr int LPW = 32 / EPT;
@@ -341,10 +348,10 @@ template <bool BF16>
 void launch_subword(int beta, unsigned blocks, cudaStream_t stream, const void* x, int64_t rows, int64_t K, int64_t ldx, bool vec_ok,
                     uint32_t* bits, int64_t ld_words, void* scales, int64_t ld_scales, int scale_bf16, int64_t G) {
   switch (beta) {
-    case 2: quantize_subword<BF16, 2><<<blocks, kThreads, 0, stream>>>(x, rows, K, ldx, vec_ok, bits, ld_words, scales, ld_scales, scale_bf16, G); break;
-    case 4: quantize_subword<BF16, 4><<<blocks, kThreads, 0, stream>>>(x, rows, K, ldx, vec_ok, bits, ld_words, scales, ld_scales, scale_bf16, G); break;
-    case 8: quantize_subword<BF16, 8><<<blocks, kThreads, 0, stream>>>(x, rows, K, ldx, vec_ok, bits, ld_words, scales, ld_scales, scale_bf16, G); break;
-    default: quantize_subword<BF16, 16><<<blocks, kThreads, 0, stream>>>(x, rows, K, ldx, vec_ok, bits, ld_words, scales, ld_scales, scale_bf16, G); break;
+    case 2: launch_pdl(quantize_subword<BF16, 2>, dim3(blocks), dim3(kThreads), 0, stream, x, rows, K, ldx, vec_ok, bits, ld_words, scales, ld_scales, scale_bf16, G); break;
+    case 4: launch_pdl(quantize_subword<BF16, 4>, dim3(blocks), dim3(kThreads), 0, stream, x, rows, K, ldx, vec_ok, bits, ld_words, scales, ld_scales, scale_bf16, G); break;
+    case 8: launch_pdl(quantize_subword<BF16, 8>, dim3(blocks), dim3(kThreads), 0, stream, x, rows, K, ldx, vec_ok, bits, ld_words, scales, ld_scales, scale_bf16, G); break;
+    default: launch_pdl(quantize_subword<BF16, 16>, dim3(blocks), dim3(kThreads), 0, stream, x, rows, K, ldx, vec_ok, bits, ld_words, scales, ld_scales, scale_bf16, G); break;
   }
 }
 
@@ -356,6 +363,8 @@ __global__ void __launch_bounds__(kThreads)
 quantize_any_beta(const void* __restrict__ x, int64_t rows, int64_t K, int64_t ldx, bool vec_ok,
                   uint32_t* __restrict__ bits, int64_t ld_words, void* __restrict__ scales, int64_t ld_scales,
                   int scale_bf16, int64_t beta_words, int64_t beta, int64_t G) {
+  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
+  pdl_wait();
   extern __shared__ float word_sum[];  // [ld_words]
   constexpr int EPT = In<BF16>::EPT;
   constexpr int LPW = 32 / EPT;
@@ -445,10 +454,10 @@ cudaError_t launch_quantize(const void* x, int x_bf16, int64_t rows, int64_t K, 
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     if (x_bf16)
-      quantize_small_beta<true><<<static_cast<unsigned>(blocks), kThreads, 0, stream>>>(
+      launch_pdl(quantize_small_beta<true>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, stream, 
           x, rows, K, ldx, vec_ok, bits, ld_words, scales, ld_scales, scale_bf16, static_cast<int>(beta_words), G);
     else
-      quantize_small_beta<false><<<static_cast<unsigned>(blocks), kThreads, 0, stream>>>(
+      launch_pdl(quantize_small_beta<false>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), 0, stream, 
           x, rows, K, ldx, vec_ok, bits, ld_words, scales, ld_scales, scale_bf16, static_cast<int>(beta_words), G);
   } else {
     const size_t smem = static_cast<size_t>(ld_words) * sizeof(float);
@@ -456,10 +465,10 @@ cudaError_t launch_quantize(const void* x, int x_bf16, int64_t rows, int64_t K, 
     int64_t blocks = rows < static_cast<int64_t>(sms) * 8 ? rows : static_cast<int64_t>(sms) * 8;
     const int64_t beta_eff = one_group ? K : beta;
     if (x_bf16)
-      quantize_any_beta<true><<<static_cast<unsigned>(blocks), kThreads, smem, stream>>>(
+      launch_pdl(quantize_any_beta<true>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), smem, stream, 
           x, rows, K, ldx, vec_ok, bits, ld_words, scales, ld_scales, scale_bf16, beta_words, beta_eff, G);
     else
-      quantize_any_beta<false><<<static_cast<unsigned>(blocks), kThreads, smem, stream>>>(
+      launch_pdl(quantize_any_beta<false>, dim3(static_cast<unsigned>(blocks)), dim3(kThreads), smem, stream, 
           x, rows, K, ldx, vec_ok, bits, ld_words, scales, ld_scales, scale_bf16, beta_words, beta_eff, G);
   }
   return cudaGetLastError();
