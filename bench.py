@@ -565,7 +565,7 @@ def side_measurements(torch, hbmm, inputs, peaks, iters: int):
         ops = 2.0 * sh.M * sh.N * sh.K
         for label, first, again in (("hbmm_umma_kernel (e4m3 operands, per-group fp32 scale step)", hbmm.PATH_TENSOR, hbmm.PATH_TENSOR_PREPARED),
                                     ("hbmm_fold_kernel (default)", hbmm.PATH_FOLDED, hbmm.PATH_FOLDED_PREPARED),
-                                    ("gemm_popc_kernel (integer pipe, no workspace)", hbmm.PATH_POPC, hbmm.PATH_POPC)):
+                                    ("gemm_popc_tile_kernel (integer pipe, no workspace)", hbmm.PATH_POPC, hbmm.PATH_POPC)):
             hbmm.gemm_ex(A, W, C, first, ws)
             ms = time_loop(torch, lambda: hbmm.gemm_ex(A, W, C, again, ws), iters)
             out.append({"kernel": "%s/%s" % (label, sh.name), "shape": [sh.M, sh.N, sh.K], "ms": round(ms, 5),

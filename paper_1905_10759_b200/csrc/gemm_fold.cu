@@ -755,14 +755,16 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
         for (int c = 0; c < TN / 32; c++) {
           uint32_t v1[32];
           load_chunk(c, v1);
-          if (c == TN / 32 - 1) {      // the accumulator is in registers: the next tile may start
+          if (WIDE && c == TN / 32 - 1) {      // the accumulator is in registers: the next tile may start
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&tempty[buf]);
           }
           finish(c, v1);
         }
+        if (!WIDE) tc_fence_before();
         __syncwarp();          // every lane is done with the warp's column factors
+        if (!WIDE && lane == 0) mbar_arrive(&tempty[buf]);
       } else if constexpr (BAL) {
         // Part of the tile's K range: the raw partial accumulator goes to this CTA's slot (first slot for the tile
         // its run starts in, second for the tile it ends in), the accumulator is handed back, and the warp
