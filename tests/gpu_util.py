@@ -86,9 +86,9 @@ def assert_close_rel_absref(c_gpu: np.ndarray, c_ref: np.ndarray, absref: np.nda
     # the second term is the rounding floor of the oracle's own double-precision sum
     strict = rtol * absref + 1e-12 * max(1.0, float(absref.max()))
     bound = strict if fine is None else strict + FOLDED_FLOOR_ULPS * U * fine
-    bad = err > bound
+    bad = ~(err <= bound)          # a NaN is outside every bound
     if bad.any():
-        i = np.unravel_index(np.argmax(err / bound), err.shape)
+        i = np.unravel_index(np.argmax(np.where(np.isnan(err), np.inf, err / bound)), err.shape)
         raise AssertionError("%s: %d elements outside rtol=%g of the magnitude reference; worst at %s: "
                              "gpu=%r ref=%r absref=%r" % (what, bad.sum(), rtol, i, c_gpu[i], c_ref[i], absref[i]))
     if fine is None:
