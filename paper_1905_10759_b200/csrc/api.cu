@@ -162,23 +162,23 @@ hbmm_status gemm_checked(const hbmm_operand* A, const hbmm_operand* W, float* C,
     case HBMM_PATH_FOLDED:
       if (!gemm_fold_supported(a, w)) return HBMM_ERR_UNSUPPORTED;
       if (!workspace_ok(workspace, workspace_bytes, fold_workspace(a, w))) return HBMM_ERR_WORKSPACE;
-      // the earlier call may have been an automatic one, which leaves no expanded weights behind for a handful of rows
-      // with sub-word groups: those take the kernel that needs none
-      if (w_prepared && gemm_subword(a, w) && gemv_popc_supported(a, w)) e = launch_gemv_popc(a, w, C, ldc, stream);
-      else e = launch_gemm_fold(a, w, C, ldc, workspace, stream, w_prepared);
+      e = launch_gemm_fold(a, w, C, ldc, workspace, stream, w_prepared);
       break;
-    default:
-      // a handful of activation rows: reading the packed weights once beats any tile kernel (and the expanded
-      // weight operand of the tensor-core paths is 32 times larger than the packed one)
-      if (gemv_popc_supported(a, w)) e = launch_gemv_popc(a, w, C, ldc, stream);
+    default: {
+      const bool fold = prefer_fold(a, w) && workspace_ok(workspace, workspace_bytes, fold_workspace(a, w));
+      // a handful of activation rows: reading the packed weights once beats any tile kernel (and the expanded weight operand
+      // of the tensor-core paths is 32 times larger than the packed one).  Not for sub-word groups where the folded kernel
+      // can run: its expanded weights are what a prepared call with more rows may rely on.
+      if (gemv_popc_supported(a, w) && !(fold && gemm_subword(a, w))) e = launch_gemv_popc(a, w, C, ldc, stream);
       // the tensor-core paths need their workspace; without one the integer-pipe path runs
-      else if (prefer_fold(a, w) && workspace_ok(workspace, workspace_bytes, fold_workspace(a, w)))
+      else if (fold)
         e = launch_gemm_fold(a, w, C, ldc, workspace, stream);
       else if (gemm_tensor_supported(a, w) && workspace_ok(workspace, workspace_bytes, tensor_workspace(a, w)))
         e = launch_gemm_tensor(a, w, C, ldc, workspace, stream);
       else
         e = popc_any(a, w, C, ldc, stream);
       break;
+    }
   }
   return e == cudaSuccess ? HBMM_OK : HBMM_ERR_CUDA;
 }

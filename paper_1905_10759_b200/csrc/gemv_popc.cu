@@ -100,9 +100,10 @@ gemv_popc_kernel(const GemvArgs g) {
 // Segments of SEG = 2, 4, 8 or 16 bits: a lane takes one word of the weight row at a time, so the 32 / SEG scales it needs
 // are one vector and a warp's loads are contiguous; the activation rows are read the same way (they are a few KB, in L1
 // after the first warp), so nothing is staged and no barrier stands between the launch and the first weight load.
-// Bound by the scales: at beta 16 they are four times the bits.  3 x 3200 x 6592 at beta 16: 24 us in 32-row tiles (three
-// rows of each used), 17 us here; with one row 7.4 us.  Against the folded tensor-core kernel with its weight expansion,
-// which the automatic choice took before when K is whole words: 8 rows of 4096 x 9216 at beta 2 / 16 1580 / 315 us -> 119 / 34.
+// Bound by the scales: at beta 16 fp32 scales are twice the bits, at beta 2 sixteen times.  3 x 3200 x 6592 at beta 16: 24 us
+// in 32-row tiles (three rows of each used), 17 us here; with one row 7.4 us.  Runs for the integer-pipe path, without a
+// workspace and where K is no whole number of words; otherwise the automatic choice is the folded kernel, whose expanded
+// weights later calls may rely on.
 template <int SEG, int MR>
 __global__ void __launch_bounds__(kWarps * 32)
 gemv_popc_sub_kernel(const GemvArgs g) {

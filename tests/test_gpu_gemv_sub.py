@@ -31,7 +31,7 @@ def test_gemv_of_sub_word_groups_matches_oracle(M, N, K, ba, bw, sdt):
 
 
 def test_prepared_call_after_an_automatic_one_on_a_few_rows():
-    """An automatic call leaves no expanded weights for these operands; a prepared call that follows has to be right."""
+    """A prepared call may follow an automatic one on the same few rows."""
     import gpu_util as gu
     from paper_1905_10759_b200 import hbmm
     M, N, K, b = 4, 40, 320, 8
@@ -45,3 +45,30 @@ def test_prepared_call_after_an_automatic_one_on_a_few_rows():
     C.fill_(float("nan"))
     hbmm.gemm_ex(A, W, C, hbmm.PATH_FOLDED_PREPARED, ws)
     gu.assert_close_rel_absref(C.cpu().numpy(), c_ref, absref, 1e-5, "prepared")
+
+
+def _junk(nbytes):
+    return torch.full((nbytes,), 0xFF, dtype=torch.uint8, device="cuda")
+
+
+@pytest.mark.parametrize("b,sdt", [(2, 0), (4, 1), (8, 0), (16, 1)])
+def test_automatic_call_on_a_few_rows_prepares_calls_on_any(b, sdt):
+    """What an automatic call on four rows leaves in a workspace that held anything before serves a prepared call on the
+    same rows and one on sixty-four; the three ways to the folded kernel give the same bits."""
+    import gpu_util as gu
+    from paper_1905_10759_b200 import hbmm
+    N, K = 40, 320
+    W, dw, sw = gu.oracle_operand(inputs.he_normal(N, K, 5300), b, sdt)
+    ops = [gu.oracle_operand(inputs.normal((M, K), 4300 + M), b, sdt) for M in (4, 64)]
+    ws = _junk(max(hbmm.gemm_workspace_bytes(A, W) for A, _, _ in ops))
+    outs = []
+    for (A, da, sa), path in ((ops[0], hbmm.PATH_AUTO), (ops[0], hbmm.PATH_FOLDED_PREPARED), (ops[1], hbmm.PATH_FOLDED_PREPARED)):
+        C = torch.full((A.rows, N), float("nan"), device="cuda")
+        hbmm.gemm_ex(A, W, C, path, ws)
+        outs.append(C)
+        assert torch.isfinite(C).all(), path
+        c_ref, absref = oracle.hbmm_from_quantized(da, sa, b, dw, sw, b)
+        gu.assert_close_rel_absref(C.cpu().numpy(), c_ref, absref, 1e-5, "path %d" % path, gu.elementwise_magnitude(da, b, dw, b, K))
+    fresh = torch.full((4, N), float("nan"), device="cuda")
+    hbmm.gemm_ex(ops[0][0], W, fresh, hbmm.PATH_FOLDED, _junk(ws.numel()))
+    assert torch.equal(outs[0], fresh) and torch.equal(outs[1], fresh)
