@@ -57,10 +57,11 @@ typedef enum {
                            scaled in the epilogue; HBWN: bf16 activations x weights written as three
                            bf16 pieces +-d_i (delta = d1 + d2 + d3), one accumulation over all of K     */
   HBMM_PATH_TENSOR_PREPARED = 4, /* HBMM_PATH_TENSOR, and the caller states that the workspace still holds
-                           the expanded weight operand an earlier HBMM_PATH_TENSOR / AUTO call with the
-                           same W, the same kind of A and this workspace left there (W unchanged
-                           since, that call completed without a device-side error): the expansion
-                           kernel is skipped.  Results are undefined otherwise.                       */
+                           the expanded weight operand an earlier HBMM_PATH_TENSOR call, or an AUTO call
+                           that picked this kernel, with the same W, the same kind of A and this
+                           workspace left there (W unchanged since, that call completed without a
+                           device-side error): the expansion kernel is skipped.  Results are undefined
+                           otherwise.                                                                 */
   HBMM_PATH_FOLDED = 5, /* tcgen05, both operands packed: every group scale, times a power of two chosen
                            per row, is split into two fp16 pieces (22 significant bits) and folded into
                            the +-1 elements, so that Eq. 7's sum over groups is one fp32 accumulation of
@@ -70,7 +71,10 @@ typedef enum {
                            largest scale).  The K products are summed one by one in fp32, so
                            the error follows sum_k |A~[m,k]| |W~[n,k]| (a few 2^-24 of it) instead of
                            vanishing where group dots cancel.  What HBMM_PATH_AUTO picks when it has
-                           the workspace and the finer grouping has at most 128 elements per group.
+                           the workspace and the finer grouping has at most 128 elements per group,
+                           except for at most eight rows of A with a finer grouping of 32, 64 or 128
+                           elements: those take a matrix-vector kernel, which leaves no expanded
+                           weights behind.
                            Callers that need Eq. 7's exact cancellation inside a group (integer
                            group dots, error relative to sum_g |dA dW D_g| alone) pass
                            HBMM_PATH_TENSOR.
@@ -78,9 +82,10 @@ typedef enum {
                            scale to 2^-17 instead of 2^-26; activations carry 2^-9), 128-column
                            tiles; what HBMM_PATH_AUTO picks for dense bf16 activations.              */
   HBMM_PATH_FOLDED_PREPARED = 6 /* HBMM_PATH_FOLDED with the expanded weights of an earlier
-                           HBMM_PATH_FOLDED / AUTO call reused, as HBMM_PATH_TENSOR_PREPARED (the
-                           arrival counters of the shared tiles, which every completed call leaves at
-                           zero, are part of what is reused)                                           */
+                           HBMM_PATH_FOLDED call reused, or of an AUTO call that picked this kernel by
+                           the rule above (no other AUTO call leaves them), as
+                           HBMM_PATH_TENSOR_PREPARED (the arrival counters of the shared tiles, which
+                           every completed call leaves at zero, are part of what is reused)            */
 } hbmm_path;
 
 /*
