@@ -317,8 +317,10 @@ hbmm_status hbmm_conv_im2col(const void *x, int32_t x_dtype, const hbmm_conv_geo
  * weights are fixed at inference time) was filled by an earlier hbmm_conv_im2col / hbmm_conv_im2col_ex
  * call with the same W, geometry, beta_a, scale type and workspace, and that nothing has written it since.
  * The call then skips the expansion; the activation part of the workspace is rewritten by every call
- * either way.  Results are undefined when the statement is false.  Paths that keep no expanded weights
- * ignore the flag.
+ * either way.  The earlier call may have had x of the other type or alignment, and may have been a fused one or
+ * not, unless the finer grouping has more than 128 elements: there the fused and the plain calls expand the
+ * weights differently.  A call with HBMM_CONV_PACK_ONLY does not count unless x was fp32 and 16-byte aligned.
+ * Results are undefined when the statement is false.  Paths that keep no expanded weights ignore the flag.
  * HBMM_CONV_PACK_ONLY (beta_a >= 2 only, otherwise HBMM_ERR_INVALID_ARG): the call stops once the packed
  * activation operand -- bits [M, ld_words] at the start of the workspace, then, from the next 256-byte
  * boundary, scales [M, ld_scales], both as hbmm_operand_bytes(M, C*kh*kw, beta_a, a_scale_dtype) lays

@@ -470,6 +470,7 @@ hbmm_status conv_checked(const void* x, int32_t x_dtype, const hbmm_conv_geom* g
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   hbmm_operand A{};
   A.rows = L.M; A.K = L.K; A.beta = beta_a; A.scale_dtype = a_scale_dtype;
+  int32_t path = HBMM_PATH_AUTO;
   if (beta_a == 1 && L.implicit) {
     return launch_hbwn_umma_conv(x, x_dtype == HBMM_BF16, workspace, L.Cp, cg, view_of(W), C_out, ldc,
                                  static_cast<char*>(workspace) + L.operand_bytes, s, w_prepared, ep ? &epi : nullptr,
@@ -512,8 +513,12 @@ hbmm_status conv_checked(const void* x, int32_t x_dtype, const hbmm_conv_geom* g
     if (pack_only) return HBMM_OK;
     if (ep)
       return launch_gemm_fold(av, wv, nullptr, 0, gemm_ws, s, w_prepared, &epi) == cudaSuccess ? HBMM_OK : HBMM_ERR_CUDA;
+    // The front end depends on the type and the alignment of x, the kernel that leaves expanded weights for a later call
+    // with HBMM_CONV_WEIGHTS_PREPARED must not: the folded kernel also for the few output pixels hbmm_gemm would hand to
+    // the matrix-vector kernel.
+    if (prefer_fold(av, wv) && L.gemm_bytes >= fold_workspace(av, wv)) path = HBMM_PATH_FOLDED;
   }
-  return gemm_checked(&A, W, C_out, ldc, HBMM_PATH_AUTO, static_cast<char*>(workspace) + L.operand_bytes, L.gemm_bytes, s);
+  return gemm_checked(&A, W, C_out, ldc, path, static_cast<char*>(workspace) + L.operand_bytes, L.gemm_bytes, s);
 }
 
 }  // namespace

@@ -50,3 +50,35 @@ def test_packed_rows_match_oracle(B, C, H, W, k, st, beta, bf16):
     # four partial sums of a word's or group's elements in turn, joined pairwise, one division
     np.testing.assert_allclose(sc[:, :G], da, rtol=(min(beta, 32) // 4 + int(np.ceil(np.log2(beta))) + 3) * gu.U, atol=0)
     assert hbmm.last_device_error() == 0
+
+
+@pytest.mark.parametrize("first", ["bf16", "off by one element"])
+@pytest.mark.parametrize("beta", [8, 16, 32, 64])
+def test_weights_of_a_first_call_serve_the_other_front_end(beta, first):
+    """At most eight output pixels: the first call's image takes the gathering front end, the prepared calls' (plain and
+    fused) the tensor-copy one; the workspace held something else before."""
+    import gpu_util as gu
+    from paper_1905_10759_b200 import hbmm
+    B, C, H, N = 2, 32, 4, 40
+    K, M = C * 9, B * 4
+    x = inputs.normal((B * C * H, H), 6100 + beta).reshape(B, C, H, H)
+    w = inputs.he_normal(N, K, 6200 + beta)
+    W = hbmm.quantize(torch.from_numpy(w).cuda(), hbmm.alloc_operand(N, K, beta))
+    geom = hbmm.make_geom(B, C, H, H, 3, 3)
+    ws = torch.full((hbmm.conv_workspace_bytes(geom, beta, hbmm.F32, W),), 0xFF, dtype=torch.uint8, device="cuda")
+    xd = torch.from_numpy(x).cuda()
+    if first == "bf16":
+        x1 = xd.bfloat16()
+    else:
+        x1 = torch.empty(xd.numel() + 1, device="cuda")[1:].view(xd.shape).copy_(xd)
+    out = torch.full((M, N), float("nan"), device="cuda")
+    hbmm.conv_im2col(x1, geom, beta, hbmm.F32, W, torch.empty((M, N), device="cuda"), ws)
+    hbmm.conv_im2col(xd, geom, beta, hbmm.F32, W, out, ws, flags=hbmm.CONV_WEIGHTS_PREPARED)
+    c_ref, absref = oracle.conv_im2col(x, w, 3, 3, (1, 1), (0, 0), beta, beta)
+    da, dw = oracle.quantize(oracle.im2col(x, 3, 3), beta)[0], oracle.quantize(w, beta)[0]
+    fine = gu.elementwise_magnitude(da, beta, dw, beta, K)
+    gu.assert_close_rel_absref(out.cpu().numpy(), c_ref, absref, 1e-5, "prepared", fine)
+    if beta >= 32:
+        z = torch.full((M, N), float("nan"), device="cuda")
+        hbmm.conv_im2col_fused(xd, geom, beta, hbmm.F32, W, hbmm.make_epilogue(out=z), ws, flags=hbmm.CONV_WEIGHTS_PREPARED)
+        gu.assert_close_rel_absref(z.cpu().numpy(), c_ref, absref, 1e-5, "fused, prepared", fine)
