@@ -84,8 +84,10 @@ typedef enum {
   HBMM_PATH_FOLDED_PREPARED = 6 /* HBMM_PATH_FOLDED with the expanded weights of an earlier
                            HBMM_PATH_FOLDED call reused, or of an AUTO call that picked this kernel by
                            the rule above (no other AUTO call leaves them), as
-                           HBMM_PATH_TENSOR_PREPARED (the arrival counters of the shared tiles, which
-                           every completed call leaves at zero, are part of what is reused)            */
+                           HBMM_PATH_TENSOR_PREPARED.  A may have another number of rows than the
+                           earlier call's; workspace_bytes of that call was at least what this one
+                           needs (the arrival counters of the shared tiles, which every completed call
+                           leaves at zero, are part of what is reused).                                */
 } hbmm_path;
 
 /*

@@ -162,7 +162,7 @@ hbmm_status gemm_checked(const hbmm_operand* A, const hbmm_operand* W, float* C,
     case HBMM_PATH_FOLDED:
       if (!gemm_fold_supported(a, w)) return HBMM_ERR_UNSUPPORTED;
       if (!workspace_ok(workspace, workspace_bytes, fold_workspace(a, w))) return HBMM_ERR_WORKSPACE;
-      e = launch_gemm_fold(a, w, C, ldc, workspace, stream, w_prepared);
+      e = launch_gemm_fold(a, w, C, ldc, workspace, workspace_bytes, stream, w_prepared);
       break;
     default: {
       const bool fold = prefer_fold(a, w) && workspace_ok(workspace, workspace_bytes, fold_workspace(a, w));
@@ -172,7 +172,7 @@ hbmm_status gemm_checked(const hbmm_operand* A, const hbmm_operand* W, float* C,
       if (gemv_popc_supported(a, w) && !(fold && gemm_subword(a, w))) e = launch_gemv_popc(a, w, C, ldc, stream);
       // the tensor-core paths need their workspace; without one the integer-pipe path runs
       else if (fold)
-        e = launch_gemm_fold(a, w, C, ldc, workspace, stream);
+        e = launch_gemm_fold(a, w, C, ldc, workspace, workspace_bytes, stream);
       else if (gemm_tensor_supported(a, w) && workspace_ok(workspace, workspace_bytes, tensor_workspace(a, w)))
         e = launch_gemm_tensor(a, w, C, ldc, workspace, stream);
       else
@@ -366,7 +366,7 @@ hbmm_status hbmm_gemm_fused(const hbmm_operand* A, const hbmm_operand* W, const 
   if (!segments_compatible(A, W) || !gemm_fold_supported(a, w) || a_subword) return HBMM_ERR_UNSUPPORTED;
   if (e.mode == kEpiPacked && !gemm_fold_next_supported(W->rows, e.nx_beta)) return HBMM_ERR_UNSUPPORTED;
   if (!workspace_ok(workspace, workspace_bytes, fold_workspace(a, w))) return HBMM_ERR_WORKSPACE;
-  return launch_gemm_fold(a, w, nullptr, 0, workspace, s, false, &e) == cudaSuccess ? HBMM_OK : HBMM_ERR_CUDA;
+  return launch_gemm_fold(a, w, nullptr, 0, workspace, workspace_bytes, s, false, &e) == cudaSuccess ? HBMM_OK : HBMM_ERR_CUDA;
 }
 
 hbmm_status hbmm_gemm_binarize_next(const hbmm_operand* A, const hbmm_operand* W, const float* bn_scale, const float* bn_shift,
@@ -504,7 +504,7 @@ hbmm_status conv_checked(const void* x, int32_t x_dtype, const hbmm_conv_geom* g
                                        w_prepared ? nullptr : &job) != cudaSuccess)
           return HBMM_ERR_CUDA;
         if (pack_only) return HBMM_OK;
-        return launch_gemm_fold(av, wv, C_out, ldc, gemm_ws, s, true, ep ? &epi : nullptr) == cudaSuccess ? HBMM_OK : HBMM_ERR_CUDA;
+        return launch_gemm_fold(av, wv, C_out, ldc, gemm_ws, L.gemm_bytes, s, true, ep ? &epi : nullptr) == cudaSuccess ? HBMM_OK : HBMM_ERR_CUDA;
       }
     }
     if (launch_im2col_quantize(x, x_dtype == HBMM_BF16, cg, beta_a, A.bits, A.ld_words, A.scales, A.ld_scales,
@@ -512,7 +512,7 @@ hbmm_status conv_checked(const void* x, int32_t x_dtype, const hbmm_conv_geom* g
       return HBMM_ERR_CUDA;
     if (pack_only) return HBMM_OK;
     if (ep)
-      return launch_gemm_fold(av, wv, nullptr, 0, gemm_ws, s, w_prepared, &epi) == cudaSuccess ? HBMM_OK : HBMM_ERR_CUDA;
+      return launch_gemm_fold(av, wv, nullptr, 0, gemm_ws, L.gemm_bytes, s, w_prepared, &epi) == cudaSuccess ? HBMM_OK : HBMM_ERR_CUDA;
     // The front end depends on the type and the alignment of x, the kernel that leaves expanded weights for a later call
     // with HBMM_CONV_WEIGHTS_PREPARED must not: the folded kernel also for the few output pixels hbmm_gemm would hand to
     // the matrix-vector kernel.

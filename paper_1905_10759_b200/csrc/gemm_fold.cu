@@ -926,14 +926,20 @@ bool balanced_possible(const Args& g, int64_t sms) {
   return sms <= kMaxBalancedCtas && n_stages >= kBalancedMinStages && tile_count<TN>(g) < kBalancedWaves * sms;
 }
 template <int TN>
-size_t counters_bytes(const Args& g) { return (static_cast<size_t>(tile_count<TN>(g)) * kEpilogueWarps * sizeof(int32_t) + 255) / 256 * 256; }
-template <int TN>
 size_t balanced_bytes(const Args& g) {
   if (!balanced_possible<TN>(g, kMaxBalancedCtas)) return 0;
   const int64_t n_stages = (g.n_words + WPS - 1) / WPS, units = tile_count<TN>(g) * n_stages;
   const int64_t ctas = units < kMaxBalancedCtas ? units : kMaxBalancedCtas;
-  return counters_bytes<TN>(g) + static_cast<size_t>(2 * ctas) * TM * TN * sizeof(float);
+  const size_t counters = (static_cast<size_t>(tile_count<TN>(g)) * kEpilogueWarps * sizeof(int32_t) + 255) / 256 * 256;
+  return counters + static_cast<size_t>(2 * ctas) * TM * TN * sizeof(float);
 }
+// The arrival counters take the first kCounterCount words of the area, for the most tiles a balanced launch may have, so
+// that they lie at the same place and are all zeroed by whichever call expands the weights, whatever its number of rows:
+// prepared calls with more and fewer rows follow it.  (Sized for the call's own tiles, they lay under another call's partial
+// tiles.)  The area holds them without being larger: of its min(units, 256) pairs of slots a launch uses at most
+// min(units / kBalancedMinStages, kMaxBalancedCtas - 1), and one pair is four times the counters.
+constexpr int64_t kCounterCount = kBalancedWaves * kMaxBalancedCtas * kEpilogueWarps;
+static_assert(2 * TM * 64 * sizeof(float) >= kCounterCount * sizeof(int32_t), "a pair of slots holds the counters");
 // [W stages][one float per weight row][counters][partial slots]
 template <int TN>
 size_t down_offset(const Args& g) { return stage_bytes<TN>(g); }
@@ -948,14 +954,19 @@ template <int TN>
 size_t prep_bytes(const Args& g) {
   return g.a_sub > 1 ? rowmax_offset<TN>(g) + static_cast<size_t>(g.M) * sizeof(float) : balanced_offset<TN>(g) + balanced_bytes<TN>(g);
 }
-// Points the argument block at the balanced schedule's part of the workspace (when the shape has one).
+// Points the argument block at the balanced schedule's part of the workspace.  A product with too many tiles for it has no
+// such part; its counters are zeroed all the same where the caller's workspace reaches that far (`have` bytes), for prepared
+// calls with fewer rows.
 template <int TN>
-void set_balanced_area(Args& g, void* workspace) {
-  if (balanced_bytes<TN>(g) == 0) return;
-  unsigned char* area = static_cast<unsigned char*>(workspace) + balanced_offset<TN>(g);
+void set_balanced_area(Args& g, void* workspace, size_t have) {
+  const bool reserved = balanced_bytes<TN>(g) != 0;
+  const int64_t n_stages = (g.n_words + WPS - 1) / WPS;
+  const size_t at = balanced_offset<TN>(g), counters = kCounterCount * sizeof(int32_t);
+  if (!reserved && (g.a_sub > 1 || n_stages < kBalancedMinStages || have < at + counters)) return;
+  unsigned char* area = static_cast<unsigned char*>(workspace) + at;
   g.sk_counters = reinterpret_cast<int32_t*>(area);
-  g.sk_counter_count = tile_count<TN>(g) * kEpilogueWarps;
-  g.sk_partials = reinterpret_cast<float*>(area + counters_bytes<TN>(g));
+  g.sk_counter_count = kCounterCount;
+  if (reserved) g.sk_partials = reinterpret_cast<float*>(area + counters);
 }
 
 // Split mode: the largest number of CTAs per tile (2 .. 8, at least two stages each) for which every tile's cluster is
@@ -1014,7 +1025,7 @@ void launch_prepare(const Args& g, unsigned char* stages, float* down, int sms, 
 }
 
 template <int TN, int ASUB, bool FUSE, bool WIDE>
-cudaError_t launch_fold_wide(Args g, void* workspace, cudaStream_t stream, bool w_prepared) {
+cudaError_t launch_fold_wide(Args g, void* workspace, size_t have, cudaStream_t stream, bool w_prepared) {
   using S = Smem<TN>;
   constexpr bool kHasBalanced = ASUB == 1;           // the balanced schedule is built for activation groups of whole words
   constexpr int kBytes = ScaleRing<TN, ASUB>::BYTES;
@@ -1039,7 +1050,7 @@ cudaError_t launch_fold_wide(Args g, void* workspace, cudaStream_t stream, bool 
   const int64_t tiles_n = (g.N + TN - 1) / TN, n_stages = (g.n_words + WPS - 1) / WPS;
   unsigned char* stages = static_cast<unsigned char*>(workspace);
   float* down = reinterpret_cast<float*>(stages + stage_bytes<TN>(g));
-  set_balanced_area<TN>(g, workspace);
+  set_balanced_area<TN>(g, workspace, have);
   if (!w_prepared) launch_prepare<TN>(g, stages, down, sms, stream);
   g.w_prep = stages;
   g.w_down = down;
@@ -1081,6 +1092,7 @@ cudaError_t launch_fold_wide(Args g, void* workspace, cudaStream_t stream, bool 
   // equal runs of (tile, stage) pairs, one per CTA, when that shortens the longest CTA's walk by a tenth or more
   const int64_t units = tiles * n_stages;
   int64_t ctas = units / kBalancedMinStages < sms ? units / kBalancedMinStages : sms;
+  if (ctas > kMaxBalancedCtas - 1) ctas = kMaxBalancedCtas - 1;
   if (ctas < 1) ctas = 1;
   int64_t run = (units + ctas - 1) / ctas;
   // a tile is shared by at most kBalancedMaxShare + 1 CTAs: the CTA that completes it adds the others' partial
@@ -1102,24 +1114,24 @@ cudaError_t launch_fold_wide(Args g, void* workspace, cudaStream_t stream, bool 
 }
 
 template <int TN, int ASUB, bool FUSE = false>
-cudaError_t launch_fold(const Args& g, void* workspace, cudaStream_t stream, bool w_prepared) {
+cudaError_t launch_fold(const Args& g, void* workspace, size_t have, cudaStream_t stream, bool w_prepared) {
   const int64_t n_stages = (g.n_words + WPS - 1) / WPS;
-  if (TN == 128 && n_stages >= kWideFromStages) return launch_fold_wide<TN, ASUB, FUSE, TN == 128>(g, workspace, stream, w_prepared);
-  return launch_fold_wide<TN, ASUB, FUSE, false>(g, workspace, stream, w_prepared);
+  if (TN == 128 && n_stages >= kWideFromStages) return launch_fold_wide<TN, ASUB, FUSE, TN == 128>(g, workspace, have, stream, w_prepared);
+  return launch_fold_wide<TN, ASUB, FUSE, false>(g, workspace, have, stream, w_prepared);
 }
 
 template <int TN>
-cudaError_t launch_fold_tn(const Args& g, void* workspace, cudaStream_t stream, bool w_prepared) {
+cudaError_t launch_fold_tn(const Args& g, void* workspace, size_t have, cudaStream_t stream, bool w_prepared) {
   if (g.ep.mode != kEpiPlain) {      // the fused epilogue is built for activation groups of whole words
     if (g.a_sub != 1) return cudaErrorNotSupported;
-    return launch_fold<TN, 1, true>(g, workspace, stream, w_prepared);
+    return launch_fold<TN, 1, true>(g, workspace, have, stream, w_prepared);
   }
   switch (g.a_sub) {
-    case 2: return launch_fold<TN, 2>(g, workspace, stream, w_prepared);
-    case 4: return launch_fold<TN, 4>(g, workspace, stream, w_prepared);
-    case 8: return launch_fold<TN, 8>(g, workspace, stream, w_prepared);
-    case 16: return launch_fold<TN, 16>(g, workspace, stream, w_prepared);
-    default: return launch_fold<TN, 1>(g, workspace, stream, w_prepared);
+    case 2: return launch_fold<TN, 2>(g, workspace, have, stream, w_prepared);
+    case 4: return launch_fold<TN, 4>(g, workspace, have, stream, w_prepared);
+    case 8: return launch_fold<TN, 8>(g, workspace, have, stream, w_prepared);
+    case 16: return launch_fold<TN, 16>(g, workspace, have, stream, w_prepared);
+    default: return launch_fold<TN, 1>(g, workspace, have, stream, w_prepared);
   }
 }
 
@@ -1148,11 +1160,11 @@ bool gemm_fold_next_supported(int64_t N, int32_t beta_next) {
           beta_next == 128) && beta_next <= tn;
 }
 
-cudaError_t launch_gemm_fold(const PackedView& A, const PackedView& W, float* C, int64_t ldc, void* workspace,
+cudaError_t launch_gemm_fold(const PackedView& A, const PackedView& W, float* C, int64_t ldc, void* workspace, size_t workspace_bytes,
                              cudaStream_t stream, bool w_prepared, const EpiArgs* ep) {
   Args g = make_args(A, W, C, ldc);
   if (ep) g.ep = *ep;
-  return g.N <= 64 ? launch_fold_tn<64>(g, workspace, stream, w_prepared) : launch_fold_tn<128>(g, workspace, stream, w_prepared);
+  return g.N <= 64 ? launch_fold_tn<64>(g, workspace, workspace_bytes, stream, w_prepared) : launch_fold_tn<128>(g, workspace, workspace_bytes, stream, w_prepared);
 }
 
 // The weight expansion of launch_gemm_fold(A, W, ..., workspace) as a job for another kernel.
@@ -1165,7 +1177,7 @@ void gemm_fold_prep_job(const PackedView& A, const PackedView& W, void* workspac
   job->n_stages = static_cast<int32_t>((n_stages + kPrepStages - 1) / kPrepStages);    // tasks per column tile
   job->tiles_n = static_cast<int32_t>((job->f.N + job->tn - 1) / job->tn);
   job->out_down = reinterpret_cast<float*>(job->out + (job->tn == 64 ? stage_bytes<64>(job->f) : stage_bytes<128>(job->f)));
-  if (job->tn == 64) set_balanced_area<64>(job->f, workspace); else set_balanced_area<128>(job->f, workspace);
+  if (job->tn == 64) set_balanced_area<64>(job->f, workspace, 0); else set_balanced_area<128>(job->f, workspace, 0);
 }
 
 cudaError_t launch_wait_expiry_selftest(cudaStream_t stream) {

@@ -136,7 +136,7 @@ struct FoldArgs {
   // part of a tile stores its raw partial accumulator in its own slot of sk_partials and counts itself in
   // sk_counters[tile][epilogue warp]; the last one to arrive adds the tile's partials in CTA order and finishes it.
   int64_t sk_units;
-  int32_t* sk_counters;          // [tiles][4]: zeroed by the weight expansion, left at zero by every launch
+  int32_t* sk_counters;          // [tiles][4], at a place no number of rows moves: zeroed by the weight expansion, left at zero by every launch
   int64_t sk_counter_count;
   float* sk_partials;            // [2 * CTAs][128][TN]
   float* a_rowmax;               // sub-word groups: largest scale of every activation row (nullptr: the scouts scan the rows)
@@ -178,7 +178,8 @@ cudaError_t gemm_fold_health(int op, int* value);
 cudaError_t launch_wait_expiry_selftest(cudaStream_t stream);
 bool gemm_fold_supported(const PackedView& A, const PackedView& W);
 size_t gemm_fold_workspace_bytes(const PackedView& A, const PackedView& W);
-cudaError_t launch_gemm_fold(const PackedView& A, const PackedView& W, float* C, int64_t ldc, void* workspace,
+// workspace_bytes: what the caller's workspace holds (at least gemm_fold_workspace_bytes).
+cudaError_t launch_gemm_fold(const PackedView& A, const PackedView& W, float* C, int64_t ldc, void* workspace, size_t workspace_bytes,
                              cudaStream_t stream, bool w_prepared = false, const EpiArgs* ep = nullptr);
 // Group sizes the fused epilogue can emit for an output of N columns.
 bool gemm_fold_next_supported(int64_t N, int32_t beta_next);

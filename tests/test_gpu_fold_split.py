@@ -92,3 +92,29 @@ def test_tiles_walked_in_blocks_of_columns():
     diff, ref = (C[:, :N] - P[:, :N]).double(), P[:, :N].double()
     assert float(diff.norm() / ref.norm()) < 1e-5
     assert float(diff.abs().max()) < 1e-3 * float(ref.abs().max())
+
+
+def test_prepared_calls_with_any_number_of_rows():
+    """One expansion serves calls of 10 to 1040 tiles in any order, split, balanced and plain, in a workspace that held
+    something else before: the same bits as a call that expands the weights itself."""
+    from paper_1905_10759_b200 import hbmm
+    N, K, b = 1280, 1024, 64
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(11)
+    W = hbmm.quantize(torch.randn((N, K), generator=gen, device="cuda"), hbmm.alloc_operand(N, K, b))
+    ops = {M: hbmm.quantize(torch.randn((M, K), generator=gen, device="cuda"), hbmm.alloc_operand(M, K, b))
+           for M in (128, 1024, 1408, 13200)}
+    nbytes = max(hbmm.gemm_workspace_bytes(A, W) for A in ops.values())
+
+    def product(M, path, ws):
+        C = torch.full((M, N), float("nan"), device="cuda")
+        hbmm.gemm_ex(ops[M], W, C, path, ws)
+        return C
+
+    junk = lambda: torch.full((nbytes,), 0xFF, dtype=torch.uint8, device="cuda")
+    fresh = {M: product(M, hbmm.PATH_FOLDED, junk()) for M in ops}
+    for first in (128, 1408, 13200):
+        ws = junk()
+        assert torch.equal(product(first, hbmm.PATH_FOLDED, ws), fresh[first])
+        for M in (1408, 1024, 1408, 128, 13200, 1024):
+            assert torch.equal(product(M, hbmm.PATH_FOLDED_PREPARED, ws), fresh[M]), (first, M)
