@@ -54,7 +54,6 @@ __device__ __forceinline__ void group_sums(const float (&a)[4], const float (&d)
 template <int BETA>
 __global__ void __launch_bounds__(kThreads)
 binarize_backward_stream(const float4* __restrict__ x, const float4* __restrict__ gy, float4* __restrict__ gx, int64_t n_vec) {
-  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
   pdl_wait();
   constexpr float inv = 1.0f / static_cast<float>(BETA);
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
@@ -90,7 +89,6 @@ template <int BETA, bool VEC>
 __global__ void __launch_bounds__(kThreads)
 binarize_backward_rows(const float* __restrict__ x, int64_t ldx, const float* __restrict__ gy, int64_t ldg, int64_t rows, int64_t K,
                        float* __restrict__ gx, int64_t ldo) {
-  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
   pdl_wait();
   const int lane = threadIdx.x & 31;
   const int64_t chunks = (K + 127) / 128, items = rows * chunks;
@@ -120,7 +118,6 @@ binarize_backward_rows(const float* __restrict__ x, int64_t ldx, const float* __
 __global__ void __launch_bounds__(kThreads)
 binarize_backward_general(const float* __restrict__ x, int64_t ldx, const float* __restrict__ gy, int64_t ldg, int64_t rows, int64_t K,
                           int64_t beta, int64_t G, float* __restrict__ gx, int64_t ldo) {
-  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
   pdl_wait();
   const int64_t total = rows * G;
   for (int64_t idx = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; idx < total;

@@ -43,7 +43,6 @@ __device__ __forceinline__ void store1(__nv_bfloat16* out, int64_t i, float v) {
 template <int BETA, int E, typename OUT>
 __global__ void __launch_bounds__(kThreads)
 binarize_dense_stream(const float4* __restrict__ x, OUT* __restrict__ out, int64_t n_items) {
-  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
   pdl_wait();
   constexpr int LANES = BETA > E ? BETA / E : 1;          // lanes per group
   constexpr int RUN = BETA < E ? BETA : E;                // elements of one group inside a lane
@@ -92,7 +91,6 @@ binarize_dense_stream(const float4* __restrict__ x, OUT* __restrict__ out, int64
 template <int BETA, bool VEC, typename OUT>
 __global__ void __launch_bounds__(kThreads)
 binarize_dense_rows(const float* __restrict__ x, int64_t ldx, int64_t rows, int64_t K, OUT* __restrict__ out, int64_t ldo) {
-  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
   pdl_wait();
   constexpr int LANES = BETA > 4 ? BETA / 4 : 1;          // lanes per group
   const int lane = threadIdx.x & 31;
@@ -137,7 +135,6 @@ template <typename OUT>
 __global__ void __launch_bounds__(kThreads)
 binarize_dense_general(const float* __restrict__ x, int64_t ldx, int64_t rows, int64_t K, int64_t beta, int64_t G,
                        OUT* __restrict__ out, int64_t ldo) {
-  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
   pdl_wait();
   const int64_t total = rows * G;
   for (int64_t idx = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; idx < total;

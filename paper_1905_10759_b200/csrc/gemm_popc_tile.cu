@@ -91,7 +91,6 @@ __device__ __forceinline__ void add_term(uint64_t& acc, uint32_t c0, uint32_t c1
 template <int SEG>
 __global__ void __launch_bounds__(kThreads, 2)
 gemm_popc_tile_kernel(const TileArgs g) {
-  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
   pdl_wait();
   using P = Cfg<SEG>;
   // The next chunk waits in registers, except for the finest segments: their counts and scales need those registers

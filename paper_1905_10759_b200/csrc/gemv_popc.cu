@@ -37,7 +37,6 @@ struct GemvArgs {
 template <int SW, int MR>
 __global__ void __launch_bounds__(kWarps * 32)
 gemv_popc_kernel(const GemvArgs g) {
-  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
   pdl_wait();
   constexpr int SEGS = 4 / SW;                          // segments per 16-byte piece
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -107,7 +106,6 @@ gemv_popc_kernel(const GemvArgs g) {
 template <int SEG, int MR>
 __global__ void __launch_bounds__(kWarps * 32)
 gemv_popc_sub_kernel(const GemvArgs g) {
-  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
   pdl_wait();
   constexpr int SPW = 32 / SEG, PARTS = SEG <= 8 ? 8 / SEG : 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

@@ -4,6 +4,11 @@
 // tensor-memory allocation, address tables) overlap the predecessor's tail.  It must execute pdl_wait in
 // every thread before it touches global memory: the wait returns when the preceding kernel has completed
 // and its writes are visible -- which also keeps the ordering transitive along a chain of such kernels.
+// Short kernels without set-up (streams, matrix-vector, integer tiles) wait and never signal: their end does.  A signal as
+// the first instruction lets every following launch of the stream move in while this one still works -- graph replays of
+// binarize_dense of 4646 x 688 at beta 48 91 us instead of 34, 1702 rows quantized at beta 8 3.1 instead of 2.0, of
+// hbmm_gemm on 3 rows of 2057 x 5248 6.6 instead of 4.4; with the wait alone all of them are at or below a plain launch.
+// The quantizer signals after its wait, for the set-up of the contraction behind it (2 % of that pair).
 #pragma once
 #include <cuda_runtime.h>
 #include <utility>

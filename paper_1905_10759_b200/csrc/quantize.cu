@@ -122,8 +122,8 @@ __global__ void __launch_bounds__(kThreads)
 quantize_small_beta(const void* __restrict__ x, int64_t rows, int64_t K, int64_t ldx, bool vec_ok,
                     uint32_t* __restrict__ bits, int64_t ld_words, void* __restrict__ scales, int64_t ld_scales,
                     int scale_bf16, int beta_words, int64_t G) {
-  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
   pdl_wait();
+  pdl_launch_dependents();      // a contraction that follows sets itself up meanwhile
   constexpr int EPT = In<BF16>::EPT;
   constexpr int LPW = 32 / EPT;  // lanes per word
   constexpr int WPW = EPT;       // words per warp item (32 lanes * EPT elements / 32)
@@ -190,8 +190,8 @@ template <bool BF16, int BETA>
 __global__ void __launch_bounds__(kThreads)
 quantize_stream(const void* __restrict__ x, int64_t total_words, uint32_t n_words, uint32_t* __restrict__ bits, int64_t ld_words,
                 void* __restrict__ scales, int64_t ld_scales, int scale_bf16, uint32_t G) {
-  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
   pdl_wait();
+  pdl_launch_dependents();      // a contraction that follows sets itself up meanwhile
   const int lane = threadIdx.x & 31;
   const int64_t warp0 = (static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x) >> 5;
   const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * kThreads) >> 5;
@@ -277,8 +277,8 @@ __global__ void __launch_bounds__(kThreads)
 quantize_subword(const void* __restrict__ x, int64_t rows, int64_t K, int64_t ldx, bool vec_ok,
                  uint32_t* __restrict__ bits, int64_t ld_words, void* __restrict__ scales, int64_t ld_scales,
                  int scale_bf16, int64_t G) {
-  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
   pdl_wait();
+  pdl_launch_dependents();      // a contraction that follows sets itself up meanwhile
   using L = In<BF16>;
   constexpr int EPT = L::EPT;
   constexpr int LPW = 32 / EPT;
@@ -363,7 +363,6 @@ __global__ void __launch_bounds__(kThreads)
 quantize_any_beta(const void* __restrict__ x, int64_t rows, int64_t K, int64_t ldx, bool vec_ok,
                   uint32_t* __restrict__ bits, int64_t ld_words, void* __restrict__ scales, int64_t ld_scales,
                   int scale_bf16, int64_t beta_words, int64_t beta, int64_t G) {
-  pdl_launch_dependents();      // the next kernel of the stream may start its own set-up
   pdl_wait();
   extern __shared__ float word_sum[];  // [ld_words]
   constexpr int EPT = In<BF16>::EPT;
