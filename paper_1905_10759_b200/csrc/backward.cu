@@ -103,13 +103,13 @@ binarize_backward_rows(const float* __restrict__ x, int64_t ldx, const float* __
 #pragma unroll
     for (int e = 0; e < 4; e++) { a[e] = fabsf(xv[e]); d[e] = signed_like(gv[e], xv[e]); }
     group_sums<BETA>(a, d, asum, dsum);
-    float o[4];
+    float am[4], dm[4], o[4];
 #pragma unroll
     for (int e = 0; e < 4; e++) {
-      const int64_t left = K - (k0 + e) / BETA * BETA;
-      const float n = static_cast<float>(left < BETA ? (left > 0 ? left : 1) : BETA);
-      const float ste = a[e] <= 1.0f ? (asum[e] / n) * gv[e] : 0.0f;
-      o[e] = signed_like(dsum[e] / n, xv[e]) + ste;
+      const bool first = e % (BETA < 4 ? BETA : 4) == 0;          // one mean per group
+      am[e] = first ? group_mean<BETA>(asum[e], k0, e, K) : am[e - 1];
+      dm[e] = first ? group_mean<BETA>(dsum[e], k0, e, K) : dm[e - 1];
+      o[e] = signed_like(dm[e], xv[e]) + (a[e] <= 1.0f ? am[e] * gv[e] : 0.0f);
     }
     store4<VEC>(gx + r * ldo, k0, K, o);
   }
@@ -186,9 +186,7 @@ cudaError_t launch_binarize_backward(const float* x, int64_t ldx, const float* g
     return cudaGetLastError();
   }
   const int64_t cap = static_cast<int64_t>(sms) * 32;
-  // rows shorter than 64 leave more than half of a warp's lanes idle: 229376 rows of 28 at beta 16 47 us in the
-  // thread-per-group kernel and 151 us in the rows kernel, 100000 rows of 56 at beta 32 71 and 69 us
-  if (pow2 && beff <= 128 && K >= 64) {
+  if (warp_per_run_pays(beff, K)) {
     const int64_t items = rows * ((K + 127) / 128);
     int64_t blocks = (items + kThreads / 32 - 1) / (kThreads / 32);
     if (blocks > cap) blocks = cap;

@@ -112,10 +112,11 @@ binarize_dense_rows(const float* __restrict__ x, int64_t ldx, int64_t rows, int6
       for (int off = 1; off < LANES; off <<= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
       sum[0] = sum[1] = sum[2] = sum[3] = s;
     }
+    float mean[4];
 #pragma unroll
     for (int e = 0; e < 4; e++) {
-      const int64_t left = K - (k0 + e) / BETA * BETA;
-      o[e] = with_sign_of(sum[e] / static_cast<float>(left < BETA ? (left > 0 ? left : 1) : BETA), xv[e]);
+      mean[e] = e % (BETA < 4 ? BETA : 4) == 0 ? group_mean<BETA>(sum[e], k0, e, K) : mean[e - 1];      // one per group
+      o[e] = with_sign_of(mean[e], xv[e]);
     }
     store4<VEC>(out + r * ldo, k0, K, o);
   }
@@ -173,9 +174,7 @@ cudaError_t launch_typed(const float* x, int64_t ldx, int64_t rows, int64_t K, i
     }
     return cudaGetLastError();
   }
-  // rows shorter than 64 leave more than half of a warp's lanes idle: 229376 rows of 28 at beta 16 36 us in the
-  // thread-per-group kernel and 94 us in the rows kernel, 100000 rows of 56 at beta 32 45 and 43 us
-  if (pow2 && beff <= 128 && K >= 64) {
+  if (warp_per_run_pays(beff, K)) {
     const int64_t items = rows * ((K + 127) / 128);
     int64_t blocks = (items + kThreads / 32 - 1) / (kThreads / 32);
     if (blocks > cap) blocks = cap;

@@ -44,5 +44,23 @@ __device__ __forceinline__ void store4(__nv_bfloat16* row, int64_t k, int64_t K,
   }
 }
 
+// A group sum as a mean, for the group that holds a lane's element e of four (the lane starts at k, k a multiple of four,
+// groups of BETA from the row's start, the last one of its own length).  A whole group's length is a power of two: the
+// product with its inverse is the quotient, bit for bit, and takes one instruction where the division takes a dozen.
+template <int BETA>
+__device__ __forceinline__ float group_mean(float sum, int64_t k, int e, int64_t K) {
+  const int64_t left = K - (BETA >= 4 ? k / BETA * BETA : k + e / BETA * BETA);      // elements from the group's start on
+  if (left >= BETA) return sum * (1.0f / static_cast<float>(BETA));
+  return sum / static_cast<float>(left > 0 ? left : 1);
+}
+
+// Whether a warp per 128 elements of a row beats a thread per group.  Rows shorter than 64 leave more than half of its lanes
+// idle, and a group of four is one 16-byte load for the thread that owns it, so that at beta 4 the warp has to be nearly
+// full: backward of 85523 x 64, padded, at beta 4 18.6 us per group and 35 per warp, of 10302 x 1728 51 and 44.
+inline bool warp_per_run_pays(int64_t beta, int64_t K) {
+  const int64_t lanes_for = (K + 127) / 128 * 128;
+  return (beta & (beta - 1)) == 0 && beta <= 128 && K >= 64 && (beta != 4 || 5 * K >= 4 * lanes_for);
+}
+
 }  // namespace rowio
 }  // namespace hbmm

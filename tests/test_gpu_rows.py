@@ -11,6 +11,7 @@ pytestmark = pytest.mark.gpu
 
 CASES = [(r, K, b, pad) for b in (1, 2, 4, 8, 16, 32, 64, 128) for r, K, pad in ((9, 131, 0), (5, 260, 4), (3, 388 - b // 2, 1))]
 CASES += [(7, 64, 128, 0), (1, 65, 64, 3), (300, 127, 16, 0)]
+CASES += [(9, 126, 4, 0), (5, 250, 4, 6), (3, 511, 4, 1)]          # nearly full warps: groups of four take them only then
 
 
 @pytest.mark.parametrize("rows,K,beta,pad", CASES)
