@@ -36,7 +36,7 @@ struct TileArgs {
   float* C;
   int64_t M, N, K, lda_w, ldw_w, lda_s, ldw_s, ldc;
   int64_t ra, rw;              // segments per A group / per W group
-  int64_t Ga, Gw;              // groups per row
+  int64_t T;                   // segments per row
   int64_t n_words, n_chunks;
   int32_t a_bf16, w_bf16;
   int32_t ks_log2;             // warps that share a tile's K range: 1 << ks_log2
@@ -80,18 +80,28 @@ __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
   return v;
 }
 __device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-// acc += (sa sw) * (counts - bias) for two neighbouring outputs; c0, c1: 2^23 + doubled count as bit patterns
+// acc += sa sw (counts - bias) for two neighbouring outputs; c0, c1: 2^23 + doubled count as bit patterns.  DOT_FIRST: the
+// first product is (counts - bias) sa, so that a segment whose signs cancel adds 0 also where the product of its scales
+// leaves the range of fp32; 4 % slower at segments of 2 and 8 bits, which take the product of the scales first.
+template <bool DOT_FIRST>
 __device__ __forceinline__ void add_term(uint64_t& acc, uint32_t c0, uint32_t c1, uint64_t neg_bias, uint64_t sa, uint64_t sw) {
-  uint64_t f = pack2(__uint_as_float(c0), __uint_as_float(c1)), s;
+  uint64_t f = pack2(__uint_as_float(c0), __uint_as_float(c1));
   asm("add.rn.f32x2 %0, %0, %1;" : "+l"(f) : "l"(neg_bias));
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(s) : "l"(sa), "l"(sw));
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(s), "l"(f));
+  if constexpr (DOT_FIRST) {
+    asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(f) : "l"(sa));
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(f), "l"(sw));
+  } else {
+    uint64_t s;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(s) : "l"(sa), "l"(sw));
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(s), "l"(f));
+  }
 }
 
 template <int SEG>
 __global__ void __launch_bounds__(kThreads, 2)
 gemm_popc_tile_kernel(const TileArgs g) {
   pdl_wait();
+  pdl_launch_dependents();      // a convolution's next front end sets itself up meanwhile
   using P = Cfg<SEG>;
   // The next chunk waits in registers, except for the finest segments: their counts and scales need those registers
   // (spills otherwise), and a chunk is 1000 instructions and more, which the other warps fill a load's latency with.
@@ -100,7 +110,7 @@ gemm_popc_tile_kernel(const TileArgs g) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int KS = 1 << g.ks_log2;
   const int part = warp & (KS - 1);
-  const int64_t m0 = (static_cast<int64_t>(blockIdx.y) * (kWarps >> g.ks_log2) + (warp >> g.ks_log2)) * TS;
+  const int64_t m0 = (static_cast<int64_t>(blockIdx.y) * (blockDim.x >> (5 + g.ks_log2)) + (warp >> g.ks_log2)) * TS;
   const int64_t n0 = static_cast<int64_t>(blockIdx.x) * TS;
   const int tx = lane & 3, ty = lane >> 2;              // columns 8 tx .., rows 4 ty ..
   uint32_t* as = smem + warp * P::SMEM_WORDS;           // [CW][32]
@@ -124,8 +134,8 @@ gemm_popc_tile_kernel(const TileArgs g) {
   auto fetch = [&](int64_t c) {
     load_words<P::CW>(arow, c * P::CW, g.lda_w, ain, pa);
     load_words<P::CW>(wrow, c * P::CW, g.ldw_w, win, pw);
-    load_scales<P::SPC>(g.a_scales, g.a_bf16, aoff, c * P::SPC, g.ra, g.Ga, ain, psa);
-    load_scales<P::SPC>(g.w_scales, g.w_bf16, woff, c * P::SPC, g.rw, g.Gw, win, psw);
+    load_scales<P::SPC>(g.a_scales, g.a_bf16, aoff, c * P::SPC, g.ra, g.T, ain, psa);
+    load_scales<P::SPC>(g.w_scales, g.w_bf16, woff, c * P::SPC, g.rw, g.T, win, psw);
   };
   if (m0 < g.M && part < g.n_chunks) {                  // warp-uniform
     if (kAhead) fetch(part);
@@ -158,7 +168,7 @@ gemm_popc_tile_kernel(const TileArgs g) {
         for (int i = 0; i < 4; i++) {
           const uint64_t sa2 = pack2(sa[i], sa[i]);
 #pragma unroll
-          for (int j = 0; j < 4; j++) add_term(acc[i][j], counts(i, 2 * j), counts(i, 2 * j + 1), neg_bias, sa2, sw[j]);
+          for (int j = 0; j < 4; j++) add_term<(SEG >= 32)>(acc[i][j], counts(i, 2 * j), counts(i, 2 * j + 1), neg_bias, sa2, sw[j]);
         }
       };
       auto words = [&](int i, uint32_t (&a)[4], uint32_t (&w)[8]) {
@@ -171,6 +181,7 @@ gemm_popc_tile_kernel(const TileArgs g) {
         constexpr int PARTS = 8 / SEG;
 #pragma unroll 1
         for (int i = 0; i < P::CW; i++) {
+          if (P::CW > 1 && left_chunk <= 32 * i) break;      // words past the row's end
 #pragma unroll 1
           for (int p = 0; p < PARTS; p++) {
             uint32_t a[4], w[8], cnt[4][8];
@@ -187,6 +198,7 @@ gemm_popc_tile_kernel(const TileArgs g) {
       } else if constexpr (SEG == 16) {
 #pragma unroll
         for (int i = 0; i < P::CW; i++) {
+          if (left_chunk <= 32 * i) break;
           uint32_t a[4], w[8];
           words(i, a, w);
           segment(2 * i, [&](int r, int j) { return 0x4B000000u + 2u * __popc((a[r] ^ w[j]) & 0xFFFFu); });
@@ -195,6 +207,7 @@ gemm_popc_tile_kernel(const TileArgs g) {
       } else if constexpr (SEG == 32) {
 #pragma unroll
         for (int i = 0; i < P::CW; i++) {
+          if (left_chunk <= 32 * i) break;
           uint32_t a[4], w[8];
           words(i, a, w);
           segment(i, [&](int r, int j) { return 0x4B000000u + 2u * __popc(a[r] ^ w[j]); });
@@ -202,6 +215,7 @@ gemm_popc_tile_kernel(const TileArgs g) {
       } else {
 #pragma unroll
         for (int s = 0; s < P::SPC; s++) {
+          if (P::SPC > 1 && left_chunk <= s * SEG) break;
           uint32_t cnt[4][8];
 #pragma unroll
           for (int q = 0; q < P::SW; q++) {
@@ -278,9 +292,12 @@ cudaError_t launch_seg(TileArgs g, int sms, cudaStream_t stream) {
   const int64_t tiles_m = (g.M + TS - 1) / TS, tiles_n = (g.N + TS - 1) / TS, want = static_cast<int64_t>(sms) * 16;
   g.ks_log2 = 0;
   while (g.ks_log2 < 3 && (tiles_m * tiles_n << g.ks_log2) < want && (2ll << g.ks_log2) <= g.n_chunks) g.ks_log2++;
-  const int64_t per_cta = kWarps >> g.ks_log2;
+  // short rows leave whole tiles to a warp; where eight of them to a CTA leave SMs without one, fewer
+  int warps = kWarps;
+  while (warps > (1 << g.ks_log2) && tiles_n * ((tiles_m * (1 << g.ks_log2) + warps - 1) / warps) < 2 * sms) warps /= 2;
+  const int64_t per_cta = warps >> g.ks_log2;
   const dim3 grid(static_cast<unsigned>(tiles_n), static_cast<unsigned>((tiles_m + per_cta - 1) / per_cta));
-  launch_pdl(gemm_popc_tile_kernel<SEG>, dim3(grid), dim3(kThreads), 0, stream, g);
+  launch_pdl(gemm_popc_tile_kernel<SEG>, dim3(grid), dim3(warps * 32), 0, stream, g);
   return cudaGetLastError();
 }
 
@@ -309,8 +326,7 @@ cudaError_t launch_gemm_popc_tile(const PackedView& A, const PackedView& W, floa
   const int64_t T = (A.K + seg - 1) / seg;
   g.ra = A.beta >= A.K ? T : A.beta / seg;
   g.rw = W.beta >= W.K ? T : W.beta / seg;
-  g.Ga = num_groups(A.K, A.beta);
-  g.Gw = num_groups(W.K, W.beta);
+  g.T = T;
   g.n_words = (A.K + 31) / 32;
   int dev = 0, sms = 0;
   if (current_device(&dev, &sms) != cudaSuccess) return cudaErrorInvalidDevice;

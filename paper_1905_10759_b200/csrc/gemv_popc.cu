@@ -28,7 +28,6 @@ struct GemvArgs {
   int64_t N, K, lda_w, ldw_w, lda_s, ldw_s, ldc;
   int32_t M, a_bf16, w_bf16;
   int32_t ra, rw;        // segments per A group / per W group
-  int64_t Ga, Gw;        // groups per row
   int32_t n_quads;       // 16-byte pieces per row: ceil(K / 128)
   int32_t T;             // segments per row
 };
@@ -119,14 +118,14 @@ gemv_popc_sub_kernel(const GemvArgs g) {
     for (int q = lane; q < n_words; q += 32) {
       const uint32_t w = __ldg(wrow + q);
       float sw[SPW];
-      load_scales<SPW>(g.w_scales, g.w_bf16, n * g.ldw_s, static_cast<int64_t>(q) * SPW, g.rw, g.Gw, true, sw);
+      load_scales<SPW>(g.w_scales, g.w_bf16, n * g.ldw_s, static_cast<int64_t>(q) * SPW, g.rw, g.T, true, sw);
       const int64_t left = g.K - static_cast<int64_t>(q) * 32;          // valid bits from the word's start
 #pragma unroll
       for (int m = 0; m < MR; m++) {
         const bool in = m < g.M;
         const uint32_t x = w ^ (in ? __ldg(g.a_bits + m * g.lda_w + q) : 0u);
         float sa[SPW];
-        load_scales<SPW>(g.a_scales, g.a_bf16, m * g.lda_s, static_cast<int64_t>(q) * SPW, g.ra, g.Ga, in, sa);
+        load_scales<SPW>(g.a_scales, g.a_bf16, m * g.lda_s, static_cast<int64_t>(q) * SPW, g.ra, g.T, in, sa);
         uint32_t cnt[PARTS];
         if constexpr (SEG <= 8) {
 #pragma unroll
@@ -172,8 +171,6 @@ bool make_args(const PackedView& A, const PackedView& W, GemvArgs& g) {
   g.M = static_cast<int32_t>(A.rows); g.a_bf16 = A.scale_bf16; g.w_bf16 = W.scale_bf16;
   g.ra = static_cast<int32_t>(a_one ? T : A.beta / seg);
   g.rw = static_cast<int32_t>(w_one ? T : W.beta / seg);
-  g.Ga = num_groups(A.K, A.beta);
-  g.Gw = num_groups(W.K, W.beta);
   g.n_quads = static_cast<int32_t>(quads);
   g.T = static_cast<int32_t>(T);
   return true;

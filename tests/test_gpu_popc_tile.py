@@ -39,3 +39,39 @@ def test_popc_tiles_match_oracle(M, N, K, ba, bw, sdt):
     # per segment two roundings, then at most one per segment and one per joined part
     T = -(-K // min(ea, ew))
     gu.assert_close_rel_absref(out[:, :N], c_ref, absref, (T + 8 + 2) * gu.U, "popc")
+
+
+@pytest.mark.parametrize("N", [1, 2, 3])
+@pytest.mark.parametrize("b", [2, 4, 8, 16, 32, 64, 128, 256])
+def test_narrowest_tiles_match_oracle(b, N):
+    """Nine rows (the fewest that reach this kernel) and columns that no vector store covers; K of less than one chunk, and
+    of several with words past the row's end in the last."""
+    import gpu_util as gu
+    from paper_1905_10759_b200 import hbmm
+    for K in (21, 1061):
+        a, w = inputs.normal((9, K), 4150 + K + b), inputs.he_normal(N, K, 5150 + N + K + b)
+        A, da, sa = gu.oracle_operand(a, b, 0)
+        W, dw, sw = gu.oracle_operand(w, b, 0)
+        e = gu.eff_beta(b, K)
+        c_ref, absref = oracle.hbmm_from_quantized(da, sa, e, dw, sw, e)
+        C = torch.full((9, 8), float("nan"), device="cuda")
+        hbmm.gemm_ex(A, W, C, hbmm.PATH_POPC)
+        assert torch.isnan(C[:, N:]).all()
+        gu.assert_close_rel_absref(C[:, :N].cpu().numpy(), c_ref, absref, (-(-K // e) + 8 + 2) * gu.U, "popc")
+
+
+@pytest.mark.parametrize("b", [32, 64, 128, 256])
+def test_cancelling_group_with_scales_beyond_the_range_of_their_product(b):
+    """A group of whole words whose signs cancel adds nothing, also where the product of its two scales is above the largest fp32."""
+    import gpu_util as gu
+    from paper_1905_10759_b200 import hbmm
+    import numpy as np
+    M, N, K = 40, 33, 4 * b
+    a, w = np.ones((M, K), np.float32), np.ones((N, K), np.float32)
+    a[:, b: 2 * b], w[:, b: 2 * b] = 1e25, 1e25
+    w[:, b: 2 * b: 2] = -1e25
+    A, da, sa = gu.oracle_operand(a, b, 0)
+    W, dw, sw = gu.oracle_operand(w, b, 0)
+    C = torch.full((M, (N + 3) // 4 * 4), float("nan"), device="cuda")
+    hbmm.gemm_ex(A, W, C, hbmm.PATH_POPC)
+    assert torch.equal(C[:, :N].cpu(), torch.full((M, N), float(3 * b)))
