@@ -204,8 +204,22 @@ cudaError_t launch_sub(const GemvArgs& g, int sms, cudaStream_t stream) {
   if (g.M <= 1) launch_pdl(gemv_popc_sub_kernel<SEG, 1>, dim3(grid), dim3(kWarps * 32), 0, stream, g);
   else if (g.M <= 2) launch_pdl(gemv_popc_sub_kernel<SEG, 2>, dim3(grid), dim3(kWarps * 32), 0, stream, g);
   else if (g.M <= 4) launch_pdl(gemv_popc_sub_kernel<SEG, 4>, dim3(grid), dim3(kWarps * 32), 0, stream, g);
-  else launch_pdl(gemv_popc_sub_kernel<SEG, 8>, dim3(grid), dim3(kWarps * 32), 0, stream, g);
+  else if constexpr (SEG < 16) launch_pdl(gemv_popc_sub_kernel<SEG, 8>, dim3(grid), dim3(kWarps * 32), 0, stream, g);
+  else return cudaErrorNotSupported;
   return cudaGetLastError();
+}
+
+// Sub-word groups: against 32 x 32 tiles (gemm_popc_tile.cu), which form 32 rows whatever M is but share each word's counts
+// and scales between them.  A warp here needs 32 words to fill its lanes and repeats the scales' work per row: many rows,
+// short K and many columns are the tiles'.  Times over those of the tiles, N = 8000 (smaller N in brackets, up to 2000):
+// one row 1.2 at one or two words, 0.9 .. 0.1 above (0.8 .. 0.1); two rows 1.7 / 0.9 .. 0.2 from five words on (0.8 .. 0.1); four
+// rows 2.8 / 0.8 .. 0.4 from 12 on, at beta 16 1.5 .. 0.8 (1.0 .. 0.2); eight rows 6 .. 0.9 (1.9 .. 0.3; beta 16 1.7 .. 0.85).
+bool sub_word_pays(int64_t rows, int64_t N, int64_t n_words, int seg) {
+  if (rows <= 2) return N <= 4096 || n_words > 2 * rows;
+  if (rows <= 4) return N <= 4096 || n_words > (seg == 16 ? 128 : 8);
+  if (seg == 16) return false;
+  if (N <= 1024) return n_words > (seg == 8 ? 8 : 2);
+  return N <= 2048 ? n_words > 8 : seg > 2 && n_words > 128;
 }
 
 }  // namespace
@@ -215,7 +229,8 @@ cudaError_t launch_sub(const GemvArgs& g, int sms, cudaStream_t stream) {
 bool gemv_popc_supported(const PackedView& A, const PackedView& W) {
   GemvArgs g;
   if (!make_args(A, W, g)) return false;
-  if (segment_of(A, W) < 32) return true;
+  const int64_t seg = segment_of(A, W);
+  if (seg < 32) return sub_word_pays(g.M, g.N, (g.K + 31) / 32, static_cast<int>(seg));
   return smem_bytes(g, 8, 1) <= 48 * 1024;
 }
 
