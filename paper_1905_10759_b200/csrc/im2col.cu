@@ -126,13 +126,15 @@ im2col_quantize_groups_kernel(const void* __restrict__ x, int x_bf16, const Conv
 // Groups shorter than a word: one thread per (row m, K-word), 32 consecutive rows per warp as above; a thread emits the word
 // and the means of its 32 / BETA groups.  One thread per row leaves most of the machine idle and walks all of K serially:
 // 3136 rows of 4608 at beta 4 from bf16 1019 us against 43 here, 3025 rows of 12800 at beta 8 2.1 ms against 86 us.
+// A block takes 1 << words_log2 words (at most eight) of as many runs of 32 rows as its other warps: rows of one word, eight
+// warps to a word, left seven of them idle (200704 rows of 8 at beta 4 31 us against 10 in the thread-per-row kernel).
 template <int BETA>
 __global__ void __launch_bounds__(256)
 im2col_quantize_words_kernel(const void* __restrict__ x, int x_bf16, const ConvGeom g, int64_t M, int64_t K, int64_t G, int64_t n_words,
-                             uint32_t* __restrict__ bits, int64_t ld_words, void* __restrict__ scales, int64_t ld_scales, int scale_bf16) {
+                             int words_log2, uint32_t* __restrict__ bits, int64_t ld_words, void* __restrict__ scales, int64_t ld_scales, int scale_bf16) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t m = static_cast<int64_t>(blockIdx.x) * 32 + lane;
-  const int64_t wi = static_cast<int64_t>(blockIdx.y) * 8 + warp;
+  const int64_t m = (static_cast<int64_t>(blockIdx.x) * (8 >> words_log2) + (warp >> words_log2)) * 32 + lane;
+  const int64_t wi = (static_cast<int64_t>(blockIdx.y) << words_log2) + (warp & ((1 << words_log2) - 1));
   if (m >= M || wi >= n_words) return;
   const int xo = static_cast<int>(m % g.Wo);
   const int yo = static_cast<int>((m / g.Wo) % g.Ho);
@@ -147,6 +149,7 @@ im2col_quantize_words_kernel(const void* __restrict__ x, int x_bf16, const ConvG
   uint32_t word = 0;
 #pragma unroll
   for (int t = 0; t < 32 / BETA; t++) {
+    if (k0 + t * BETA >= K) break;
     float s[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int e = 0; e < BETA; e++) {
@@ -160,8 +163,7 @@ im2col_quantize_words_kernel(const void* __restrict__ x, int x_bf16, const ConvG
       }
     }
     const int64_t left = K - (k0 + t * BETA);
-    if (left > 0)
-      store_scale(scales, scale_bf16, m * ld_scales + wi * (32 / BETA) + t, ((s[0] + s[1]) + (s[2] + s[3])) / static_cast<float>(left < BETA ? left : BETA));
+    store_scale(scales, scale_bf16, m * ld_scales + wi * (32 / BETA) + t, ((s[0] + s[1]) + (s[2] + s[3])) / static_cast<float>(left < BETA ? left : BETA));
   }
   bits[m * ld_words + wi] = word;
   if (wi == n_words - 1) {
@@ -455,10 +457,17 @@ cudaError_t launch_im2col_quantize(const void* x, int x_bf16, const ConvGeom& g,
                                                              ld_words, scales, ld_scales, scale_bf16);
     return cudaGetLastError();
   }
-  const int64_t n_words = (K + 31) / 32, word_blocks = (n_words + 7) / 8;
-  if (beta < K && (beta == 2 || beta == 4 || beta == 8 || beta == 16) && word_blocks <= 65535) {
-    const dim3 grid(static_cast<unsigned>((M + 31) / 32), static_cast<unsigned>(word_blocks));
-#define HBMM_IW(B) case B: im2col_quantize_words_kernel<B><<<grid, 256, 0, stream>>>(x, x_bf16, g, M, K, G, n_words, bits, ld_words, scales, ld_scales, scale_bf16); break;
+  const int64_t n_words = (K + 31) / 32;
+  int words_log2 = 0;
+  while (words_log2 < 3 && (1 << words_log2) < n_words) words_log2++;
+  const int64_t word_blocks = (n_words + (1 << words_log2) - 1) >> words_log2;
+  // rows of up to three words keep a machine full of rows busy by themselves: 466 thousand rows of 75 at beta 16 81 us in
+  // words, 63 in rows; 50176 rows are level
+  const bool words_pay = n_words > 3 || M < 65536 || (beta == 2 && n_words > 1);
+  if (words_pay && beta < K && (beta == 2 || beta == 4 || beta == 8 || beta == 16) && word_blocks <= 65535) {
+    const int64_t rows = 32 * (8 >> words_log2);
+    const dim3 grid(static_cast<unsigned>((M + rows - 1) / rows), static_cast<unsigned>(word_blocks));
+#define HBMM_IW(B) case B: im2col_quantize_words_kernel<B><<<grid, 256, 0, stream>>>(x, x_bf16, g, M, K, G, n_words, words_log2, bits, ld_words, scales, ld_scales, scale_bf16); break;
     switch (beta) { HBMM_IW(2) HBMM_IW(4) HBMM_IW(8) HBMM_IW(16) }
 #undef HBMM_IW
     return cudaGetLastError();
