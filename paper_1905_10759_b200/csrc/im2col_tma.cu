@@ -462,11 +462,27 @@ bool make_plan(const ConvGeom& g, int sms, bool flat, int32_t beta, Plan* out, s
   return false;
 }
 
+// Strided filters: a tile holds every input row and column between the taps and may leave only a few pixels to an item, so
+// the kernels that gather from global memory win where a filter has many taps that skip much of the image.  Groups of whole
+// words: up to 3 x 3 always staged (stride 2 to 8, 0.1 .. 1.05 of the gather's time), up to 5 x 5 where neighbouring filters
+// overlap (256 x 28 x 28, 5 x 5: stride 2 0.6 .. 1.1, stride 8 1.3 .. 2.0), 7 x 7 at stride 2 (0.4 .. 1.3, large images 0.6; at
+// stride 4 1.0 .. 1.6), above not (11 x 11 1.4 .. 3.8).  Groups shorter than a word, whose gather has a thread per word: the
+// filters with a gather of their own (3 x 3 0.4 .. 1.2), 2 x 2 for as many words as leave that gather to its latency (0.6 .. 0.8;
+// above, or at stride 5, 1.1 .. 2.0), 5 x 5 not (1.4 .. 1.8), nor rows of less than a word (63 images of 8 x 56 x 56, 1 x 1 at stride 3: 2.2).
+bool stage_strided(const ConvGeom& g, int32_t beta) {
+  const int taps = g.kh * g.kw;
+  if (beta >= 32) return taps <= 9 || (taps <= 25 && g.sw < g.kw) || (taps <= 49 && 3 * g.sw <= g.kw);
+  if (g.C * taps < 32) return false;
+  const int64_t words = static_cast<int64_t>(g.B) * g.Ho * g.Wo * ((static_cast<int64_t>(g.C) * taps + 31) / 32);
+  return (g.kh == 3 && g.kw == 3) || taps == 1 || (taps <= 9 && g.sw <= 2 * g.kw && words <= 24576);
+}
+
 // 0: not supported, 1: tensor-copy tiles with halo, 2: flat channel planes
 int tma_mode(const void* x, int x_bf16, const ConvGeom& g, int32_t beta) {
   const int64_t K = static_cast<int64_t>(g.C) * g.kh * g.kw;
   const bool beta_ok = beta == 2 || beta == 4 || beta == 8 || beta == 16 || (beta >= 32 && beta % 32 == 0 && beta / 32 <= 64);
   if (x_bf16 || !beta_ok || beta >= K || reinterpret_cast<uintptr_t>(x) % 16 != 0) return 0;
+  if (g.sw != 1 && !stage_strided(g, beta)) return 0;
   Plan p;
   size_t smem;
   int dev = 0, sms = 0;
