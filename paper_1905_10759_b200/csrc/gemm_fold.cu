@@ -914,10 +914,13 @@ constexpr int64_t kBalancedMaxShare = 4;
 // stages win (64 x 1024 x 1024, 16 stages: 17.4 -> 8.0 us in eight parts).
 constexpr int64_t kSplitMinStages = 2;
 constexpr int64_t kSplitFromStages = 6;
-// 128-column tiles: the wide accumulator from this many stages per tile on.  50176 x 128 x 1152 (18 stages) 40.4 -> 43.5 us,
-// 4096 x 4096 x 512 (8) 47 -> 52, 4096 x 4096 x 1024 (16) 84 -> 85; 3000 x 3000 x 1472 (23) 75 -> 68, 4096 x 4096 x 2048 (32)
-// 159 -> 152, 3136 x 512 x 4608 (72) 50 -> 45 us.
-constexpr int64_t kWideFromStages = 20;
+// 128-column tiles: the wide accumulator from this many stages per tile on.  Its epilogue is exposed at the end of every tile
+// but a CTA's last, so that the line lies further out the more tiles a CTA walks and the slower they leave it.  Wide over
+// narrow at 20 / 27 / 36 / 50 stages (K = 1280 / 1728 / 2304 / 3200): at most two tiles per CTA 0.85 .. 1.0 / 0.94 .. 0.99 / 0.92 ..
+// 0.97 / 0.86 .. 0.94; more 0.96 .. 1.09 / 0.94 .. 1.06 / 0.91 .. 1.01 / 0.89 .. 0.98; fused, more than one tile per CTA: rows
+// stored as vectors 0.98 .. 1.08 / 0.97 .. 1.05 / 0.95 .. 1.03 / 0.93 .. 1.0, packed rows and rows off 16 bytes 0.98 .. 1.18 / 0.97
+// .. 1.15 / 0.98 .. 1.14 / 0.95 .. 1.08 (and 0.92 .. 1.03 at 72).
+constexpr int64_t kWideFromStages = 20, kWideFromManyTiles = 30, kWideFromSlowRows = 60;
 // Plain schedule: above this many bytes of expanded weights the tiles are walked in blocks of as many columns as hold
 // kBlockBytes of them.  Row by row over all columns every wave of CTAs read all of the weights again, from memory once they
 // exceed the L2 (8192^3: 268 MB a wave, 7.5 GB in all, under the power cap): 3.29 -> 2.49 ms with blocks of 8, 18 or 36 MB
@@ -1121,8 +1124,16 @@ cudaError_t launch_fold_wide(Args g, void* workspace, size_t have, cudaStream_t 
 
 template <int TN, int ASUB, bool FUSE = false>
 cudaError_t launch_fold(const Args& g, void* workspace, size_t have, cudaStream_t stream, bool w_prepared) {
-  const int64_t n_stages = (g.n_words + WPS - 1) / WPS;
-  if (TN == 128 && n_stages >= kWideFromStages) return launch_fold_wide<TN, ASUB, FUSE, TN == 128>(g, workspace, have, stream, w_prepared);
+  if constexpr (TN == 128) {
+    int dev = 0, sms = 0;
+    if (current_device(&dev, &sms) != cudaSuccess) return cudaErrorInvalidDevice;
+    const int64_t n_stages = (g.n_words + WPS - 1) / WPS, tiles = tile_count<TN>(g);
+    const bool vector_rows = g.ep.mode == kEpiDense && reinterpret_cast<uintptr_t>(g.ep.out) % 16 == 0 &&
+                             g.ep.ld_out * (g.ep.out_bf16 ? 2 : 4) % 16 == 0;
+    const int64_t from = FUSE && tiles > sms ? (vector_rows ? kWideFromManyTiles : kWideFromSlowRows)
+                                             : (tiles > 2 * static_cast<int64_t>(sms) ? kWideFromManyTiles : kWideFromStages);
+    if (n_stages >= from) return launch_fold_wide<TN, ASUB, FUSE, true>(g, workspace, have, stream, w_prepared);
+  }
   return launch_fold_wide<TN, ASUB, FUSE, false>(g, workspace, have, stream, w_prepared);
 }
 
