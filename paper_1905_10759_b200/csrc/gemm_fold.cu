@@ -344,9 +344,11 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
 
   // The first tile's row factors are found by the producer warps, two threads per row, while their first words and scales
   // are on the way: nothing can be expanded before they are known, and the scouts (two rows per thread) take several
-  // memory round trips for a long row.  (Where a row has few scales and a CTA many tiles this costs 1 %: the scouts' later
-  // tiles start later.  It runs for split tiles and for sub-word groups.)
-  const bool scan_first = (SPLIT || ASUB > 1) && my_tiles > 0 && !(ASUB > 1 && g.a_rowmax);
+  // memory round trips for a long row.  Runs for split tiles and for sub-word groups, where a row's scales are long enough for
+  // it to pay (off over on: 256 x 1000, beta 32 fp32, 144 / 576 / 1152 bytes 0.98 / 1.06 / 1.11; beta 4, 2088 x 64, 64 / 128 / 192 /
+  // 384 bytes 0.95 / 1.00 / 1.05 / 1.09, of bf16 scales 128 / 192 / 320 0.95 / 1.06 / 1.13).
+  const int64_t row_bytes = g.lda_s * (g.a_bf16 ? 2 : 4);
+  const bool scan_first = (SPLIT || ASUB > 1) && row_bytes >= (ASUB > 1 ? 192 : 288) && my_tiles > 0 && !(ASUB > 1 && g.a_rowmax);
 
   // The CTA is persistent: it walks tiles blockIdx.x, blockIdx.x + gridDim.x, ... and the stage ring
   // simply continues across tiles (gst counts stages since launch).
