@@ -87,7 +87,7 @@ binarize_dense_stream(const float4* __restrict__ x, OUT* __restrict__ out, int64
 // Rows that end inside a group, or are padded, or start off a 16-byte boundary (beta a power of two up to 128): a warp
 // takes 128 consecutive elements of a row, so groups never leave it; absent elements are zeros, the last group divides by
 // its own length.  One thread per group, as below, walks its group serially, 4-byte loads beta elements apart:
-// 173 x 3180 at beta 128 to bf16 69 us against 3.4 us here; 8192 x 1000 at beta 64 118 against 19 us.
+// 173 x 3180 at beta 128 to bf16 68 us against 2.0 here; 8192 x 1000 at beta 64 95 against 12.
 template <int BETA, bool VEC, typename OUT>
 __global__ void __launch_bounds__(kThreads)
 binarize_dense_rows(const float* __restrict__ x, int64_t ldx, int64_t rows, int64_t K, OUT* __restrict__ out, int64_t ldo) {
@@ -174,7 +174,7 @@ cudaError_t launch_typed(const float* x, int64_t ldx, int64_t rows, int64_t K, i
     }
     return cudaGetLastError();
   }
-  if (warp_per_run_pays(beff, K)) {
+  if (warp_per_run_pays(beff, K, sizeof(OUT) == 2)) {
     const int64_t items = rows * ((K + 127) / 128);
     int64_t blocks = (items + kThreads / 32 - 1) / (kThreads / 32);
     if (blocks > cap) blocks = cap;

@@ -56,10 +56,12 @@ __device__ __forceinline__ float group_mean(float sum, int64_t k, int e, int64_t
 
 // Whether a warp per 128 elements of a row beats a thread per group.  Rows shorter than 64 leave more than half of its lanes
 // idle, and a group of four is one 16-byte load for the thread that owns it, so that at beta 4 the warp has to be nearly
-// full: backward of 85523 x 64, padded, at beta 4 18.6 us per group and 35 per warp, of 10302 x 1728 51 and 44.
-inline bool warp_per_run_pays(int64_t beta, int64_t K) {
+// full: backward of 85523 x 64, padded, at beta 4 16 us per group and 28 per warp, of 10302 x 1728 51 and 40.  Groups of
+// eight that leave as bf16 want it well above half full: dense of 73938 x 64 15.4 and 17.6 us.
+inline bool warp_per_run_pays(int64_t beta, int64_t K, bool half_out = false) {
   const int64_t lanes_for = (K + 127) / 128 * 128;
-  return (beta & (beta - 1)) == 0 && beta <= 128 && K >= 64 && (beta != 4 || 5 * K >= 4 * lanes_for);
+  if ((beta & (beta - 1)) != 0 || beta > 128 || K < 64) return false;
+  return beta == 4 ? 5 * K >= 4 * lanes_for : beta != 8 || !half_out || 5 * K >= 3 * lanes_for;
 }
 
 }  // namespace rowio
