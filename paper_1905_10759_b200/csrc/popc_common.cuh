@@ -12,9 +12,10 @@ __device__ __forceinline__ float load_scale(const void* s, int bf16, int64_t idx
   return __ldg(reinterpret_cast<const float*>(s) + idx);
 }
 
-// s / r for segment numbers: the 64-bit division is a tenth of a chunk's instructions (5104 x 536 x 6912 at beta 256 / 16
-// 549 against 484 us without it), and segments hardly ever need it.
+// s / r for segment numbers.  The 64-bit division is a noticeable part of a chunk's instructions (5104 x 536 x 6912 at beta
+// 256 / 16 550 us with it, 520 with the 32-bit one); r is a power of two unless a group is three words or the like.
 __device__ __forceinline__ int64_t div_segments(int64_t s, int64_t r) {
+  if ((r & (r - 1)) == 0) return s >> (63 - __clzll(r));
   if (((s | r) >> 32) == 0) return static_cast<uint32_t>(s) / static_cast<uint32_t>(r);
   return s / r;
 }
