@@ -39,6 +39,7 @@
 #include <cuda_fp16.h>
 #include <atomic>
 #include "kernels.h"
+#include "split_choice.h"
 #include "tensor_map.h"
 #include "umma_common.cuh"
 #include "gemm_fold_prep.cuh"
@@ -229,7 +230,6 @@ __device__ __forceinline__ void first_rows_barrier() {
 }
 
 // Split mode: byte offset of the 16-byte piece u of row `row` of a partial tile.
-constexpr int kMaxSplit = 8;            // CTAs that may share a tile (the portable cluster size)
 template <int TN>
 __device__ __forceinline__ int split_piece(int row, int u) { return row * (TN * 4) + ((u ^ (row & 7)) << 4); }
 __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
@@ -912,10 +912,7 @@ constexpr int64_t kMaxBalancedCtas = 256;
 constexpr int64_t kBalancedWaves = 4;
 constexpr int64_t kBalancedMinStages = 4;
 constexpr int64_t kBalancedMaxShare = 4;
-// Split mode: 256 x 256 x 256 (four stages) takes 7.4 us whole and 7.8 us in two parts; from six stages on parts of two
-// stages win (64 x 1024 x 1024, 16 stages: 17.4 -> 8.0 us in eight parts).
-constexpr int64_t kSplitMinStages = 2;
-constexpr int64_t kSplitFromStages = 6;
+std::atomic<int> g_resident_clusters[64][kMaxSplit + 1];        // per device, see choose_split
 // 128-column tiles: the wide accumulator from this many stages per tile on.  Its epilogue is exposed at the end of every tile
 // but a CTA's last, so that the line lies further out the more tiles a CTA walks and the slower they leave it.  Wide over
 // narrow at 20 / 27 / 36 / 50 stages (K = 1280 / 1728 / 2304 / 3200): at most two tiles per CTA 0.85 .. 1.0 / 0.94 .. 0.99 / 0.92 ..
@@ -980,39 +977,22 @@ void set_balanced_area(Args& g, void* workspace, size_t have) {
   if (reserved) g.sk_partials = reinterpret_cast<float*>(area + counters);
 }
 
-// Split mode: the largest number of CTAs per tile (2 .. 8, at least two stages each) for which every tile's cluster is
-// resident at once; 1: not worth it.  Taken where the tiles cover at most half of the machine.  Against the balanced
-// schedule, whose last CTA adds the partial tiles through global memory (12 .. 20 rounds of loads by four warps):
-// 256 x 1000 x 4096 28.4 -> 16.2 us, 256 x 4096 x 4096 39 -> 30, 256 x 4096 x 9216 61.5 -> 56, 49 x 512 x 4608 26.6 -> 12.2,
-// 1024^3 24.2 -> 13.2 us; and the second accumulator brings the error of a result from 4e-7 .. 4e-6 to 1e-7 .. 1.8e-6.  (All instantiations take a whole SM per CTA, so they share what was asked once.)
+// Clusters of `size` CTAs of the kernel that the current device holds at once.
 template <typename Kernel>
-int choose_split(Kernel kernel, int smem_bytes, int dev, int sms, int64_t tiles, int64_t n_stages) {
-  static std::atomic<int> resident[64][kMaxSplit + 1];           // clusters of each size the device holds, plus one; 0: not asked yet
-  if (2 * tiles > sms || n_stages < kSplitFromStages || dev < 0 || dev >= 64) return 1;
-  int64_t most = n_stages / kSplitMinStages;
-  if (most > kMaxSplit) most = kMaxSplit;
-  for (int s = static_cast<int>(most); s >= 2; s--) {
-    if (tiles * s > sms) continue;
-    int n = resident[dev][s].load(std::memory_order_relaxed);
-    if (n == 0) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(static_cast<unsigned>(s));
-      cfg.blockDim = dim3(kThreads);
-      cfg.dynamicSmemBytes = static_cast<size_t>(smem_bytes);
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = static_cast<unsigned>(s);
-      attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      int got = 0;
-      if (cudaOccupancyMaxActiveClusters(&got, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); got = 0; }
-      n = got + 1;
-      resident[dev][s].store(n, std::memory_order_relaxed);
-    }
-    if (tiles <= n - 1) return s;
-  }
-  return 1;
+bool resident_clusters(Kernel kernel, int smem_bytes, int size, int* clusters) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(size));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = static_cast<size_t>(smem_bytes);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(size);
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaOccupancyMaxActiveClusters(clusters, kernel, &cfg) == cudaSuccess) return true;
+  cudaGetLastError();
+  return false;
 }
 
 // Launched without programmatic serialization: its few CTAs would all land on the first SMs the kernel before leaves (that
@@ -1093,7 +1073,9 @@ cudaError_t launch_fold_wide(Args g, void* workspace, size_t have, cudaStream_t 
   }
   const int64_t tiles = ((g.M + TM - 1) / TM) * tiles_n;
   if constexpr (!FUSE) {
-    const int split = choose_split(hbmm_fold_kernel<TN, ASUB, FUSE, kSplit, kSplitWide>, kBytes, dev, sms, tiles, n_stages);
+    // (all instantiations take a whole SM per CTA, so they share what was asked once)
+    const auto ask = [](int size, int* clusters) { return resident_clusters(hbmm_fold_kernel<TN, ASUB, FUSE, kSplit, kSplitWide>, kBytes, size, clusters); };
+    const int split = dev >= 0 && dev < 64 ? choose_split(g_resident_clusters[dev], sms, tiles, n_stages, ask) : 1;
     if (split > 1) {
       g.split = split;
       return launch_pdl_cluster(hbmm_fold_kernel<TN, ASUB, FUSE, kSplit, kSplitWide>, dim3(static_cast<unsigned>(tiles * split)), dim3(kThreads),
