@@ -107,12 +107,21 @@ def _dtype_code(dt: torch.dtype) -> int:
     raise TypeError("only float32 and bfloat16 tensors are accepted, got %s" % dt)
 
 
+# The current stream's raw handle, asked for directly: building the stream object torch.cuda.current_stream() returns takes
+# 3.2 us, a third of a whole call (9.1 us), the handle 0.2 us.  Neither function is part of torch's public interface, so a
+# torch without them takes the stream object, and so does a process in which CUDA is not up yet (the object brings it up, or
+# says why it cannot: no driver, a forked child).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device_index = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream: Optional[torch.cuda.Stream]) -> int:
-    """Raw handle of `stream`, or of the current device's current stream.  The handle is asked for directly: building the
-    stream object torch.cuda.current_stream() returns takes 3.2 us, a third of a whole call (9.1 us), the handle 0.2 us."""
+    """Raw handle of `stream`, or of the current device's current stream."""
     if stream is not None:
         return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if _raw_stream is None or _device_index is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_device_index())
 
 
 def _dev_ptr(t: Optional[torch.Tensor]) -> Optional[int]:

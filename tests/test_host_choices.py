@@ -1,6 +1,9 @@
-"""Host-side choices that need no GPU: the split of a tile between CTAs when the occupancy query fails."""
+"""Host-side choices that need no GPU: the split of a tile between CTAs when the occupancy query fails, and the stream handle
+the binding passes on."""
 import os
 import subprocess
+
+import torch
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -27,3 +30,19 @@ def test_failed_occupancy_query_is_not_kept(tmp_path):
     src.write_text(SPLIT)
     subprocess.run(["g++", "-std=c++17", "-O1", "-I", os.path.join(ROOT, "paper_1905_10759_b200", "csrc"), str(src), "-o", str(exe)], check=True)
     assert subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split() == ["1", "8", "8", "0", "1"]
+
+
+def test_stream_handle_without_private_functions_or_before_cuda_is_up(monkeypatch):
+    from paper_1905_10759_b200 import hbmm
+
+    class Stream:
+        cuda_stream = 7
+
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: Stream())
+    monkeypatch.setattr(hbmm, "_device_index", lambda: 3)
+    monkeypatch.setattr(hbmm, "_raw_stream", lambda device: 40 + device)
+    for up, raw, want in ((True, hbmm._raw_stream, 43), (False, hbmm._raw_stream, 7), (True, None, 7)):
+        monkeypatch.setattr(torch.cuda, "is_initialized", lambda up=up: up)
+        monkeypatch.setattr(hbmm, "_raw_stream", raw)
+        assert hbmm._stream(None) == want
+        assert hbmm._stream(Stream()) == 7
