@@ -10,7 +10,11 @@ runs the four HBMM calls on one stream and the four HBWN calls on a second one, 
 step (the one-stream time is reported beside it).  The metric is effective binary TOPS =
 2*M*N*K summed over the eight products / step time.
 
-    python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
+    python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--rows FILE]
+
+The last line of standard output is one JSON object of a few KB: the timed step, its end-to-end leg, the clocks, the dominant
+kernel's roofline, and one short row per kernel and per configuration.  `--rows FILE` writes the whole record there (every
+field of those rows, and the side measurements, which are taken only then).
 
 With N > 1 (torchrun, one rank per GPU) every rank runs its own batch of 64 images (weak
 scaling, no data-path collective); the time is the max over ranks.  `--impl reference` times
@@ -953,6 +957,47 @@ def run_reference(args):
     return 0
 
 
+# ----------------------------------------------------------------------------- what is printed
+# Fields of a configuration's row that the printed line keeps.
+ROW_KEEP = ("name", "beta", "scale_dtype", "hbmm_gemm_ms", "conv_call_ms", "warm_l2_ms", "cold_l2_ms_median", "tops", "tops_warm",
+            "frac_of_popcount_hbm_roofline", "frac_of_fp32_add_hbm_roofline", "frac_of_popcount_hbm_roofline_cold")
+LINE_BYTES = 16000          # a longer line is cut by readers that keep the end of the output
+
+
+def short_numbers(v):
+    """Floats to six significant digits, all the way down."""
+    if isinstance(v, float):
+        return float("%.6g" % v)
+    if isinstance(v, dict):
+        return {k: short_numbers(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [short_numbers(x) for x in v]
+    return v
+
+
+def printed_line(record, rows_file=None):
+    """The record as the one line that is printed: the contract's fields as they are, the rows cut to what ROW_KEEP names."""
+    line = dict(record)
+    line.pop("other_rows", None)
+    line.pop("context", None)
+    rates = line.pop("measured_alu_rates", None) or {}
+    line["measured_alu_rates"] = {k: v.get("ops_per_s") if isinstance(v, dict) else v for k, v in rates.items() if k != "planning_figures"}
+    line["kernels"] = {k: [{f: r[f] for f in ("layer", "ms", "frac") if f in r} if isinstance(r, dict) else r for r in v]
+                       for k, v in (record.get("kernels") or {}).items()}
+    line["configs"] = [{k: r[k] for k in ROW_KEEP if k in r} for r in record.get("configs") or []] or None
+    if rows_file:
+        line["rows_file"] = rows_file
+    contract = {k: line[k] for k in ("value", "ms_per_step", "e2e")}
+    line = short_numbers(line)
+    line.update(contract)
+    text = json.dumps(line, allow_nan=False)
+    if len(text) > LINE_BYTES:                       # the contract's fields come first
+        for k in ("configs", "kernels", "measured_alu_rates"):
+            line.pop(k, None)
+        text = json.dumps(line, allow_nan=False)
+    return text
+
+
 # ----------------------------------------------------------------------------- main arm
 def run_ours(args):
     import torch
@@ -1107,7 +1152,8 @@ def run_ours(args):
     configs = None
     if world == 1:
         configs = config_rows(torch, hbmm, inputs, layers, brk, rates, peaks, 10)
-        side = side_measurements(torch, hbmm, inputs, peaks, max(5, min(args.steps, 20)))
+        if args.rows:
+            side = side_measurements(torch, hbmm, inputs, peaks, max(5, min(args.steps, 20)))
         base, _, _ = cpu_baseline(shapes, 12.0)
         err = hbmm.last_device_error()
         if err != 0:
@@ -1148,7 +1194,10 @@ def run_ours(args):
     }
     if base is not None:
         line["cpu_baseline"] = base
-    print(json.dumps(line))
+    if args.rows:
+        with open(args.rows, "w") as f:
+            json.dump(line, f, indent=1)
+    print(printed_line(line, args.rows))
     if world > 1:
         import torch.distributed as dist
         dist.barrier()
@@ -1166,6 +1215,8 @@ def main():
                     help="run the warm-up and the timed steps only, no measurement: for a profiler's launch list")
     ap.add_argument("--profile-layer", default=None,
                     help="run only this layer (conv2_x .. conv5_x), few launches, no measurement: for profiler captures")
+    ap.add_argument("--rows", default=None, metavar="FILE",
+                    help="write the whole record there, side measurements included (they run only with this)")
     args = ap.parse_args()
     if args.impl == "reference":
         return run_reference(args)
