@@ -109,8 +109,7 @@ def _dtype_code(dt: torch.dtype) -> int:
 
 # The current stream's raw handle, asked for directly: building the stream object torch.cuda.current_stream() returns takes
 # 3.2 us, a third of a whole call (9.1 us), the handle 0.2 us.  Neither function is part of torch's public interface, so a
-# torch without them takes the stream object, and so does a process in which CUDA is not up yet (the object brings it up, or
-# says why it cannot: no driver, a forked child).
+# torch without them takes the stream object.
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 _device_index = getattr(torch._C, "_cuda_getDevice", None)
 
@@ -119,7 +118,7 @@ def _stream(stream: Optional[torch.cuda.Stream]) -> int:
     """Raw handle of `stream`, or of the current device's current stream."""
     if stream is not None:
         return stream.cuda_stream
-    if _raw_stream is None or _device_index is None or not torch.cuda.is_initialized():
+    if _raw_stream is None or _device_index is None:
         return torch.cuda.current_stream().cuda_stream
     return _raw_stream(_device_index())
 

@@ -32,7 +32,7 @@ def test_failed_occupancy_query_is_not_kept(tmp_path):
     assert subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split() == ["1", "8", "8", "0", "1"]
 
 
-def test_stream_handle_without_private_functions_or_before_cuda_is_up(monkeypatch):
+def test_stream_handle_without_private_functions(monkeypatch):
     from paper_1905_10759_b200 import hbmm
 
     class Stream:
@@ -40,9 +40,7 @@ def test_stream_handle_without_private_functions_or_before_cuda_is_up(monkeypatc
 
     monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: Stream())
     monkeypatch.setattr(hbmm, "_device_index", lambda: 3)
-    monkeypatch.setattr(hbmm, "_raw_stream", lambda device: 40 + device)
-    for up, raw, want in ((True, hbmm._raw_stream, 43), (False, hbmm._raw_stream, 7), (True, None, 7)):
-        monkeypatch.setattr(torch.cuda, "is_initialized", lambda up=up: up)
+    for raw, want in ((lambda device: 40 + device, 43), (None, 7)):
         monkeypatch.setattr(hbmm, "_raw_stream", raw)
         assert hbmm._stream(None) == want
         assert hbmm._stream(Stream()) == 7
