@@ -32,7 +32,8 @@
 //   warp  13    : one thread streams the prepared W stages (cp.async.bulk, completion on the stage's
 //                 mbarrier); W is expanded once per call (or once per weight tensor) into a workspace
 // A stage holds 64 K-elements (two packed words): 64 TMEM columns of A pieces and the W stage in shared
-// memory.  Tensor memory: two accumulators of TN columns, the rest is the ring of A stages.  Stages and the
+// memory.  Tensor memory: two accumulators (of TN columns; of 2 TN for the 64-column tile) or, for long and split
+// 128-column tiles, one of 256 columns; the rest is the ring of A stages.  Stages and the
 // accumulators are mbarrier rings.  Every wait is bounded: on expiry the thread records a code, raises a
 // CTA-wide abort flag that all other waits observe, and the kernel drains and frees its TMEM before returning.
 #include <cuda_bf16.h>
@@ -309,7 +310,7 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
   // Plain schedule: where the expanded weights are larger than what the L2 keeps, the tiles are walked in blocks of
   // g.group_n column tiles, row by row inside a block, so that all row tiles of a block read the same few columns' weights.
   auto in_blocks = [&](int64_t t) -> int64_t {
-    if (!WIDE || g.group_n == 0 || t >= n_tiles) return t;      // short tiles have small weights; the test there costs them 2 %
+    if (!WIDE || g.group_n == 0 || t >= n_tiles) return t;      // short tiles: the test costs them 2 %, and only tens of thousands of columns give them weights this large
     const int64_t blk = t / (g.group_n * tiles_m), r = t - blk * (g.group_n * tiles_m);
     const int64_t n0 = blk * g.group_n, w = tiles_n - n0 < g.group_n ? tiles_n - n0 : g.group_n;
     return (r / w) * tiles_n + n0 + r % w;

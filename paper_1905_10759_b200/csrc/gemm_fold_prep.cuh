@@ -14,6 +14,7 @@
 #include <cuda_fp16.h>
 #include <cstdint>
 #include "kernels.h"
+#include "popc_common.cuh"
 #include "umma_common.cuh"
 
 namespace hbmm {
@@ -34,8 +35,9 @@ struct Smem {
   static constexpr int A_COLS = 2 * (KB / 2);             // TMEM columns of one A stage: two pieces x 64 fp16 (two per 32-bit column)
   // A tensor-core instruction costs about the same for 64 and for 128 columns, so the narrow tile stacks
   // the two weight pieces along N: one MMA of 2 TN columns forms A1 W1 and A1 W2 side by side (the epilogue
-  // adds the two blocks) and a second one of TN columns adds A2 W1.  The wide tile has no room for a
-  // 256-column accumulator pair beside the A ring and adds all three products into the same TN columns.
+  // adds the two blocks) and a second one of TN columns adds A2 W1.  For 128-column tiles the accumulators'
+  // 256 columns are either two accumulators into which all three products add, or, for long and for split
+  // tiles, one accumulator of 256 columns stacked like the narrow tile's (WIDE in the kernel).
   static constexpr bool STACKED = TN == 64;
   static constexpr int ACC_COLS = STACKED ? 2 * TN : TN;  // one fp32 accumulator
   static constexpr int STAGES = (512 - 2 * ACC_COLS) / A_COLS;        // 4: the rest of the 512 columns
@@ -56,10 +58,7 @@ struct Smem {
   static_assert(STAGES >= 3 && A_BASE + STAGES * A_COLS <= 512, "accumulators and the A ring share 512 columns");
 };
 
-__device__ __forceinline__ float load_scale(const void* s, int bf16, int64_t idx) {
-  if (bf16) return __uint_as_float(static_cast<uint32_t>(__ldg(reinterpret_cast<const unsigned short*>(s) + idx)) << 16);
-  return __ldg(reinterpret_cast<const float*>(s) + idx);
-}
+using popc::load_scale;
 
 // Largest scale of one operand row.  Rows are 16-byte vectors (the leading dimension is a multiple of 4
 // fp32 / 8 bf16 entries) and entries past the last group are stored zeros.  Scales are >= 0, so their bit

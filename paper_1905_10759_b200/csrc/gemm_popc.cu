@@ -3,18 +3,15 @@
 // word segments.  For every output element and every 32-bit K-word: p = popc(a ^ w); the signed +-1 dot of a K-segment is
 // D = n_valid - 2 * sum(p); C += (deltaA * deltaW) * D in fp32.  The segment is min(beta_a, beta_w); the operand with the
 // coarser groups reuses its scale across segments.  Pad bits are zero in both operands.
-#include <cuda_bf16.h>
 #include "kernels.h"
+#include "popc_common.cuh"
 
 namespace hbmm {
 namespace {
 
-constexpr int kThreads = 256;
+using popc::load_scale;
 
-__device__ __forceinline__ float load_scale(const void* s, int bf16, int64_t idx) {
-  if (bf16) return __uint_as_float(static_cast<uint32_t>(__ldg(reinterpret_cast<const unsigned short*>(s) + idx)) << 16);
-  return __ldg(reinterpret_cast<const float*>(s) + idx);
-}
+constexpr int kThreads = 256;
 
 struct GemmArgs {
   const uint32_t* a_bits; const void* a_scales;
@@ -23,7 +20,6 @@ struct GemmArgs {
   int64_t M, N, K, lda_w, ldw_w, lda_s, ldw_s, ldc;
   int32_t a_bf16, w_bf16;
   int32_t ra, rw;        // groups: A group = segment / ra, W group = segment / rw
-  int64_t Ga, Gw;        // number of groups per row
   int64_t n_words;       // ceil(K/32)
   int64_t T;             // number of segments
   int32_t seg_words;     // words per segment
@@ -119,8 +115,6 @@ GemmArgs make_args(const PackedView& A, const PackedView& W, float* C, int64_t l
   g.T = (A.K + seg - 1) / seg;
   g.ra = static_cast<int32_t>(a_one ? g.T : A.beta / seg);
   g.rw = static_cast<int32_t>(w_one ? g.T : W.beta / seg);
-  g.Ga = num_groups(A.K, A.beta);
-  g.Gw = num_groups(W.K, W.beta);
   return g;
 }
 

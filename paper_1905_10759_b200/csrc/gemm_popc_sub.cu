@@ -7,14 +7,11 @@ namespace hbmm {
 namespace {
 
 struct SubArgs {
-  const uint32_t* a_bits; const void* a_scales;
-  const uint32_t* w_bits; const void* w_scales;
-  float* C;
-  int64_t M, N, K, lda_w, ldw_w, lda_s, ldw_s, ldc;
-  int32_t a_bf16, w_bf16;
+  const uint32_t* a_bits;
+  const uint32_t* w_bits;
+  int64_t M, N, K, lda_w, ldw_w;
   int32_t seg;                 // bits per segment: 2, 4, 8 or 16
-  int64_t a_beta, w_beta;      // group length in elements (K when there is one group per row)
-  int64_t n_words, T;          // ceil(K / 32), ceil(K / seg)
+  int64_t T;                   // segments per row: ceil(K / seg)
 };
 
 // D[m,n,t] = n_valid(t) - 2 * popc over the bits of segment t.
@@ -33,16 +30,13 @@ partials_popc_sub_kernel(const SubArgs g, int32_t* __restrict__ D) {
   }
 }
 
-SubArgs make_args(const PackedView& A, const PackedView& W, float* C, int64_t ldc) {
+SubArgs make_args(const PackedView& A, const PackedView& W) {
+  const int64_t a = A.beta >= A.K ? A.K : A.beta, w = W.beta >= W.K ? W.K : W.beta;
   SubArgs g;
-  g.a_bits = A.bits; g.a_scales = A.scales; g.w_bits = W.bits; g.w_scales = W.scales; g.C = C;
+  g.a_bits = A.bits; g.w_bits = W.bits;
   g.M = A.rows; g.N = W.rows; g.K = A.K;
-  g.lda_w = A.ld_words; g.ldw_w = W.ld_words; g.lda_s = A.ld_scales; g.ldw_s = W.ld_scales; g.ldc = ldc;
-  g.a_bf16 = A.scale_bf16; g.w_bf16 = W.scale_bf16;
-  g.a_beta = A.beta >= A.K ? A.K : A.beta;
-  g.w_beta = W.beta >= W.K ? W.K : W.beta;
-  g.seg = static_cast<int32_t>(g.a_beta < g.w_beta ? g.a_beta : g.w_beta);
-  g.n_words = (A.K + 31) / 32;
+  g.lda_w = A.ld_words; g.ldw_w = W.ld_words;
+  g.seg = static_cast<int32_t>(a < w ? a : w);
   g.T = (A.K + g.seg - 1) / g.seg;
   return g;
 }
@@ -57,7 +51,7 @@ bool gemm_subword(const PackedView& A, const PackedView& W) {
 }
 
 cudaError_t launch_partials_popc_sub(const PackedView& A, const PackedView& W, int32_t* D, cudaStream_t stream) {
-  const SubArgs g = make_args(A, W, nullptr, 0);
+  const SubArgs g = make_args(A, W);
   const int64_t total = g.M * g.N * g.T;
   int64_t blocks = (total + 255) / 256;
   if (blocks > 148 * 32) blocks = 148 * 32;
