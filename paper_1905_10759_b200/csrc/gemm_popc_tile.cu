@@ -52,6 +52,79 @@ struct Cfg {
   static constexpr int SMEM_WORDS = WARP_WORDS > TS * TS ? WARP_WORDS : TS * TS;   // ... which its partial sums reuse
 };
 
+// s / r for segment numbers.  The 64-bit division is a noticeable part of a chunk's instructions (5104 x 536 x 6912 at beta
+// 256 / 16 550 us with it, 520 with the 32-bit one); r is a power of two unless a group is three words or the like.
+__device__ __forceinline__ int64_t div_segments(int64_t s, int64_t r) {
+  if ((r & (r - 1)) == 0) return s >> (63 - __clzll(r));
+  if (((s | r) >> 32) == 0) return static_cast<uint32_t>(s) / static_cast<uint32_t>(r);
+  return s / r;
+}
+
+// The scales of SPC consecutive segments of one row from segment s0 on, r segments to a group; 0 past the last of the T
+// segments.  One group per segment, in order: 16-byte loads of fp32 scales, 4-byte loads of bf16 pairs (s0 is a multiple of
+// SPC, rows are 16-byte vectors); otherwise one load per segment, or one for all.
+template <int SPC>
+__device__ __forceinline__ void chunk_scales(const void* s, int bf16, int64_t row_off, int64_t s0, int64_t r, int64_t T, bool in, float (&v)[SPC]) {
+#pragma unroll
+  for (int i = 0; i < SPC; i++) v[i] = 0.0f;
+  if (!in) return;
+  if (SPC >= 4 && r == 1 && !bf16) {
+#pragma unroll
+    for (int q = 0; q < SPC / 4; q++)
+      if (s0 + 4 * q < T) {
+        const float4 x = __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(s) + row_off + s0 + 4 * q));
+        v[(4 * q) % SPC] = x.x;
+        if (s0 + 4 * q + 1 < T) v[(4 * q + 1) % SPC] = x.y;
+        if (s0 + 4 * q + 2 < T) v[(4 * q + 2) % SPC] = x.z;
+        if (s0 + 4 * q + 3 < T) v[(4 * q + 3) % SPC] = x.w;
+      }
+    return;
+  }
+  if (SPC == 2 && r == 1 && !bf16) {
+    if (s0 < T) {
+      const float2 x = __ldg(reinterpret_cast<const float2*>(reinterpret_cast<const float*>(s) + row_off + s0));
+      v[0] = x.x;
+      if (s0 + 1 < T) v[SPC - 1] = x.y;
+    }
+    return;
+  }
+  if (SPC >= 2 && r == 1 && bf16) {
+#pragma unroll
+    for (int q = 0; q < SPC / 2; q++)
+      if (s0 + 2 * q < T) {
+        const uint32_t x = __ldg(reinterpret_cast<const uint32_t*>(reinterpret_cast<const unsigned short*>(s) + row_off + s0 + 2 * q));
+        v[(2 * q) % SPC] = __uint_as_float(x << 16);
+        if (s0 + 2 * q + 1 < T) v[(2 * q + 1) % SPC] = __uint_as_float(x & 0xFFFF0000u);
+      }
+    return;
+  }
+  if (s0 >= T) return;
+  if (r == 1) {
+#pragma unroll
+    for (int i = 0; i < SPC; i++)
+      if (s0 + i < T) v[i] = load_scale(s, bf16, row_off + s0 + i);
+    return;
+  }
+  if (r % SPC == 0 || SPC % r == 0) {          // whole groups, or all inside one: a load per group
+    const int64_t g0 = div_segments(s0, r);
+    const int mask = r < SPC ? static_cast<int>(r) - 1 : SPC - 1;
+    int64_t g = row_off + g0;
+    float x = 0.0f;
+#pragma unroll
+    for (int i = 0; i < SPC; i++) {
+      if ((i & mask) == 0 && s0 + i < T) x = load_scale(s, bf16, g++);
+      if (s0 + i < T) v[i] = x;
+    }
+    return;
+  }
+  int64_t g = div_segments(s0, r), rem = s0 - g * r;
+#pragma unroll
+  for (int i = 0; i < SPC; i++) {
+    if (s0 + i < T) v[i] = load_scale(s, bf16, row_off + g);
+    if (++rem >= r) { rem = 0; g++; }
+  }
+}
+
 // The CW packed words of one row from word w0 on (rows are padded to a multiple of four words).
 template <int CW>
 __device__ __forceinline__ void load_words(const uint32_t* row, int64_t w0, int64_t ld, bool in, uint32_t (&v)[CW]) {
@@ -97,7 +170,9 @@ __device__ __forceinline__ void add_term(uint64_t& acc, uint32_t c0, uint32_t c1
   }
 }
 
-template <int SEG>
+// MIXED: some group spans several segments (ra, rw not both 1).  The lookup for that, in every kernel, costs the uniform
+// groupings registers: 2 % at 2-bit segments, 5 % at 32.
+template <int SEG, bool MIXED>
 __global__ void __launch_bounds__(kThreads, 2)
 gemm_popc_tile_kernel(const TileArgs g) {
   pdl_wait();
@@ -134,8 +209,13 @@ gemm_popc_tile_kernel(const TileArgs g) {
   auto fetch = [&](int64_t c) {
     load_words<P::CW>(arow, c * P::CW, g.lda_w, ain, pa);
     load_words<P::CW>(wrow, c * P::CW, g.ldw_w, win, pw);
-    load_scales<P::SPC>(g.a_scales, g.a_bf16, aoff, c * P::SPC, g.ra, g.T, ain, psa);
-    load_scales<P::SPC>(g.w_scales, g.w_bf16, woff, c * P::SPC, g.rw, g.T, win, psw);
+    if constexpr (MIXED) {
+      chunk_scales<P::SPC>(g.a_scales, g.a_bf16, aoff, c * P::SPC, g.ra, g.T, ain, psa);
+      chunk_scales<P::SPC>(g.w_scales, g.w_bf16, woff, c * P::SPC, g.rw, g.T, win, psw);
+    } else {
+      load_scales<P::SPC>(g.a_scales, g.a_bf16, aoff, c * P::SPC, 1, g.T, ain, psa);
+      load_scales<P::SPC>(g.w_scales, g.w_bf16, woff, c * P::SPC, 1, g.T, win, psw);
+    }
   };
   if (m0 < g.M && part < g.n_chunks) {                  // warp-uniform
     if (kAhead) fetch(part);
@@ -207,7 +287,6 @@ gemm_popc_tile_kernel(const TileArgs g) {
       } else if constexpr (SEG == 32) {
 #pragma unroll
         for (int i = 0; i < P::CW; i++) {
-          if (left_chunk <= 32 * i) break;
           uint32_t a[4], w[8];
           words(i, a, w);
           segment(i, [&](int r, int j) { return 0x4B000000u + 2u * __popc(a[r] ^ w[j]); });
@@ -215,7 +294,6 @@ gemm_popc_tile_kernel(const TileArgs g) {
       } else {
 #pragma unroll
         for (int s = 0; s < P::SPC; s++) {
-          if (P::SPC > 1 && left_chunk <= s * SEG) break;
           uint32_t cnt[4][8];
 #pragma unroll
           for (int q = 0; q < P::SW; q++) {
@@ -297,7 +375,8 @@ cudaError_t launch_seg(TileArgs g, int sms, cudaStream_t stream) {
   while (warps > (1 << g.ks_log2) && tiles_n * ((tiles_m * (1 << g.ks_log2) + warps - 1) / warps) < 2 * sms) warps /= 2;
   const int64_t per_cta = warps >> g.ks_log2;
   const dim3 grid(static_cast<unsigned>(tiles_n), static_cast<unsigned>((tiles_m + per_cta - 1) / per_cta));
-  launch_pdl(gemm_popc_tile_kernel<SEG>, dim3(grid), dim3(warps * 32), 0, stream, g);
+  if (g.ra == 1 && g.rw == 1) launch_pdl(gemm_popc_tile_kernel<SEG, false>, dim3(grid), dim3(warps * 32), 0, stream, g);
+  else launch_pdl(gemm_popc_tile_kernel<SEG, true>, dim3(grid), dim3(warps * 32), 0, stream, g);
   return cudaGetLastError();
 }
 

@@ -28,6 +28,7 @@ struct GemvArgs {
   int64_t N, K, lda_w, ldw_w, lda_s, ldw_s, ldc;
   int32_t M, a_bf16, w_bf16;
   int32_t ra, rw;        // segments per A group / per W group
+  int64_t Ga, Gw;        // groups per row
   int32_t n_quads;       // 16-byte pieces per row: ceil(K / 128)
   int32_t T;             // segments per row
 };
@@ -118,14 +119,14 @@ gemv_popc_sub_kernel(const GemvArgs g) {
     for (int q = lane; q < n_words; q += 32) {
       const uint32_t w = __ldg(wrow + q);
       float sw[SPW];
-      load_scales<SPW>(g.w_scales, g.w_bf16, n * g.ldw_s, static_cast<int64_t>(q) * SPW, g.rw, g.T, true, sw);
+      load_scales<SPW>(g.w_scales, g.w_bf16, n * g.ldw_s, static_cast<int64_t>(q) * SPW, g.rw, g.Gw, true, sw);
       const int64_t left = g.K - static_cast<int64_t>(q) * 32;          // valid bits from the word's start
 #pragma unroll
       for (int m = 0; m < MR; m++) {
         const bool in = m < g.M;
         const uint32_t x = w ^ (in ? __ldg(g.a_bits + m * g.lda_w + q) : 0u);
         float sa[SPW];
-        load_scales<SPW>(g.a_scales, g.a_bf16, m * g.lda_s, static_cast<int64_t>(q) * SPW, g.ra, g.T, in, sa);
+        load_scales<SPW>(g.a_scales, g.a_bf16, m * g.lda_s, static_cast<int64_t>(q) * SPW, g.ra, g.Ga, in, sa);
         uint32_t cnt[PARTS];
         if constexpr (SEG <= 8) {
 #pragma unroll
@@ -171,6 +172,8 @@ bool make_args(const PackedView& A, const PackedView& W, GemvArgs& g) {
   g.M = static_cast<int32_t>(A.rows); g.a_bf16 = A.scale_bf16; g.w_bf16 = W.scale_bf16;
   g.ra = static_cast<int32_t>(a_one ? T : A.beta / seg);
   g.rw = static_cast<int32_t>(w_one ? T : W.beta / seg);
+  g.Ga = num_groups(A.K, A.beta);
+  g.Gw = num_groups(W.K, W.beta);
   g.n_quads = static_cast<int32_t>(quads);
   g.T = static_cast<int32_t>(T);
   return true;
@@ -204,22 +207,23 @@ cudaError_t launch_sub(const GemvArgs& g, int sms, cudaStream_t stream) {
   if (g.M <= 1) launch_pdl(gemv_popc_sub_kernel<SEG, 1>, dim3(grid), dim3(kWarps * 32), 0, stream, g);
   else if (g.M <= 2) launch_pdl(gemv_popc_sub_kernel<SEG, 2>, dim3(grid), dim3(kWarps * 32), 0, stream, g);
   else if (g.M <= 4) launch_pdl(gemv_popc_sub_kernel<SEG, 4>, dim3(grid), dim3(kWarps * 32), 0, stream, g);
-  else if constexpr (SEG < 16) launch_pdl(gemv_popc_sub_kernel<SEG, 8>, dim3(grid), dim3(kWarps * 32), 0, stream, g);
-  else return cudaErrorNotSupported;
+  else launch_pdl(gemv_popc_sub_kernel<SEG, 8>, dim3(grid), dim3(kWarps * 32), 0, stream, g);
   return cudaGetLastError();
 }
 
 // Sub-word groups: against 32 x 32 tiles (gemm_popc_tile.cu), which form 32 rows whatever M is but share each word's counts
 // and scales between them.  A warp here needs 32 words to fill its lanes and repeats the scales' work per row: many rows,
-// short K and many columns are the tiles'.  Times over those of the tiles, N = 8000 (smaller N in brackets, up to 2000):
-// one row 1.2 at one or two words, 0.9 .. 0.1 above (0.8 .. 0.1); two rows 1.7 / 0.9 .. 0.2 from five words on (0.8 .. 0.1); four
-// rows 2.8 / 0.8 .. 0.4 from 12 on, at beta 16 1.5 .. 0.8 (1.0 .. 0.2); eight rows 6 .. 0.9 (1.9 .. 0.3; beta 16 1.7 .. 0.85).
-bool sub_word_pays(int64_t rows, int64_t N, int64_t n_words, int seg) {
-  if (rows <= 2) return N <= 4096 || n_words > 2 * rows;
-  if (rows <= 4) return N <= 4096 || n_words > (seg == 16 ? 128 : 8);
-  if (seg == 16) return false;
-  if (N <= 1024) return n_words > (seg == 8 ? 8 : 2);
-  return N <= 2048 ? n_words > 8 : seg > 2 && n_words > 128;
+// short K and many columns are the tiles'.  Time here over theirs, measured at 1, 2, 4, 5 and 8 rows, 64 to 9000 columns and 24
+// to 9216 elements: one and two rows 0.1 .. 1.1, over 4096 columns 1.0 .. 2.0 up to two words per row and below one above; four
+// rows 0.2 .. 1.0 up to 2048 columns, above 1.0 .. 2.7 at up to four (eight) words, then 0.3 .. 0.95, but at beta 16 0.9 .. 1.6 to
+// 60 words; eight rows 1.0 .. 1.4 to four words and 0.3 .. 1.0 above, beyond 2048 columns 1.0 .. 4.5 to 16 words and 0.5 .. 1.5
+// above; at beta 16 five rows 0.65 .. 1.3, eight 0.9 .. 3.4.
+bool sub_word_pays(int64_t rows, int64_t N, int64_t n_words, int64_t seg) {
+  const bool wide = N > 4096;
+  if (rows <= 2) return !wide || n_words > 2 * rows;
+  if (rows <= 4) return N <= 2048 || n_words > (seg == 16 ? 60 : (wide ? 8 : 4));
+  if (seg == 16) return rows <= 6 && !wide && n_words > 3;
+  return n_words > (N <= 2048 ? 6 : 16);
 }
 
 }  // namespace
@@ -230,7 +234,7 @@ bool gemv_popc_supported(const PackedView& A, const PackedView& W) {
   GemvArgs g;
   if (!make_args(A, W, g)) return false;
   const int64_t seg = segment_of(A, W);
-  if (seg < 32) return sub_word_pays(g.M, g.N, (g.K + 31) / 32, static_cast<int>(seg));
+  if (seg < 32) return sub_word_pays(g.M, g.N, (g.K + 31) / 32, seg);
   return smem_bytes(g, 8, 1) <= 48 * 1024;
 }
 

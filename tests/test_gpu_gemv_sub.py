@@ -9,6 +9,7 @@ from paper_1905_10759_b200 import inputs
 pytestmark = pytest.mark.gpu
 
 CASES = [(M, N, K, b, b, 0) for b in (2, 4, 8, 16) for M, N, K in ((1, 9, 31), (3, 33, 1056), (8, 17, 2055))]
+CASES += [(6, 21, 301, 16, 16, 0), (5, 30, 1111, 16, 16, 1)]      # five and six rows at 16: beyond, the tiles take them
 CASES += [(5, 40, 777, 2, 64, 0), (2, 41, 777, 32, 8, 1), (4, 7, 333, 333, 16, 0), (6, 8, 100, 4, 4, 1), (7, 1500, 96, 16, 2, 0)]
 
 
