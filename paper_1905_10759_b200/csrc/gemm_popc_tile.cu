@@ -14,9 +14,11 @@
 // popcount instruction.  (One masked popcount per 2-bit segment would keep that unit busy for 128 clk per word and warp
 // against ~75 issue slots this way; at 16 bits the two are level.)
 // Measured against one 64 x 64 (sub-word) or 128 x 128 (word) tile per CTA, which this replaces: 333 x 720 x 1000 at
-// beta 16 28.5 -> 9.7 us, 82 x 536 x 3768 at beta 64 90 -> 9.2 us, 4050 x 280 x 4368 at beta 16 203 -> 104 us; on the
-// conv3_x matrix (50176 x 128 x 1152) beta 2 / 4 / 8 / 16 / 32 / 128: 1337 / 660 / 332 / 172 / 90 / 81 ->
-// 926 / 640 / 326 / 153 / 83 / 71 us.  Scalar fp32 instead of the paired instructions: 5 % slower.
+// beta 16 27.8 -> 8.9 us, 82 x 536 x 3768 at beta 64 90 -> 9.4 us, 4050 x 280 x 4368 at beta 16 203 -> 107 us; on the
+// conv3_x matrix (50176 x 128 x 1152) beta 2 / 4 / 8 / 16 / 32 / 128: 1337 / 662 / 334 / 172 / 89 / 81 ->
+// 926 / 546 / 327 / 159 / 83 / 67 us.  Slower than those tiles only at mixed groupings of sub-word segments over long K (5104 x
+// 536 x 6912 at beta 256 / 16 487 -> 516), whose scales each warp loads for itself.  Scalar fp32 instead of the paired
+// instructions: 5 % slower.
 #include "kernels.h"
 #include "pdl.cuh"
 #include "popc_common.cuh"
@@ -53,7 +55,7 @@ struct Cfg {
 };
 
 // s / r for segment numbers.  The 64-bit division is a noticeable part of a chunk's instructions (5104 x 536 x 6912 at beta
-// 256 / 16 550 us with it, 520 with the 32-bit one); r is a power of two unless a group is three words or the like.
+// 256 / 16 550 us with it, 516 without); r is a power of two unless a group is three words or the like.
 __device__ __forceinline__ int64_t div_segments(int64_t s, int64_t r) {
   if ((r & (r - 1)) == 0) return s >> (63 - __clzll(r));
   if (((s | r) >> 32) == 0) return static_cast<uint32_t>(s) / static_cast<uint32_t>(r);
