@@ -1,5 +1,6 @@
-"""The matrix-vector kernel on groups shorter than a word (gemv_popc.cu): one to eight rows, K ending inside a word and
-inside a group, a row shorter than a warp's stride, mixed groups, one group per row, bf16 scales -- against the oracle."""
+"""Products of one to eight rows on groups shorter than a word: the matrix-vector kernel (gemv_popc.cu) and, for many rows of
+few words, the tiles; K ending inside a word and inside a group, a row shorter than a warp's stride, mixed groups, one group per
+row, bf16 scales -- against the oracle.  And what an automatic call on such rows leaves for prepared ones."""
 import pytest
 import torch
 
