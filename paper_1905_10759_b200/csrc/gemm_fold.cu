@@ -539,7 +539,7 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
     }
   } else if (warp == kLoaderWarp) {
     // =========================== W loader ===========================
-    if (lane == 0) {
+    if (elect_one()) {
       int64_t gst = 0;
       bool ok = true;
       // sub-word groups: the next scale block to request -- [128 rows][2 ASUB scales] of one stage; rows past M and groups
@@ -596,20 +596,20 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
   } else if (warp == kMmaWarp) {
     // =========================== MMA issuer ===========================
     // The tensor core's queue holds a few MMAs, whatever their size: with 128-column instructions (64 clk each) the barrier,
-    // the fence and the commit around a stage's twelve, and the producers' stores to tensor memory in between, drain it --
-    // 1100 clk per stage instead of the 768 the MMAs take.  WIDE forms A1 [W1; W2] as one instruction of 256 columns
+    // the fence and the commit around a stage's twelve drain it.  The stage's data is always there (it arrives 3700 clk before
+    // its first MMA, the slot is free 120 clk after the last one has been issued): what this one thread does between two MMAs
+    // is the kernel's time, so it runs behind elect_one (per stage 1260 clk with lane == 0, of which 625 the eight
+    // instructions of the 64-column tile; 4096^3 335 -> 306 us, 50176 x 128 x 1152 38.8 -> 36.3, 200704 x 64 x 576 55.8 ->
+    // 50.4).  WIDE forms A1 [W1; W2] as one instruction of 256 columns
     // (128 clk), which rides over these, and as a side effect keeps the large products' sum apart from the small ones'.  Its
     // accumulator takes the room of both: the epilogue is then exposed at every tile's end, so a tile has to be long.
-    // The whole warp walks the loop so that ring indices and descriptors stay warp-uniform values; one
-    // lane issues the MMAs and commits.
-    {
+    if (elect_one()) {
       constexpr uint32_t idesc = instr_desc(TN, kFmtF16);
       constexpr uint32_t idesc2 = instr_desc(2 * TN, kFmtF16);     // stacked: both weight pieces in one instruction
       const uint64_t db0 = smem_desc(smem_u32(smem + S::OFF_B));
       const uint64_t db_hi = db0 & 0xFFFFFFFF00000000ull;
       const uint32_t db_lo = static_cast<uint32_t>(db0);
       const uint32_t full_a = smem_u32(full), empty_a = smem_u32(empty), tfull_a = smem_u32(tfull), tempty_a = smem_u32(tempty);
-      const bool leader = lane == 0;
       uint32_t s = 0, full_par = 0;
       bool ok = true;
       for (int64_t ti = 0; ti < my_tiles && ok; ti++) {
@@ -625,35 +625,29 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
           tc_fence_after();
           const uint32_t a1 = tmem_base + S::A_BASE + s * S::A_COLS, a2 = a1 + KB / 2;
           const uint32_t b1_lo = db_lo + s * (S::B_STAGE >> 4), b2_lo = b1_lo + (S::B_PIECE >> 4);
-          if (leader) {
 #pragma unroll
-            for (int ks = 0; ks < KB / 16; ks++) {        // 16 K-elements = 8 TMEM columns of A, 32 bytes along the swizzled rows of W
-              if constexpr (STACK) {
-                umma_f16_ts(d_tmem, a1 + ks * 8, db_hi | (b1_lo + ks * 2), idesc2, (st | ks) != 0 ? 1u : 0u);   // A1 [W1; W2]
-                umma_f16_ts(d_tmem + TN, a2 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, 1u);                      // A2 W1, to A1 W2
-              } else {
-                umma_f16_ts(d_tmem, a1 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, (st | ks) != 0 ? 1u : 0u);
-                umma_f16_ts(d_tmem, a2 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, 1u);
-                umma_f16_ts(d_tmem, a1 + ks * 8, db_hi | (b2_lo + ks * 2), idesc, 1u);
-              }
+          for (int ks = 0; ks < KB / 16; ks++) {          // 16 K-elements = 8 TMEM columns of A, 32 bytes along the swizzled rows of W
+            if constexpr (STACK) {
+              umma_f16_ts(d_tmem, a1 + ks * 8, db_hi | (b1_lo + ks * 2), idesc2, (st | ks) != 0 ? 1u : 0u);   // A1 [W1; W2]
+              umma_f16_ts(d_tmem + TN, a2 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, 1u);                      // A2 W1, to A1 W2
+            } else {
+              umma_f16_ts(d_tmem, a1 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, (st | ks) != 0 ? 1u : 0u);
+              umma_f16_ts(d_tmem, a2 + ks * 8, db_hi | (b1_lo + ks * 2), idesc, 1u);
+              umma_f16_ts(d_tmem, a1 + ks * 8, db_hi | (b2_lo + ks * 2), idesc, 1u);
             }
-            umma_commit_a(empty_a + s * 8);     // the stage (TMEM columns and W bytes) is free once these MMAs have read it
           }
-          __syncwarp();
+          umma_commit_a(empty_a + s * 8);       // the stage (TMEM columns and W bytes) is free once these MMAs have read it
           if (++s == STAGES) { s = 0; full_par ^= 1; }
         }
-        if (ok && leader) umma_commit_a(tfull_a + buf * 8);
-        __syncwarp();
+        if (ok) umma_commit_a(tfull_a + buf * 8);
       }
-      if (leader) {
-        // every MMA issued so far has retired before TMEM is released -- also after an abort, so this wait
-        // does not look at the abort flag (the commit arrives once the tensor core is done, whatever the
-        // other warps do)
-        umma_commit(drain);
-        if (!mbar_wait_quiet(drain, 0, g_spin_limit < kDrainPolls ? kDrainPolls : g_spin_limit)) {
-          atomicCAS(&g_error_word, 0, 4);
-          *abort_flag = 1;
-        }
+      // every MMA issued so far has retired before TMEM is released -- also after an abort, so this wait
+      // does not look at the abort flag (the commit arrives once the tensor core is done, whatever the
+      // other warps do)
+      umma_commit(drain);
+      if (!mbar_wait_quiet(drain, 0, g_spin_limit < kDrainPolls ? kDrainPolls : g_spin_limit)) {
+        atomicCAS(&g_error_word, 0, 4);
+        *abort_flag = 1;
       }
     }
     __syncwarp();

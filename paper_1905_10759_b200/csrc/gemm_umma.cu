@@ -166,7 +166,7 @@ hbmm_umma_kernel(const Args g) {
   } else if (warp == kLoaderWarp) {
     // =========================== W loader ===========================
     reg_dec<kRegsIssuer>();
-    if (lane == 0) {
+    if (elect_one()) {
       int64_t gst = 0;
       bool ok = true;
       for (int64_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
@@ -193,7 +193,7 @@ hbmm_umma_kernel(const Args g) {
   } else if (warp == kMmaWarp) {
     // =========================== MMA issuer ===========================
     reg_dec<kRegsIssuer>();
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc_sign = instr_desc(TN, kFmtE4M3), idesc_scale = instr_desc(TN, kFmtBF16);
       // Descriptors of stage 0 / word slot 0; every other slot differs only by its start address, so
       // the low descriptor word is stepped by bytes/16.

@@ -217,7 +217,7 @@ hbwn_umma_kernel(const Args g, const __grid_constant__ CUtensorMap a_map) {
 
   if (warp == kLoaderWarp) {
     // =========================== loader ===========================
-    if (lane == 0) {
+    if (elect_one()) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&a_map) : "memory");
       // One thread feeds the whole CTA, so the loop carries its indices along instead of dividing:
       // ring slot and round, K block -> (filter tap row, column, channel block).
@@ -276,7 +276,7 @@ hbwn_umma_kernel(const Args g, const __grid_constant__ CUtensorMap a_map) {
     __syncwarp();
   } else if (warp == kMmaWarp) {
     // =========================== MMA issuer ===========================
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc = instr_desc(S::NST, kFmtBF16);
       const uint64_t da0 = smem_desc(smem_u32(smem + S::OFF_A)), db0 = smem_desc(smem_u32(smem + off_b));
       const uint64_t da_hi = da0 & 0xFFFFFFFF00000000ull, db_hi = db0 & 0xFFFFFFFF00000000ull;
@@ -457,7 +457,7 @@ hbwn_pair_kernel(const Args g, const __grid_constant__ CUtensorMap a_map, const 
 
   if (warp == kLoaderWarp) {
     // =========================== loader (both CTAs) ===========================
-    if (lane == 0) {
+    if (elect_one()) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&a_map) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(&b_map) : "memory");
       const uint32_t full0 = mapa_rank(smem_u32(full), 0);          // rank 0's `full` barriers
@@ -513,7 +513,7 @@ hbwn_pair_kernel(const Args g, const __grid_constant__ CUtensorMap a_map, const 
     __syncwarp();
   } else if (warp == kMmaWarp) {
     // =========================== MMA issuer (rank 0) ===========================
-    if (lane == 0 && rank == 0) {
+    if (rank == 0 && elect_one()) {
       constexpr uint32_t idesc = instr_desc_pair(S::NST, kFmtBF16);
       const uint64_t da0 = smem_desc(smem_u32(smem + S::OFF_A)), db0 = smem_desc(smem_u32(smem + S::OFF_B));
       const uint64_t da_hi = da0 & 0xFFFFFFFF00000000ull, db_hi = db0 & 0xFFFFFFFF00000000ull;
@@ -692,7 +692,7 @@ hbwn_halo_kernel(const Args g, const HaloArgs h, const __grid_constant__ CUtenso
   const uint32_t tmem_base = *tmem_base_ptr;
 
   if (warp == kLoaderWarp) {
-    if (lane == 0) {
+    if (elect_one()) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&a_map) : "memory");
       int64_t issued = 0;
       bool ok = true;
@@ -730,7 +730,7 @@ hbwn_halo_kernel(const Args g, const HaloArgs h, const __grid_constant__ CUtenso
     }
     __syncwarp();
   } else if (warp == kMmaWarp) {
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc = instr_desc(S::NST, kFmtBF16);
       const uint64_t da0 = smem_desc(smem_u32(smem)), db0 = smem_desc(smem_u32(smem + off_b));
       const uint64_t da_hi = da0 & 0xFFFFFFFF00000000ull, db_hi = db0 & 0xFFFFFFFF00000000ull;

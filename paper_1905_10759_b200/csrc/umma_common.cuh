@@ -95,6 +95,16 @@ __device__ __forceinline__ void tma_load_im2col_4d(void* dst, const void* tensor
                : "memory");
 }
 
+// True in one lane of a converged warp, always the same one.  For the roles of a single thread: behind elect.sync the compiler
+// knows that one thread runs and keeps ring indices, descriptors and tensor-memory addresses in the uniform registers the
+// tensor-core and copy instructions take their operands from; behind lane == 0 each of them is moved there first, one after
+// the other, in front of every instruction (folded contraction, 200704 x 64 x 576: 55.8 -> 50.4 us; 4096^3: 335 -> 306).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 // ---- tcgen05 helpers
 __device__ __forceinline__ bool mbar_wait_a(uint32_t bar, uint32_t parity, volatile int* abort_flag, int code) {
   if (mbar_try_wait_a(bar, parity)) return true;
