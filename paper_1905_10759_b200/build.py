@@ -5,10 +5,12 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libhbmm.so")
+BINDING = os.path.join(HERE, "_binding.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
 NVCC_FLAGS = [
@@ -29,10 +31,10 @@ def sources():
 
 
 def is_stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(BINDING):
         return True
     t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
+    deps = sources() + glob.glob(os.path.join(CSRC, "*.cpp")) + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
         glob.glob(os.path.join(INCLUDE, "*.h"))
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -61,8 +63,22 @@ def build_lib(force: bool = False, verbose: bool = False) -> str:
             raise RuntimeError("nvcc failed on %s" % src)
     tmp = LIB + ".tmp.%d" % os.getpid()
     subprocess.check_call([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", tmp] + objs)
+    build_binding()
     os.replace(tmp, LIB)
     return LIB
+
+
+def build_binding() -> None:
+    """The native marshalling of hbmm.py's hot calls (csrc/binding.cpp), against the running torch and Python."""
+    import torch
+    from torch.utils import cpp_extension as ext
+    tmp = BINDING + ".tmp.%d" % os.getpid()
+    include = ext.include_paths("cuda") + [sysconfig.get_paths()["include"], INCLUDE]
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", os.path.join(CSRC, "binding.cpp"), "-o", tmp]
+    cmd += ["-D_GLIBCXX_USE_CXX11_ABI=%d" % torch.compiled_with_cxx11_abi()]
+    cmd += [a for d in include for a in ("-isystem", d)] + ["-L" + d for d in ext.library_paths("cuda")]
+    subprocess.check_call(cmd + ["-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
+    os.replace(tmp, BINDING)
 
 
 if __name__ == "__main__":

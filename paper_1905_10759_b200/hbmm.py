@@ -24,6 +24,8 @@ if not os.path.exists(LIB_PATH):
 
 _lib = ctypes.CDLL(LIB_PATH)
 
+from . import _binding  # noqa: E402  (native marshalling of the hot calls; built beside the library)
+
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_ALIGNMENT, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT = range(7)
 F32, BF16 = 0, 1
 PATH_AUTO, PATH_POPC, PATH_B1MMA, PATH_TENSOR, PATH_TENSOR_PREPARED, PATH_FOLDED, PATH_FOLDED_PREPARED = 0, 1, 2, 3, 4, 5, 6
@@ -84,6 +86,20 @@ class HbmmError(RuntimeError):
     def __init__(self, status: int, where: str):
         self.status = status
         super().__init__("%s: %s (status %d)" % (where, status_string(status), status))
+
+
+# The calls a program makes once per layer and pass are native functions (csrc/binding.cpp: the marshalling took a third of a
+# small call's host time); the rest of this file marshals in Python.
+_binding.connect(HbmmError, *(ctypes.cast(getattr(_lib, _n), ctypes.c_void_p).value for _n in (
+    "hbmm_quantize", "hbmm_gemm", "hbmm_gemm_ex", "hbmm_conv_im2col_ex", "hbmm_conv_im2col_fused", "hbmm_binarize_dense",
+    "hbmm_binarize_backward")))
+quantize = _binding.quantize
+gemm = _binding.gemm
+gemm_ex = _binding.gemm_ex
+conv_im2col = _binding.conv_im2col
+conv_im2col_fused = _binding.conv_im2col_fused
+binarize_dense = _binding.binarize_dense
+binarize_backward = _binding.binarize_backward
 
 
 def _check(status: int, where: str) -> None:
@@ -185,38 +201,10 @@ def wrap_dense(a: torch.Tensor) -> Operand:
     return Operand(d, dense=a)
 
 
-def quantize(x: torch.Tensor, out: Operand, stream=None) -> Operand:
-    """hbmm_quantize: Hadamard-binarize and pack the rows of ``x`` [rows, K] into ``out``."""
-    if x.dim() != 2 or x.stride(1) != 1:
-        raise ValueError("x must be a row-major 2-D tensor")
-    rows, K = x.shape
-    _check(_lib.hbmm_quantize(_dev_ptr(x), _dtype_code(x.dtype), rows, K, x.stride(0), ctypes.byref(out.desc), _stream(stream)),
-           "hbmm_quantize")
-    return out
-
-
 def gemm_workspace_bytes(A: Operand, W: Operand) -> int:
     n = _sz()
     _check(_lib.hbmm_gemm_workspace_bytes(ctypes.byref(A.desc), ctypes.byref(W.desc), n), "hbmm_gemm_workspace_bytes")
     return n.value
-
-
-def gemm(A: Operand, W: Operand, C: torch.Tensor, workspace: Optional[torch.Tensor] = None, stream=None):
-    """hbmm_gemm: C[M, N] (fp32, row-major, caller-allocated) = A~ W~^T."""
-    ws_ptr = _dev_ptr(workspace)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(_lib.hbmm_gemm(ctypes.byref(A.desc), ctypes.byref(W.desc), _dev_ptr(C), C.stride(0), ws_ptr, ws_bytes,
-                          _stream(stream)), "hbmm_gemm")
-    return C
-
-
-def gemm_ex(A: Operand, W: Operand, C: torch.Tensor, path: int, workspace: Optional[torch.Tensor] = None,
-            stream=None):
-    ws_ptr = _dev_ptr(workspace)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(_lib.hbmm_gemm_ex(ctypes.byref(A.desc), ctypes.byref(W.desc), _dev_ptr(C), C.stride(0), ws_ptr, ws_bytes,
-                             path, _stream(stream)), "hbmm_gemm_ex")
-    return C
 
 
 def gemm_partials(A: Operand, W: Operand, D: torch.Tensor, path: int = PATH_AUTO, stream=None):
@@ -265,33 +253,6 @@ def gemm_binarize_next(A: "Operand", W: "Operand", nxt: "Operand", workspace: to
     return nxt
 
 
-def binarize_backward(x: torch.Tensor, gy: torch.Tensor, beta: int, gx: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
-    """hbmm_binarize_backward: x, gy fp32 [rows, K] (row stride >= K, unit column stride); returns gx = dC/dX."""
-    if x.dtype != torch.float32 or gy.dtype != torch.float32 or x.shape != gy.shape or x.dim() != 2:
-        raise ValueError("x and gy must be fp32 matrices of one shape")
-    if x.stride(1) != 1 or gy.stride(1) != 1:
-        raise ValueError("rows must be contiguous")
-    if gx is None:
-        gx = torch.empty(x.shape, dtype=torch.float32, device=x.device)
-    _check(_lib.hbmm_binarize_backward(_dev_ptr(x), x.stride(0), _dev_ptr(gy), gy.stride(0), x.shape[0], x.shape[1], beta,
-                                       _dev_ptr(gx), gx.stride(0), _stream(stream)), "hbmm_binarize_backward")
-    return gx
-
-
-def binarize_dense(x: torch.Tensor, beta: int, out_dtype: int = F32, out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
-    """hbmm_binarize_dense: x fp32 [rows, K] (row stride >= K, unit column stride); returns delta (.) Sign(x) as fp32 or bf16."""
-    if x.dtype != torch.float32 or x.dim() != 2 or x.stride(1) != 1:
-        raise ValueError("x must be an fp32 matrix with contiguous rows")
-    tdt = torch.bfloat16 if out_dtype == BF16 else torch.float32
-    if out is None:
-        out = torch.empty(x.shape, dtype=tdt, device=x.device)
-    if out.dtype != tdt or out.shape != x.shape or out.stride(1) != 1:
-        raise ValueError("out must match x's shape and the requested type")
-    _check(_lib.hbmm_binarize_dense(_dev_ptr(x), x.stride(0), x.shape[0], x.shape[1], beta, _dev_ptr(out), out_dtype, out.stride(0),
-                                    _stream(stream)), "hbmm_binarize_dense")
-    return out
-
-
 def binarize_map(x: torch.Tensor, beta_a: int, out_dtype: int = F32, stream=None) -> torch.Tensor:
     """Eq. 3-4 on a contiguous NCHW activation map: groups of beta_a neighbours along each map row.  Argument
     marshalling only: the map is passed to hbmm_binarize_dense as [batch*channels*height, width]."""
@@ -299,23 +260,6 @@ def binarize_map(x: torch.Tensor, beta_a: int, out_dtype: int = F32, stream=None
         raise ValueError("x must be a contiguous NCHW tensor")
     B, C, H, W = x.shape
     return binarize_dense(x.view(B * C * H, W), beta_a, out_dtype, stream=stream).view(B, C, H, W)
-
-
-def conv_im2col(x: torch.Tensor, geom: hbmm_conv_geom, beta_a: int, a_scale_dtype: int, W: Operand,
-                C_out: torch.Tensor, workspace: torch.Tensor, stream=None, flags: int = 0):
-    """hbmm_conv_im2col (flags == 0) / hbmm_conv_im2col_ex: x NCHW contiguous; C_out fp32 [B*Ho*Wo, N]."""
-    if not x.is_contiguous():
-        raise ValueError("x must be a contiguous NCHW tensor")
-    if flags:
-        _check(_lib.hbmm_conv_im2col_ex(_dev_ptr(x), _dtype_code(x.dtype), ctypes.byref(geom), beta_a, a_scale_dtype,
-                                        ctypes.byref(W.desc), _dev_ptr(C_out), 0 if C_out is None else C_out.stride(0),
-                                        _dev_ptr(workspace), workspace.numel() * workspace.element_size(), flags, _stream(stream)),
-               "hbmm_conv_im2col_ex")
-        return C_out
-    _check(_lib.hbmm_conv_im2col(_dev_ptr(x), _dtype_code(x.dtype), ctypes.byref(geom), beta_a, a_scale_dtype,
-                                 ctypes.byref(W.desc), _dev_ptr(C_out), C_out.stride(0), _dev_ptr(workspace),
-                                 workspace.numel() * workspace.element_size(), _stream(stream)), "hbmm_conv_im2col")
-    return C_out
 
 
 def conv_im2col_static(x: torch.Tensor, geom: hbmm_conv_geom, beta_a: int, a_scale_dtype: int, W: Operand,
@@ -418,13 +362,3 @@ def gemm_fused(A: Operand, W: Operand, ep: hbmm_epilogue, workspace: torch.Tenso
     """hbmm_gemm_fused: the product goes through activation, affine map and dense / binarized output in the epilogue."""
     _check(_lib.hbmm_gemm_fused(ctypes.byref(A.desc), ctypes.byref(W.desc), ctypes.byref(ep), _dev_ptr(workspace),
                                 workspace.numel() * workspace.element_size(), _stream(stream)), "hbmm_gemm_fused")
-
-
-def conv_im2col_fused(x: torch.Tensor, geom: hbmm_conv_geom, beta_a: int, a_scale_dtype: int, W: Operand, ep: hbmm_epilogue,
-                      workspace: torch.Tensor, stream=None, flags: int = 0) -> None:
-    """hbmm_conv_im2col_fused: x NCHW contiguous (or NHWC bf16 with CONV_INPUT_NHWC)."""
-    if not x.is_contiguous():
-        raise ValueError("x must be contiguous")
-    _check(_lib.hbmm_conv_im2col_fused(_dev_ptr(x), _dtype_code(x.dtype), ctypes.byref(geom), beta_a, a_scale_dtype,
-                                       ctypes.byref(W.desc), ctypes.byref(ep), _dev_ptr(workspace),
-                                       workspace.numel() * workspace.element_size(), flags, _stream(stream)), "hbmm_conv_im2col_fused")

@@ -1,0 +1,44 @@
+"""The native entry points (csrc/binding.cpp): arguments by position and by keyword, and the errors raised before anything
+reaches the library (no GPU needed)."""
+import inspect
+
+import pytest
+import torch
+
+from paper_1905_10759_b200 import hbmm
+
+
+def test_signatures():
+    want = {
+        "quantize": "(x, out, stream=None)", "gemm": "(A, W, C, workspace=None, stream=None)",
+        "gemm_ex": "(A, W, C, path, workspace=None, stream=None)",
+        "conv_im2col": "(x, geom, beta_a, a_scale_dtype, W, C_out, workspace, stream=None, flags=0)",
+        "conv_im2col_fused": "(x, geom, beta_a, a_scale_dtype, W, ep, workspace, stream=None, flags=0)",
+        "binarize_dense": "(x, beta, out_dtype=0, out=None, stream=None)",
+        "binarize_backward": "(x, gy, beta, gx=None, stream=None)",
+    }
+    assert {n: str(inspect.signature(getattr(hbmm, n))) for n in want} == want
+
+
+@pytest.mark.parametrize("call,error,text", [
+    (lambda x, op: hbmm.quantize(x, op), ValueError, "device tensor expected"),
+    (lambda x, op: hbmm.quantize(out=op, x=x), ValueError, "device tensor expected"),
+    (lambda x, op: hbmm.quantize(x.t(), op), ValueError, "row-major"),
+    (lambda x, op: hbmm.quantize(x[0], op), ValueError, "row-major"),
+    (lambda x, op: hbmm.gemm(op, op, x), ValueError, "device tensor expected"),
+    (lambda x, op: hbmm.gemm_ex(op, op, x, hbmm.PATH_AUTO, workspace=x), ValueError, "device tensor expected"),
+    (lambda x, op: hbmm.binarize_dense(x.double(), 4), ValueError, "fp32 matrix"),
+    (lambda x, op: hbmm.binarize_dense(x, 4, hbmm.BF16, x), ValueError, "requested type"),
+    (lambda x, op: hbmm.binarize_backward(x, x[:1], 4), ValueError, "one shape"),
+    (lambda x, op: hbmm.binarize_backward(x.t(), x.t(), 4), ValueError, "contiguous"),
+    (lambda x, op: hbmm.conv_im2col(x.t(), hbmm.make_geom(1, 1, 2, 32, 1, 1), 32, hbmm.F32, op, x, x), ValueError, "contiguous"),
+    (lambda x, op: hbmm.quantize(x), TypeError, "out"),
+    (lambda x, op: hbmm.quantize(x, op, None, None), TypeError, "positional"),
+    (lambda x, op: hbmm.quantize(x, op, x=x), TypeError, "multiple values"),
+    (lambda x, op: hbmm.gemm(op, op, x, ws=None), TypeError, "unexpected"),
+    (lambda x, op: hbmm.quantize([1.0], op), TypeError, "Tensor"),
+])
+def test_errors_before_the_library(call, error, text):
+    x = torch.ones((2, 32))
+    with pytest.raises(error, match=text):
+        call(x, hbmm.alloc_operand(2, 32, 32, device="cpu"))
