@@ -441,7 +441,7 @@ hbmm_status conv_checked(const void* x, int32_t x_dtype, const hbmm_conv_geom* g
   const bool pack_only = (flags & HBMM_CONV_PACK_ONLY) != 0;
   const bool input_nhwc = (flags & HBMM_CONV_INPUT_NHWC) != 0;
   if (pack_only && beta_a < 2) return HBMM_ERR_INVALID_ARG;     // only a packed activation operand can be left behind
-  // honoured on the two tensor-copy paths below; every other path expands the weights again (still correct)
+  // honoured on the paths below whose front end expands the weights; every other path expands the weights again (still correct)
   const bool w_prepared = (flags & HBMM_CONV_WEIGHTS_PREPARED) != 0;
   ConvGeom cg;
   hbmm_status st = check_geom(g, &cg);
@@ -495,13 +495,16 @@ hbmm_status conv_checked(const void* x, int32_t x_dtype, const hbmm_conv_geom* g
       const bool a_subword = beta_a < 32 && beta_a < L.K;
       if (!gemm_fold_supported(av, wv) || a_subword || L.gemm_bytes < fold_workspace(av, wv)) return HBMM_ERR_UNSUPPORTED;
     }
+    const bool walk = im2col_walk_supported(x_dtype == HBMM_BF16, cg, beta_a, A.ld_words, A.ld_scales);
     if ((ep || prefer_fold(av, wv)) && L.gemm_bytes > 0 && L.gemm_bytes >= fold_workspace(av, wv) &&
-        im2col_quantize_tma_supported(x, x_dtype == HBMM_BF16, cg, beta_a)) {
+        (walk || im2col_quantize_tma_supported(x, x_dtype == HBMM_BF16, cg, beta_a))) {
       UmmaPrepJob job{};
       gemm_fold_prep_job(av, wv, gemm_ws, &job);
       if (job.n_stages * job.tiles_n <= 4096) {
-        if (launch_im2col_quantize_tma(x, cg, beta_a, A.bits, A.ld_words, A.scales, A.ld_scales, a_scale_dtype == HBMM_BF16, s,
-                                       w_prepared ? nullptr : &job) != cudaSuccess)
+        const UmmaPrepJob* expand = w_prepared ? nullptr : &job;
+        const int s_bf16 = a_scale_dtype == HBMM_BF16;
+        if ((walk ? launch_im2col_walk(x, x_dtype == HBMM_BF16, cg, beta_a, A.bits, A.ld_words, A.scales, A.ld_scales, s_bf16, s, expand)
+                  : launch_im2col_quantize_tma(x, cg, beta_a, A.bits, A.ld_words, A.scales, A.ld_scales, s_bf16, s, expand)) != cudaSuccess)
           return HBMM_ERR_CUDA;
         if (pack_only) return HBMM_OK;
         return launch_gemm_fold(av, wv, C_out, ldc, gemm_ws, L.gemm_bytes, s, true, ep ? &epi : nullptr) == cudaSuccess ? HBMM_OK : HBMM_ERR_CUDA;

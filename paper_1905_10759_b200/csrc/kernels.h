@@ -216,7 +216,12 @@ cudaError_t launch_hbwn_umma_conv(const void* x, int x_bf16, void* x_nhwc, int C
 cudaError_t launch_im2col_quantize(const void* x, int x_bf16, const ConvGeom& g, int32_t beta,
                                    uint32_t* bits, int64_t ld_words, void* scales, int64_t ld_scales,
                                    int scale_bf16, cudaStream_t stream);
-// The packed front end with its input tile staged by tensor copies (fp32 input, beta = 32).
+// 3 x 3 filters at stride 1, groups of 2, 4, 8, 16 elements or of whole K-words, fp32 or bf16 images of any width and alignment.
+bool im2col_walk_supported(int x_bf16, const ConvGeom& g, int32_t beta, int64_t ld_words, int64_t ld_scales);
+// `prep` as for launch_im2col_quantize_tma (folded operands only).
+cudaError_t launch_im2col_walk(const void* x, int x_bf16, const ConvGeom& g, int32_t beta, uint32_t* bits, int64_t ld_words, void* scales,
+                               int64_t ld_scales, int scale_bf16, cudaStream_t stream, const UmmaPrepJob* prep = nullptr);
+// The packed front end with its input tile staged by tensor copies (fp32 input).
 bool im2col_quantize_tma_supported(const void* x, int x_bf16, const ConvGeom& g, int32_t beta);
 // prep (optional): weight-expansion tasks of the contraction that follows, run by extra CTAs of the launch.
 cudaError_t launch_im2col_quantize_tma(const void* x, const ConvGeom& g, int32_t beta, uint32_t* bits, int64_t ld_words, void* scales,
