@@ -72,6 +72,8 @@ template <int SUBW> struct DepthFor { static constexpr int value = SUBW == 1 ? 4
 // pieces (by the row number, as wide as the row is long), so 8 consecutive rows read 8 different bank groups.
 constexpr int kStagedFrom = 4;          // groups per word from which the scales go through shared memory (beta_a <= 8)
 constexpr int64_t kRowMaxFrom = 512;    // scales per row from which a kernel of its own finds the rows' largest scales
+constexpr int kOutBlock = 32 * 128;     // 32 rows of 32 fp32 outputs
+constexpr int kMaxSmem = 227 * 1024;
 template <int TN, int ASUB>
 struct ScaleRing {
   static constexpr int ROW_BYTES = 8 * ASUB;                       // two words' scales
@@ -82,7 +84,12 @@ struct ScaleRing {
   static constexpr int LEAD = NS - Smem<TN>::STAGES;
   static constexpr int OFF = (Smem<TN>::USED + 1023) / 1024 * 1024;
   static constexpr int OFF_BAR = OFF + NS * STAGE;                 // sfull[NS]
-  static constexpr int BYTES = ASUB == 1 ? Smem<TN>::BYTES : OFF_BAR + NS * 8 + 16;
+  // The epilogue warps' staging of finished 32 x 32 blocks: two or one of 4 KB each, as far as there is room.
+  static constexpr int RINGS = ASUB == 1 ? Smem<TN>::USED : OFF_BAR + NS * 8 + 16;
+  static constexpr int OFF_OUT = (RINGS + 1023) / 1024 * 1024;
+  static constexpr int OUT_BUFS = OFF_OUT + kEpilogueWarps * 2 * kOutBlock <= kMaxSmem ? 2 : (OFF_OUT + kEpilogueWarps * kOutBlock <= kMaxSmem ? 1 : 0);
+  static constexpr int OUT_END = OUT_BUFS > 0 ? OFF_OUT + kEpilogueWarps * OUT_BUFS * kOutBlock : RINGS;
+  static constexpr int BYTES = OUT_END > 120 * 1024 ? OUT_END : 120 * 1024;        // one CTA per SM, see Smem
   // byte offset of the 16-byte piece c of row p inside a stage block
   __device__ static __forceinline__ int piece(int p, int c) {
     if (ASUB == 16) return p * 128 + ((c ^ (p & 7)) << 4);
@@ -259,7 +266,7 @@ enum Mode : int { kPlain = 0, kBalanced = 1, kSplit = 2 };
 // WIDE (128-column tiles): one accumulator of 256 columns instead of two of 128 (see the MMA issuer).
 template <int TN, int ASUB, bool FUSE, int MODE, bool WIDE>
 __global__ void __launch_bounds__(kThreads, 1)
-hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
+hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map, const __grid_constant__ CUtensorMap c_map) {
   using S = Smem<TN>;
   using SR = ScaleRing<TN, ASUB>;
   const bool staged = ASUB > 1 && g.a_staged;                    // the stage's scales come through shared memory
@@ -655,6 +662,7 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
     // =========================== epilogue ===========================
     const int row = warp * 32 + lane;               // TMEM lane = tile row
     const uint32_t t_lane = static_cast<uint32_t>(warp * 32) << 16;
+    uint32_t out_count = 0;                         // blocks handed to the copy engine
     for (int64_t ti = 0; ti < my_tiles; ti++) {
       const uint32_t buf = static_cast<uint32_t>(ti % NBUF);
       const int slot = static_cast<int>(ti & (kRowSlots - 1));
@@ -685,7 +693,6 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&rowempty[slot]);
-      float* dst = g.C + m * g.ldc + nb;
       float carry = 0.0f;                                   // |z| sum of a group wider than a 32-column chunk
       // raw accumulator of chunk c (32 columns of this thread's row): the block of A1 W1 and the block of the cross
       // products added, where they are apart
@@ -723,7 +730,32 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
             }
             epi::finish_chunk(g.ep, cv, fs, fh, m, nb + c * 32, g.N, c == TN / 32 - 1, nb + TN, carry);
           }
+        } else if (SR::OUT_BUFS > 0 && ((g.N & 3) == 0 || nb + c * 32 + 32 <= g.N)) {
+          // The block goes to shared memory (as the copy's 128-byte swizzle has it: eight rows, eight bank groups) and leaves by
+          // a tensor copy, which drops what lies outside the matrix.  Sixteen bytes of a row per lane straight to the matrix
+          // are 32 lines an instruction: a tile of 128 x 128 took 7400 clk that way.  (The copy clips a row to 16 bytes: the block in which
+          // N ends inside four columns leaves by the stores below, which touch nothing behind it.)
+          unsigned char* out = smem + SR::OFF_OUT + (warp * SR::OUT_BUFS + (SR::OUT_BUFS == 2 ? out_count & 1 : 0)) * kOutBlock;
+          if (lane == 0) bulk_wait_read<SR::OUT_BUFS == 2 ? 1 : 0>();          // the copy that read this buffer last is done with it
+          __syncwarp();
+#pragma unroll
+          for (int j = 0; j < 32; j += 4) {
+            const float4 fw = *reinterpret_cast<const float4*>(cf + c * 32 + j);
+            float o[4];
+#pragma unroll
+            for (int e = 0; e < 4; e++) o[e] = __uint_as_float(v1[j + e]) * fa;
+            *reinterpret_cast<float4*>(out + lane * 128 + (((j >> 2) ^ (lane & 7)) << 4)) = make_float4(o[0] * fw.x, o[1] * fw.y, o[2] * fw.z, o[3] * fw.w);
+          }
+          fence_async_proxy();
+          __syncwarp();
+          if (lane == 0) {
+            const int64_t m0 = m - lane, n0 = nb + c * 32;
+            if (m0 < g.M && n0 < g.N) tma_store_2d(&c_map, out, static_cast<int32_t>(n0), static_cast<int32_t>(m0));
+            bulk_commit();
+          }
+          out_count++;
         } else if (m < g.M) {
+          float* dst = g.C + m * g.ldc + nb;
 #pragma unroll
           for (int j = 0; j < 32; j += 4) {
             const float4 fw = *reinterpret_cast<const float4*>(cf + c * 32 + j);
@@ -812,6 +844,7 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map) {
       }
 
     }
+    if (!FUSE && !SPLIT && SR::OUT_BUFS > 0 && lane == 0) bulk_wait_all();      // the rows are in memory before the CTA ends
   }
 
   if constexpr (SPLIT) {
@@ -1016,7 +1049,7 @@ cudaError_t launch_fold_wide(Args g, void* workspace, size_t have, cudaStream_t 
   constexpr bool kHasBalanced = ASUB == 1;           // the balanced schedule is built for activation groups of whole words
   constexpr int kBytes = ScaleRing<TN, ASUB>::BYTES;
   constexpr bool kSplitWide = TN == 128 && !FUSE;
-  static_assert(kBytes <= 227 * 1024, "weight stages and the scale ring fit one CTA's shared memory");
+  static_assert(kBytes <= kMaxSmem, "weight stages and the scale ring fit one CTA's shared memory");
   static DeviceOnce configured;
   int dev = 0, sms = 0;
   if (current_device(&dev, &sms) != cudaSuccess) return cudaErrorInvalidDevice;
@@ -1067,6 +1100,7 @@ cudaError_t launch_fold_wide(Args g, void* workspace, size_t have, cudaStream_t 
     if (e != cudaSuccess) return e;
   }
   const int64_t tiles = ((g.M + TM - 1) / TM) * tiles_n;
+  CUtensorMap c_map = {};
   if constexpr (!FUSE) {
     // (all instantiations take a whole SM per CTA, so they share what was asked once)
     const auto ask = [](int size, int* clusters) { return resident_clusters(hbmm_fold_kernel<TN, ASUB, FUSE, kSplit, kSplitWide>, kBytes, size, clusters); };
@@ -1074,8 +1108,19 @@ cudaError_t launch_fold_wide(Args g, void* workspace, size_t have, cudaStream_t 
     if (split > 1) {
       g.split = split;
       return launch_pdl_cluster(hbmm_fold_kernel<TN, ASUB, FUSE, kSplit, kSplitWide>, dim3(static_cast<unsigned>(tiles * split)), dim3(kThreads),
-                                static_cast<unsigned>(split), kBytes, stream, g, s_map);
+                                static_cast<unsigned>(split), kBytes, stream, g, s_map, c_map);
     }
+  }
+  if (!FUSE && ScaleRing<TN, ASUB>::OUT_BUFS > 0) {
+    // the product as a 2-D tensor for the epilogue's copies: 32 x 32 blocks
+    EncodeTiledFn fn = encode_tiled_fn();
+    const cuuint64_t dims[2] = {static_cast<cuuint64_t>(g.N), static_cast<cuuint64_t>(g.M)};
+    const cuuint64_t strides[1] = {static_cast<cuuint64_t>(g.ldc) * 4};
+    const cuuint32_t box[2] = {32, 32};
+    const cuuint32_t elem[2] = {1, 1};
+    if (!fn || fn(&c_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, g.C, dims, strides, box, elem, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return cudaErrorNotSupported;
   }
   // equal runs of (tile, stage) pairs, one per CTA, when that shortens the longest CTA's walk by a tenth or more
   const int64_t units = tiles * n_stages;
@@ -1091,14 +1136,14 @@ cudaError_t launch_fold_wide(Args g, void* workspace, size_t have, cudaStream_t 
   if (kHasBalanced && balanced_possible<TN>(g, sms) && run * 10 <= plain_walk * 9) {
     ctas = (units + run - 1) / run;                     // no CTA without work
     g.sk_units = run;
-    return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kHasBalanced ? kBalanced : kPlain, WIDE>, dim3(static_cast<unsigned>(ctas)), dim3(kThreads), kBytes, stream, g, s_map);
+    return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kHasBalanced ? kBalanced : kPlain, WIDE>, dim3(static_cast<unsigned>(ctas)), dim3(kThreads), kBytes, stream, g, s_map, c_map);
   }
   const unsigned grid = static_cast<unsigned>(tiles < sms ? tiles : sms);   // one persistent CTA per SM
   if (WIDE && stage_bytes<TN>(g) > kWeightsInL2) {
     g.group_n = static_cast<int64_t>(kBlockBytes / (static_cast<size_t>(n_stages) * S::B_STAGE));
     if (g.group_n < 1) g.group_n = 1;
   }
-  return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kPlain, WIDE>, dim3(grid), dim3(kThreads), kBytes, stream, g, s_map);
+  return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kPlain, WIDE>, dim3(grid), dim3(kThreads), kBytes, stream, g, s_map, c_map);
 }
 
 template <int TN, int ASUB, bool FUSE = false>
@@ -1158,6 +1203,19 @@ bool gemm_fold_next_supported(int64_t N, int32_t beta_next) {
 
 cudaError_t launch_gemm_fold(const PackedView& A, const PackedView& W, float* C, int64_t ldc, void* workspace, size_t workspace_bytes,
                              cudaStream_t stream, bool w_prepared, const EpiArgs* ep) {
+  // the copies that store the product take 32-bit row numbers
+  constexpr int64_t kMostRows = int64_t{1} << 30;
+  if (!ep && A.rows > kMostRows) {
+    PackedView part = A;
+    for (int64_t m = 0; m < A.rows; m += kMostRows) {
+      part.bits = A.bits + m * A.ld_words;
+      part.scales = static_cast<const char*>(A.scales) + m * A.ld_scales * (A.scale_bf16 ? 2 : 4);
+      part.rows = A.rows - m < kMostRows ? A.rows - m : kMostRows;
+      const cudaError_t e = launch_gemm_fold(part, W, C + m * ldc, ldc, workspace, workspace_bytes, stream, w_prepared || m > 0, nullptr);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
   Args g = make_args(A, W, C, ldc);
   if (ep) g.ep = *ep;
   return g.N <= 64 ? launch_fold_tn<64>(g, workspace, workspace_bytes, stream, w_prepared) : launch_fold_tn<128>(g, workspace, workspace_bytes, stream, w_prepared);

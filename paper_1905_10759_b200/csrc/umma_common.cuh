@@ -84,6 +84,17 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const void* tensor_map, i
   asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
                ::"r"(smem_u32(dst)), "l"(tensor_map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar)) : "memory");
 }
+// Tiled 2-D tensor copy shared memory -> global; what lies outside the tensor is dropped, in pieces of 16 bytes (a row of
+// 1030 fp32 is written to its 1032nd).  Neither coordinate is negative, x times
+// the element size is a multiple of 16 bytes.  One thread issues, commits and waits for its own groups of copies.
+__device__ __forceinline__ void tma_store_2d(const void* tensor_map, const void* src, int32_t x, int32_t y) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
+               ::"l"(tensor_map), "r"(x), "r"(y), "r"(smem_u32(src)) : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// ... until at most N of its groups have not read their shared memory yet / until all have written
+template <int N> __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // im2col-mode tensor copy of an NHWC image: `pixels-per-column` consecutive base pixels starting at
 // (w, h, n) (walking W, then H, then N inside the map's bounding box), each displaced by the filter
 // offsets (w_off, h_off), `channels-per-pixel` channels from c.  c times the element size must be a
