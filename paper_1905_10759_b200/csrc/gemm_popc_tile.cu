@@ -2,23 +2,24 @@
 // path of every K that is no whole number of words.  A segment is the finer of the two groupings: 2, 4, 8 or 16 bits
 // of a word, or 1, 2, 4 or 8 words; per output and segment  C += (deltaA deltaW) D,  D = n_valid - 2 popc(a ^ w).
 //
-// What bounds it: per output and word one XOR and the population counts (16 /clk/SM), per output and segment three
-// fp32 operations (issued two outputs at a time) -- and, for the products this path really gets (a few hundred rows,
-// K some thousand), how many warps have work at all.  So a warp owns a whole 32 x 32 tile of C (4 x 8 outputs per
-// lane), stages its own operands (no barrier between warps in the K loop; the next chunk's loads are in flight while
-// the current one is computed), and up to eight warps of a CTA split the K range of a tile; their partial sums meet
-// in shared memory at the end, always in the same order.
-// Population counts of 2-, 4- and 8-bit segments are formed for all of a word at once by adding neighbouring fields
-// (2, 3 or 4 levels); the doubled count of a segment is then a byte, and one byte permutation puts it under the
-// exponent of 2^23, so that float - (2^23 + n_valid) = 2 popc - n_valid exactly.  Segments of 16 bits and more use the
-// popcount instruction.  (One masked popcount per 2-bit segment would keep that unit busy for 128 clk per word and warp
-// against ~75 issue slots this way; at 16 bits the two are level.)
-// Measured against one 64 x 64 (sub-word) or 128 x 128 (word) tile per CTA, which this replaces: 333 x 720 x 1000 at
-// beta 16 27.8 -> 8.9 us, 82 x 536 x 3768 at beta 64 90 -> 9.4 us, 4050 x 280 x 4368 at beta 16 203 -> 107 us; on the
-// conv3_x matrix (50176 x 128 x 1152) beta 2 / 4 / 8 / 16 / 32 / 128: 1337 / 662 / 334 / 172 / 89 / 81 ->
-// 926 / 546 / 327 / 159 / 83 / 67 us.  Slower than those tiles only at mixed groupings of sub-word segments over long K (5104 x
-// 536 x 6912 at beta 256 / 16 487 -> 516), whose scales each warp loads for itself.  Scalar fp32 instead of the paired
-// instructions: 5 % slower.
+// The dots D of a word's segments are formed by mma.sync on bytes of +-64: exact integers, in the registers that scale them (a
+// tcgen05 accumulator would have to come out of tensor memory once per segment), and, started from the bits of 1.5 2^23, already
+// floats.  16 x 8 outputs over 32 elements cost 8.4 clk of a scheduler's tensor unit; the population counts they replace, at 16
+// /clk/SM, 32 clk for whole words, and 75 issue slots for all of a word's segments of 2 to 8 bits.  Segments shorter than a word
+// take one product each, the first operand zeroed outside the segment.  Which element sits at which K index of the instruction
+// is free as long as both operands agree: byte j of register r of lane t of a quad holds bit 8 j + 2 t + r of the word, so that
+// expanding a register is one shift and one three-input operation, and the segments of 16 and 8 bits are bytes, those of 4 and
+// 2 bits bytes of some lanes.  (e4m3 bytes, whose products are fp32 by themselves, run at 0.8 of the rate of s8 and are
+// converted on the way: 0.8 .. 1.0 of the counts' speed.)
+// What bounds it: the loads of a warp's own operands and scales, the three fp32 operations per output and segment (issued two
+// outputs at a time); and, for the products this path really gets (a few hundred rows, K some thousand), how many warps have
+// work at all.  So a warp owns a whole 32 x 32 tile of C, stages its own operands (no barrier between warps in the K loop; the
+// next chunk's loads are in flight while the current one is computed), and up to eight warps of a CTA split the K range of a
+// tile; their partial sums meet in shared memory at the end, always in the same order.
+// Against the same tiles on population counts, us: conv3_x matrix (50176 x 128 x 1152) at beta 2 / 4 / 8 / 16 / 32 / 64 / 128 / 256
+// 922 / 543 / 325 / 158 / 82.6 / 74.8 / 66.8 / 72.5 -> 815 / 446 / 241 / 124 / 82.5 / 63.3 / 50.7 / 47.0; 333 x 720 x 1000 at beta
+// 16 9.0 -> 7.8; 691 x 1216 x 5032 at beta 8 194 -> 146; 3325 x 872 x 2946 at beta 64 104 -> 92; 320 x 1480 x 8376 at beta 2 553 ->
+// 483; 5104 x 536 x 6912 at beta 256 / 16 504 -> 426; 82 x 536 x 3768 at beta 64 9.2 -> 8.5; 9 x 1000 x 4097 at beta 32 10.0 -> 10.3.
 #include "kernels.h"
 #include "pdl.cuh"
 #include "popc_common.cuh"
@@ -155,22 +156,32 @@ __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
   return v;
 }
 __device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-// acc += sa sw (counts - bias) for two neighbouring outputs; c0, c1: 2^23 + doubled count as bit patterns.  DOT_FIRST: the
-// first product is (counts - bias) sa, so that a segment whose signs cancel adds 0 also where the product of its scales
-// leaves the range of fp32; 4 % slower at segments of 2 and 8 bits, which take the product of the scales first.
+// acc += sa sw D for two neighbouring outputs.  DOT_FIRST: the first product is D sa, so that a segment whose signs cancel adds
+// 0 also where the product of its scales leaves the range of fp32 (groups of whole words; shorter ones take the product of the
+// scales first).
 template <bool DOT_FIRST>
-__device__ __forceinline__ void add_term(uint64_t& acc, uint32_t c0, uint32_t c1, uint64_t neg_bias, uint64_t sa, uint64_t sw) {
-  uint64_t f = pack2(__uint_as_float(c0), __uint_as_float(c1));
-  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(f) : "l"(neg_bias));
+__device__ __forceinline__ void add_term(uint64_t& acc, uint32_t d0, uint32_t d1, uint64_t sa, uint64_t sw) {
+  uint64_t f, d = pack2(__uint_as_float(d0), __uint_as_float(d1));
+  const uint64_t unit = pack2(0x1p-12f, 0x1p-12f), bias = pack2(-3072.0f, -3072.0f);
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(d), "l"(unit), "l"(bias));      // the dot, exactly
   if constexpr (DOT_FIRST) {
-    asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(f) : "l"(sa));
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(f) : "l"(d), "l"(sa));
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(f), "l"(sw));
   } else {
-    uint64_t s;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(s) : "l"(sa), "l"(sw));
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(s), "l"(f));
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(f) : "l"(sa), "l"(sw));
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(f), "l"(d));
   }
 }
+
+// d = c + a b^T, 16 x 8 outputs over 32 elements of +-64: 4096 times the dot
+__device__ __forceinline__ void mma_s8(uint32_t (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2], const uint32_t (&c)[4]) {
+  asm("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %11, %12, %13};"
+      : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "r"(c[0]), "r"(c[1]), "r"(c[2]), "r"(c[3]));
+}
+// Bits 8 j + b of a word (b = 7 - shift) as four bytes: 1 -> +64, 0 -> -64.
+__device__ __forceinline__ uint32_t expand(uint32_t word, int shift) { return ((word << shift) & 0x80808080u) ^ 0xC0C0C0C0u; }
+constexpr uint32_t kBias = 0x4B400000u;      // 1.5 2^23: an integer sum started from here is that float plus the sum
 
 // MIXED: some group spans several segments (ra, rw not both 1).  The lookup for that, in every kernel, costs the uniform
 // groupings registers: 2 % at 2-bit segments, 5 % at 32.
@@ -189,10 +200,10 @@ gemm_popc_tile_kernel(const TileArgs g) {
   const int part = warp & (KS - 1);
   const int64_t m0 = (static_cast<int64_t>(blockIdx.y) * (blockDim.x >> (5 + g.ks_log2)) + (warp >> g.ks_log2)) * TS;
   const int64_t n0 = static_cast<int64_t>(blockIdx.x) * TS;
-  const int tx = lane & 3, ty = lane >> 2;              // columns 8 tx .., rows 4 ty ..
+  const int qt = lane & 3, qg = lane >> 2;              // lane of its quad, quad: rows qg + 8 i, columns 8 j + 2 qt and the next
   uint32_t* as = smem + warp * P::SMEM_WORDS;           // [CW][32]
   uint32_t* ws = as + P::CW * TS;                       // [CW][32]
-  float* sa_s = reinterpret_cast<float*>(ws + P::CW * TS);   // [SPC][32], negated
+  float* sa_s = reinterpret_cast<float*>(ws + P::CW * TS);   // [SPC][32]
   float* sw_s = sa_s + P::SPC * TS;                     // [SPC][32]
   const int64_t m = m0 + lane, n = n0 + lane;           // the rows this lane stages
   const bool ain = m < g.M, win = n < g.N;
@@ -200,7 +211,7 @@ gemm_popc_tile_kernel(const TileArgs g) {
   const uint32_t* wrow = g.w_bits + (win ? n : 0) * g.ldw_w;
   const int64_t aoff = (ain ? m : 0) * g.lda_s, woff = (win ? n : 0) * g.ldw_s;
 
-  uint64_t acc[4][4];                                   // two neighbouring columns each
+  uint64_t acc[4][4];                                   // [8 rows apart][8 columns apart], two neighbouring columns each
 #pragma unroll
   for (int i = 0; i < 4; i++)
 #pragma unroll
@@ -227,141 +238,131 @@ gemm_popc_tile_kernel(const TileArgs g) {
 #pragma unroll
       for (int i = 0; i < P::CW; i++) { as[i * TS + lane] = pa[i]; ws[i * TS + lane] = pw[i]; }
 #pragma unroll
-      for (int i = 0; i < P::SPC; i++) { sa_s[i * TS + lane] = -psa[i]; sw_s[i * TS + lane] = psw[i]; }
+      for (int i = 0; i < P::SPC; i++) { sa_s[i * TS + lane] = psa[i]; sw_s[i * TS + lane] = psw[i]; }
       __syncwarp();
       if (kAhead && c + KS < g.n_chunks) fetch(c + KS);
       const int64_t left_chunk = g.K - c * (P::CW * 32);              // elements from the chunk's start to the row's end
-      // one segment of all 32 outputs: counts(i, j) gives 2^23 + 2 popc as a bit pattern
-      auto segment = [&](int s, auto counts) {
-        const int64_t left = left_chunk - s * SEG;
-        const int nv = left >= SEG ? SEG : (left > 0 ? static_cast<int>(left) : 0);
-        const float nb = -(8388608.0f + static_cast<float>(nv));
-        const uint64_t neg_bias = pack2(nb, nb);
-        const float4 sa4 = *reinterpret_cast<const float4*>(sa_s + s * TS + 4 * ty);
-        const float sa[4] = {sa4.x, sa4.y, sa4.z, sa4.w};
-        uint64_t sw[4];
+      // the dots of one segment in 16 rows from 16 r on, d[column block of 8], into the sums
+      auto segment = [&](int s, int r, const uint32_t (&d)[4][4]) {
+        uint64_t sa[2], sw[4];
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-          const float4 v = *reinterpret_cast<const float4*>(sw_s + s * TS + 8 * tx + 4 * h);
-          sw[2 * h] = pack2(v.x, v.y);
-          sw[2 * h + 1] = pack2(v.z, v.w);
+        for (int i = 0; i < 2; i++) {
+          const float v = sa_s[s * TS + 16 * r + 8 * i + qg];
+          sa[i] = pack2(v, v);
         }
 #pragma unroll
-        for (int i = 0; i < 4; i++) {
-          const uint64_t sa2 = pack2(sa[i], sa[i]);
+        for (int j = 0; j < 4; j++) {
+          const float2 u = *reinterpret_cast<const float2*>(sw_s + s * TS + 8 * j + 2 * qt);
+          sw[j] = pack2(u.x, u.y);
+        }
 #pragma unroll
-          for (int j = 0; j < 4; j++) add_term<(SEG >= 32)>(acc[i][j], counts(i, 2 * j), counts(i, 2 * j + 1), neg_bias, sa2, sw[j]);
+        for (int i = 0; i < 2; i++)
+#pragma unroll
+          for (int j = 0; j < 4; j++) add_term<(SEG >= 32)>(acc[2 * r + i][j], d[j][2 * i], d[j][2 * i + 1], sa[i], sw[j]);
+      };
+      // word i of the chunk as operand registers; elements past the row's end are 0 in the first operand
+      auto words = [&](int i, uint32_t (&a)[2][4], uint32_t (&w)[4][2]) {
+        const int s0 = 7 - 2 * qt, s1 = s0 - 1;
+#pragma unroll
+        for (int r = 0; r < 4; r++) {
+          const uint32_t av = as[i * TS + 8 * r + qg], wv = ws[i * TS + 8 * r + qg];
+          a[r >> 1][r & 1] = expand(av, s0);
+          a[r >> 1][2 + (r & 1)] = expand(av, s1);
+          w[r][0] = expand(wv, s0);
+          w[r][1] = expand(wv, s1);
+        }
+        const int64_t left = left_chunk - 32 * i;
+        if (left < 32) {
+          uint32_t k0 = 0u, k1 = 0u;
+#pragma unroll
+          for (int j = 0; j < 4; j++) {
+            if (8 * j + 2 * qt < left) k0 |= 0xFFu << (8 * j);
+            if (8 * j + 2 * qt + 1 < left) k1 |= 0xFFu << (8 * j);
+          }
+#pragma unroll
+          for (int r = 0; r < 2; r++) { a[r][0] &= k0; a[r][1] &= k0; a[r][2] &= k1; a[r][3] &= k1; }
         }
       };
-      auto words = [&](int i, uint32_t (&a)[4], uint32_t (&w)[8]) {
-        const uint4 av = *reinterpret_cast<const uint4*>(as + i * TS + 4 * ty);
-        const uint4 w0 = *reinterpret_cast<const uint4*>(ws + i * TS + 8 * tx), w1 = *reinterpret_cast<const uint4*>(ws + i * TS + 8 * tx + 4);
-        a[0] = av.x; a[1] = av.y; a[2] = av.z; a[3] = av.w;
-        w[0] = w0.x; w[1] = w0.y; w[2] = w0.z; w[3] = w0.w; w[4] = w1.x; w[5] = w1.y; w[6] = w1.z; w[7] = w1.w;
-      };
-      if constexpr (SEG <= 8) {
-        constexpr int PARTS = 8 / SEG;
+      const uint32_t bias[4] = {kBias, kBias, kBias, kBias};
+      if constexpr (SEG < 32) {
 #pragma unroll 1
         for (int i = 0; i < P::CW; i++) {
           if (P::CW > 1 && left_chunk <= 32 * i) break;      // words past the row's end
-#pragma unroll 1
-          for (int p = 0; p < PARTS; p++) {
-            uint32_t a[4], w[8], cnt[4][8];
-            words(i, a, w);
+          uint32_t a[2][4], w[4][2];
+          words(i, a, w);
+          constexpr int PER_BYTE = SEG < 8 ? 8 / SEG : 1, BYTES = SEG < 8 ? 1 : SEG / 8;     // segments of a byte, bytes of a segment
+#pragma unroll 2
+          for (int s = 0; s < P::SPW; s++) {
+            const uint32_t bytes = (BYTES == 2 ? 0xFFFFu : 0xFFu) << (8 * BYTES * (s / PER_BYTE));
+            const uint32_t keep = PER_BYTE == 1 || qt / (4 / PER_BYTE) == s % PER_BYTE ? bytes : 0u;
 #pragma unroll
-            for (int r = 0; r < 4; r++)
+            for (int r = 0; r < 2; r++) {
+              const uint32_t part[4] = {a[r][0] & keep, a[r][1] & keep, a[r][2] & keep, a[r][3] & keep};
+              uint32_t d[4][4];
 #pragma unroll
-              for (int j = 0; j < 8; j++) cnt[r][j] = doubled_counts<SEG>(a[r] ^ w[j], p);
-#pragma unroll
-            for (int b = 0; b < 4; b++)
-              segment(i * P::SPW + b * PARTS + p, [&](int r, int j) { return __byte_perm(cnt[r][j], 0x4B000000u, 0x7540u + b); });
+              for (int j = 0; j < 4; j++) mma_s8(d[j], part, w[j], bias);
+              segment(i * P::SPW + s, r, d);
+            }
           }
-        }
-      } else if constexpr (SEG == 16) {
-#pragma unroll
-        for (int i = 0; i < P::CW; i++) {
-          if (left_chunk <= 32 * i) break;
-          uint32_t a[4], w[8];
-          words(i, a, w);
-          segment(2 * i, [&](int r, int j) { return 0x4B000000u + 2u * __popc((a[r] ^ w[j]) & 0xFFFFu); });
-          segment(2 * i + 1, [&](int r, int j) { return 0x4B000000u + 2u * __popc((a[r] ^ w[j]) >> 16); });
-        }
-      } else if constexpr (SEG == 32) {
-#pragma unroll
-        for (int i = 0; i < P::CW; i++) {
-          uint32_t a[4], w[8];
-          words(i, a, w);
-          segment(i, [&](int r, int j) { return 0x4B000000u + 2u * __popc(a[r] ^ w[j]); });
         }
       } else {
-#pragma unroll
+#pragma unroll 2
         for (int s = 0; s < P::SPC; s++) {
-          uint32_t cnt[4][8];
+          if (left_chunk <= s * SEG) break;
+          uint32_t d[2][4][4];
 #pragma unroll
           for (int q = 0; q < P::SW; q++) {
-            uint32_t a[4], w[8];
+            if (P::SW > 1 && left_chunk <= 32 * (s * P::SW + q)) break;
+            uint32_t a[2][4], w[4][2];
             words(s * P::SW + q, a, w);
 #pragma unroll
-            for (int r = 0; r < 4; r++)
+            for (int r = 0; r < 2; r++)
 #pragma unroll
-              for (int j = 0; j < 8; j++) {
-                const uint32_t p = __popc(a[r] ^ w[j]);
-                cnt[r][j] = q == 0 ? p : cnt[r][j] + p;
+              for (int j = 0; j < 4; j++) {
+                if (q == 0) mma_s8(d[r][j], a[r], w[j], bias);
+                else mma_s8(d[r][j], a[r], w[j], d[r][j]);
               }
           }
-          segment(s, [&](int r, int j) { return 0x4B000000u + 2u * cnt[r][j]; });
+          segment(s, 0, d[0]);
+          segment(s, 1, d[1]);
         }
       }
     }
   }
+  auto store = [&](int i, int j, float x, float y) {
+    const int64_t row = m0 + 8 * i + qg, col = n0 + 8 * j + 2 * qt;
+    if (row >= g.M) return;
+    float* dst = g.C + row * g.ldc + col;
+    if (col + 1 < g.N) *reinterpret_cast<float2*>(dst) = make_float2(x, y);
+    else if (col < g.N) dst[0] = x;
+  };
   if (KS == 1) {
 #pragma unroll
-    for (int i = 0; i < 4; i++) {
-      const int64_t row = m0 + 4 * ty + i;
-      if (row >= g.M) continue;
+    for (int i = 0; i < 4; i++)
 #pragma unroll
-      for (int h = 0; h < 2; h++) {
-        const int64_t col = n0 + 8 * tx + 4 * h;
-        float o[4];
-        unpack2(acc[i][2 * h], o[0], o[1]);
-        unpack2(acc[i][2 * h + 1], o[2], o[3]);
-        float* dst = g.C + row * g.ldc + col;
-        if (col + 3 < g.N) *reinterpret_cast<float4*>(dst) = make_float4(o[0], o[1], o[2], o[3]);
-        else
-          for (int e = 0; e < 4; e++)
-            if (col + e < g.N) dst[e] = o[e];
+      for (int j = 0; j < 4; j++) {
+        float x, y;
+        unpack2(acc[i][j], x, y);
+        store(i, j, x, y);
       }
-    }
     return;
   }
-  // the KS partial tiles, added in order of their part: [4-column block of a lane: 2 i + h][lane] as 16-byte vectors
+  // the KS partial tiles, added in order of their part: [4 i + j][lane] as pairs of columns
   __syncwarp();                                         // the staging area is this warp's own
-  float4* mine = reinterpret_cast<float4*>(smem + warp * P::SMEM_WORDS);
+  uint64_t* mine = reinterpret_cast<uint64_t*>(smem + warp * P::SMEM_WORDS);
 #pragma unroll
   for (int i = 0; i < 4; i++)
 #pragma unroll
-    for (int h = 0; h < 2; h++) {
-      float o[4];
-      unpack2(acc[i][2 * h], o[0], o[1]);
-      unpack2(acc[i][2 * h + 1], o[2], o[3]);
-      mine[(2 * i + h) * 32 + lane] = make_float4(o[0], o[1], o[2], o[3]);
-    }
+    for (int j = 0; j < 4; j++) mine[(4 * i + j) * 32 + lane] = acc[i][j];
   __syncthreads();
   const int first = warp - part;                        // the warps first .. first + KS - 1 hold this tile
-  for (int b = part; b < 8; b += KS) {                  // 8 blocks shared out among the KS warps
-    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int b = part; b < 16; b += KS) {                 // 16 blocks shared out among the KS warps
+    float2 sum = make_float2(0.f, 0.f);
     for (int q = 0; q < KS; q++) {
-      const float4 v = reinterpret_cast<const float4*>(smem + (first + q) * P::SMEM_WORDS)[b * 32 + lane];
-      sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
+      const float2 v = reinterpret_cast<const float2*>(smem + (first + q) * P::SMEM_WORDS)[b * 32 + lane];
+      sum.x += v.x; sum.y += v.y;
     }
-    const int64_t row = m0 + 4 * ty + (b >> 1), col = n0 + 8 * tx + 4 * (b & 1);
-    if (row >= g.M) continue;
-    float* dst = g.C + row * g.ldc + col;
-    const float o[4] = {sum.x, sum.y, sum.z, sum.w};
-    if (col + 3 < g.N) *reinterpret_cast<float4*>(dst) = sum;
-    else
-      for (int e = 0; e < 4; e++)
-        if (col + e < g.N) dst[e] = o[e];
+    store(b >> 2, b & 3, sum.x, sum.y);
   }
 }
 
