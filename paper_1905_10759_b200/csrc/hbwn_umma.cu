@@ -37,11 +37,14 @@ using namespace umma;
 constexpr int kThreads = 6 * 32;
 constexpr int kLoaderWarp = 4, kMmaWarp = 5;
 constexpr int KB = 64;            // K elements per stage (128 bytes of bf16 per row)
+// Epilogue staging (see finish_block): two 4 KB blocks and 64 affine factors for each of the four epilogue warps.
+constexpr int kOutBlock = 32 * 128, kOutBlocks = 4 * 2 * kOutBlock, kOutFactors = 4 * 64 * 4;
 
 struct Args {
   const __nv_bfloat16* a; int64_t lda;
   const uint32_t* w_bits; const void* w_scales; int64_t ldw_w, ldw_s; int32_t w_bf16;
   float* C; int64_t ldc; int32_t c_vec;   // c_vec: rows of C allow 16-byte stores
+  int32_t o_copy;                 // finished blocks leave by tensor copies (see finish_block)
   int64_t M, N, K, Gw;
   int64_t beta;                   // weight group length (>= K: one group per row)
   const unsigned char* w_prep;    // [n tile][k block][3 pieces][TN rows x 128 bytes]
@@ -64,6 +67,7 @@ __device__ __forceinline__ float load_scale(const void* s, int bf16, int64_t idx
 // TN: columns of the CTA tile.  NP: bf16 pieces per weight -- 3 carry the fp32 group scale to 2^-26 (64-column
 // tiles: 192 stacked rows per MMA), 2 carry it to 2^-17 (128-column tiles: 256 stacked rows per MMA, which
 // moves 40 % fewer shared-memory bytes per output, the resource that bounds this kernel).
+constexpr int kResBytes = 225 * 1024;
 template <int TN, int NP>
 struct Smem {
   static constexpr int A_STAGE = TM * 128;
@@ -75,13 +79,16 @@ struct Smem {
   static constexpr int OFF_BAR = OFF_B + STAGES * B_STAGE;
   static constexpr int NBAR = 2 * STAGES + 4 + 2;      // full, empty, tfull[2], tempty[2], drain, wfull
   static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
-  static constexpr int USED = OFF_MISC + 16;
+  static constexpr int OFF_FACTORS = (OFF_MISC + 16 + 15) / 16 * 16;       // read as 16-byte vectors
+  static constexpr int OFF_OUT = (OFF_FACTORS + kOutFactors + 1023) / 1024 * 1024;
+  static constexpr bool COPIES = OFF_OUT + kOutBlocks <= 227 * 1024;
+  static constexpr int USED = COPIES ? OFF_OUT + kOutBlocks : OFF_OUT;
   static constexpr int BYTES = USED > 120 * 1024 ? USED : 120 * 1024;   // one CTA per SM
   static constexpr int NST = NP * TN;                  // MMA N: the pieces side by side
   static constexpr int TMEM_COLS = 512;                // two accumulator buffers of NST columns
   // Resident mode (one column tile whose weight pieces fit beside the activation ring): the pieces of all
   // K blocks are copied into shared memory once per CTA and only activation tiles stream afterwards.
-  static constexpr int RES_STAGES = 4;
+  static constexpr int RES_STAGES = 4;                 // (kResBytes and the epilogue's factors in all)
   static constexpr int RES_OFF_B = RES_STAGES * A_STAGE;
   static constexpr int RES_MAX_B = 225 * 1024 - RES_OFF_B - 512;        // bytes of weight pieces that fit
   static_assert(NST <= 256 && NST % 16 == 0 && 2 * NST <= TMEM_COLS, "one MMA covers the stacked pieces");
@@ -169,9 +176,114 @@ nhwc_and_pieces_kernel(const CopyArgs c, const Args g, unsigned char* __restrict
   }
 }
 
+// The epilogue's part of shared memory: per warp the affine factors of 32 columns and, where there is room, two 4 KB blocks that
+// leave by tensor copies.
+// One epilogue warp's way of finishing 32 x 32 outputs at a time.
+struct OutWarp {
+  unsigned char* blocks;         // this warp's two
+  float* factors;                // scale of 32 columns, shift of 32 columns
+  uint32_t count;                // blocks handed to the copy engine
+  __device__ __forceinline__ OutWarp(unsigned char* all_blocks, unsigned char* all_factors, int warp)
+      : blocks(all_blocks + warp * 2 * kOutBlock), factors(reinterpret_cast<float*>(all_factors) + warp * 64), count(0) {}
+};
+// v: the pieces' accumulators of columns n0 .. n0 + 31 of row m (valid: an output).  fsc, fsh: this lane's column's affine factors.
+// Whole blocks (o_copy: consecutive rows, which start on 16 bytes) go through shared memory and leave by a tensor copy: sixteen
+// bytes of a row per lane straight to the output are 32 lines an instruction, 4600 clk for 128 columns, 8100 with the affine
+// factors loaded one by one, at the end of every CTA's last tile -- and beside the next tile's MMAs, whose operands come through
+// the same shared-memory path (13400 instead of 9500 clk per tile of 18 stages).
+template <int NP, bool COPIES>
+__device__ __forceinline__ void finish_block(const Args& g, const CUtensorMap& o_map, OutWarp& out, const uint32_t (&v)[NP][32], float fsc, float fsh,
+                                             bool valid, int64_t m, int64_t n0, int lane, bool last_chunk, int64_t tile_end, float& carry) {
+  float z[32];
+#pragma unroll
+  for (int e = 0; e < 32; e++) {           // smallest pieces first
+    z[e] = __uint_as_float(v[NP - 1][e]);
+#pragma unroll
+    for (int i = NP - 2; i >= 0; i--) z[e] += __uint_as_float(v[i][e]);
+  }
+  const bool plain = g.ep.mode == kEpiPlain;
+  if (!plain) {
+    __syncwarp();                          // the factors of the block before are read
+    out.factors[lane] = fsc;
+    out.factors[32 + lane] = fsh;
+    __syncwarp();
+  }
+  const int per_copy = !plain && g.ep.out_bf16 ? 8 : 4;          // outputs per 16 bytes: the copy clips a row to them
+  if (COPIES && g.o_copy && (n0 + 32 <= g.N || g.N % per_copy == 0)) {
+    unsigned char* block = out.blocks + (out.count & 1) * kOutBlock;
+    if (lane == 0) bulk_wait_read<1>();
+    __syncwarp();
+    if (!plain) {
+#pragma unroll
+      for (int e = 0; e < 32; e += 4) {
+        const float4 fs = *reinterpret_cast<const float4*>(out.factors + e), fh = *reinterpret_cast<const float4*>(out.factors + 32 + e);
+        const float s4[4] = {fs.x, fs.y, fs.z, fs.w}, h4[4] = {fh.x, fh.y, fh.z, fh.w};
+#pragma unroll
+        for (int q = 0; q < 4; q++) z[e + q] = fmaf(g.ep.act == 1 ? fmaxf(z[e + q], 0.0f) : z[e + q], s4[q], h4[q]);
+      }
+    }
+    if (per_copy == 8) {                   // 64 bytes a row, pieces permuted as the copy's 64-byte swizzle has them
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        uint32_t w[4];
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+          const __nv_bfloat162 h = __floats2bfloat162_rn(z[8 * j + 2 * e], z[8 * j + 2 * e + 1]);
+          w[e] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+        *reinterpret_cast<uint4*>(block + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; j++)
+        *reinterpret_cast<float4*>(block + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_float4(z[4 * j], z[4 * j + 1], z[4 * j + 2], z[4 * j + 3]);
+    }
+    fence_async_proxy();
+    __syncwarp();
+    if (lane == 0) {
+      const int64_t m0 = m - lane;
+      if (m0 < g.M && n0 < g.N) tma_store_2d(&o_map, block, static_cast<int32_t>(n0), static_cast<int32_t>(m0));
+      bulk_commit();
+    }
+    out.count++;
+    return;
+  }
+  if (!valid) return;
+  if (!plain) {
+    // activation, affine map, then a dense (fp32 / bf16) or binarized row instead of the fp32 product
+    float fs[32], fh[32];
+#pragma unroll
+    for (int e = 0; e < 32; e += 4) {
+      const float4 a = *reinterpret_cast<const float4*>(out.factors + e), b = *reinterpret_cast<const float4*>(out.factors + 32 + e);
+      fs[e] = a.x; fs[e + 1] = a.y; fs[e + 2] = a.z; fs[e + 3] = a.w;
+      fh[e] = b.x; fh[e + 1] = b.y; fh[e + 2] = b.z; fh[e + 3] = b.w;
+    }
+    epi::finish_chunk(g.ep, z, fs, fh, m, n0, g.N, last_chunk, tile_end, carry);
+    return;
+  }
+  float* dst = g.C + m * g.ldc + n0;
+#pragma unroll
+  for (int j = 0; j < 32; j += 4) {
+    if (g.c_vec && n0 + j + 3 < g.N) *reinterpret_cast<float4*>(dst + j) = make_float4(z[j], z[j + 1], z[j + 2], z[j + 3]);
+    else
+      for (int e = 0; e < 4; e++)
+        if (n0 + j + e < g.N) dst[j + e] = z[j + e];
+  }
+}
+// This lane's column's affine factors for each block of 32 columns of a tile.
+template <int BLOCKS>
+__device__ __forceinline__ void load_factors(const Args& g, int64_t nb, int lane, float (&fsc)[BLOCKS], float (&fsh)[BLOCKS]) {
+#pragma unroll
+  for (int c = 0; c < BLOCKS; c++) {
+    const int64_t n = nb + c * 32 + lane;
+    fsc[c] = (g.ep.bn_scale && n < g.N) ? __ldg(g.ep.bn_scale + n) : 1.0f;
+    fsh[c] = (g.ep.bn_shift && n < g.N) ? __ldg(g.ep.bn_shift + n) : 0.0f;
+  }
+}
+
 template <int TN, int NP, bool RES>
 __global__ void __launch_bounds__(kThreads, 1)
-hbwn_umma_kernel(const Args g, const __grid_constant__ CUtensorMap a_map) {
+hbwn_umma_kernel(const Args g, const __grid_constant__ CUtensorMap a_map, const __grid_constant__ CUtensorMap o_map) {
   using S = Smem<TN, NP>;
   constexpr int STAGES = RES ? S::RES_STAGES : S::STAGES;
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -318,13 +430,15 @@ hbwn_umma_kernel(const Args g, const __grid_constant__ CUtensorMap a_map) {
     // =========================== epilogue ===========================
     const int row = warp * 32 + lane;
     const uint32_t t_lane = static_cast<uint32_t>(warp * 32) << 16;
+    OutWarp out(smem + S::OFF_OUT, RES ? smem + kResBytes : smem + S::OFF_FACTORS, warp);
     for (int64_t ti = 0; ti < my_tiles; ti++) {
       const uint32_t buf = static_cast<uint32_t>(ti & 1);
-      if (!mbar_wait(&tfull[buf], static_cast<uint32_t>((ti >> 1) & 1), abort_flag, 5)) break;
-      tc_fence_after();
       const int64_t tile = blockIdx.x + ti * gridDim.x;
       const int64_t m = (tile / tiles_n) * TM + row, nb = (tile % tiles_n) * TN;
-      float* dst = g.C + m * g.ldc + nb;
+      float fsc[TN / 32], fsh[TN / 32];
+      load_factors<TN / 32>(g, nb, lane, fsc, fsh);
+      if (!mbar_wait(&tfull[buf], static_cast<uint32_t>((ti >> 1) & 1), abort_flag, 5)) break;
+      tc_fence_after();
       float carry = 0.0f;                                   // |z| sum of a next-layer group wider than a 32-column chunk
 #pragma unroll
       for (int c = 0; c < TN / 32; c++) {
@@ -333,44 +447,13 @@ hbwn_umma_kernel(const Args g, const __grid_constant__ CUtensorMap a_map) {
 #pragma unroll
         for (int i = 0; i < NP; i++) tmem_ld32(t_addr + i * TN, v[i]);
         tmem_ld_wait();
-        if (m < g.M && g.ep.mode != kEpiPlain) {
-          // activation, affine map, then a dense (fp32 / bf16) or binarized row instead of the fp32 product
-          float cv[32], fs[32], fh[32];
-#pragma unroll
-          for (int e = 0; e < 32; e++) {
-            float acc = __uint_as_float(v[NP - 1][e]);
-#pragma unroll
-            for (int i = NP - 2; i >= 0; i--) acc += __uint_as_float(v[i][e]);
-            cv[e] = acc;
-            const int64_t n = nb + c * 32 + e;
-            fs[e] = (g.ep.bn_scale && n < g.N) ? __ldg(g.ep.bn_scale + n) : 1.0f;
-            fh[e] = (g.ep.bn_shift && n < g.N) ? __ldg(g.ep.bn_shift + n) : 0.0f;
-          }
-          epi::finish_chunk(g.ep, cv, fs, fh, m, nb + c * 32, g.N, c == TN / 32 - 1, nb + TN, carry);
-        } else if (m < g.M) {
-#pragma unroll
-          for (int j = 0; j < 32; j += 4) {
-            float o[4];
-#pragma unroll
-            for (int e = 0; e < 4; e++) {    // smallest pieces first
-              float acc = __uint_as_float(v[NP - 1][j + e]);
-#pragma unroll
-              for (int i = NP - 2; i >= 0; i--) acc += __uint_as_float(v[i][j + e]);
-              o[e] = acc;
-            }
-            const int64_t n = nb + c * 32 + j;
-            if (g.c_vec && n + 3 < g.N)
-              *reinterpret_cast<float4*>(dst + c * 32 + j) = make_float4(o[0], o[1], o[2], o[3]);
-            else
-              for (int e = 0; e < 4; e++)
-                if (n + e < g.N) dst[c * 32 + j + e] = o[e];
-          }
-        }
+        finish_block<NP, !RES && S::COPIES>(g, o_map, out, v, fsc[c], fsh[c], m < g.M, m, nb + c * 32, lane, c == TN / 32 - 1, nb + TN, carry);
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[buf]);
     }
+    if (!RES && S::COPIES && lane == 0) bulk_wait_all();     // the rows are in memory before the CTA ends
   }
 
   tc_fence_before();
@@ -401,19 +484,23 @@ struct PairSmem {
   static constexpr int A_STAGE = TM * 128;                 // this CTA's 128 activation rows
   static constexpr int B_HALF = (NST / 2) * 128;           // this CTA's half of the stacked weight rows
   static constexpr int STAGE = A_STAGE + B_HALF;
-  static constexpr int STAGES = (200 * 1024) / STAGE;
+  static constexpr int STAGES = (192 * 1024) / STAGE;
   static constexpr int OFF_A = 0;
   static constexpr int OFF_B = STAGES * A_STAGE;
   static constexpr int OFF_BAR = STAGES * STAGE;
   static constexpr int NBAR = 2 * STAGES + 4 + 1;          // full, empty, tfull[2], tempty[2], drain
-  static constexpr int BYTES = OFF_BAR + NBAR * 8 + 16;
+  static constexpr int OFF_FACTORS = (OFF_BAR + NBAR * 8 + 16 + 15) / 16 * 16;       // read as 16-byte vectors
+  static constexpr int OFF_OUT = (OFF_FACTORS + kOutFactors + 1023) / 1024 * 1024;
+  static constexpr int BYTES = OFF_OUT + kOutBlocks;
   static constexpr int TMEM_COLS = 512;
-  static_assert(NST == 256 && B_HALF == Smem<TN, NP>::B_PIECE, "each CTA of the pair stages exactly one weight piece");
+  static_assert(NP == 2 && 2 * NST <= TMEM_COLS && BYTES <= 227 * 1024, "each CTA of the pair stages exactly one weight piece");
 };
 
+constexpr int kPairPrep = 128;     // rows of a column tile in the prepared weights, whatever the pair kernel's own tile
 template <int TN, int NP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-hbwn_pair_kernel(const Args g, const __grid_constant__ CUtensorMap a_map, const __grid_constant__ CUtensorMap b_map) {
+hbwn_pair_kernel(const Args g, const __grid_constant__ CUtensorMap a_map, const __grid_constant__ CUtensorMap b_map,
+                 const __grid_constant__ CUtensorMap o_map) {
   using S = PairSmem<TN, NP>;
   constexpr int STAGES = S::STAGES;
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -469,8 +556,8 @@ hbwn_pair_kernel(const Args g, const __grid_constant__ CUtensorMap a_map, const 
         const int64_t tile = pair + ti * n_pairs;
         const int64_t tile_m = tile / tiles_n, tile_n = tile - tile_m * tiles_n;
         const int64_t m0 = tile_m * (2 * TM) + rank * TM;
-        // rows of the weight-piece matrix: [column tile][k block][piece][TN rows]; this CTA stages piece `rank`
-        int32_t b_row = static_cast<int32_t>((tile_n * n_kb * NP + rank) * TN);
+        // rows of the weight-piece matrix: [column tile of 128][k block][piece][128 rows]; this CTA stages piece `rank`
+        int32_t b_row = static_cast<int32_t>((tile_n / (kPairPrep / TN) * n_kb * NP + rank) * kPairPrep + tile_n % (kPairPrep / TN) * TN);
         int32_t b = 0, h0 = 0, w0 = 0;
         if (g.conv) {
           b = static_cast<int32_t>(m0 / g.HoWo);
@@ -490,7 +577,7 @@ hbwn_pair_kernel(const Args g, const __grid_constant__ CUtensorMap a_map, const 
           else
             tma_load_2d_pair(smem + S::OFF_A + s * S::A_STAGE, &a_map, kb * KB, static_cast<int32_t>(m0), bar);
           tma_load_2d_pair(smem + S::OFF_B + s * S::B_HALF, &b_map, 0, b_row, bar);
-          b_row += NP * TN;
+          b_row += NP * kPairPrep;
           issued++;
           if (++cb == g.cblocks) { cb = 0; if (++fj == g.kw) { fj = 0; fi++; } }
           if (++s == STAGES) { s = 0; round++; }
@@ -554,13 +641,15 @@ hbwn_pair_kernel(const Args g, const __grid_constant__ CUtensorMap a_map, const 
     const int row = warp * 32 + lane;
     const uint32_t t_lane = static_cast<uint32_t>(warp * 32) << 16;
     const uint32_t tempty0 = mapa_rank(smem_u32(tempty), 0);        // rank 0's `tempty` barriers
+    OutWarp out(smem + S::OFF_OUT, smem + S::OFF_FACTORS, warp);
     for (int64_t ti = 0; ti < my_tiles; ti++) {
       const uint32_t buf = static_cast<uint32_t>(ti & 1);
-      if (!mbar_wait(&tfull[buf], static_cast<uint32_t>((ti >> 1) & 1), abort_flag, 5)) break;
-      tc_fence_after();
       const int64_t tile = pair + ti * n_pairs;
       const int64_t m = (tile / tiles_n) * (2 * TM) + rank * TM + row, nb = (tile % tiles_n) * TN;
-      float* dst = g.C + m * g.ldc + nb;
+      float fsc[TN / 32], fsh[TN / 32];
+      load_factors<TN / 32>(g, nb, lane, fsc, fsh);
+      if (!mbar_wait(&tfull[buf], static_cast<uint32_t>((ti >> 1) & 1), abort_flag, 5)) break;
+      tc_fence_after();
       float carry = 0.0f;
 #pragma unroll
       for (int c = 0; c < TN / 32; c++) {
@@ -569,43 +658,13 @@ hbwn_pair_kernel(const Args g, const __grid_constant__ CUtensorMap a_map, const 
 #pragma unroll
         for (int i = 0; i < NP; i++) tmem_ld32(t_addr + i * TN, v[i]);
         tmem_ld_wait();
-        if (m < g.M && g.ep.mode != kEpiPlain) {
-          float cv[32], fs[32], fh[32];
-#pragma unroll
-          for (int e = 0; e < 32; e++) {
-            float acc = __uint_as_float(v[NP - 1][e]);
-#pragma unroll
-            for (int i = NP - 2; i >= 0; i--) acc += __uint_as_float(v[i][e]);
-            cv[e] = acc;
-            const int64_t n = nb + c * 32 + e;
-            fs[e] = (g.ep.bn_scale && n < g.N) ? __ldg(g.ep.bn_scale + n) : 1.0f;
-            fh[e] = (g.ep.bn_shift && n < g.N) ? __ldg(g.ep.bn_shift + n) : 0.0f;
-          }
-          epi::finish_chunk(g.ep, cv, fs, fh, m, nb + c * 32, g.N, c == TN / 32 - 1, nb + TN, carry);
-        } else if (m < g.M) {
-#pragma unroll
-          for (int j = 0; j < 32; j += 4) {
-            float o[4];
-#pragma unroll
-            for (int e = 0; e < 4; e++) {    // smallest pieces first
-              float acc = __uint_as_float(v[NP - 1][j + e]);
-#pragma unroll
-              for (int i = NP - 2; i >= 0; i--) acc += __uint_as_float(v[i][j + e]);
-              o[e] = acc;
-            }
-            const int64_t n = nb + c * 32 + j;
-            if (g.c_vec && n + 3 < g.N)
-              *reinterpret_cast<float4*>(dst + c * 32 + j) = make_float4(o[0], o[1], o[2], o[3]);
-            else
-              for (int e = 0; e < 4; e++)
-                if (n + e < g.N) dst[c * 32 + j + e] = o[e];
-          }
-        }
+        finish_block<NP, true>(g, o_map, out, v, fsc[c], fsh[c], m < g.M, m, nb + c * 32, lane, c == TN / 32 - 1, nb + TN, carry);
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(tempty0 + buf * 8);
     }
+    if (lane == 0) bulk_wait_all();      // the rows are in memory before the CTA ends
   }
 
   // Neither CTA may leave while the other can still reach into it (rank 0's MMAs read rank 1's shared memory and
@@ -771,6 +830,9 @@ hbwn_halo_kernel(const Args g, const HaloArgs h, const __grid_constant__ CUtenso
   } else if (warp < 4) {
     const int row = warp * 32 + lane;
     const uint32_t t_lane = static_cast<uint32_t>(warp * 32) << 16;
+    OutWarp out(nullptr, smem + off_bar + 256, warp);
+    float fsc[TN / 32], fsh[TN / 32];
+    load_factors<TN / 32>(g, 0, lane, fsc, fsh);
     for (int64_t ti = 0; ti < my_tiles; ti++) {
       const uint32_t buf = static_cast<uint32_t>(ti & 1);
       // where this thread's position lies in the padded image, and whether it is an output at all
@@ -782,7 +844,6 @@ hbwn_halo_kernel(const Args g, const HaloArgs h, const __grid_constant__ CUtenso
       const int64_t m = (static_cast<int64_t>(b) * h.Ho + y) * h.Wo + x;
       if (!mbar_wait(&tfull[buf], static_cast<uint32_t>((ti >> 1) & 1), abort_flag, 5)) break;
       tc_fence_after();
-      float* dst = g.C + m * g.ldc;
       float carry = 0.0f;
 #pragma unroll
       for (int c = 0; c < TN / 32; c++) {
@@ -791,38 +852,7 @@ hbwn_halo_kernel(const Args g, const HaloArgs h, const __grid_constant__ CUtenso
 #pragma unroll
         for (int i = 0; i < NP; i++) tmem_ld32(t_addr + i * TN, v[i]);
         tmem_ld_wait();
-        if (valid && g.ep.mode != kEpiPlain) {
-          float cv[32], fs[32], fh[32];
-#pragma unroll
-          for (int e = 0; e < 32; e++) {
-            float acc = __uint_as_float(v[NP - 1][e]);
-#pragma unroll
-            for (int i = NP - 2; i >= 0; i--) acc += __uint_as_float(v[i][e]);
-            cv[e] = acc;
-            const int64_t n = c * 32 + e;
-            fs[e] = (g.ep.bn_scale && n < g.N) ? __ldg(g.ep.bn_scale + n) : 1.0f;
-            fh[e] = (g.ep.bn_shift && n < g.N) ? __ldg(g.ep.bn_shift + n) : 0.0f;
-          }
-          epi::finish_chunk(g.ep, cv, fs, fh, m, c * 32, g.N, c == TN / 32 - 1, TN, carry);
-        } else if (valid) {
-#pragma unroll
-          for (int j = 0; j < 32; j += 4) {
-            float o[4];
-#pragma unroll
-            for (int e = 0; e < 4; e++) {    // smallest pieces first
-              float acc = __uint_as_float(v[NP - 1][j + e]);
-#pragma unroll
-              for (int i = NP - 2; i >= 0; i--) acc += __uint_as_float(v[i][j + e]);
-              o[e] = acc;
-            }
-            const int64_t n = c * 32 + j;
-            if (g.c_vec && n + 3 < g.N)
-              *reinterpret_cast<float4*>(dst + n) = make_float4(o[0], o[1], o[2], o[3]);
-            else
-              for (int e = 0; e < 4; e++)
-                if (n + e < g.N) dst[n + e] = o[e];
-          }
-        }
+        finish_block<NP, false>(g, a_map, out, v, fsc[c], fsh[c], valid, m, c * 32, lane, c == TN / 32 - 1, TN, carry);
       }
       tc_fence_before();
       __syncwarp();
@@ -852,6 +882,7 @@ Args make_args(const DenseView& A, const PackedView& W, float* C, int64_t ldc) {
   g.conv = 0; g.taps = 1; g.kw = 1; g.cblocks = static_cast<int32_t>(g.n_kb); g.Cin = 0;
   g.HoWo = 1; g.Wo = 1; g.sh = g.sw = 1; g.ph = g.pw = 0;
   g.ep = plain_epilogue();
+  g.o_copy = 0;
   return g;
 }
 
@@ -924,6 +955,24 @@ bool make_pieces_map(const void* w_prep, int64_t rows, int box_rows, CUtensorMap
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The output (the product, or the dense tensor of the epilogue chain) as a 2-D tensor for the epilogue's copies: 32 x 32 blocks.
+// false: its rows do not start on 16 bytes, or it is not dense.
+bool make_out_map(const Args& g, CUtensorMap* map) {
+  if (g.ep.mode == kEpiPacked) return false;
+  const bool plain = g.ep.mode == kEpiPlain, bf16 = !plain && g.ep.out_bf16;
+  void* out = plain ? static_cast<void*>(g.C) : g.ep.out;
+  const int64_t pitch = (plain ? g.ldc : g.ep.ld_out) * (bf16 ? 2 : 4);
+  EncodeTiledFn fn = encode_tiled_fn();
+  if (!fn || reinterpret_cast<uintptr_t>(out) % 16 != 0 || pitch % 16 != 0) return false;
+  const cuuint64_t dims[2] = {static_cast<cuuint64_t>(g.N), static_cast<cuuint64_t>(g.M)};
+  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(pitch)};
+  const cuuint32_t box[2] = {32, 32};
+  const cuuint32_t elem[2] = {1, 1};
+  return fn(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, out, dims, strides, box, elem,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, bf16 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 constexpr int kHaloSmemMax = 227 * 1024;
 
 // Whether the shared-rows kernel takes this convolution, and its geometry: stride 1, exactly one 64-channel
@@ -933,7 +982,7 @@ bool plan_halo(const ConvGeom& c, int64_t N, HaloArgs* h) {
   if (c.sh != 1 || c.sw != 1 || c.C != KB || N > 64 || c.ph > 127 || c.pw > 127) return false;
   const int64_t Wp = static_cast<int64_t>(c.W) + 2 * c.pw, Hp = static_cast<int64_t>(c.H) + 2 * c.ph;
   if (static_cast<int64_t>(c.kh - 1) * Wp + (c.kw - 1) > TM || Hp * Wp >= (int64_t{1} << 31)) return false;
-  const int64_t smem = static_cast<int64_t>(kRing + 1) * kBlockBytes + static_cast<int64_t>(c.kh) * c.kw * Smem<64, 2>::B_STAGE + 256;
+  const int64_t smem = static_cast<int64_t>(kRing + 1) * kBlockBytes + static_cast<int64_t>(c.kh) * c.kw * Smem<64, 2>::B_STAGE + 256 + kOutFactors;
   if (smem > kHaloSmemMax) return false;
   h->Wp = static_cast<int32_t>(Wp); h->Hp = static_cast<int32_t>(Hp); h->HpWp = static_cast<int32_t>(Hp * Wp);
   h->Ho = c.Ho; h->Wo = c.Wo; h->B = c.B;
@@ -957,21 +1006,45 @@ Args make_conv_args(const ConvGeom& c, const PackedView& W, float* C, int64_t ld
   g.n_kb = static_cast<int64_t>(g.taps) * g.cblocks;
   g.HoWo = c.Ho * c.Wo; g.Wo = c.Wo; g.sh = c.sh; g.sw = c.sw; g.ph = c.ph; g.pw = c.pw;
   g.ep = plain_epilogue();
+  g.o_copy = 0;
   return g;
+}
+
+// CTA pairs walk tiles of 256 x 128, or of 256 x 64 where that keeps more pairs busy or leaves them a shorter last turn: clocks of
+// a stage and of a tile's exposed epilogue.  A stage of half the columns takes three quarters of the time (it brings the same
+// activations), so the narrow tile only pays where it takes fewer than 1.4 turns for one.  Wide / narrow, us: 3136 x 256 x 2304
+// (26 / 52 tiles for 74 pairs) 16.0 / 12.9, 784 x 128 x 1152 11.0 / 8.3, 11760 x 192 x 1728 (92 / 138) 21.7 / 17.9; 50176 x 128 x
+// 1152 (196 / 392) 23.6 / 32.1, 6272 x 256 x 1728 (50 / 100) 14.2 / 17.3, 7840 x 256 x 1152 (62 / 124) 11.9 / 13.7.
+constexpr int64_t kWideStage = 512, kWideTile = 2500, kNarrowStage = 375, kNarrowTile = 1500;
+
+// prep_rows: rows of the prepared weight pieces' matrix.
+template <int TN, int NP>
+cudaError_t launch_pair(const Args& g, const CUtensorMap& a_map, const CUtensorMap& o_map, int64_t prep_rows, int dev, int64_t pairs, cudaStream_t stream) {
+  using P = PairSmem<TN, NP>;
+  static DeviceOnce configured;
+  if (configured.pending(dev)) {
+    const cudaError_t e = cudaFuncSetAttribute(hbwn_pair_kernel<TN, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, P::BYTES);
+    if (e != cudaSuccess) return e;
+    configured.mark(dev);
+  }
+  CUtensorMap b_map;
+  if (!make_pieces_map(g.w_prep, prep_rows, TN, &b_map)) return cudaErrorNotSupported;
+  const int64_t tiles = ((g.M + 2 * TM - 1) / (2 * TM)) * ((g.N + TN - 1) / TN);
+  if (tiles < pairs) pairs = tiles;
+  return launch_pdl(hbwn_pair_kernel<TN, NP>, dim3(static_cast<unsigned>(2 * pairs)), dim3(kThreads), P::BYTES, stream, g, a_map, b_map, o_map);
 }
 
 template <int TN, int NP>
 cudaError_t launch(Args g, const CUtensorMap& a_map, void* workspace, cudaStream_t stream, const CopyArgs* copy = nullptr,
                    bool w_prepared = false, const HaloArgs* halo = nullptr) {
   using S = Smem<TN, NP>;
-  constexpr int kResBytes = 225 * 1024;
   static DeviceOnce configured;
   int dev = 0, sms = 0;
   if (current_device(&dev, &sms) != cudaSuccess) return cudaErrorInvalidDevice;
   if (configured.pending(dev)) {
     cudaError_t e = cudaFuncSetAttribute(hbwn_umma_kernel<TN, NP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::BYTES);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(hbwn_umma_kernel<TN, NP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kResBytes);
+    e = cudaFuncSetAttribute(hbwn_umma_kernel<TN, NP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kResBytes + kOutFactors);
     if (e != cudaSuccess) return e;
     configured.mark(dev);
   }
@@ -998,7 +1071,7 @@ cudaError_t launch(Args g, const CUtensorMap& a_map, void* workspace, cudaStream
         if (e != cudaSuccess) return e;
         halo_configured.mark(dev);
       }
-      const int64_t used = static_cast<int64_t>(kRing + 1) * kBlockBytes + static_cast<int64_t>(g.taps) * S::B_STAGE + 256;
+      const int64_t used = static_cast<int64_t>(kRing + 1) * kBlockBytes + static_cast<int64_t>(g.taps) * S::B_STAGE + 256 + kOutFactors;
       const int bytes = static_cast<int>(used > 120 * 1024 ? used : 120 * 1024);          // one CTA per SM
       const int64_t tiles = (halo->positions + TM - 1) / TM;
       HaloArgs hh = *halo;
@@ -1007,29 +1080,25 @@ cudaError_t launch(Args g, const CUtensorMap& a_map, void* workspace, cudaStream
       return launch_pdl(hbwn_halo_kernel<NP>, dim3(static_cast<unsigned>(ctas)), dim3(kThreads), bytes, stream, g, hh, a_map);
     }
   }
+  CUtensorMap o_map = {};
+  g.o_copy = S::COPIES && g.M < (int64_t{1} << 31) && make_out_map(g, &o_map) ? 1 : 0;
   if constexpr (TN == 128 && NP == 2) {
-    // at least two row tiles: CTA pairs that share each weight stage
-    if (g.M > TM && sms >= 2) {
-      using P = PairSmem<TN, NP>;
-      static DeviceOnce pair_configured;
-      if (pair_configured.pending(dev)) {
-        const cudaError_t e = cudaFuncSetAttribute(hbwn_pair_kernel<TN, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, P::BYTES);
-        if (e != cudaSuccess) return e;
-        pair_configured.mark(dev);
-      }
-      CUtensorMap b_map;
-      if (!make_pieces_map(g.w_prep, tiles_n * n_kb * NP * TN, TN, &b_map)) return cudaErrorNotSupported;
-      const int64_t pair_tiles = ((g.M + 2 * TM - 1) / (2 * TM)) * tiles_n;
-      const int64_t pairs = pair_tiles < sms / 2 ? pair_tiles : sms / 2;
-      return launch_pdl(hbwn_pair_kernel<TN, NP>, dim3(static_cast<unsigned>(2 * pairs)), dim3(kThreads), P::BYTES, stream, g, a_map, b_map);
+    // CTA pairs that share each weight stage (a product of one row tile only where it is cut into narrow ones)
+    if (sms >= 2) {
+      const int64_t tiles_m = (g.M + 2 * TM - 1) / (2 * TM), pairs = sms / 2;
+      const auto turns = [&](int64_t tiles) { return (tiles + pairs - 1) / pairs; };
+      const bool narrow = !(g.ep.mode == kEpiPacked && g.ep.nx_beta > 64) &&
+                          turns(tiles_m * ((g.N + 63) / 64)) * (n_kb * kNarrowStage + kNarrowTile) < turns(tiles_m * tiles_n) * (n_kb * kWideStage + kWideTile);
+      if (narrow) return launch_pair<64, NP>(g, a_map, o_map, tiles_n * n_kb * NP * TN, dev, pairs, stream);
+      if (g.M > TM) return launch_pair<TN, NP>(g, a_map, o_map, tiles_n * n_kb * NP * TN, dev, pairs, stream);
     }
   }
   const int64_t tiles = ((g.M + TM - 1) / TM) * tiles_n;
   const unsigned grid = static_cast<unsigned>(tiles < sms ? tiles : sms);
   // a single column tile whose pieces fit beside the activation ring stays resident in shared memory
   if (tiles_n == 1 && n_kb * S::B_STAGE <= S::RES_MAX_B && tiles > sms)
-    return launch_pdl(hbwn_umma_kernel<TN, NP, true>, dim3(grid), dim3(kThreads), kResBytes, stream, g, a_map);
-  return launch_pdl(hbwn_umma_kernel<TN, NP, false>, dim3(grid), dim3(kThreads), S::BYTES, stream, g, a_map);
+    return launch_pdl(hbwn_umma_kernel<TN, NP, true>, dim3(grid), dim3(kThreads), kResBytes + kOutFactors, stream, g, a_map, o_map);
+  return launch_pdl(hbwn_umma_kernel<TN, NP, false>, dim3(grid), dim3(kThreads), S::BYTES, stream, g, a_map, o_map);
 }
 
 // exact: three pieces, 64-column tiles.  Otherwise two pieces: 128-column tiles when there are more than 64 columns.
