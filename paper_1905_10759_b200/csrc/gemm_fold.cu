@@ -1043,6 +1043,35 @@ void launch_prepare(const Args& g, unsigned char* stages, float* down, int sms, 
   }
 }
 
+// Equal runs of (tile, stage) pairs, one per CTA: they pay when they shorten the longest CTA's walk by a tenth or more.
+struct Runs { int64_t run, ctas, walk; bool pay; };
+template <int TN>
+Runs balanced_runs(const Args& g, int64_t sms) {
+  Runs r{};
+  const int64_t n_stages = (g.n_words + WPS - 1) / WPS, tiles = tile_count<TN>(g), units = tiles * n_stages;
+  r.ctas = units / kBalancedMinStages < sms ? units / kBalancedMinStages : sms;
+  if (r.ctas > kMaxBalancedCtas - 1) r.ctas = kMaxBalancedCtas - 1;
+  if (r.ctas < 1) r.ctas = 1;
+  r.run = (units + r.ctas - 1) / r.ctas;
+  // a tile is shared by at most kBalancedMaxShare + 1 CTAs: the CTA that completes it adds the others' partial
+  // accumulators one after the other, which costs more than the shorter walk saves beyond that
+  const int64_t min_run = (n_stages + kBalancedMaxShare - 1) / kBalancedMaxShare;
+  if (r.run < min_run) r.run = min_run;
+  r.walk = (tiles + sms - 1) / sms * n_stages;
+  r.pay = balanced_possible<TN>(g, sms) && r.run * 10 <= r.walk * 9;
+  r.ctas = (units + r.run - 1) / r.run;                     // no CTA without work
+  return r;
+}
+// Whole short 128-column tiles with the wide accumulator instead of the balanced schedule of narrow ones, whose reduction costs
+// some 9 us.  In hundredths of a us: a stage 46 of a whole tile, 42 of a run, a turn's exposed epilogue 150.  Balanced / whole
+// wide, us: 25088 x 128 x 576 21.4 / 17.3, 12544 x 128 x 1152 19.7 / 15.5, 4096 x 960 x 256 21.0 / 13.5, 1000 x 3000 x 640 27.3 /
+// 18.3, 50176 x 128 x 576 27.0 / 24.0; level at 12544 x 256 x 1152, slower at 50176 x 128 x 1152 (34.4 / 35.6) and 2048 x 4096 x
+// 768 (40.9 / 45.2).  The error against 64 bits falls to a third.  (Whole narrow tiles take 14.8 us of the first, but sum all of
+// K in one accumulator with the small products: 6.5e-7 balanced, 7.7e-7 narrow, 2.3e-7 wide.)
+inline bool whole_wide_pays(const Runs& r, int64_t n_stages) {
+  return r.pay && 46 * r.walk + 150 * (r.walk / n_stages) < 900 + 42 * r.run;
+}
+
 template <int TN, int ASUB, bool FUSE, bool WIDE>
 cudaError_t launch_fold_wide(Args g, void* workspace, size_t have, cudaStream_t stream, bool w_prepared) {
   using S = Smem<TN>;
@@ -1122,21 +1151,12 @@ cudaError_t launch_fold_wide(Args g, void* workspace, size_t have, cudaStream_t 
                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return cudaErrorNotSupported;
   }
-  // equal runs of (tile, stage) pairs, one per CTA, when that shortens the longest CTA's walk by a tenth or more
-  const int64_t units = tiles * n_stages;
-  int64_t ctas = units / kBalancedMinStages < sms ? units / kBalancedMinStages : sms;
-  if (ctas > kMaxBalancedCtas - 1) ctas = kMaxBalancedCtas - 1;
-  if (ctas < 1) ctas = 1;
-  int64_t run = (units + ctas - 1) / ctas;
-  // a tile is shared by at most kBalancedMaxShare + 1 CTAs: the CTA that completes it adds the others' partial
-  // accumulators one after the other, which costs more than the shorter walk saves beyond that
-  const int64_t min_run = (n_stages + kBalancedMaxShare - 1) / kBalancedMaxShare;
-  if (run < min_run) run = min_run;
-  const int64_t plain_walk = ((tiles + sms - 1) / sms) * n_stages;
-  if (kHasBalanced && balanced_possible<TN>(g, sms) && run * 10 <= plain_walk * 9) {
-    ctas = (units + run - 1) / run;                     // no CTA without work
-    g.sk_units = run;
-    return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kHasBalanced ? kBalanced : kPlain, WIDE>, dim3(static_cast<unsigned>(ctas)), dim3(kThreads), kBytes, stream, g, s_map, c_map);
+  if (kHasBalanced && !(WIDE && n_stages < kWideFromStages)) {
+    const Runs runs = balanced_runs<TN>(g, sms);
+    if (runs.pay) {
+      g.sk_units = runs.run;
+      return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kHasBalanced ? kBalanced : kPlain, WIDE>, dim3(static_cast<unsigned>(runs.ctas)), dim3(kThreads), kBytes, stream, g, s_map, c_map);
+    }
   }
   const unsigned grid = static_cast<unsigned>(tiles < sms ? tiles : sms);   // one persistent CTA per SM
   if (WIDE && stage_bytes<TN>(g) > kWeightsInL2) {
@@ -1156,7 +1176,8 @@ cudaError_t launch_fold(const Args& g, void* workspace, size_t have, cudaStream_
                              g.ep.ld_out * (g.ep.out_bf16 ? 2 : 4) % 16 == 0;
     const int64_t from = FUSE && tiles > sms ? (vector_rows ? kWideFromManyTiles : kWideFromSlowRows)
                                              : (tiles > 2 * static_cast<int64_t>(sms) ? kWideFromManyTiles : kWideFromStages);
-    if (n_stages >= from) return launch_fold_wide<TN, ASUB, FUSE, true>(g, workspace, have, stream, w_prepared);
+    const bool whole = !FUSE && ASUB == 1 && n_stages < from && n_stages < kWideFromStages && whole_wide_pays(balanced_runs<TN>(g, sms), n_stages);
+    if (n_stages >= from || whole) return launch_fold_wide<TN, ASUB, FUSE, true>(g, workspace, have, stream, w_prepared);
   }
   return launch_fold_wide<TN, ASUB, FUSE, false>(g, workspace, have, stream, w_prepared);
 }
