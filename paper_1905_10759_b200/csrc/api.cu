@@ -495,15 +495,16 @@ hbmm_status conv_checked(const void* x, int32_t x_dtype, const hbmm_conv_geom* g
       const bool a_subword = beta_a < 32 && beta_a < L.K;
       if (!gemm_fold_supported(av, wv) || a_subword || L.gemm_bytes < fold_workspace(av, wv)) return HBMM_ERR_UNSUPPORTED;
     }
-    const bool walk = im2col_walk_supported(x_dtype == HBMM_BF16, cg, beta_a, A.ld_words, A.ld_scales);
+    const bool walk = im2col_walk_supported(x_dtype == HBMM_BF16, cg, beta_a, A.ld_words, A.ld_scales), point = im2col_point_supported(cg, beta_a);
     if ((ep || prefer_fold(av, wv)) && L.gemm_bytes > 0 && L.gemm_bytes >= fold_workspace(av, wv) &&
-        (walk || im2col_quantize_tma_supported(x, x_dtype == HBMM_BF16, cg, beta_a))) {
+        (walk || point || im2col_quantize_tma_supported(x, x_dtype == HBMM_BF16, cg, beta_a))) {
       UmmaPrepJob job{};
       gemm_fold_prep_job(av, wv, gemm_ws, &job);
       if (job.n_stages * job.tiles_n <= 4096) {
         const UmmaPrepJob* expand = w_prepared ? nullptr : &job;
         const int s_bf16 = a_scale_dtype == HBMM_BF16;
         if ((walk ? launch_im2col_walk(x, x_dtype == HBMM_BF16, cg, beta_a, A.bits, A.ld_words, A.scales, A.ld_scales, s_bf16, s, expand)
+             : point ? launch_im2col_point(x, x_dtype == HBMM_BF16, cg, beta_a, A.bits, A.ld_words, A.scales, A.ld_scales, s_bf16, s, expand)
                   : launch_im2col_quantize_tma(x, cg, beta_a, A.bits, A.ld_words, A.scales, A.ld_scales, s_bf16, s, expand)) != cudaSuccess)
           return HBMM_ERR_CUDA;
         if (pack_only) return HBMM_OK;

@@ -429,6 +429,8 @@ cudaError_t launch_im2col_quantize(const void* x, int x_bf16, const ConvGeom& g,
   const int64_t G = num_groups(K, beta);
   if (im2col_walk_supported(x_bf16, g, beta, ld_words, ld_scales))
     return launch_im2col_walk(x, x_bf16, g, beta, bits, ld_words, scales, ld_scales, scale_bf16, stream);
+  if (im2col_point_supported(g, beta))
+    return launch_im2col_point(x, x_bf16, g, beta, bits, ld_words, scales, ld_scales, scale_bf16, stream);
   if (im2col_quantize_tma_supported(x, x_bf16, g, beta))
     return launch_im2col_quantize_tma(x, g, beta, bits, ld_words, scales, ld_scales, scale_bf16, stream);
   if (beta == 32 && beta < K && g.sw == 1) {

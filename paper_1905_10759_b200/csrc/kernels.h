@@ -221,6 +221,10 @@ bool im2col_walk_supported(int x_bf16, const ConvGeom& g, int32_t beta, int64_t 
 // `prep` as for launch_im2col_quantize_tma (folded operands only).
 cudaError_t launch_im2col_walk(const void* x, int x_bf16, const ConvGeom& g, int32_t beta, uint32_t* bits, int64_t ld_words, void* scales,
                                int64_t ld_scales, int scale_bf16, cudaStream_t stream, const UmmaPrepJob* prep = nullptr);
+// 1 x 1 filters, groups of 2, 4, 8, 16 elements or of up to eight whole K-words, fp32 or bf16 images of any stride and padding.
+bool im2col_point_supported(const ConvGeom& g, int32_t beta);
+cudaError_t launch_im2col_point(const void* x, int x_bf16, const ConvGeom& g, int32_t beta, uint32_t* bits, int64_t ld_words, void* scales,
+                                int64_t ld_scales, int scale_bf16, cudaStream_t stream, const UmmaPrepJob* prep = nullptr);
 // The packed front end with its input tile staged by tensor copies (fp32 input).
 bool im2col_quantize_tma_supported(const void* x, int x_bf16, const ConvGeom& g, int32_t beta);
 // prep (optional): weight-expansion tasks of the contraction that follows, run by extra CTAs of the launch.

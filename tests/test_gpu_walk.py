@@ -1,6 +1,6 @@
-"""Packed convolution front end of 3 x 3 filters at stride 1 (columns walked down the image): the packed operand left in
-the workspace against the oracle's binarization of the im2col rows, at the edges of its lanes, strips, row segments, channel
-pieces and ranges."""
+"""Packed convolution front ends of 3 x 3 filters at stride 1 (columns walked down the image) and of 1 x 1 filters: the packed
+operand left in the workspace against the oracle's binarization of the im2col rows, at the edges of their lanes, strips, row
+segments, channel pieces and ranges."""
 import numpy as np
 import pytest
 import torch
@@ -26,11 +26,34 @@ CASES = [
 ]
 
 
+POINT_CASES = [
+    # the same for 1 x 1 filters, with their stride
+    (2, 64, 9, 31, 1, 0, 32, False, False),
+    (1, 100, 7, 13, 2, 0, 4, True, True),     # the last word of four channels
+    (3, 48, 5, 5, 2, 1, 16, False, False),    # padding: rows of zeros
+    (1, 33, 3, 3, 1, 0, 8, False, False),
+    (1, 70, 8, 8, 3, 0, 2, True, False),
+    (2, 260, 6, 6, 1, 0, 64, False, True),    # a last group of four channels
+    (1, 512, 4, 4, 1, 0, 256, False, False),
+    (2, 64, 6, 6, 1, 0, 64, True, False),     # one group per row
+    (2, 10, 6, 6, 1, 0, 16, False, False),
+]
+
+
 @pytest.mark.parametrize("B,C,H,W,pad,beta,bf16,sbf16", CASES)
 def test_packed_rows_match_oracle(B, C, H, W, pad, beta, bf16, sbf16):
+    packed_rows(B, C, H, W, 3, 1, pad, beta, bf16, sbf16)
+
+
+@pytest.mark.parametrize("B,C,H,W,st,pad,beta,bf16,sbf16", POINT_CASES)
+def test_packed_pixels_match_oracle(B, C, H, W, st, pad, beta, bf16, sbf16):
+    packed_rows(B, C, H, W, 1, st, pad, beta, bf16, sbf16)
+
+
+def packed_rows(B, C, H, W, k, st, pad, beta, bf16, sbf16):
     import gpu_util as gu
     from paper_1905_10759_b200 import hbmm
-    K = C * 9
+    K = C * k * k
     x = inputs.normal((B * C * H, W), 760 + C + W).reshape(B, C, H, W).copy()
     x.reshape(-1)[::7] = 0.0
     x.reshape(-1)[::11] = -0.0
@@ -38,8 +61,8 @@ def test_packed_rows_match_oracle(B, C, H, W, pad, beta, bf16, sbf16):
         x = torch.from_numpy(x).bfloat16().float().numpy()
     sdt = hbmm.BF16 if sbf16 else hbmm.F32
     Wop = hbmm.quantize(torch.from_numpy(inputs.he_normal(40, K, 761)).cuda(), hbmm.alloc_operand(40, K, max(beta, 32)))
-    geom = hbmm.make_geom(B, C, H, W, 3, 3, (1, 1), (pad, pad))
-    M = B * (H + 2 * pad - 2) * (W + 2 * pad - 2)
+    geom = hbmm.make_geom(B, C, H, W, k, k, (st, st), (pad, pad))
+    M = B * ((H + 2 * pad - k) // st + 1) * ((W + 2 * pad - k) // st + 1)
     ws = torch.empty(hbmm.conv_workspace_bytes(geom, beta, sdt, Wop), dtype=torch.uint8, device="cuda").fill_(0xAB)
     # an image off any vector's alignment: only the element's own is asked for
     xd = torch.empty(x.size + 1, dtype=torch.bfloat16 if bf16 else torch.float32, device="cuda")[1:].view(x.shape).copy_(torch.from_numpy(x))
@@ -48,7 +71,7 @@ def test_packed_rows_match_oracle(B, C, H, W, pad, beta, bf16, sbf16):
     bits = ws[:bb].view(torch.int32).reshape(M, lw)
     off = (bb + 255) // 256 * 256
     sc = ws[off: off + sb].view(torch.bfloat16 if sbf16 else torch.float32).reshape(M, ls).float().cpu().numpy().astype(np.float64)
-    da, sa = oracle.quantize(oracle.im2col(x, 3, 3, (1, 1), (pad, pad)), beta)
+    da, sa = oracle.quantize(oracle.im2col(x, k, k, (st, st), (pad, pad)), gu.eff_beta(beta, K))
     assert np.array_equal(gu.host_bits(bits), oracle.pack(sa, lw))
     G = da.shape[1]
     assert np.all(sc[:, G:] == 0.0)
