@@ -49,7 +49,8 @@ typedef enum { HBMM_F32 = 0, HBMM_BF16 = 1 } hbmm_dtype;
  * dense activations x packed weights (HBWN, beta_a == 1). */
 typedef enum {
   HBMM_PATH_AUTO = 0,   /* the fastest path that supports the operands (and has its workspace)         */
-  HBMM_PATH_POPC = 1,   /* XOR + __popc on the integer pipe, fp32 group-scale epilogue in registers;
+  HBMM_PATH_POPC = 1,   /* integer dots per group in registers (mma.sync on bytes, XOR + __popc for few
+                           rows and long groups), scaled in fp32;
                            HBWN: weight sign XOR-ed into fp32 activations on the fp32 pipe              */
   HBMM_PATH_B1MMA = 2,  /* legacy warp-level mma.sync: b1 xor.popc, beta multiple of 128;
                            HBWN: bf16 mma.sync with per-group partial sums (bf16 activations only)      */
@@ -193,7 +194,7 @@ hbmm_status hbmm_binarize_dense(const float *x, int64_t ldx, int64_t rows, int64
  * three bf16 pieces); 0 when no path needs scratch.  For products of few output tiles (fewer than about
  * a thousand tiles of 128 x 128 or 128 x 64 outputs) the packed x packed figure also holds the slots in
  * which CTAs that share a tile's K range exchange partial sums (up to 32 MB).  hbmm_gemm still works
- * without a workspace (NULL or too small): it then runs the integer-pipe path (HBMM) or the warp-level
+ * without a workspace (NULL or too small): it then runs HBMM_PATH_POPC (HBMM) or the warp-level
  * kernels (HBWN).  The workspace must be 16-byte aligned. */
 hbmm_status hbmm_gemm_workspace_bytes(const hbmm_operand *A, const hbmm_operand *W, size_t *bytes);
 

@@ -97,7 +97,7 @@ inline bool workspace_ok(const void* ws, size_t have, size_t need) {
   return need == 0 || (ws != nullptr && have >= need && (reinterpret_cast<uintptr_t>(ws) & 15u) == 0);
 }
 
-// The integer-pipe contraction that fits the operands: matrix-vector shaped, sub-word segments, or tiled.
+// The workspace-free contraction that fits the operands: matrix-vector shaped, sub-word segments, or tiled.
 cudaError_t popc_any(const PackedView& a, const PackedView& w, float* C, int64_t ldc, cudaStream_t stream) {
   if (gemv_popc_supported(a, w)) return launch_gemv_popc(a, w, C, ldc, stream);
   return gemm_popc_tile_supported(a, w) ? launch_gemm_popc_tile(a, w, C, ldc, stream) : launch_gemm_popc(a, w, C, ldc, stream);
@@ -170,7 +170,7 @@ hbmm_status gemm_checked(const hbmm_operand* A, const hbmm_operand* W, float* C,
       // of the tensor-core paths is 32 times larger than the packed one).  Not for sub-word groups where the folded kernel
       // can run: its expanded weights are what a prepared call with more rows may rely on.
       if (gemv_popc_supported(a, w) && !(fold && gemm_subword(a, w))) e = launch_gemv_popc(a, w, C, ldc, stream);
-      // the tensor-core paths need their workspace; without one the integer-pipe path runs
+      // the tensor-core paths need their workspace; without one the workspace-free path runs
       else if (fold)
         e = launch_gemm_fold(a, w, C, ldc, workspace, workspace_bytes, stream);
       else if (gemm_tensor_supported(a, w) && workspace_ok(workspace, workspace_bytes, tensor_workspace(a, w)))

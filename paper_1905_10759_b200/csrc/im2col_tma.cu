@@ -43,16 +43,11 @@ struct Plan {
 // One K-word of a full 32-channel chunk whose groups are shorter than a word: the packed word, and the word's SUB
 // group means stored straight to the operand's scale row (`dst`: the word's first scale).
 template <int SUB>
-__device__ __forceinline__ void gather_word_sub(int taps, bool flat, int w, uint32_t addr, uint32_t cs_bytes, uint32_t pitch_bytes,
+__device__ __forceinline__ void gather_word_sub(bool flat, int w, uint32_t addr, uint32_t cs_bytes, uint32_t pitch_bytes,
                                                 uint32_t pm, uint32_t& word, void* scales, int scale_bf16, int64_t idx, bool vec) {
   float sums[SUB];
-  if (taps == 9) {
-    if (flat) gather_word_dispatch_sub<3, 3, true, SUB>(w, addr, cs_bytes, pitch_bytes, pm, word, sums);
-    else gather_word_dispatch_sub<3, 3, false, SUB>(w, addr, cs_bytes, pitch_bytes, 0u, word, sums);
-  } else {
-    if (flat) gather_word_dispatch_sub<1, 1, true, SUB>(w, addr, cs_bytes, pitch_bytes, pm, word, sums);
-    else gather_word_dispatch_sub<1, 1, false, SUB>(w, addr, cs_bytes, pitch_bytes, 0u, word, sums);
-  }
+  if (flat) gather_word_dispatch_sub<3, 3, true, SUB>(w, addr, cs_bytes, pitch_bytes, pm, word, sums);
+  else gather_word_dispatch_sub<3, 3, false, SUB>(w, addr, cs_bytes, pitch_bytes, 0u, word, sums);
   constexpr float inv = static_cast<float>(SUB) / 32.0f;          // 1 / beta
 #pragma unroll
   for (int i = 0; i < SUB; i++) sums[i] *= inv;
@@ -248,16 +243,16 @@ im2col_quantize_tma_kernel(const __grid_constant__ CUtensorMap x_map, const floa
           float mean = 0.0f;
           const int word_abs = static_cast<int>(static_cast<int64_t>(ic.chunk_first) * kCC * taps / 32) + words_done + w;
           const int64_t m_pix = (static_cast<int64_t>(ic.b) * g.Ho + ic.yo0) * g.Wo + pix;
-          if (GROUPS == 1 && cc == kCC && (taps == 9 ? (g.kh == 3 && g.kw == 3) : taps == 1)) {
+          if (GROUPS == 1 && cc == kCC && g.kh == 3 && g.kw == 3) {
             // groups shorter than a word: the word's means go straight to the scale row
             const int64_t sidx = m_pix * ld_scales + static_cast<int64_t>(word_abs) * tp.sub;
             const uint32_t a = t_addr + po * 4;
             const bool vec = tp.vec_scales != 0;
             switch (tp.sub) {
-              case 2: gather_word_sub<2>(taps, tp.flat != 0, w, a, cs * 4, tp.pitch * 4, pm, word, scales, scale_bf16, sidx, vec); break;
-              case 4: gather_word_sub<4>(taps, tp.flat != 0, w, a, cs * 4, tp.pitch * 4, pm, word, scales, scale_bf16, sidx, vec); break;
-              case 8: gather_word_sub<8>(taps, tp.flat != 0, w, a, cs * 4, tp.pitch * 4, pm, word, scales, scale_bf16, sidx, vec); break;
-              default: gather_word_sub<16>(taps, tp.flat != 0, w, a, cs * 4, tp.pitch * 4, pm, word, scales, scale_bf16, sidx, vec); break;
+              case 2: gather_word_sub<2>(tp.flat != 0, w, a, cs * 4, tp.pitch * 4, pm, word, scales, scale_bf16, sidx, vec); break;
+              case 4: gather_word_sub<4>(tp.flat != 0, w, a, cs * 4, tp.pitch * 4, pm, word, scales, scale_bf16, sidx, vec); break;
+              case 8: gather_word_sub<8>(tp.flat != 0, w, a, cs * 4, tp.pitch * 4, pm, word, scales, scale_bf16, sidx, vec); break;
+              default: gather_word_sub<16>(tp.flat != 0, w, a, cs * 4, tp.pitch * 4, pm, word, scales, scale_bf16, sidx, vec); break;
             }
           } else if (GROUPS == 1) {
             // any filter size, short last chunk: group by group (the last group of the row may be short)
@@ -279,7 +274,7 @@ im2col_quantize_tma_kernel(const __grid_constant__ CUtensorMap x_map, const floa
             if (tp.flat) gather_word_dispatch<3, 3, true>(w, t_addr + po * 4, cs * 4, tp.pitch * 4, pm, word, sum);
             else gather_word_dispatch<3, 3, false>(w, t_addr + po * 4, cs * 4, tp.pitch * 4, 0u, word, sum);
             mean = GROUPS == 2 ? sum : sum * 0.03125f;
-          } else if (cc == kCC && taps == 1) {
+          } else if (GROUPS == 2 && cc == kCC && taps == 1) {      // groups of more words than the kernel for 1 x 1 filters takes
             float sum;
             if (tp.flat) gather_word_dispatch<1, 1, true>(w, t_addr + po * 4, cs * 4, tp.pitch * 4, pm, word, sum);
             else gather_word_dispatch<1, 1, false>(w, t_addr + po * 4, cs * 4, tp.pitch * 4, 0u, word, sum);
@@ -468,13 +463,13 @@ bool make_plan(const ConvGeom& g, int sms, bool flat, int32_t beta, Plan* out, s
 // overlap (256 x 28 x 28, 5 x 5: stride 2 0.6 .. 1.1, stride 8 1.3 .. 2.0), 7 x 7 at stride 2 (0.4 .. 1.3, large images 0.6; at
 // stride 4 1.0 .. 1.6), above not (11 x 11 1.4 .. 3.8).  Groups shorter than a word, whose gather has a thread per word: the
 // filters with a gather of their own (3 x 3 0.4 .. 1.2), 2 x 2 for as many words as leave that gather to its latency (0.6 .. 0.8;
-// above, or at stride 5, 1.1 .. 2.0), 5 x 5 not (1.4 .. 1.8), nor rows of less than a word (63 images of 8 x 56 x 56, 1 x 1 at stride 3: 2.2).
+// above, or at stride 5, 1.1 .. 2.0), 5 x 5 not (1.4 .. 1.8), nor rows of less than a word.
 bool stage_strided(const ConvGeom& g, int32_t beta) {
   const int taps = g.kh * g.kw;
   if (beta >= 32) return taps <= 9 || (taps <= 25 && g.sw < g.kw) || (taps <= 49 && 3 * g.sw <= g.kw);
   if (g.C * taps < 32) return false;
   const int64_t words = static_cast<int64_t>(g.B) * g.Ho * g.Wo * ((static_cast<int64_t>(g.C) * taps + 31) / 32);
-  return (g.kh == 3 && g.kw == 3) || taps == 1 || (taps <= 9 && g.sw <= 2 * g.kw && words <= 24576);
+  return (g.kh == 3 && g.kw == 3) || (taps <= 9 && g.sw <= 2 * g.kw && words <= 24576);
 }
 
 // 0: not supported, 1: tensor-copy tiles with halo, 2: flat channel planes
@@ -489,7 +484,7 @@ int tma_mode(const void* x, int x_bf16, const ConvGeom& g, int32_t beta) {
   if (current_device(&dev, &sms) != cudaSuccess) return 0;       // the plan's channel split follows the device's SM count
   if (g.W % 4 == 0 && encode_tiled_fn() != nullptr && make_plan(g, sms, false, beta, &p, &smem)) return 1;
   // small images whose rows are not multiples of 16 bytes: whole planes, masked 3x3 / 1x1 gather
-  const bool filt = (g.kh == 3 && g.kw == 3) || (g.kh == 1 && g.kw == 1);
+  const bool filt = (g.kh == 3 && g.kw == 3) || (g.kh == 1 && g.kw == 1 && beta >= 32);
   if (filt && g.C % kCC == 0 && (static_cast<int64_t>(g.C) * g.H * g.W) % 4 == 0 && make_plan(g, sms, true, beta, &p, &smem)) return 2;
   return 0;
 }

@@ -74,7 +74,7 @@ cudaError_t launch_partials_popc(const PackedView& A, const PackedView& W, int32
 bool gemv_popc_supported(const PackedView& A, const PackedView& W);
 cudaError_t launch_gemv_popc(const PackedView& A, const PackedView& W, float* C, int64_t ldc, cudaStream_t stream);
 
-// The same in 32 x 32 warp tiles with the K range split between warps: segments of 2, 4, 8, 16 bits or 1, 2, 4, 8 words.
+// The same in 32 x 32 warp tiles with the K range split between warps, the dots by mma.sync on bytes: segments of 2, 4, 8, 16 bits or 1, 2, 4, 8 words.
 bool gemm_popc_tile_supported(const PackedView& A, const PackedView& W);
 cudaError_t launch_gemm_popc_tile(const PackedView& A, const PackedView& W, float* C, int64_t ldc, cudaStream_t stream);
 
