@@ -74,6 +74,35 @@ def test_long_tiles_match_oracle(M, N, K, ba, bw):
     assert float(diff.norm() / P[:, :N].double().norm()) < 1e-5
 
 
+@pytest.mark.parametrize("M,N,K,ba,bw,sdt", [
+    (2900, 1001, 256, 32, 32, 0),     # 184 tiles of four stages
+    (4000, 700, 288, 32, 16, 1),      # 192 tiles, the last stage of one word, bf16 scales
+    (5000, 900, 224, 224, 32, 0),     # 320 tiles: three turns, one activation group per row
+    (2560, 1030, 928, 32, 32, 0),     # 15 stages: the longest taken whole at 180 tiles
+    (2560, 1030, 1024, 64, 32, 0),    # 16: the balanced schedule
+])
+def test_short_whole_tiles_match_oracle(M, N, K, ba, bw, sdt):
+    """Short 128-column tiles that are walked whole with the wide accumulator, and the first that are not."""
+    import gpu_util as gu
+    from paper_1905_10759_b200 import hbmm
+    a, w = inputs.normal((M, K), 4600 + M + K + ba), inputs.he_normal(N, K, 5600 + N + K + bw)
+    A, da, sa = gu.oracle_operand(a, ba, sdt)
+    W, dw, sw = gu.oracle_operand(w, bw, sdt)
+    ws = torch.empty(hbmm.gemm_workspace_bytes(A, W), dtype=torch.uint8, device="cuda")
+    C = torch.full((M, (N + 3) // 4 * 4 + 4), float("nan"), device="cuda")
+    D = torch.full_like(C, float("nan"))
+    hbmm.gemm_ex(A, W, C, hbmm.PATH_FOLDED, ws)
+    hbmm.gemm_ex(A, W, D, hbmm.PATH_FOLDED_PREPARED, ws)
+    assert torch.isnan(C[:, N:]).all() and torch.isnan(D[:, N:]).all() and torch.equal(C[:, :N], D[:, :N])
+    rows = list(range(0, M, 97)) + [M - 1]
+    ea, ew = gu.eff_beta(ba, K), gu.eff_beta(bw, K)
+    c_ref, absref = oracle.hbmm_from_quantized(da[rows], sa[rows], ea, dw, sw, ew)
+    fine = gu.elementwise_magnitude(da[rows], ea, dw, ew, K)
+    gu.assert_close_rel_absref(C[rows, :N].cpu().numpy(), c_ref, absref, 1e-5, "short whole tiles", fine)
+    hbmm.gemm_ex(A, W, D, hbmm.PATH_POPC)      # all the other rows: on the integer pipe, which the oracle holds to 1e-5 as well
+    assert float((C - D)[:, :N].double().norm() / D[:, :N].double().norm()) < 1e-5
+
+
 def test_tiles_walked_in_blocks_of_columns():
     """More expanded weights than the L2 keeps: every tile is still formed once (blocks of 11 columns, a last one of 10; row
     and column remainders).  Against the integer pipe, which the oracle holds to 1e-5 elsewhere."""
