@@ -20,7 +20,7 @@
 // What bounds it: the load / shuffle / shared-memory pipe (some 120 instructions per row of 32 channels, against 290 gathered
 // loads), then memory.  Against the staged tiles and the gathers it replaces, beta 32 unless said, us: 64 x 64 x 56 x 56
 // 48.1 -> 22.6 (bf16 119 -> 23.6); 64 x 128 x 28 x 28 29.3 -> 14.2, at beta 16 / 8 / 4 / 2 42.5 / 46.1 / 63.2 / 90.3 -> 20.0 /
-// 19.5 / 29.6 / 44.0; 64 x 256 x 14 x 14 17.5 -> 9.5; 20 x 192 x 55 x 55 at beta 2 434 -> 94; 16 x 100 x 27 x 27 bf16 at beta 16
+// 19.5 / 27.1 / 40.3; 64 x 256 x 14 x 14 17.5 -> 9.5; 20 x 192 x 55 x 55 at beta 2 434 -> 75; 16 x 100 x 27 x 27 bf16 at beta 16
 // 26.4 -> 11.1; one image of 512 x 7 x 7 4.1 -> 3.5.  The same at stride 2, two columns per lane, was level with the staged tiles
 // (32 x 64 x 56 x 56 12.0 against 12.3, one image of 512 x 7 x 7 3.5 against 5.5) and is not built.
 #include <cuda_bf16.h>
@@ -33,9 +33,9 @@ namespace hbmm {
 namespace {
 
 constexpr int kMaxWarps = 8;
-// Below this many warps an SM waits for its loads whatever their number (64 x 64 x 56 x 56: 40.3 us in segments of 14 rows, 8
-// warps per SM; 22.6 in segments of 7).
-constexpr double kLatencyWarps = 16.0;
+// Warps an SM holds at once (128 registers a thread).  A row takes a warp the same time whether 8 or 16 of them are there
+// (64 x 64 x 56 x 56: 40.3 us in segments of 14 rows, 8 warps per SM; 22.6 in segments of 7), so time goes in turns of 16.
+constexpr int kWarpsAtOnce = 16;
 
 // Channels a lane holds: a whole chunk of 32 where the registers take its groups' sums, else as few as leave whole bytes of
 // packed words (8 channels = 72 bits).
@@ -376,17 +376,19 @@ bool make_walk_plan(const ConvGeom& g, int32_t beta, int elem_bytes, int sms, in
   p.words = chunks * 9;
   p.groups = static_cast<int32_t>(p.gw > 1 ? chunks * 9 / p.gw : static_cast<int64_t>(chunks) * 288 / beta);
   if (p.ranges == 1) { p.words = static_cast<int32_t>(ld_words); p.groups = static_cast<int32_t>(ld_scales); }
-  // rows of a segment: every segment reads two rows more than it leaves, a CTA more than the machine holds costs
-  // a turn
-  double cost = 0.0;
+  // rows of a segment: every segment reads two rows more than it leaves, a CTA more than the machine holds costs a turn.  (With
+  // the warps per SM counted one by one instead of in turns, beta 32 unless said, us: 33 x 96 x 40 x 40 at beta 8 25.7 against
+  // 19.3, 20 x 192 x 55 x 55 at beta 2 94 / 75, 128 x 64 x 56 x 56 47.2 / 41.4, 100 x 256 x 14 x 14 15.1 / 12.6, 64 x 512 x 7 x 7
+  // 9.9 / 9.0, 64 x 128 x 28 x 28 at beta 4 29.9 / 27.1; none slower.)
+  int64_t cost = 0;
   for (int r = 1; r <= g.Ho; r++) {
     const int nseg = (g.Ho + r - 1) / r;
     if (r > 1 && (g.Ho + r - 2) / (r - 1) == nseg) continue;      // the same segments, less evenly
     const int64_t units = static_cast<int64_t>(g.B) * nseg * p.strips;
     const int64_t ctas = (units + p.sets * p.L - 1) / (p.sets * p.L) * p.ranges;
-    const double per_sm = static_cast<double>((ctas + sms - 1) / sms) * p.sets * p.pieces;
-    const double c = (r + 2) * (per_sm < kLatencyWarps ? kLatencyWarps : per_sm);
-    if (cost == 0.0 || c < cost) { cost = c; p.R = r; p.nseg = nseg; }
+    const int64_t at_once = static_cast<int64_t>(sms) * (kWarpsAtOnce / (p.sets * p.pieces));
+    const int64_t c = (r + 2) * ((ctas + at_once - 1) / at_once);
+    if (cost == 0 || c < cost) { cost = c; p.R = r; p.nseg = nseg; }
   }
   const int64_t units = static_cast<int64_t>(g.B) * p.nseg * p.strips;
   if (units >= (int64_t{1} << 28)) return false;
