@@ -499,7 +499,7 @@ hbmm_status conv_checked(const void* x, int32_t x_dtype, const hbmm_conv_geom* g
     if ((ep || prefer_fold(av, wv)) && L.gemm_bytes > 0 && L.gemm_bytes >= fold_workspace(av, wv) &&
         (walk || point || im2col_quantize_tma_supported(x, x_dtype == HBMM_BF16, cg, beta_a))) {
       UmmaPrepJob job{};
-      gemm_fold_prep_job(av, wv, gemm_ws, &job);
+      gemm_fold_prep_job(av, wv, gemm_ws, L.gemm_bytes, &job);
       if (job.n_stages * job.tiles_n <= 4096) {
         const UmmaPrepJob* expand = w_prepared ? nullptr : &job;
         const int s_bf16 = a_scale_dtype == HBMM_BF16;

@@ -39,6 +39,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <atomic>
+#include "fold_plan.h"
 #include "kernels.h"
 #include "split_choice.h"
 #include "tensor_map.h"
@@ -53,7 +54,6 @@ namespace {
 using namespace umma;
 using namespace fold;
 
-constexpr int kEpilogueWarps = 4;
 constexpr int kProducerWarps = 8;
 constexpr int kFirstProducerWarp = kEpilogueWarps;
 constexpr int kMmaWarp = kEpilogueWarps + kProducerWarps;   // 12
@@ -730,7 +730,7 @@ hbmm_fold_kernel(const Args g, const __grid_constant__ CUtensorMap s_map, const 
             }
             epi::finish_chunk(g.ep, cv, fs, fh, m, nb + c * 32, g.N, c == TN / 32 - 1, nb + TN, carry);
           }
-        } else if (SR::OUT_BUFS > 0 && ((g.N & 3) == 0 || nb + c * 32 + 32 <= g.N)) {
+        } else if (SR::OUT_BUFS > 0 && g.c_copy && ((g.N & 3) == 0 || nb + c * 32 + 32 <= g.N)) {
           // The block goes to shared memory (as the copy's 128-byte swizzle has it: eight rows, eight bank groups) and leaves by
           // a tensor copy, which drops what lies outside the matrix.  Sixteen bytes of a row per lane straight to the matrix
           // are 32 lines an instruction: a tile of 128 x 128 took 7400 clk that way.  (The copy clips a row to 16 bytes: the block in which
@@ -926,20 +926,14 @@ Args make_args(const PackedView& A, const PackedView& W, float* C, int64_t ldc) 
   g.a_staged = 0; g.a_rowmax = nullptr;
   g.split = 1;
   g.group_n = 0;
+  g.c_copy = 0;
   return g;
 }
 
-template <int TN>
-size_t stage_bytes(const Args& g) {
-  const int64_t tiles_n = (g.N + TN - 1) / TN, n_stages = (g.n_words + WPS - 1) / WPS;
-  return static_cast<size_t>(tiles_n * n_stages) * Smem<TN>::B_STAGE;
-}
-// Balanced schedule: worth its reduction traffic when the tiles are few waves of the machine and a tile's K walk is
-// long enough to cut.  The workspace is sized for any device of up to kMaxBalancedCtas multiprocessors.
-constexpr int64_t kMaxBalancedCtas = 256;
-constexpr int64_t kBalancedWaves = 4;
-constexpr int64_t kBalancedMinStages = 4;
-constexpr int64_t kBalancedMaxShare = 4;
+FoldShape shape_of(const Args& g, int tn) { return FoldShape{g.M, g.N, g.n_words, tn, g.a_sub > 1}; }
+static_assert(FoldShape::kRows == TM && FoldShape::kWords == WPS && Smem<64>::B_STAGE == 64 * FoldShape::kRowBytes &&
+              Smem<128>::B_STAGE == 128 * FoldShape::kRowBytes, "the plan counts the kernel's tiles and stages");
+
 std::atomic<int> g_resident_clusters[64][kMaxSplit + 1];        // per device, see choose_split
 // 128-column tiles: the wide accumulator from this many stages per tile on.  Its epilogue is exposed at the end of every tile
 // but a CTA's last, so that the line lies further out the more tiles a CTA walks and the slower they leave it.  Wide over
@@ -954,55 +948,16 @@ constexpr int64_t kWideFromStages = 20, kWideFromManyTiles = 30, kWideFromSlowRo
 // (2.49 / 2.51 / 2.53), 4096^3 (67 MB) 304 -> 289 us.  Below, the L2 holds them whatever the order.
 constexpr size_t kWeightsInL2 = size_t{48} << 20;
 constexpr size_t kBlockBytes = size_t{18} << 20;
-template <int TN>
-int64_t tile_count(const Args& g) { return ((g.M + TM - 1) / TM) * ((g.N + TN - 1) / TN); }
-template <int TN>
-bool balanced_possible(const Args& g, int64_t sms) {
-  const int64_t n_stages = (g.n_words + WPS - 1) / WPS;
-  return sms <= kMaxBalancedCtas && n_stages >= kBalancedMinStages && tile_count<TN>(g) < kBalancedWaves * sms;
-}
-template <int TN>
-size_t balanced_bytes(const Args& g) {
-  if (!balanced_possible<TN>(g, kMaxBalancedCtas)) return 0;
-  const int64_t n_stages = (g.n_words + WPS - 1) / WPS, units = tile_count<TN>(g) * n_stages;
-  const int64_t ctas = units < kMaxBalancedCtas ? units : kMaxBalancedCtas;
-  const size_t counters = (static_cast<size_t>(tile_count<TN>(g)) * kEpilogueWarps * sizeof(int32_t) + 255) / 256 * 256;
-  return counters + static_cast<size_t>(2 * ctas) * TM * TN * sizeof(float);
-}
-// The arrival counters take the first kCounterCount words of the area, for the most tiles a balanced launch may have, so
-// that they lie at the same place and are all zeroed by whichever call expands the weights, whatever its number of rows:
-// prepared calls with more and fewer rows follow it.  (Sized for the call's own tiles, they lay under another call's partial
-// tiles.)  The area holds them without being larger: of its min(units, 256) pairs of slots a launch uses at most
-// min(units / kBalancedMinStages, kMaxBalancedCtas - 1), and one pair is four times the counters.
-constexpr int64_t kCounterCount = kBalancedWaves * kMaxBalancedCtas * kEpilogueWarps;
-static_assert(2 * TM * 64 * sizeof(float) >= kCounterCount * sizeof(int32_t), "a pair of slots holds the counters");
-// [W stages][one float per weight row][counters][partial slots]
-template <int TN>
-size_t down_offset(const Args& g) { return stage_bytes<TN>(g); }
-template <int TN>
-size_t balanced_offset(const Args& g) {
-  return (stage_bytes<TN>(g) + static_cast<size_t>((g.N + TN - 1) / TN) * TN * sizeof(float) + 255) / 256 * 256;
-}
-// ... then, for activation groups shorter than a word, one float per activation row (its largest scale)
-template <int TN>
-size_t rowmax_offset(const Args& g) { return (balanced_offset<TN>(g) + balanced_bytes<TN>(g) + 255) / 256 * 256; }
-template <int TN>
-size_t prep_bytes(const Args& g) {
-  return g.a_sub > 1 ? rowmax_offset<TN>(g) + static_cast<size_t>(g.M) * sizeof(float) : balanced_offset<TN>(g) + balanced_bytes<TN>(g);
-}
-// Points the argument block at the balanced schedule's part of the workspace.  A product with too many tiles for it has no
-// such part; its counters are zeroed all the same where the caller's workspace reaches that far (`have` bytes), for prepared
-// calls with fewer rows.
+// Points the argument block at the balanced schedule's part of the workspace, as far as there is one.
 template <int TN>
 void set_balanced_area(Args& g, void* workspace, size_t have) {
-  const bool reserved = balanced_bytes<TN>(g) != 0;
-  const int64_t n_stages = (g.n_words + WPS - 1) / WPS;
-  const size_t at = balanced_offset<TN>(g), counters = kCounterCount * sizeof(int32_t);
-  if (!reserved && (g.a_sub > 1 || n_stages < kBalancedMinStages || have < at + counters)) return;
-  unsigned char* area = static_cast<unsigned char*>(workspace) + at;
-  g.sk_counters = reinterpret_cast<int32_t*>(area);
-  g.sk_counter_count = kCounterCount;
-  if (reserved) g.sk_partials = reinterpret_cast<float*>(area + counters);
+  const FoldArea area = fold_area(shape_of(g, TN), have);
+  unsigned char* base = static_cast<unsigned char*>(workspace);
+  if (area.counters) {
+    g.sk_counters = reinterpret_cast<int32_t*>(base + area.at);
+    g.sk_counter_count = kCounterCount;
+  }
+  if (area.slots) g.sk_partials = reinterpret_cast<float*>(base + area.slots_at);
 }
 
 // Clusters of `size` CTAs of the kernel that the current device holds at once.
@@ -1043,35 +998,6 @@ void launch_prepare(const Args& g, unsigned char* stages, float* down, int sms, 
   }
 }
 
-// Equal runs of (tile, stage) pairs, one per CTA: they pay when they shorten the longest CTA's walk by a tenth or more.
-struct Runs { int64_t run, ctas, walk; bool pay; };
-template <int TN>
-Runs balanced_runs(const Args& g, int64_t sms) {
-  Runs r{};
-  const int64_t n_stages = (g.n_words + WPS - 1) / WPS, tiles = tile_count<TN>(g), units = tiles * n_stages;
-  r.ctas = units / kBalancedMinStages < sms ? units / kBalancedMinStages : sms;
-  if (r.ctas > kMaxBalancedCtas - 1) r.ctas = kMaxBalancedCtas - 1;
-  if (r.ctas < 1) r.ctas = 1;
-  r.run = (units + r.ctas - 1) / r.ctas;
-  // a tile is shared by at most kBalancedMaxShare + 1 CTAs: the CTA that completes it adds the others' partial
-  // accumulators one after the other, which costs more than the shorter walk saves beyond that
-  const int64_t min_run = (n_stages + kBalancedMaxShare - 1) / kBalancedMaxShare;
-  if (r.run < min_run) r.run = min_run;
-  r.walk = (tiles + sms - 1) / sms * n_stages;
-  r.pay = balanced_possible<TN>(g, sms) && r.run * 10 <= r.walk * 9;
-  r.ctas = (units + r.run - 1) / r.run;                     // no CTA without work
-  return r;
-}
-// Whole short 128-column tiles with the wide accumulator instead of the balanced schedule of narrow ones, whose reduction costs
-// some 9 us.  In hundredths of a us: a stage 46 of a whole tile, 42 of a run, a turn's exposed epilogue 150.  Balanced / whole
-// wide, us: 25088 x 128 x 576 21.4 / 17.3, 12544 x 128 x 1152 19.7 / 15.5, 4096 x 960 x 256 21.0 / 13.5, 1000 x 3000 x 640 27.3 /
-// 18.3, 50176 x 128 x 576 27.0 / 24.0; level at 12544 x 256 x 1152, slower at 50176 x 128 x 1152 (34.4 / 35.6) and 2048 x 4096 x
-// 768 (40.9 / 45.2).  The error against 64 bits falls to a third.  (Whole narrow tiles take 14.8 us of the first, but sum all of
-// K in one accumulator with the small products: 6.5e-7 balanced, 7.7e-7 narrow, 2.3e-7 wide.)
-inline bool whole_wide_pays(const Runs& r, int64_t n_stages) {
-  return r.pay && 46 * r.walk + 150 * (r.walk / n_stages) < 900 + 42 * r.run;
-}
-
 template <int TN, int ASUB, bool FUSE, bool WIDE>
 cudaError_t launch_fold_wide(Args g, void* workspace, size_t have, cudaStream_t stream, bool w_prepared) {
   using S = Smem<TN>;
@@ -1095,9 +1021,10 @@ cudaError_t launch_fold_wide(Args g, void* workspace, size_t have, cudaStream_t 
     }
     configured.mark(dev);
   }
-  const int64_t tiles_n = (g.N + TN - 1) / TN, n_stages = (g.n_words + WPS - 1) / WPS;
+  const FoldShape shape = shape_of(g, TN);
+  const int64_t n_stages = shape.stages(), tiles = shape.tiles();
   unsigned char* stages = static_cast<unsigned char*>(workspace);
-  float* down = reinterpret_cast<float*>(stages + stage_bytes<TN>(g));
+  float* down = reinterpret_cast<float*>(stages + shape.weight_bytes());
   set_balanced_area<TN>(g, workspace, have);
   if (!w_prepared) launch_prepare<TN>(g, stages, down, sms, stream);
   g.w_prep = stages;
@@ -1123,12 +1050,11 @@ cudaError_t launch_fold_wide(Args g, void* workspace, size_t have, cudaStream_t 
   g.a_rowmax = nullptr;
   if (ASUB > 1 && !g.a_bf16 && g.lda_s % 4 == 0 && g.lda_s >= kRowMaxFrom && reinterpret_cast<uintptr_t>(g.a_scales) % 16 == 0) {
     // many scales per row: reduce the rows to their largest scale in a kernel of its own, at streaming bandwidth
-    g.a_rowmax = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + rowmax_offset<TN>(g));
+    g.a_rowmax = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + rowmax_offset(shape));
     const cudaError_t e = launch_pdl(row_max_kernel, dim3(static_cast<unsigned>((g.M + 7) / 8)), dim3(256), 0, stream,
                                      reinterpret_cast<const float*>(g.a_scales), g.lda_s, g.M, g.a_rowmax);
     if (e != cudaSuccess) return e;
   }
-  const int64_t tiles = ((g.M + TM - 1) / TM) * tiles_n;
   CUtensorMap c_map = {};
   if constexpr (!FUSE) {
     // (all instantiations take a whole SM per CTA, so they share what was asked once)
@@ -1140,26 +1066,25 @@ cudaError_t launch_fold_wide(Args g, void* workspace, size_t have, cudaStream_t 
                                 static_cast<unsigned>(split), kBytes, stream, g, s_map, c_map);
     }
   }
-  if (!FUSE && ScaleRing<TN, ASUB>::OUT_BUFS > 0) {
-    // the product as a 2-D tensor for the epilogue's copies: 32 x 32 blocks
+  if (!FUSE && ScaleRing<TN, ASUB>::OUT_BUFS > 0 && copies_reach(shape)) {
+    // the product as a 2-D tensor for the epilogue's copies: 32 x 32 blocks (not a row pitch that such a tensor cannot have)
     EncodeTiledFn fn = encode_tiled_fn();
     const cuuint64_t dims[2] = {static_cast<cuuint64_t>(g.N), static_cast<cuuint64_t>(g.M)};
     const cuuint64_t strides[1] = {static_cast<cuuint64_t>(g.ldc) * 4};
     const cuuint32_t box[2] = {32, 32};
     const cuuint32_t elem[2] = {1, 1};
-    if (!fn || fn(&c_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, g.C, dims, strides, box, elem, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaErrorNotSupported;
+    g.c_copy = fn && fn(&c_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, g.C, dims, strides, box, elem, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
   }
   if (kHasBalanced && !(WIDE && n_stages < kWideFromStages)) {
-    const Runs runs = balanced_runs<TN>(g, sms);
+    const Runs runs = balanced_runs(shape, sms, have);
     if (runs.pay) {
       g.sk_units = runs.run;
       return launch_pdl(hbmm_fold_kernel<TN, ASUB, FUSE, kHasBalanced ? kBalanced : kPlain, WIDE>, dim3(static_cast<unsigned>(runs.ctas)), dim3(kThreads), kBytes, stream, g, s_map, c_map);
     }
   }
   const unsigned grid = static_cast<unsigned>(tiles < sms ? tiles : sms);   // one persistent CTA per SM
-  if (WIDE && stage_bytes<TN>(g) > kWeightsInL2) {
+  if (WIDE && shape.weight_bytes() > kWeightsInL2) {
     g.group_n = static_cast<int64_t>(kBlockBytes / (static_cast<size_t>(n_stages) * S::B_STAGE));
     if (g.group_n < 1) g.group_n = 1;
   }
@@ -1171,12 +1096,13 @@ cudaError_t launch_fold(const Args& g, void* workspace, size_t have, cudaStream_
   if constexpr (TN == 128) {
     int dev = 0, sms = 0;
     if (current_device(&dev, &sms) != cudaSuccess) return cudaErrorInvalidDevice;
-    const int64_t n_stages = (g.n_words + WPS - 1) / WPS, tiles = tile_count<TN>(g);
+    const FoldShape shape = shape_of(g, TN);
+    const int64_t n_stages = shape.stages(), tiles = shape.tiles();
     const bool vector_rows = g.ep.mode == kEpiDense && reinterpret_cast<uintptr_t>(g.ep.out) % 16 == 0 &&
                              g.ep.ld_out * (g.ep.out_bf16 ? 2 : 4) % 16 == 0;
     const int64_t from = FUSE && tiles > sms ? (vector_rows ? kWideFromManyTiles : kWideFromSlowRows)
                                              : (tiles > 2 * static_cast<int64_t>(sms) ? kWideFromManyTiles : kWideFromStages);
-    const bool whole = !FUSE && ASUB == 1 && n_stages < from && n_stages < kWideFromStages && whole_wide_pays(balanced_runs<TN>(g, sms), n_stages);
+    const bool whole = !FUSE && ASUB == 1 && n_stages < from && n_stages < kWideFromStages && whole_wide_pays(balanced_runs(shape, sms, have), n_stages);
     if (n_stages >= from || whole) return launch_fold_wide<TN, ASUB, FUSE, true>(g, workspace, have, stream, w_prepared);
   }
   return launch_fold_wide<TN, ASUB, FUSE, false>(g, workspace, have, stream, w_prepared);
@@ -1211,7 +1137,7 @@ bool gemm_fold_supported(const PackedView& A, const PackedView& W) {
 // Bytes of workspace: the weight operand as fp16 piece tiles (4 bytes per element) + one float per row.
 size_t gemm_fold_workspace_bytes(const PackedView& A, const PackedView& W) {
   const Args g = make_args(A, W, nullptr, 0);
-  return g.N <= 64 ? prep_bytes<64>(g) : prep_bytes<128>(g);
+  return fold_bytes(shape_of(g, g.N <= 64 ? 64 : 128));
 }
 
 // workspace: device, 16-byte aligned, at least gemm_fold_workspace_bytes.
@@ -1224,35 +1150,22 @@ bool gemm_fold_next_supported(int64_t N, int32_t beta_next) {
 
 cudaError_t launch_gemm_fold(const PackedView& A, const PackedView& W, float* C, int64_t ldc, void* workspace, size_t workspace_bytes,
                              cudaStream_t stream, bool w_prepared, const EpiArgs* ep) {
-  // the copies that store the product take 32-bit row numbers
-  constexpr int64_t kMostRows = int64_t{1} << 30;
-  if (!ep && A.rows > kMostRows) {
-    PackedView part = A;
-    for (int64_t m = 0; m < A.rows; m += kMostRows) {
-      part.bits = A.bits + m * A.ld_words;
-      part.scales = static_cast<const char*>(A.scales) + m * A.ld_scales * (A.scale_bf16 ? 2 : 4);
-      part.rows = A.rows - m < kMostRows ? A.rows - m : kMostRows;
-      const cudaError_t e = launch_gemm_fold(part, W, C + m * ldc, ldc, workspace, workspace_bytes, stream, w_prepared || m > 0, nullptr);
-      if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-  }
   Args g = make_args(A, W, C, ldc);
   if (ep) g.ep = *ep;
   return g.N <= 64 ? launch_fold_tn<64>(g, workspace, workspace_bytes, stream, w_prepared) : launch_fold_tn<128>(g, workspace, workspace_bytes, stream, w_prepared);
 }
 
 // The weight expansion of launch_gemm_fold(A, W, ..., workspace) as a job for another kernel.
-void gemm_fold_prep_job(const PackedView& A, const PackedView& W, void* workspace, UmmaPrepJob* job) {
+void gemm_fold_prep_job(const PackedView& A, const PackedView& W, void* workspace, size_t workspace_bytes, UmmaPrepJob* job) {
   job->f = make_args(A, W, nullptr, 0);
   job->folded = 1;
   job->out = static_cast<unsigned char*>(workspace);
   job->tn = job->f.N <= 64 ? 64 : 128;
-  const int64_t n_stages = (job->f.n_words + WPS - 1) / WPS;
-  job->n_stages = static_cast<int32_t>((n_stages + kPrepStages - 1) / kPrepStages);    // tasks per column tile
-  job->tiles_n = static_cast<int32_t>((job->f.N + job->tn - 1) / job->tn);
-  job->out_down = reinterpret_cast<float*>(job->out + (job->tn == 64 ? stage_bytes<64>(job->f) : stage_bytes<128>(job->f)));
-  if (job->tn == 64) set_balanced_area<64>(job->f, workspace, 0); else set_balanced_area<128>(job->f, workspace, 0);
+  const FoldShape shape = shape_of(job->f, job->tn);
+  job->n_stages = static_cast<int32_t>((shape.stages() + kPrepStages - 1) / kPrepStages);    // tasks per column tile
+  job->tiles_n = static_cast<int32_t>(shape.tiles_n());
+  job->out_down = reinterpret_cast<float*>(job->out + shape.weight_bytes());
+  if (job->tn == 64) set_balanced_area<64>(job->f, workspace, workspace_bytes); else set_balanced_area<128>(job->f, workspace, workspace_bytes);
 }
 
 cudaError_t launch_wait_expiry_selftest(cudaStream_t stream) {

@@ -143,6 +143,7 @@ struct FoldArgs {
   int64_t group_n;               // column tiles per block of the plain schedule's walk; 0: row by row over all columns
   int32_t split;                 // CTAs (one cluster) that share a tile's K range in split mode
   int32_t a_staged;              // sub-word groups: the activation scales of a stage reach the producers through shared memory
+  int32_t c_copy;                // finished blocks of the product leave by tensor copies
 };
 // The weight expansion as a job another kernel can run: n_stages x tiles_n tasks of tn threads each
 // (n_stages counts tasks per column tile: single stages of the e4m3 layout, runs of stages of the folded one).
@@ -183,7 +184,7 @@ cudaError_t launch_gemm_fold(const PackedView& A, const PackedView& W, float* C,
                              cudaStream_t stream, bool w_prepared = false, const EpiArgs* ep = nullptr);
 // Group sizes the fused epilogue can emit for an output of N columns.
 bool gemm_fold_next_supported(int64_t N, int32_t beta_next);
-void gemm_fold_prep_job(const PackedView& A, const PackedView& W, void* workspace, UmmaPrepJob* job);
+void gemm_fold_prep_job(const PackedView& A, const PackedView& W, void* workspace, size_t workspace_bytes, UmmaPrepJob* job);
 
 // Dense x packed contraction (HBWN), three kernels:
 //   select : sign bit XOR-ed into fp32 activations on the fp32 pipe (any dense dtype);

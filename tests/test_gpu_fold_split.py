@@ -103,6 +103,20 @@ def test_short_whole_tiles_match_oracle(M, N, K, ba, bw, sdt):
     assert float((C - D)[:, :N].double().norm() / D[:, :N].double().norm()) < 1e-5
 
 
+def test_row_pitch_that_no_tensor_copy_takes():
+    """One row whose pitch (2^38 elements) is beyond a tensor copy's: the blocks leave by plain stores, with the same values."""
+    import gpu_util as gu
+    from paper_1905_10759_b200 import hbmm
+    N, K = 103, 256
+    A, _, _ = gu.oracle_operand(inputs.normal((1, K), 4700), 32, 0)
+    W, _, _ = gu.oracle_operand(inputs.he_normal(N, K, 5700), 32, 0)
+    ws = torch.empty(hbmm.gemm_workspace_bytes(A, W), dtype=torch.uint8, device="cuda")
+    C, D = torch.full((1, 108), float("nan"), device="cuda"), torch.full((1, 108), float("nan"), device="cuda")
+    hbmm.gemm_ex(A, W, C, hbmm.PATH_FOLDED, ws)
+    hbmm.gemm_ex(A, W, D.as_strided((1, 108), (1 << 38, 1)), hbmm.PATH_FOLDED_PREPARED, ws)
+    assert torch.equal(C[:, :N], D[:, :N]) and torch.isnan(C[:, N:]).all() and torch.isnan(D[:, N:]).all()
+
+
 def test_tiles_walked_in_blocks_of_columns():
     """More expanded weights than the L2 keeps: every tile is still formed once (blocks of 11 columns, a last one of 10; row
     and column remainders).  Against the integer pipe, which the oracle holds to 1e-5 elsewhere."""
