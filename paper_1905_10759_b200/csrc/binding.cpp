@@ -19,6 +19,7 @@ decltype(&hbmm_conv_im2col_fused) f_conv_fused;
 decltype(&hbmm_binarize_dense) f_dense;
 decltype(&hbmm_binarize_backward) f_backward;
 PyObject* g_error;                 // HbmmError
+PyTypeObject *t_operand, *t_geom, *t_epilogue;      // the ctypes structures that stand for hbmm_operand, hbmm_conv_geom, hbmm_epilogue
 PyObject *s_desc, *s_cuda_stream;
 
 // Arguments of a METH_FASTCALL | METH_KEYWORDS call in the order of `names`; absent ones stay null.
@@ -85,16 +86,20 @@ bool small_integer(PyObject* o, int32_t* v) {
   *v = static_cast<int32_t>(w);               // as ctypes passes it on
   return true;
 }
-// The bytes behind a ctypes structure.
+// The bytes behind a ctypes structure, of the type it is declared as and no other: what they hold is taken for sizes and addresses.
 template <typename T>
 struct Struct {
   Py_buffer view{};
   const T* p = nullptr;
   ~Struct() { if (view.obj) PyBuffer_Release(&view); }
-  bool open(PyObject* o) {
+  bool open(PyObject* o, PyTypeObject* type) {
+    if (!PyObject_TypeCheck(o, type)) {
+      PyErr_Format(PyExc_TypeError, "%s expected, got %s", type->tp_name, Py_TYPE(o)->tp_name);
+      return false;
+    }
     if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) return false;
     if (view.len < static_cast<Py_ssize_t>(sizeof(T))) {
-      PyErr_SetString(PyExc_TypeError, "a structure of the wrong type");
+      PyErr_Format(PyExc_TypeError, "%s is shorter than the library's", type->tp_name);
       return false;
     }
     p = static_cast<const T*>(view.buf);
@@ -103,7 +108,7 @@ struct Struct {
   bool open_desc(PyObject* operand) {
     PyObject* d = PyObject_GetAttr(operand, s_desc);
     if (!d) return false;
-    const bool ok = open(d);
+    const bool ok = open(d, t_operand);
     Py_DECREF(d);                             // the view holds it
     return ok;
   }
@@ -168,7 +173,7 @@ PyObject* py_quantize(PyObject*, PyObject* const* args, Py_ssize_t nargs, PyObje
   void *p, *s;
   int32_t dt;
   Struct<hbmm_operand> out;
-  if (!device_ptr(*x, &p) || !dtype_code(*x, &dt) || !out.open_desc(a[1]) || !stream_of(a[2], &s)) return nullptr;
+  if (!out.open_desc(a[1]) || !device_ptr(*x, &p) || !dtype_code(*x, &dt) || !stream_of(a[2], &s)) return nullptr;
   const int64_t rows = x->size(0), K = x->size(1), ld = x->stride(0);
   HBMM_CALL(f_quantize(p, dt, rows, K, ld, out.p, s));
   return done(status, "hbmm_quantize", a[1]);
@@ -222,8 +227,8 @@ PyObject* py_conv_im2col(PyObject*, PyObject* const* args, Py_ssize_t nargs, PyO
   Struct<hbmm_conv_geom> geom;
   Struct<hbmm_operand> W;
   Buffer ws;
-  if (!device_ptr(*x, &p) || !dtype_code(*x, &dt) || !geom.open(a[1]) || !small_integer(a[2], &beta) || !small_integer(a[3], &sdt) ||
-      !W.open_desc(a[4]) || (a[8] && !integer(a[8], &flags)))
+  if (!geom.open(a[1], t_geom) || !W.open_desc(a[4]) || !device_ptr(*x, &p) || !dtype_code(*x, &dt) || !small_integer(a[2], &beta) ||
+      !small_integer(a[3], &sdt) || (!none(a[8]) && !integer(a[8], &flags)))
     return nullptr;
   if (!none(a[5])) {
     const at::Tensor* C = tensor_of(a[5]);
@@ -254,8 +259,8 @@ PyObject* py_conv_im2col_fused(PyObject*, PyObject* const* args, Py_ssize_t narg
   Struct<hbmm_operand> W;
   Struct<hbmm_epilogue> ep;
   Buffer ws;
-  if (!device_ptr(*x, &p) || !dtype_code(*x, &dt) || !geom.open(a[1]) || !small_integer(a[2], &beta) || !small_integer(a[3], &sdt) ||
-      !W.open_desc(a[4]) || !ep.open(a[5]) || !ws.open(a[6]) || !stream_of(a[7], &s) || (a[8] && !integer(a[8], &flags)))
+  if (!geom.open(a[1], t_geom) || !W.open_desc(a[4]) || !ep.open(a[5], t_epilogue) || !device_ptr(*x, &p) || !dtype_code(*x, &dt) ||
+      !small_integer(a[2], &beta) || !small_integer(a[3], &sdt) || !ws.open(a[6]) || !stream_of(a[7], &s) || (a[8] && !integer(a[8], &flags)))
     return nullptr;
   HBMM_CALL(f_conv_fused(p, dt, geom.p, beta, sdt, W.p, ep.p, ws.p, ws.bytes, static_cast<uint32_t>(flags), s));
   return done(status, "hbmm_conv_im2col_fused", Py_None);
@@ -334,11 +339,13 @@ PyObject* py_binarize_dense(PyObject*, PyObject* const* args, Py_ssize_t nargs, 
   END_HANDLE_TH_ERRORS
 }
 
-// connect(HbmmError, addresses of the C functions in the order of the f_ pointers above)
+// connect(HbmmError, hbmm_operand, hbmm_conv_geom, hbmm_epilogue, addresses of the C functions in the order of the f_ pointers above)
 PyObject* py_connect(PyObject*, PyObject* args) {
-  PyObject* err;
+  PyObject *err, *types[3];
   unsigned long long p[7];
-  if (!PyArg_ParseTuple(args, "OKKKKKKK", &err, &p[0], &p[1], &p[2], &p[3], &p[4], &p[5], &p[6])) return nullptr;
+  if (!PyArg_ParseTuple(args, "OO!O!O!KKKKKKK", &err, &PyType_Type, &types[0], &PyType_Type, &types[1], &PyType_Type, &types[2], &p[0], &p[1],
+                        &p[2], &p[3], &p[4], &p[5], &p[6]))
+    return nullptr;
   f_quantize = reinterpret_cast<decltype(f_quantize)>(p[0]);
   f_gemm = reinterpret_cast<decltype(f_gemm)>(p[1]);
   f_gemm_ex = reinterpret_cast<decltype(f_gemm_ex)>(p[2]);
@@ -348,6 +355,11 @@ PyObject* py_connect(PyObject*, PyObject* args) {
   f_backward = reinterpret_cast<decltype(f_backward)>(p[6]);
   Py_INCREF(err);
   Py_XSETREF(g_error, err);
+  PyTypeObject** const held[] = {&t_operand, &t_geom, &t_epilogue};
+  for (int i = 0; i < 3; i++) {
+    Py_INCREF(types[i]);
+    Py_XSETREF(*held[i], reinterpret_cast<PyTypeObject*>(types[i]));
+  }
   Py_RETURN_NONE;
 }
 

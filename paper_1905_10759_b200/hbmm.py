@@ -57,6 +57,16 @@ class hbmm_conv_geom(ctypes.Structure):
                 ("B", "C", "H", "W", "kh", "kw", "stride_h", "stride_w", "pad_h", "pad_w")]
 
 
+class hbmm_epilogue(ctypes.Structure):
+    _fields_ = [
+        ("activation", ctypes.c_int32), ("out_kind", ctypes.c_int32),
+        ("bn_scale", ctypes.c_void_p), ("bn_shift", ctypes.c_void_p),
+        ("out", ctypes.c_void_p), ("ld_out", ctypes.c_int64),
+        ("out_dtype", ctypes.c_int32), ("reserved", ctypes.c_int32),
+        ("next", ctypes.POINTER(hbmm_operand)),
+    ]
+
+
 _i32, _i64, _vp, _sz = ctypes.c_int32, ctypes.c_int64, ctypes.c_void_p, ctypes.c_size_t
 _P = ctypes.POINTER
 _lib.hbmm_operand_bytes.argtypes = [_i64, _i64, _i32, _i32, _P(_sz), _P(_sz), _P(_i64), _P(_i64)]
@@ -90,7 +100,7 @@ class HbmmError(RuntimeError):
 
 # The calls a program makes once per layer and pass are native functions (csrc/binding.cpp: the marshalling took a third of a
 # small call's host time); the rest of this file marshals in Python.
-_binding.connect(HbmmError, *(ctypes.cast(getattr(_lib, _n), ctypes.c_void_p).value for _n in (
+_binding.connect(HbmmError, hbmm_operand, hbmm_conv_geom, hbmm_epilogue, *(ctypes.cast(getattr(_lib, _n), ctypes.c_void_p).value for _n in (
     "hbmm_quantize", "hbmm_gemm", "hbmm_gemm_ex", "hbmm_conv_im2col_ex", "hbmm_conv_im2col_fused", "hbmm_binarize_dense",
     "hbmm_binarize_backward")))
 quantize = _binding.quantize
@@ -319,16 +329,6 @@ def bench_alu_rate(kind: int, blocks: int, iters: int, sink: torch.Tensor, strea
     ops = _i64(0)
     _check(_lib.hbmm_bench_alu_rate(kind, blocks, iters, _dev_ptr(sink), ctypes.byref(ops), _stream(stream)), "hbmm_bench_alu_rate")
     return int(ops.value)
-
-
-class hbmm_epilogue(ctypes.Structure):
-    _fields_ = [
-        ("activation", ctypes.c_int32), ("out_kind", ctypes.c_int32),
-        ("bn_scale", ctypes.c_void_p), ("bn_shift", ctypes.c_void_p),
-        ("out", ctypes.c_void_p), ("ld_out", ctypes.c_int64),
-        ("out_dtype", ctypes.c_int32), ("reserved", ctypes.c_int32),
-        ("next", ctypes.POINTER(hbmm_operand)),
-    ]
 
 
 _lib.hbmm_gemm_fused.argtypes = [_P(hbmm_operand), _P(hbmm_operand), _P(hbmm_epilogue), _vp, _sz, _vp]

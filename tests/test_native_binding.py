@@ -37,8 +37,36 @@ def test_signatures():
     (lambda x, op: hbmm.quantize(x, op, x=x), TypeError, "multiple values"),
     (lambda x, op: hbmm.gemm(op, op, x, ws=None), TypeError, "unexpected"),
     (lambda x, op: hbmm.quantize([1.0], op), TypeError, "Tensor"),
+    (lambda x, op: hbmm.conv_im2col(x, hbmm.make_geom(1, 1, 2, 32, 1, 1), 32, hbmm.F32, op, x, x, flags=None), ValueError, "device tensor"),
 ])
 def test_errors_before_the_library(call, error, text):
     x = torch.ones((2, 32))
     with pytest.raises(error, match=text):
         call(x, hbmm.alloc_operand(2, 32, 32, device="cpu"))
+
+
+GEOM, EP, OPERAND = hbmm.make_geom(1, 1, 2, 32, 1, 1), hbmm.hbmm_epilogue(), hbmm.hbmm_operand()
+
+
+@pytest.mark.parametrize("desc", [GEOM, EP, bytes(256), bytearray(256), None])
+def test_operands_of_another_type(desc):
+    x, bad = torch.ones((2, 32)), hbmm.Operand(desc)
+    good = hbmm.alloc_operand(2, 32, 32, device="cpu")
+    for call in (lambda: hbmm.quantize(x, bad), lambda: hbmm.gemm(bad, good, x), lambda: hbmm.gemm(good, bad, x),
+                 lambda: hbmm.gemm_ex(good, bad, x, hbmm.PATH_AUTO), lambda: hbmm.conv_im2col(x, GEOM, 32, hbmm.F32, bad, x, x),
+                 lambda: hbmm.conv_im2col_fused(x, GEOM, 32, hbmm.F32, bad, EP, x)):
+        with pytest.raises(TypeError, match="hbmm_operand expected"):
+            call()
+
+
+@pytest.mark.parametrize("other", [OPERAND, bytes(256), (1, 1, 2, 32, 1, 1, 1, 1, 0, 0)])
+def test_geometries_and_epilogues_of_another_type(other):
+    x, op = torch.ones((2, 32)), hbmm.alloc_operand(2, 32, 32, device="cpu")
+    for geom in (other, EP):
+        with pytest.raises(TypeError, match="hbmm_conv_geom expected"):
+            hbmm.conv_im2col(x, geom, 32, hbmm.F32, op, x, x)
+        with pytest.raises(TypeError, match="hbmm_conv_geom expected"):
+            hbmm.conv_im2col_fused(x, geom, 32, hbmm.F32, op, EP, x)
+    for ep in (other, GEOM):
+        with pytest.raises(TypeError, match="hbmm_epilogue expected"):
+            hbmm.conv_im2col_fused(x, GEOM, 32, hbmm.F32, op, ep, x)
