@@ -30,19 +30,37 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-def is_stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(BINDING):
+def _older(target: str, deps) -> bool:
+    return not os.path.exists(target) or any(os.path.getmtime(d) > os.path.getmtime(target) for d in deps)
+
+
+def lib_is_stale() -> bool:
+    return _older(LIB, sources() + [f for e in ("*.h", "*.cuh") for f in glob.glob(os.path.join(CSRC, e))] + glob.glob(os.path.join(INCLUDE, "*.h")))
+
+
+def built_for() -> str:
+    """What the binding is compiled against; the module carries it as BUILT_FOR."""
+    import torch
+    return "torch %s, Python %s" % (torch.__version__, sysconfig.get_config_var("SOABI"))
+
+
+def binding_is_stale() -> bool:
+    if _older(BINDING, glob.glob(os.path.join(CSRC, "*.cpp")) + glob.glob(os.path.join(INCLUDE, "*.h"))):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cpp")) + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
-        glob.glob(os.path.join(INCLUDE, "*.h"))
-    return any(os.path.getmtime(d) > t for d in deps)
+    with open(BINDING, "rb") as f:
+        return built_for().encode() + b"\0" not in f.read()
 
 
 def build_lib(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ into libhbmm.so (one object per file, in parallel)."""
-    if not force and not is_stale():
-        return LIB
+    """Compile what is out of date: libhbmm.so from every .cu under csrc/ (one object per file, in parallel), and the binding."""
+    if force or lib_is_stale():
+        _build_cuda(verbose)
+    if force or binding_is_stale():
+        build_binding()
+    return LIB
+
+
+def _build_cuda(verbose: bool) -> None:
     nvcc = _nvcc()
     objdir = os.path.join(HERE, "_build")
     os.makedirs(objdir, exist_ok=True)
@@ -63,9 +81,7 @@ def build_lib(force: bool = False, verbose: bool = False) -> str:
             raise RuntimeError("nvcc failed on %s" % src)
     tmp = LIB + ".tmp.%d" % os.getpid()
     subprocess.check_call([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", tmp] + objs)
-    build_binding()
     os.replace(tmp, LIB)
-    return LIB
 
 
 def build_binding() -> None:
@@ -75,7 +91,7 @@ def build_binding() -> None:
     tmp = BINDING + ".tmp.%d" % os.getpid()
     include = ext.include_paths("cuda") + [sysconfig.get_paths()["include"], INCLUDE]
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", os.path.join(CSRC, "binding.cpp"), "-o", tmp]
-    cmd += ["-D_GLIBCXX_USE_CXX11_ABI=%d" % torch.compiled_with_cxx11_abi()]
+    cmd += ["-D_GLIBCXX_USE_CXX11_ABI=%d" % torch.compiled_with_cxx11_abi(), '-DHBMM_BUILT_FOR="%s"' % built_for()]
     cmd += [a for d in include for a in ("-isystem", d)] + ["-L" + d for d in ext.library_paths("cuda")]
     subprocess.check_call(cmd + ["-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
     os.replace(tmp, BINDING)

@@ -393,5 +393,7 @@ PyMODINIT_FUNC PyInit__binding() {
   s_desc = PyUnicode_InternFromString("desc");
   s_cuda_stream = PyUnicode_InternFromString("cuda_stream");
   if (!s_desc || !s_cuda_stream) return nullptr;
-  return PyModule_Create(&module_def);
+  PyObject* m = PyModule_Create(&module_def);
+  if (m && PyModule_AddStringConstant(m, "BUILT_FOR", HBMM_BUILT_FOR) != 0) Py_CLEAR(m);
+  return m;
 }

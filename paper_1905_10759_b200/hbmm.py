@@ -24,7 +24,16 @@ if not os.path.exists(LIB_PATH):
 
 _lib = ctypes.CDLL(LIB_PATH)
 
-from . import _binding  # noqa: E402  (native marshalling of the hot calls; built beside the library)
+from .build import built_for  # noqa: E402
+
+try:
+    from . import _binding  # noqa: E402  (native marshalling of the hot calls; built beside the library)
+except ImportError as e:
+    raise ImportError("_binding.so is missing or does not load (%s); build it with `python -m paper_1905_10759_b200.build` "
+                      "or __graft_entry__.build()" % e) from e
+if _binding.BUILT_FOR != built_for():      # another torch lays its tensors out as it likes
+    raise ImportError("_binding.so is built for %s, this is %s; build it again with `python -m paper_1905_10759_b200.build` "
+                      "or __graft_entry__.build()" % (_binding.BUILT_FOR, built_for()))
 
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_ALIGNMENT, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT = range(7)
 F32, BF16 = 0, 1

@@ -1,11 +1,15 @@
-"""The native entry points (csrc/binding.cpp): arguments by position and by keyword, and the errors raised before anything
-reaches the library (no GPU needed)."""
+"""The native entry points (csrc/binding.cpp): arguments by position and by keyword, the errors raised before anything reaches
+the library, and what a binding that is missing or of another torch says (no GPU needed)."""
 import inspect
+import os
+import shutil
+import subprocess
+import sys
 
 import pytest
 import torch
 
-from paper_1905_10759_b200 import hbmm
+from paper_1905_10759_b200 import build, hbmm
 
 
 def test_signatures():
@@ -70,3 +74,32 @@ def test_geometries_and_epilogues_of_another_type(other):
     for ep in (other, GEOM):
         with pytest.raises(TypeError, match="hbmm_epilogue expected"):
             hbmm.conv_im2col_fused(x, GEOM, 32, hbmm.F32, op, ep, x)
+
+
+def import_copy(where, change):
+    """Imports a copy of the package whose _binding.so has been changed; the error it ends with."""
+    pkg = where / "paper_1905_10759_b200"
+    pkg.mkdir()
+    for f in ("__init__.py", "hbmm.py", "build.py", "libhbmm.so", "_binding.so"):
+        src = os.path.join(build.HERE, f)
+        (os.symlink if f == "libhbmm.so" else shutil.copy)(src, pkg / f)
+    change(pkg / "_binding.so")
+    run = subprocess.run([sys.executable, "-c", "import paper_1905_10759_b200.hbmm"], cwd=where, capture_output=True, text=True)
+    assert run.returncode != 0
+    return run.stderr.strip().splitlines()[-1]
+
+
+def test_missing_or_foreign_binding(tmp_path):
+    hint = "python -m paper_1905_10759_b200.build"
+    for name, change, text in (("a", os.remove, "missing or does not load"), ("b", lambda p: p.write_bytes(b"no library"), "missing or does not load"),
+                               ("c", lambda p: p.write_bytes(p.read_bytes().replace(build.built_for().encode(), build.built_for().encode()[::-1])), "is built for")):
+        where = tmp_path / name
+        where.mkdir()
+        error = import_copy(where, change)
+        assert error.startswith("ImportError: _binding.so") and text in error and hint in error
+
+
+def test_binding_of_another_torch_is_stale(monkeypatch):
+    assert not build.binding_is_stale()
+    monkeypatch.setattr(torch, "__version__", "0.0")
+    assert build.binding_is_stale() and not build.lib_is_stale()
