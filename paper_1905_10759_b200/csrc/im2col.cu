@@ -6,6 +6,7 @@
 // variant writes bf16 rows for the HBWN mode.
 #include <cuda_bf16.h>
 #include "kernels.h"
+#include "im2col_gather.cuh"
 
 namespace hbmm {
 namespace {
@@ -376,7 +377,12 @@ im2col_quantize_tiled_kernel(const void* __restrict__ x, int x_bf16, const ConvG
       const unsigned short* o = off + k_begin;
       uint32_t word = 0;
       float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-      if (nk == 32) {
+      if (cc == kTileCC && g.kh == 3 && g.kw == 3) {
+        // 3 x 3 filters that the kernel of im2col_walk.cu does not take (stride over the rows, wide padding): constant offsets
+        // instead of the table.  Table / constant, us, bf16: 8 x 64 x 56 x 56 with padding 3 30.7 / 28.3, at stride 2 over the rows
+        // 33 x 192 x 28 x 28 55.4 / 51.6, 33 x 128 x 55 x 55 118.9 / 113.4, 64 x 256 x 14 x 14 40.3 / 38.8.
+        gather_word_dispatch<3, 3>(w, static_cast<uint32_t>(__cvta_generic_to_shared(base)), tp.rows_in * tp.span * 4, tp.span * 4, 0u, word, s0);
+      } else if (nk == 32) {
 #pragma unroll
         for (int e = 0; e < 32; e += 4) {
           const float v0 = base[o[e]], v1 = base[o[e + 1]], v2 = base[o[e + 2]], v3 = base[o[e + 3]];

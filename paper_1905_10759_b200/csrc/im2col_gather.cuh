@@ -1,5 +1,5 @@
 // Inner loop of the packed convolution front end for a full 32-channel chunk whose filter size is
-// known at compile time (the staged tiles of im2col_tma.cu).
+// known at compile time (the staged tiles of im2col_tma.cu and im2col.cu).
 #pragma once
 #include <cstdint>
 

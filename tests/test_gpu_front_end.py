@@ -27,15 +27,29 @@ CASES = [
 
 @pytest.mark.parametrize("B,C,H,W,k,st,beta,bf16", CASES)
 def test_packed_rows_match_oracle(B, C, H, W, k, st, beta, bf16):
+    packed_rows(B, C, H, W, k, (st, st), k // 2, beta, bf16)
+
+
+@pytest.mark.parametrize("B,C,H,W,sh,pad,bf16", [
+    (2, 64, 9, 13, 2, 1, True),           # stride over the rows only
+    (1, 40, 7, 10, 1, 3, True),           # wide padding, short last channel chunk
+    (1, 33, 11, 6, 2, 0, False),          # a chunk of one channel
+])
+def test_tiles_with_constant_offsets_match_oracle(B, C, H, W, sh, pad, bf16):
+    """3 x 3 filters at beta 32 that neither the walked columns nor the tensor copies take."""
+    packed_rows(B, C, H, W, 3, (sh, 1), pad, 32, bf16)
+
+
+def packed_rows(B, C, H, W, k, st, pad, beta, bf16):
     import gpu_util as gu
     from paper_1905_10759_b200 import hbmm
-    K, pad = C * k * k, k // 2
+    K = C * k * k
     x = inputs.normal((B * C * H, W), 650 + C + H).reshape(B, C, H, W)
     if bf16:
         x = torch.from_numpy(x).bfloat16().float().numpy()
     Wop = hbmm.quantize(torch.from_numpy(inputs.he_normal(40, K, 651)).cuda(), hbmm.alloc_operand(40, K, max(beta, 32)))
-    geom = hbmm.make_geom(B, C, H, W, k, k, (st, st), (pad, pad))
-    M = B * ((H + 2 * pad - k) // st + 1) * ((W + 2 * pad - k) // st + 1)
+    geom = hbmm.make_geom(B, C, H, W, k, k, st, (pad, pad))
+    M = B * ((H + 2 * pad - k) // st[0] + 1) * ((W + 2 * pad - k) // st[1] + 1)
     ws = torch.empty(hbmm.conv_workspace_bytes(geom, beta, hbmm.F32, Wop), dtype=torch.uint8, device="cuda").fill_(0xAB)
     xd = torch.from_numpy(x).cuda()
     hbmm.conv_im2col(xd.bfloat16() if bf16 else xd, geom, beta, hbmm.F32, Wop, None, ws, flags=hbmm.CONV_PACK_ONLY)
@@ -43,7 +57,7 @@ def test_packed_rows_match_oracle(B, C, H, W, k, st, beta, bf16):
     bits = ws[:bb].view(torch.int32).reshape(M, lw)
     off = (bb + 255) // 256 * 256
     sc = ws[off: off + sb].view(torch.float32).reshape(M, ls).cpu().numpy().astype(np.float64)
-    da, sa = oracle.quantize(oracle.im2col(x, k, k, (st, st), (pad, pad)), beta)
+    da, sa = oracle.quantize(oracle.im2col(x, k, k, st, (pad, pad)), beta)
     assert np.array_equal(gu.host_bits(bits), oracle.pack(sa, lw))
     G = da.shape[1]
     assert np.all(sc[:, G:] == 0.0)
