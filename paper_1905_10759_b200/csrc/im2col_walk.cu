@@ -19,9 +19,9 @@
 //
 // What bounds it: the load / shuffle / shared-memory pipe (some 120 instructions per row of 32 channels, against 290 gathered
 // loads), then memory.  Against the staged tiles and the gathers it replaces, beta 32 unless said, us: 64 x 64 x 56 x 56
-// 48.1 -> 22.6 (bf16 119 -> 23.6); 64 x 128 x 28 x 28 29.3 -> 14.2, at beta 16 / 8 / 4 / 2 42.5 / 46.1 / 63.2 / 90.3 -> 20.0 /
-// 19.5 / 27.1 / 40.3; 64 x 256 x 14 x 14 17.5 -> 9.5; 20 x 192 x 55 x 55 at beta 2 434 -> 75; 16 x 100 x 27 x 27 bf16 at beta 16
-// 26.4 -> 11.1; one image of 512 x 7 x 7 4.1 -> 3.5.  The same at stride 2, two columns per lane, was level with the staged tiles
+// 48.1 -> 22.6 (bf16 119 -> 23.6); 64 x 128 x 28 x 28 29.3 -> 14.2, at beta 16 / 8 / 4 / 2 42.9 / 46.3 / 63.4 / 90.3 -> 15.5 /
+// 18.8 / 27.5 / 40.3; 64 x 256 x 14 x 14 17.5 -> 9.5; 20 x 192 x 55 x 55 at beta 2 434 -> 75; 16 x 100 x 27 x 27 bf16 at beta 16
+// 26.4 -> 7.5; one image of 512 x 7 x 7 4.1 -> 3.5.  The same at stride 2, two columns per lane, was level with the staged tiles
 // (32 x 64 x 56 x 56 12.0 against 12.3, one image of 512 x 7 x 7 3.5 against 5.5) and is not built.
 #include <cuda_bf16.h>
 #include "kernels.h"
@@ -37,9 +37,10 @@ constexpr int kMaxWarps = 8;
 // (64 x 64 x 56 x 56: 40.3 us in segments of 14 rows, 8 warps per SM; 22.6 in segments of 7), so time goes in turns of 16.
 constexpr int kWarpsAtOnce = 16;
 
-// Channels a lane holds: a whole chunk of 32 where the registers take its groups' sums, else as few as leave whole bytes of
-// packed words (8 channels = 72 bits).
-__host__ __device__ constexpr int channels_for(int beta) { return beta >= 16 ? 32 : (beta == 8 ? 16 : 8); }
+// Channels a lane holds: a whole chunk of 32 where its groups are those of whole words (nine), else as few as leave whole bytes
+// of packed words (8 channels = 72 bits) and two groups per channel or fewer.  At beta 16, 32 / 16 channels, us: 64 x 128 x 28 x
+// 28 20.2 / 15.5, 64 x 64 x 56 x 56 35.5 / 27.8, 8 x 48 x 16 x 16 6.9 / 3.5, one image of 512 x 7 x 7 5.5 / 3.7.
+__host__ __device__ constexpr int channels_for(int beta) { return beta >= 32 ? 32 : (beta >= 8 ? 16 : 8); }
 
 struct FastDiv {
   uint32_t d, magic;             // quotients of numbers below 2^16 by d below 2^16
@@ -87,7 +88,10 @@ template <> __device__ __forceinline__ float load_elem<__nv_bfloat16>(const char
   return __uint_as_float(static_cast<uint32_t>(v) << 16);
 }
 
-template <int BETA, typename T>
+// LIVE: no channel beyond it in any lane.  An image of fewer channels than a lane holds spent the time of a full chunk on them,
+// more than the tiles and gathers before it.  Those / all channels / LIVE of them, us: 8 x 8 x 56 x 56 at beta 32 4.6 / 7.4 /
+// 3.1, 33 x 20 x 28 x 28 at beta 96 7.5 / 8.9 / 7.2, 64 x 16 x 7 x 7 bf16 at beta 16 7.8 / 9.8 / 3.5.
+template <int BETA, int LIVE, typename T>
 __global__ void __launch_bounds__(kMaxWarps * 32, 2)
 im2col_walk_kernel(const T* __restrict__ x, const ConvGeom g, const WalkPlan p, const FastDiv by_bits, const FastDiv by_scales,
                    const __grid_constant__ UmmaPrepJob prep, int n_prep, uint32_t* __restrict__ bits, int64_t ld_words,
@@ -162,12 +166,12 @@ im2col_walk_kernel(const T* __restrict__ x, const ConvGeom g, const WalkPlan p, 
 #pragma unroll
     for (int c = 0; c < CH; c++) v[c] = 0.0f;
     if (col_ok && r >= 0 && r < g.H) {
-      if (nch == CH) {
+      if (LIVE == CH && nch == CH) {
 #pragma unroll
         for (int c = 0; c < CH; c++) v[c] = load_elem<T>(xb + static_cast<size_t>(c) * plane_bytes + off);
       } else {
 #pragma unroll
-        for (int c = 0; c < CH; c++)
+        for (int c = 0; c < LIVE; c++)
           if (c < nch) v[c] = load_elem<T>(xb + static_cast<size_t>(c) * plane_bytes + off);
       }
     }
@@ -187,6 +191,7 @@ im2col_walk_kernel(const T* __restrict__ x, const ConvGeom g, const WalkPlan p, 
       const uint32_t le = bl & m4, lo = (bl >> 4) & m4, ce = (bo & m4) << 1, co = (bo >> 3) & (m4 << 1), re = (br & m4) << 2, ro = (br >> 2) & (m4 << 2);
 #pragma unroll
       for (int q = 0; q < Q; q++) {
+        if (4 * q >= LIVE) { h[q] = 0u; continue; }
         const uint32_t sel = 0x1111u * (q >> 1);
         uint32_t o = __byte_perm((q & 1) ? lo : le, 0, sel) & 0x08040201u;
         o |= __byte_perm((q & 1) ? co : ce, 0, sel) & 0x10080402u;
@@ -208,7 +213,7 @@ im2col_walk_kernel(const T* __restrict__ x, const ConvGeom g, const WalkPlan p, 
         bool any = false;
 #pragma unroll
         for (int c = 0; c < BETA; c++)
-          if (C::whole(c) && C::group(c, 0) == q) { col = any ? col + fabsf(v[u * BETA + c]) : fabsf(v[u * BETA + c]); any = true; }
+          if (C::whole(c) && C::group(c, 0) == q && u * BETA + c < LIVE) { col = any ? col + fabsf(v[u * BETA + c]) : fabsf(v[u * BETA + c]); any = true; }
         if (any) {
           const float s = (__shfl_up_sync(0xFFFFFFFFu, col, 1) + col) + __shfl_down_sync(0xFFFFFFFFu, col, 1);
           add(0, u * 9 + q, s); add(1, u * 9 + q, s); add(2, u * 9 + q, s);
@@ -216,7 +221,7 @@ im2col_walk_kernel(const T* __restrict__ x, const ConvGeom g, const WalkPlan p, 
       }
 #pragma unroll
       for (int c = 0; c < BETA; c++) {
-        if (C::whole(c)) continue;
+        if (C::whole(c) || u * BETA + c >= LIVE) continue;
         const float m = v[u * BETA + c], l = __shfl_up_sync(0xFFFFFFFFu, m, 1), rr = __shfl_down_sync(0xFFFFFFFFu, m, 1);
         const float lm = fabsf(l) + fabsf(m), mr = fabsf(m) + fabsf(rr), all = lm + fabsf(rr);
 #pragma unroll
@@ -267,8 +272,16 @@ im2col_walk_kernel(const T* __restrict__ x, const ConvGeom g, const WalkPlan p, 
       if constexpr (CH == 32) {
 #pragma unroll
         for (int q = 0; q < 9; q++) {
-          if (nch == CH) sb[piece * 9 + q] = wd[q];
+          if (LIVE == CH && nch == CH) sb[piece * 9 + q] = wd[q];
           else if (32 * q < valid) sb[piece * 9 + q] = valid - 32 * q >= 32 ? wd[q] : wd[q] & ((1u << (valid - 32 * q)) - 1u);
+        }
+      } else if constexpr (CH == 16) {
+        unsigned short* by = reinterpret_cast<unsigned short*>(sb) + piece * 9;
+#pragma unroll
+        for (int q = 0; q < 9; q++) {
+          const uint32_t o = (wd[q >> 1] >> (16 * (q & 1))) & 0xFFFFu;
+          if (LIVE == CH && nch == CH) by[q] = static_cast<unsigned short>(o);
+          else if (16 * q < valid) by[q] = static_cast<unsigned short>(valid - 16 * q >= 16 ? o : o & ((1u << (valid - 16 * q)) - 1u));
         }
       } else {
         unsigned char* by = reinterpret_cast<unsigned char*>(sb) + piece * (9 * CH / 8);
@@ -280,13 +293,18 @@ im2col_walk_kernel(const T* __restrict__ x, const ConvGeom g, const WalkPlan p, 
         }
       }
       const float inv = p.gw > 1 ? 1.0f : 1.0f / BETA;      // groups of several words are divided when their words are added
-      if (nch == CH) {
+      if (LIVE == CH && nch == CH) {
 #pragma unroll
         for (int q = 0; q < G; q++) ss[q] = fin[q] * inv;
       } else {
+        float last = 0.0f;       // of the row's short last group
 #pragma unroll
-        for (int q = 0; q < G; q++)
-          if (BETA * q < valid) ss[q] = p.gw > 1 || valid - BETA * q >= BETA ? fin[q] * inv : fin[q] / static_cast<float>(valid - BETA * q);
+        for (int q = 0; q < (9 * LIVE + BETA - 1) / BETA; q++) {
+          if (BETA * (q + 1) <= valid) ss[q] = fin[q] * inv;
+          else if (BETA * q < valid) last = fin[q];
+        }
+        const int n = valid % BETA;
+        if (n != 0) ss[valid / BETA] = p.gw > 1 ? last : last / static_cast<float>(n);
       }
     }
 #pragma unroll
@@ -405,12 +423,12 @@ bool make_walk_plan(const ConvGeom& g, int32_t beta, int elem_bytes, int sms, in
   return walk_smem_bytes(p) <= 100 * 1024;
 }
 
-template <int BETA, typename T>
-cudaError_t launch_walk(const void* x, const ConvGeom& g, WalkPlan p, const UmmaPrepJob* prep, uint32_t* bits, int64_t ld_words, void* scales,
+template <int BETA, int LIVE, typename T>
+cudaError_t launch_walk_live(const void* x, const ConvGeom& g, WalkPlan p, const UmmaPrepJob* prep, uint32_t* bits, int64_t ld_words, void* scales,
                                int64_t ld_scales, int scale_bf16, int dev, cudaStream_t stream) {
   static DeviceOnce configured;
   if (configured.pending(dev)) {
-    const cudaError_t e = cudaFuncSetAttribute(im2col_walk_kernel<BETA, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+    const cudaError_t e = cudaFuncSetAttribute(im2col_walk_kernel<BETA, LIVE, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
     if (e != cudaSuccess) return e;
     configured.mark(dev);
   }
@@ -427,8 +445,22 @@ cudaError_t launch_walk(const void* x, const ConvGeom& g, WalkPlan p, const Umma
   const FastDiv by_bits = FastDiv::make(p.vec_bits ? (p.max_words + 3) / 4 : p.max_words);
   const FastDiv by_scales = FastDiv::make(p.vec_scales ? (p.max_groups + 3) / 4 : p.max_groups);
   const int64_t ctas = (static_cast<int64_t>(p.n_units) + p.sets * p.L - 1) / (p.sets * p.L) * p.ranges;
-  return launch_pdl(im2col_walk_kernel<BETA, T>, dim3(static_cast<unsigned>(ctas + n_prep)), dim3(static_cast<unsigned>(p.sets * p.pieces * 32)),
+  return launch_pdl(im2col_walk_kernel<BETA, LIVE, T>, dim3(static_cast<unsigned>(ctas + n_prep)), dim3(static_cast<unsigned>(p.sets * p.pieces * 32)),
                     walk_smem_bytes(p), stream, static_cast<const T*>(x), g, p, by_bits, by_scales, job, n_prep, bits, ld_words, scales, ld_scales, scale_bf16);
+}
+
+// The kernel for as few channels as the image has.
+template <int BETA, typename T, typename... Rest>
+cudaError_t launch_walk(const void* x, const ConvGeom& g, Rest... rest) {
+  constexpr int CH = channels_for(BETA);
+  if constexpr (CH >= 16) {
+    if (g.C <= 8) return launch_walk_live<BETA, 8, T>(x, g, rest...);
+  }
+  if constexpr (CH == 32) {
+    if (g.C <= 16) return launch_walk_live<BETA, 16, T>(x, g, rest...);
+    if (g.C <= 24) return launch_walk_live<BETA, 24, T>(x, g, rest...);
+  }
+  return launch_walk_live<BETA, CH, T>(x, g, rest...);
 }
 
 template <typename T>

@@ -23,6 +23,16 @@ CASES = [
     (1, 256, 13, 13, 1, 256, False, True), # a group of eight words spans four chunks
     (1, 96, 3, 90, 1, 96, True, False),    # groups of three words
     (5, 20, 2, 1, 1, 16, False, False),    # one input column
+    (2, 8, 6, 9, 1, 32, False, False),     # images of fewer channels than a lane holds: all of 8,
+    (1, 7, 5, 8, 1, 16, True, False),      # ... 7 of 8,
+    (2, 16, 6, 9, 1, 32, True, True),      # 16,
+    (1, 9, 5, 7, 2, 64, False, False),     # 9 of 16, a short group of two words,
+    (2, 24, 6, 9, 1, 96, False, False),    # 24,
+    (1, 17, 9, 9, 1, 32, False, False),    # 17 of 24
+    (2, 3, 7, 7, 1, 16, False, False),
+    (1, 3, 5, 5, 0, 16, False, True),      # K = 27: a short second group
+    (2, 25, 6, 9, 1, 32, False, False),    # ... and one channel more: all 32
+    (1, 130, 6, 9, 1, 16, False, False),   # two channel ranges at beta 16, the last of two channels
 ]
 
 
