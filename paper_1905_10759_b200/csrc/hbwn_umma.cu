@@ -1016,6 +1016,12 @@ Args make_conv_args(const ConvGeom& c, const PackedView& W, float* C, int64_t ld
 // (26 / 52 tiles for 74 pairs) 16.0 / 12.9, 784 x 128 x 1152 11.0 / 8.3, 11760 x 192 x 1728 (92 / 138) 21.7 / 17.9; 50176 x 128 x
 // 1152 (196 / 392) 23.6 / 32.1, 6272 x 256 x 1728 (50 / 100) 14.2 / 17.3, 7840 x 256 x 1152 (62 / 124) 11.9 / 13.7.
 constexpr int64_t kWideStage = 512, kWideTile = 2500, kNarrowStage = 375, kNarrowTile = 1500;
+// The most narrow tiles of a product of few rows.  All its CTAs ask the L2 for the same few lines at the same time, and with one CTA
+// per 128 columns, which is what it takes else, there are half as many of them.  Wide / narrow, us (mean over placements, which
+// count for up to 40 % here), K = 1984: 1 row, N = 1000 / 2000 / 3000 13.4 / 10.3, 13.4 / 14.1, 13.4 / 17.6; 4 rows, N = 2000 /
+// 3000 / 4600 13.4 / 10.2, 13.4 / 13.9, 14.0 / 14.7; 33 rows, N = 3000 / 4600 13.4 / 13.7, 14.0 / 15.5; from 64 rows on narrow
+// wherever the turns below say so.
+inline int64_t narrow_limit(int64_t rows) { return rows < 4 ? 16 : rows < 64 ? 32 : INT64_MAX; }
 
 // prep_rows: rows of the prepared weight pieces' matrix.
 template <int TN, int NP>
@@ -1087,7 +1093,7 @@ cudaError_t launch(Args g, const CUtensorMap& a_map, void* workspace, cudaStream
     if (sms >= 2) {
       const int64_t tiles_m = (g.M + 2 * TM - 1) / (2 * TM), pairs = sms / 2;
       const auto turns = [&](int64_t tiles) { return (tiles + pairs - 1) / pairs; };
-      const bool narrow = !(g.ep.mode == kEpiPacked && g.ep.nx_beta > 64) &&
+      const bool narrow = (g.N + 63) / 64 <= narrow_limit(g.M) && !(g.ep.mode == kEpiPacked && g.ep.nx_beta > 64) &&
                           turns(tiles_m * ((g.N + 63) / 64)) * (n_kb * kNarrowStage + kNarrowTile) < turns(tiles_m * tiles_n) * (n_kb * kWideStage + kWideTile);
       if (narrow) return launch_pair<64, NP>(g, a_map, o_map, tiles_n * n_kb * NP * TN, dev, pairs, stream);
       if (g.M > TM) return launch_pair<TN, NP>(g, a_map, o_map, tiles_n * n_kb * NP * TN, dev, pairs, stream);

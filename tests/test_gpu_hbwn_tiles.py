@@ -72,3 +72,23 @@ def test_tiles_match_oracle(B, C, H, N, kind, extra):
     assert (out[:, N:] == 7.0).all()
     got = out[:, :N].float().cpu().numpy().astype(np.float64)
     assert (np.abs(got - z) <= band + (2.0 ** -8 * np.abs(z) if kind == "bf16" else 0.0) + 1e-12).all()
+
+
+@pytest.mark.parametrize("M,N", [(1, 1024), (1, 1025), (3, 1100), (4, 1025), (5, 2048), (5, 2049), (63, 2100), (64, 2100)])
+def test_few_rows_match_oracle(M, N):
+    """One row tile, at the limits of rows and columns between narrow tiles of CTA pairs and one CTA per 128 columns."""
+    import gpu_util as gu
+    from paper_1905_10759_b200 import hbmm
+    K, beta = 128, 32
+    a = torch.from_numpy(inputs.normal((M, K), 8400 + N)).bfloat16()
+    w = inputs.he_normal(N, K, 8500 + N)
+    A, W = hbmm.wrap_dense(a.cuda()), hbmm.quantize(torch.from_numpy(w).cuda(), hbmm.alloc_operand(N, K, beta))
+    ws = torch.empty(hbmm.gemm_workspace_bytes(A, W), dtype=torch.uint8, device="cuda").fill_(0xFF)
+    C = torch.full((M, (N + 3) // 4 * 4 + 4), float("nan"), device="cuda")
+    hbmm.gemm_ex(A, W, C, hbmm.PATH_FOLDED, ws)
+    dw, sw = oracle.quantize(w, beta)
+    wb = np.repeat(dw, beta, axis=1)[:, :K] * sw
+    x = a.float().numpy().astype(np.float64)
+    tol = (K + 4) * gu.U * (np.abs(x) @ np.abs(wb).T) + 2.0 ** -18 * (np.abs(x) @ np.abs(wb).T)
+    assert (np.abs(C[:, :N].cpu().numpy() - x @ wb.T) <= tol).all() and torch.isnan(C[:, N:]).all()
+    assert hbmm.last_device_error() == 0
