@@ -25,10 +25,6 @@ struct PointArgs {
   int32_t vec;                         // a word's scales are stored as vectors
 };
 
-__device__ __forceinline__ float load_elem(const float* p) { return __ldg(p); }
-__device__ __forceinline__ float load_elem(const __nv_bfloat16* p) {
-  return __uint_as_float(static_cast<uint32_t>(__ldg(reinterpret_cast<const unsigned short*>(p))) << 16);
-}
 __device__ __forceinline__ void store_one(void* scales, int bf16, int64_t idx, float v) {
   if (bf16) reinterpret_cast<__nv_bfloat16*>(scales)[idx] = __float2bfloat16_rn(v);
   else reinterpret_cast<float*>(scales)[idx] = v;
@@ -65,10 +61,10 @@ im2col_point_kernel(const T* __restrict__ x, const ConvGeom g, const PointArgs p
     float v[32];
     if (nk == 32 && inside) {
 #pragma unroll
-      for (int e = 0; e < 32; e++) v[e] = load_elem(pc + e * plane);
+      for (int e = 0; e < 32; e++) v[e] = load_elem<T>(pc + e * plane);
     } else {
 #pragma unroll
-      for (int e = 0; e < 32; e++) v[e] = inside && e < nk ? load_elem(pc + e * plane) : 0.0f;
+      for (int e = 0; e < 32; e++) v[e] = inside && e < nk ? load_elem<T>(pc + e * plane) : 0.0f;
     }
     uint32_t pat = 0;
 #pragma unroll

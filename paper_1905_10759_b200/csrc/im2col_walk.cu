@@ -75,19 +75,6 @@ struct Cut {
   __host__ __device__ static constexpr bool whole(int c) { return group(c, 0) == group(c, 8); }
 };
 
-// (volatile: the next row's loads stay where they are written, ahead of the barrier and the stores of this one)
-template <typename T> __device__ __forceinline__ float load_elem(const char* p);
-template <> __device__ __forceinline__ float load_elem<float>(const char* p) {
-  float v;
-  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
-  return v;
-}
-template <> __device__ __forceinline__ float load_elem<__nv_bfloat16>(const char* p) {
-  unsigned short v;
-  asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p));
-  return __uint_as_float(static_cast<uint32_t>(v) << 16);
-}
-
 // LIVE: no channel beyond it in any lane.  An image of fewer channels than a lane holds spent the time of a full chunk on them,
 // more than the tiles and gathers before it.  Those / all channels / LIVE of them, us: 8 x 8 x 56 x 56 at beta 32 4.6 / 7.4 /
 // 3.1, 33 x 20 x 28 x 28 at beta 96 7.5 / 8.9 / 7.2, 64 x 16 x 7 x 7 bf16 at beta 16 7.8 / 9.8 / 3.5.

@@ -10,13 +10,30 @@
 // hbmm_gemm on 3 rows of 2057 x 5248 6.6 instead of 4.4; with the wait alone all of them are at or below a plain launch.
 // The quantizer signals after its wait, for the set-up of the contraction behind it (2 % of that pair).
 #pragma once
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <cstdint>
 #include <utility>
 
 namespace hbmm {
 
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// One element, as fp32, of a tensor that the kernel before may have written.  Volatile, so that it stays behind pdl_wait (and where
+// it is written, among other such loads), and a plain load: the read-only kind (__ldg, ld.global.nc) promises memory that nobody
+// writes while this kernel lives, and its life began before the wait.
+template <typename T> __device__ __forceinline__ float load_elem(const void* p);
+template <> __device__ __forceinline__ float load_elem<float>(const void* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+template <> __device__ __forceinline__ float load_elem<__nv_bfloat16>(const void* p) {
+  unsigned short v;
+  asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+  return __uint_as_float(static_cast<uint32_t>(v) << 16);
+}
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args&&... args) {
