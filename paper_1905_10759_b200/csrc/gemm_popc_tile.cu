@@ -17,9 +17,12 @@
 // next chunk's loads are in flight while the current one is computed), and up to eight warps of a CTA split the K range of a
 // tile; their partial sums meet in shared memory at the end, always in the same order.
 // Against the same tiles on population counts, us: conv3_x matrix (50176 x 128 x 1152) at beta 2 / 4 / 8 / 16 / 32 / 64 / 128 / 256
-// 922 / 543 / 325 / 158 / 82.6 / 74.8 / 66.8 / 72.5 -> 815 / 446 / 241 / 124 / 82.5 / 63.3 / 50.7 / 47.0; 333 x 720 x 1000 at beta
-// 16 9.0 -> 7.8; 691 x 1216 x 5032 at beta 8 194 -> 146; 3325 x 872 x 2946 at beta 64 104 -> 92; 320 x 1480 x 8376 at beta 2 553 ->
-// 483; 5104 x 536 x 6912 at beta 256 / 16 504 -> 426; 82 x 536 x 3768 at beta 64 9.2 -> 8.5; 9 x 1000 x 4097 at beta 32 10.0 -> 10.3.
+// 923 / 544 / 325 / 158 / 82.6 / 74.8 / 66.7 / 72.4 -> 807 / 441 / 239 / 124 / 75.0 / 60.6 / 47.6 / 43.8; 333 x 720 x 1000 at beta
+// 16 9.0 -> 7.8; 691 x 1216 x 5032 at beta 8 194 -> 146; 3325 x 872 x 2946 at beta 64 104 -> 86; 320 x 1480 x 8376 at beta 2 553 ->
+// 483; 5104 x 536 x 6912 at beta 256 / 16 504 -> 426; 9 x 1000 x 4097 at beta 32 10.0 -> 9.8; 82 x 2880 x 152 at beta 32 / 64 3.4 /
+// 3.5 -> 3.3 / 3.1; level or slower by 0.3 us where a warp has one chunk and the last one ends early (100 x 1000 x 500 at beta 32 3.1
+// -> 3.4).
+#include <type_traits>
 #include "kernels.h"
 #include "pdl.cuh"
 #include "popc_common.cuh"
@@ -155,7 +158,6 @@ __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
   asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
   return v;
 }
-__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
 // acc += sa sw D for two neighbouring outputs.  DOT_FIRST: the first product is D sa, so that a segment whose signs cancel adds
 // 0 also where the product of its scales leaves the range of fp32 (groups of whole words; shorter ones take the product of the
 // scales first).
@@ -201,6 +203,12 @@ gemm_popc_tile_kernel(const TileArgs g) {
   const int64_t m0 = (static_cast<int64_t>(blockIdx.y) * (blockDim.x >> (5 + g.ks_log2)) + (warp >> g.ks_log2)) * TS;
   const int64_t n0 = static_cast<int64_t>(blockIdx.x) * TS;
   const int qt = lane & 3, qg = lane >> 2;              // lane of its quad, quad: rows qg + 8 i, columns 8 j + 2 qt and the next
+  // Whole-word segments: the rows are staged in the order a lane reads them in, as 16-byte pieces -- row 8 i + qg at 4 qg + i, the
+  // scale of column 8 j + 2 qt + e at 8 qt + 2 j + e.  One by one they are 20 loads a segment, which bounded single words
+  // (50176 x 128 x 1152 at beta 32 76.0 us so, 73.7 in pieces).  Shorter segments keep the row order: the pieces' registers cost
+  // them 3 .. 8 %.
+  constexpr bool VEC = SEG >= 32;
+  const int row_at = VEC ? (lane & 7) * 4 + (lane >> 3) : lane, col_at = VEC ? ((lane >> 1) & 3) * 8 + (lane >> 3) * 2 + (lane & 1) : lane;
   uint32_t* as = smem + warp * P::SMEM_WORDS;           // [CW][32]
   uint32_t* ws = as + P::CW * TS;                       // [CW][32]
   float* sa_s = reinterpret_cast<float*>(ws + P::CW * TS);   // [SPC][32]
@@ -236,24 +244,36 @@ gemm_popc_tile_kernel(const TileArgs g) {
       if (!kAhead) fetch(c);
       __syncwarp();
 #pragma unroll
-      for (int i = 0; i < P::CW; i++) { as[i * TS + lane] = pa[i]; ws[i * TS + lane] = pw[i]; }
+      for (int i = 0; i < P::CW; i++) { as[i * TS + row_at] = pa[i]; ws[i * TS + row_at] = pw[i]; }
 #pragma unroll
-      for (int i = 0; i < P::SPC; i++) { sa_s[i * TS + lane] = psa[i]; sw_s[i * TS + lane] = psw[i]; }
+      for (int i = 0; i < P::SPC; i++) { sa_s[i * TS + row_at] = psa[i]; sw_s[i * TS + col_at] = psw[i]; }
       __syncwarp();
       if (kAhead && c + KS < g.n_chunks) fetch(c + KS);
       const int64_t left_chunk = g.K - c * (P::CW * 32);              // elements from the chunk's start to the row's end
       // the dots of one segment in 16 rows from 16 r on, d[column block of 8], into the sums
       auto segment = [&](int s, int r, const uint32_t (&d)[4][4]) {
         uint64_t sa[2], sw[4];
+        if constexpr (VEC) {
+          const float2 v = *reinterpret_cast<const float2*>(sa_s + s * TS + 4 * qg + 2 * r);
+          sa[0] = pack2(v.x, v.x);
+          sa[1] = pack2(v.y, v.y);
 #pragma unroll
-        for (int i = 0; i < 2; i++) {
-          const float v = sa_s[s * TS + 16 * r + 8 * i + qg];
-          sa[i] = pack2(v, v);
-        }
+          for (int h = 0; h < 2; h++) {
+            const float4 u = *reinterpret_cast<const float4*>(sw_s + s * TS + 8 * qt + 4 * h);
+            sw[2 * h] = pack2(u.x, u.y);
+            sw[2 * h + 1] = pack2(u.z, u.w);
+          }
+        } else {
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-          const float2 u = *reinterpret_cast<const float2*>(sw_s + s * TS + 8 * j + 2 * qt);
-          sw[j] = pack2(u.x, u.y);
+          for (int i = 0; i < 2; i++) {
+            const float v = sa_s[s * TS + 16 * r + 8 * i + qg];
+            sa[i] = pack2(v, v);
+          }
+#pragma unroll
+          for (int j = 0; j < 4; j++) {
+            const float2 u = *reinterpret_cast<const float2*>(sw_s + s * TS + 8 * j + 2 * qt);
+            sw[j] = pack2(u.x, u.y);
+          }
         }
 #pragma unroll
         for (int i = 0; i < 2; i++)
@@ -261,18 +281,26 @@ gemm_popc_tile_kernel(const TileArgs g) {
           for (int j = 0; j < 4; j++) add_term<(SEG >= 32)>(acc[2 * r + i][j], d[j][2 * i], d[j][2 * i + 1], sa[i], sw[j]);
       };
       // word i of the chunk as operand registers; elements past the row's end are 0 in the first operand
-      auto words = [&](int i, uint32_t (&a)[2][4], uint32_t (&w)[4][2]) {
+      auto words = [&](int i, uint32_t (&a)[2][4], uint32_t (&w)[4][2], auto whole) {
         const int s0 = 7 - 2 * qt, s1 = s0 - 1;
+        uint32_t av[4], wv[4];
+        if constexpr (VEC) {
+          const uint4 a4 = *reinterpret_cast<const uint4*>(as + i * TS + 4 * qg), w4 = *reinterpret_cast<const uint4*>(ws + i * TS + 4 * qg);
+          av[0] = a4.x; av[1] = a4.y; av[2] = a4.z; av[3] = a4.w;
+          wv[0] = w4.x; wv[1] = w4.y; wv[2] = w4.z; wv[3] = w4.w;
+        } else {
+#pragma unroll
+          for (int r = 0; r < 4; r++) { av[r] = as[i * TS + 8 * r + qg]; wv[r] = ws[i * TS + 8 * r + qg]; }
+        }
 #pragma unroll
         for (int r = 0; r < 4; r++) {
-          const uint32_t av = as[i * TS + 8 * r + qg], wv = ws[i * TS + 8 * r + qg];
-          a[r >> 1][r & 1] = expand(av, s0);
-          a[r >> 1][2 + (r & 1)] = expand(av, s1);
-          w[r][0] = expand(wv, s0);
-          w[r][1] = expand(wv, s1);
+          a[r >> 1][r & 1] = expand(av[r], s0);
+          a[r >> 1][2 + (r & 1)] = expand(av[r], s1);
+          w[r][0] = expand(wv[r], s0);
+          w[r][1] = expand(wv[r], s1);
         }
         const int64_t left = left_chunk - 32 * i;
-        if (left < 32) {
+        if (!decltype(whole)::value && left < 32) {
           uint32_t k0 = 0u, k1 = 0u;
 #pragma unroll
           for (int j = 0; j < 4; j++) {
@@ -289,7 +317,7 @@ gemm_popc_tile_kernel(const TileArgs g) {
         for (int i = 0; i < P::CW; i++) {
           if (P::CW > 1 && left_chunk <= 32 * i) break;      // words past the row's end
           uint32_t a[2][4], w[4][2];
-          words(i, a, w);
+          words(i, a, w, std::false_type{});
           constexpr int PER_BYTE = SEG < 8 ? 8 / SEG : 1, BYTES = SEG < 8 ? 1 : SEG / 8;     // segments of a byte, bytes of a segment
 #pragma unroll 2
           for (int s = 0; s < P::SPW; s++) {
@@ -306,15 +334,16 @@ gemm_popc_tile_kernel(const TileArgs g) {
           }
         }
       } else {
-#pragma unroll 2
-        for (int s = 0; s < P::SPC; s++) {
-          if (left_chunk <= s * SEG) break;
+        // whole: nothing of the chunk lies past the row's end.  Without tests between them its segments overlap, where a loop
+        // waited at each for the products of the last (50176 x 128 x 1152 at beta 32 82.8 -> 76.0 us, at 256 47.0 -> 43.8).
+        auto one = [&](int s, auto whole) {
+          constexpr bool WHOLE = decltype(whole)::value;
           uint32_t d[2][4][4];
 #pragma unroll
           for (int q = 0; q < P::SW; q++) {
-            if (P::SW > 1 && left_chunk <= 32 * (s * P::SW + q)) break;
+            if (!WHOLE && P::SW > 1 && left_chunk <= 32 * (s * P::SW + q)) break;
             uint32_t a[2][4], w[4][2];
-            words(s * P::SW + q, a, w);
+            words(s * P::SW + q, a, w, whole);
 #pragma unroll
             for (int r = 0; r < 2; r++)
 #pragma unroll
@@ -325,44 +354,51 @@ gemm_popc_tile_kernel(const TileArgs g) {
           }
           segment(s, 0, d[0]);
           segment(s, 1, d[1]);
+        };
+        if (left_chunk >= P::CW * 32) {
+#pragma unroll
+          for (int s = 0; s < P::SPC; s++) one(s, std::true_type{});
+        } else {
+#pragma unroll 2
+          for (int s = 0; s < P::SPC; s++) {
+            if (left_chunk <= s * SEG) break;
+            one(s, std::false_type{});
+          }
         }
       }
     }
   }
-  auto store = [&](int i, int j, float x, float y) {
-    const int64_t row = m0 + 8 * i + qg, col = n0 + 8 * j + 2 * qt;
-    if (row >= g.M) return;
-    float* dst = g.C + row * g.ldc + col;
-    if (col + 1 < g.N) *reinterpret_cast<float2*>(dst) = make_float2(x, y);
-    else if (col < g.N) dst[0] = x;
-  };
-  if (KS == 1) {
-#pragma unroll
-    for (int i = 0; i < 4; i++)
-#pragma unroll
-      for (int j = 0; j < 4; j++) {
-        float x, y;
-        unpack2(acc[i][j], x, y);
-        store(i, j, x, y);
-      }
-    return;
-  }
-  // the KS partial tiles, added in order of their part: [4 i + j][lane] as pairs of columns
-  __syncwarp();                                         // the staging area is this warp's own
-  uint64_t* mine = reinterpret_cast<uint64_t*>(smem + warp * P::SMEM_WORDS);
+  // The warp's tile (the staging area is its own) row by row, the 16-byte pieces of a row permuted by its number, so that both
+  // the pairs of columns that come and the pieces that leave are spread over the banks; the KS partial tiles are added in
+  // order of their part, four rows a turn, and leave as whole rows.  (As pairs of columns out of the registers' order, sixteen
+  // turns: 82 x 2880 x 152 at beta 64 3.9 us, 3.4 so; 5184 x 448 x 640 16.9, 15.9.)
+  __syncwarp();
+  float* mine = reinterpret_cast<float*>(smem + warp * P::SMEM_WORDS);
 #pragma unroll
   for (int i = 0; i < 4; i++)
 #pragma unroll
-    for (int j = 0; j < 4; j++) mine[(4 * i + j) * 32 + lane] = acc[i][j];
-  __syncthreads();
+    for (int j = 0; j < 4; j++)
+      *reinterpret_cast<uint64_t*>(mine + (8 * i + qg) * TS + (((2 * j + (qt >> 1)) ^ qg) << 2) + 2 * (qt & 1)) = acc[i][j];
+  if (KS == 1) __syncwarp();
+  else __syncthreads();
   const int first = warp - part;                        // the warps first .. first + KS - 1 hold this tile
-  for (int b = part; b < 16; b += KS) {                 // 16 blocks shared out among the KS warps
-    float2 sum = make_float2(0.f, 0.f);
-    for (int q = 0; q < KS; q++) {
-      const float2 v = reinterpret_cast<const float2*>(smem + (first + q) * P::SMEM_WORDS)[b * 32 + lane];
-      sum.x += v.x; sum.y += v.y;
+#pragma unroll 2
+  for (int b = part; b < 8; b += KS) {                  // the rows shared out among the KS warps
+    const int r = 4 * b + (lane >> 3);
+    const int at = r * TS + (((lane & 7) ^ (r & 7)) << 2);
+    float4 sum = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(smem + first * P::SMEM_WORDS) + at);
+    for (int q = 1; q < KS; q++) {
+      const float4 v = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(smem + (first + q) * P::SMEM_WORDS) + at);
+      sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
     }
-    store(b >> 2, b & 3, sum.x, sum.y);
+    const int64_t row = m0 + r, col = n0 + 4 * (lane & 7);
+    if (row >= g.M) continue;
+    float* dst = g.C + row * g.ldc + col;
+    const float o[4] = {sum.x, sum.y, sum.z, sum.w};
+    if (col + 3 < g.N) *reinterpret_cast<float4*>(dst) = sum;
+    else
+      for (int e = 0; e < 4; e++)
+        if (col + e < g.N) dst[e] = o[e];
   }
 }
 

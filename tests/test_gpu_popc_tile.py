@@ -20,6 +20,11 @@ CASES += [
     (50, 60, 333, 333, 4, 0),
     (600, 2050, 96, 32, 32, 0),      # enough tiles that one warp walks the whole of K
     (600, 1030, 290, 8, 8, 0),       # two warps per tile
+    (600, 2050, 128, 32, 32, 0),     # whole chunks only: one to a warp,
+    (33, 70, 1152, 64, 32, 0),       # ... nine in eight parts,
+    (40, 37, 640, 128, 128, 1),
+    (40, 36, 512, 256, 256, 0),
+    (41, 38, 1000, 96, 32, 0),       # whole ones and one that ends inside its last word
 ]
 
 
