@@ -47,6 +47,12 @@ POINT_CASES = [
     (1, 512, 4, 4, 1, 0, 256, False, False),
     (2, 64, 6, 6, 1, 0, 64, True, False),     # one group per row
     (2, 10, 6, 6, 1, 0, 16, False, False),
+    (2, 3, 7, 7, 1, 1, 96, True, True),       # rows of one word and one group, stored whole
+    (2, 8, 7, 7, 1, 0, 2, True, False),       # all of eight channels, one of them, one more
+    (1, 2, 6, 7, 1, 0, 16, False, False),
+    (1, 9, 6, 7, 1, 1, 4, False, False),
+    (1, 32, 9, 15, 2, 0, 32, False, False),
+    (3, 31, 5, 5, 1, 0, 4, False, True),
 ]
 
 
