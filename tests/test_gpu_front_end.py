@@ -1,6 +1,7 @@
-"""Packed convolution front end on strided filters (tensor-copy tiles of fewer rows, whole channel planes) and on the gather
-for groups shorter than a word (bf16 images, odd widths, large filters, K ending inside a word): the packed operand left in
-the workspace against the oracle's binarization of the im2col rows."""
+"""Packed convolution front end on strided filters (tensor-copy tiles of fewer rows, whole channel planes), on the gather for
+groups shorter than a word (bf16 images, odd widths, large filters, K ending inside a word; 3 x 3 at stride 1 and 1 x 1 have
+kernels of their own) and on the staged tiles of 3 x 3 filters that are not walked: the packed operand left in the workspace
+against the oracle's binarization of the im2col rows."""
 import numpy as np
 import pytest
 import torch
@@ -22,6 +23,7 @@ CASES = [
     (2, 33, 7, 7, 5, 1, 2, False),        # K = 825
     (2, 48, 12, 12, 3, 2, 4, True),       # bf16 image
     (1, 5, 11, 10, 3, 1, 8, True),        # K = 45: two words, a short group
+    (1, 3, 11, 10, 5, 1, 8, True),        # K = 75: three words, a short group
 ]
 
 
@@ -68,17 +70,19 @@ def packed_rows(B, C, H, W, k, st, pad, beta, bf16):
 
 @pytest.mark.parametrize("first", ["bf16", "off by one element"])
 @pytest.mark.parametrize("beta", [8, 16, 32, 64])
-def test_weights_of_a_first_call_serve_the_other_front_end(beta, first):
-    """At most eight output pixels: the first call's image takes the gathering front end, the prepared calls' (plain and
-    fused) the tensor-copy one; the workspace held something else before."""
+@pytest.mark.parametrize("B,H,Wd,st", [(2, 4, 4, 1), (1, 5, 8, 2)])
+def test_weights_of_a_first_call_serve_the_other_front_end(B, H, Wd, st, beta, first):
+    """At most eight output pixels.  At stride 2 the first call's image takes the gathering front end, the prepared calls' (plain
+    and fused) the tensor-copy one; at stride 1 both are walked, from images of another type or alignment.  The workspace held
+    something else before."""
     import gpu_util as gu
     from paper_1905_10759_b200 import hbmm
-    B, C, H, N = 2, 32, 4, 40
-    K, M = C * 9, B * 4
-    x = inputs.normal((B * C * H, H), 6100 + beta).reshape(B, C, H, H)
+    C, N = 32, 40
+    K, M = C * 9, B * ((H - 3) // st + 1) * ((Wd - 3) // st + 1)
+    x = inputs.normal((B * C * H, Wd), 6100 + beta).reshape(B, C, H, Wd)
     w = inputs.he_normal(N, K, 6200 + beta)
     W = hbmm.quantize(torch.from_numpy(w).cuda(), hbmm.alloc_operand(N, K, beta))
-    geom = hbmm.make_geom(B, C, H, H, 3, 3)
+    geom = hbmm.make_geom(B, C, H, Wd, 3, 3, (st, st))
     ws = torch.full((hbmm.conv_workspace_bytes(geom, beta, hbmm.F32, W),), 0xFF, dtype=torch.uint8, device="cuda")
     xd = torch.from_numpy(x).cuda()
     if first == "bf16":
@@ -88,8 +92,8 @@ def test_weights_of_a_first_call_serve_the_other_front_end(beta, first):
     out = torch.full((M, N), float("nan"), device="cuda")
     hbmm.conv_im2col(x1, geom, beta, hbmm.F32, W, torch.empty((M, N), device="cuda"), ws)
     hbmm.conv_im2col(xd, geom, beta, hbmm.F32, W, out, ws, flags=hbmm.CONV_WEIGHTS_PREPARED)
-    c_ref, absref = oracle.conv_im2col(x, w, 3, 3, (1, 1), (0, 0), beta, beta)
-    da, dw = oracle.quantize(oracle.im2col(x, 3, 3), beta)[0], oracle.quantize(w, beta)[0]
+    c_ref, absref = oracle.conv_im2col(x, w, 3, 3, (st, st), (0, 0), beta, beta)
+    da, dw = oracle.quantize(oracle.im2col(x, 3, 3, (st, st)), beta)[0], oracle.quantize(w, beta)[0]
     fine = gu.elementwise_magnitude(da, beta, dw, beta, K)
     gu.assert_close_rel_absref(out.cpu().numpy(), c_ref, absref, 1e-5, "prepared", fine)
     if beta >= 32:
