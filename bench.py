@@ -459,7 +459,7 @@ def side_measurements(torch, hbmm, inputs, peaks, iters: int):
         out.append({"kernel": "hbmm_fold_kernel/beta_a%d_beta_w%d" % (ba, bw), "shape": [M, N, K], "ms": round(ms, 5), "bound": "tensor",
                     "achieved": ach, "peak": bf16_tflops, "unit": "TFLOP/s", "frac": ach / bf16_tflops})
         if ba != 8:
-            # the same product with no workspace: masked popcounts on the integer pipe, one multiply-add per output and group
+            # the same product with no workspace: mma.sync on bytes, one multiply-add per output and group
             msp = time_loop(torch, lambda: hbmm.gemm_ex(A, W, C, hbmm.PATH_POPC), max(3, iters // 4))
             out.append({"kernel": "gemm_popc_tile_kernel (no workspace)/beta_a%d_beta_w%d" % (ba, bw), "shape": [M, N, K], "ms": round(msp, 5),
                         "tops": 2.0 * M * N * K / (msp * 1e-3) / 1e12, "multiply_adds_per_output": K // min(ba, bw)})
@@ -569,7 +569,7 @@ def side_measurements(torch, hbmm, inputs, peaks, iters: int):
         ops = 2.0 * sh.M * sh.N * sh.K
         for label, first, again in (("hbmm_umma_kernel (e4m3 operands, per-group fp32 scale step)", hbmm.PATH_TENSOR, hbmm.PATH_TENSOR_PREPARED),
                                     ("hbmm_fold_kernel (default)", hbmm.PATH_FOLDED, hbmm.PATH_FOLDED_PREPARED),
-                                    ("gemm_popc_tile_kernel (integer pipe, no workspace)", hbmm.PATH_POPC, hbmm.PATH_POPC)):
+                                    ("gemm_popc_tile_kernel (mma.sync s8, no workspace)", hbmm.PATH_POPC, hbmm.PATH_POPC)):
             hbmm.gemm_ex(A, W, C, first, ws)
             ms = time_loop(torch, lambda: hbmm.gemm_ex(A, W, C, again, ws), iters)
             out.append({"kernel": "%s/%s" % (label, sh.name), "shape": [sh.M, sh.N, sh.K], "ms": round(ms, 5),

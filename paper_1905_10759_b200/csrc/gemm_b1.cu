@@ -3,7 +3,7 @@
 // One mma.sync.m16n8k128 adds popc(a ^ w) over 128 K-bits to a 16 x 8 tile of int32 counters, so a
 // segment must be a whole number of 128-bit chunks (beta a multiple of 128, or one group per row).
 // The signed dot of a segment is n_valid - 2 * count (Section 4.2, Eq. 7; pad bits are zero in both
-// operands and never count); the fp32 scale epilogue is the same as on the integer-pipe path.
+// operands and never count); the fp32 scale epilogue is the same as on the workspace-free path.
 // On B200 this instruction runs far below the other two paths (it is kept for comparison): the
 // kernel is a plain one, fragments are read straight from global memory through L1.
 #include <cuda_bf16.h>

@@ -1,6 +1,6 @@
-// HBMM contraction of two packed operands on the integer pipe (Section 4.2, Eq. 7): the workspace-free path, and the
-// path of every K that is no whole number of words.  A segment is the finer of the two groupings: 2, 4, 8 or 16 bits
-// of a word, or 1, 2, 4 or 8 words; per output and segment  C += (deltaA deltaW) D,  D = n_valid - 2 popc(a ^ w).
+// HBMM contraction of two packed operands by warp-level integer matrix instructions (Section 4.2, Eq. 7): the workspace-free
+// path, and the path of every K that is no whole number of words.  A segment is the finer of the two groupings: 2, 4, 8 or 16
+// bits of a word, or 1, 2, 4 or 8 words; per output and segment  C += (deltaA deltaW) D,  D the segment's dot of signs.
 //
 // The dots D of a word's segments are formed by mma.sync on bytes of +-64: exact integers, in the registers that scale them (a
 // tcgen05 accumulator would have to come out of tensor memory once per segment), and, started from the bits of 1.5 2^23, already
@@ -193,8 +193,9 @@ gemm_popc_tile_kernel(const TileArgs g) {
   pdl_wait();
   pdl_launch_dependents();      // a convolution's next front end sets itself up meanwhile
   using P = Cfg<SEG>;
-  // The next chunk waits in registers, except for the finest segments: their counts and scales need those registers
-  // (spills otherwise), and a chunk is 1000 instructions and more, which the other warps fill a load's latency with.
+  // The next chunk waits in registers, except for the finest segments, whose scales are 16 and 8 to a word and operand: at 2-bit
+  // segments they do not fit (36 and 156 bytes of spills), and a chunk is 1000 instructions and more there, which the other
+  // warps fill a load's latency with.
   constexpr bool kAhead = SEG > 4;
   __shared__ __align__(16) uint32_t smem[kWarps * P::SMEM_WORDS];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

@@ -63,7 +63,7 @@ cudaError_t launch_binarize_backward(const float* x, int64_t ldx, const float* g
 cudaError_t launch_binarize_dense(const float* x, int64_t ldx, int64_t rows, int64_t K, int32_t beta, void* out, bool out_bf16,
                                   int64_t ldo, cudaStream_t stream);
 
-// Packed x packed contraction on the integer pipe (XOR + POPC).
+// Packed x packed contraction on the integer pipe (XOR + POPC), for segments the tiles below do not take.
 cudaError_t launch_gemm_popc(const PackedView& A, const PackedView& W, float* C, int64_t ldc,
                              cudaStream_t stream);
 cudaError_t launch_partials_popc(const PackedView& A, const PackedView& W, int32_t* D,

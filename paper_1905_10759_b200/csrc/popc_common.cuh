@@ -1,4 +1,4 @@
-// Pieces shared by the integer-pipe contractions: scales of consecutive segments of a row, and the counts of all
+// Pieces shared by the workspace-free contractions: scales of consecutive segments of a row, and the counts of all
 // sub-word segments of a word at once.
 #pragma once
 #include <cstdint>

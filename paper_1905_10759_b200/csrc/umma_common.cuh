@@ -106,10 +106,9 @@ __device__ __forceinline__ void tma_load_im2col_4d(void* dst, const void* tensor
                : "memory");
 }
 
-// True in one lane of a converged warp, always the same one.  For the roles of a single thread: behind elect.sync the compiler
-// knows that one thread runs and keeps ring indices, descriptors and tensor-memory addresses in the uniform registers the
-// tensor-core and copy instructions take their operands from; behind lane == 0 each of them is moved there first, one after
-// the other, in front of every instruction (folded contraction, 200704 x 64 x 576: 55.8 -> 50.4 us; 4096^3: 335 -> 306).
+// True in one lane of a converged warp, always the same one.  For the roles of a single thread, which run faster behind it than
+// behind lane == 0 (folded contraction, 200704 x 64 x 576: 55.8 -> 50.4 us; 4096^3: 335 -> 306): supposedly because the compiler
+// knows that one thread runs, and the tensor-core and copy instructions take their operands from registers of the whole warp.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));

@@ -67,7 +67,7 @@ def test_long_tiles_match_oracle(M, N, K, ba, bw):
     c_ref, absref = oracle.hbmm_from_quantized(da[rows], sa[rows], ba, dw, sw, bw)
     fine = gu.elementwise_magnitude(da[rows], ba, dw, bw, K)
     gu.assert_close_rel_absref(C[rows, :N].cpu().numpy(), c_ref, absref, 1e-5, "long tiles", fine)
-    # all the other rows: the same product on the integer pipe, which the oracle holds to 1e-5 as well
+    # all the other rows: the same product without a workspace, which the oracle holds to 1e-5 as well
     P = torch.empty_like(C)
     hbmm.gemm_ex(A, W, P, hbmm.PATH_POPC)
     diff = (C[:, :N] - P[:, :N]).double()
@@ -99,7 +99,7 @@ def test_short_whole_tiles_match_oracle(M, N, K, ba, bw, sdt):
     c_ref, absref = oracle.hbmm_from_quantized(da[rows], sa[rows], ea, dw, sw, ew)
     fine = gu.elementwise_magnitude(da[rows], ea, dw, ew, K)
     gu.assert_close_rel_absref(C[rows, :N].cpu().numpy(), c_ref, absref, 1e-5, "short whole tiles", fine)
-    hbmm.gemm_ex(A, W, D, hbmm.PATH_POPC)      # all the other rows: on the integer pipe, which the oracle holds to 1e-5 as well
+    hbmm.gemm_ex(A, W, D, hbmm.PATH_POPC)      # all the other rows: without a workspace, which the oracle holds to 1e-5 as well
     assert float((C - D)[:, :N].double().norm() / D[:, :N].double().norm()) < 1e-5
 
 
@@ -119,7 +119,7 @@ def test_row_pitch_that_no_tensor_copy_takes():
 
 def test_tiles_walked_in_blocks_of_columns():
     """More expanded weights than the L2 keeps: every tile is still formed once (blocks of 11 columns, a last one of 10; row
-    and column remainders).  Against the integer pipe, which the oracle holds to 1e-5 elsewhere."""
+    and column remainders).  Against the workspace-free tiles, which the oracle holds to 1e-5 elsewhere."""
     from paper_1905_10759_b200 import hbmm
     M, N, K, b = 2500, 4090, 3200, 32
     gen = torch.Generator(device="cuda")

@@ -1,4 +1,4 @@
-"""The integer-pipe contraction in warp tiles (gemm_popc_tile.cu) at the sizes where it can go wrong: edges of the 32 x 32
+"""The workspace-free contraction in warp tiles (gemm_popc_tile.cu) at the sizes where it can go wrong: edges of the 32 x 32
 tile, every segment length, chunks and K ranges that end inside a word, a segment or a warp's share, one group per row,
 mixed groups, both scale types -- against the oracle."""
 import pytest
